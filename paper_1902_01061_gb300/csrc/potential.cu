@@ -18,6 +18,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "pointsum.cuh"
 
 namespace scgr {
 
@@ -189,68 +190,252 @@ __global__ void adjoint_finish_kernel(const double* __restrict__ tot, const doub
 // ---- vector-Jacobian product of the force field ---------------------------
 // f_i depends on Y_i only (X fixed, descriptors fixed), so dF/dY is block
 // diagonal with J_ii = -aY sum_j w_ij [I + (p - 1) r r^T / d^2], r = Y_i - X_j,
-// w_ij = g d^(p-1).  grad_i = J_ii v_i (J_ii is symmetric).  One thread per
-// template point; reference tiles of the force records are recomputed.
+// w_ij = g d^(p-1).  grad_i = J_ii v_i (J_ii is symmetric).
+//
+// Per point only C = sum_j c_ij r r^T with c = w / d^2 = g d^(p-3) is
+// accumulated: its trace is sum_j w (r r^T / d^2 has trace 1), so
+// J = -aY [tr(C) I + (p - 1) C].  A coincident pair has r = 0 and adds
+// nothing, as its w = 0 for p > 1 asks.  For p = 1, J = -aY (sum_j w) I with
+// w = g also for coincident pairs, so that form sums w alone (C[0]).
+//
+// Bound: the FP32 pipe.  A pair costs 18 FP32 lane operations (3 differences,
+// 3 for d^2, 2 for the exponent, 1 weight, 3 + 6 for the products and sums)
+// and two special-function results (ex2 and rsqrt for p = 2): 126 / 18 = 7
+// pairs per clock per SM, 2.2e12 pairs/s.  The layout is the force kernel's:
+// reference tiles in shared memory read as 128-bit broadcasts, two reference
+// points per packed .f32x2 instruction, P template points per thread (their
+// independent chains hide the special-function latency), the reference range
+// split over grid.y so that a small template still fills the GPU, and the
+// tile sums added across tiles with Kahan compensation.  Measured on GB300 at
+// 10,007 x 9,001, p = 2: 91 us a call (5.2 ms with one scalar thread per
+// template point, no split, and exp2f, log2f and a division per pair); the
+// error against float64 went from 2.5e-7 to 1.4e-7.
 constexpr int VJP_TPB = 128;
-constexpr int VJP_TILE = FORCE_TJ;
+constexpr int VJP_NC = 6;                 // C: xx xy xz yy yz zz
+constexpr float VJP_D2_MIN = 1e-37f;      // keeps rsqrt and lg2 of d^2 = 0 finite (the products with r are 0)
 
+__device__ __forceinline__ float vjp_ex2_neg(float x) {
+  float y;
+  asm("{ .reg .f32 t; neg.f32 t, %1; ex2.approx.ftz.f32 %0, t; }" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float vjp_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float vjp_lg2(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Reference points (j, j+1) against one template point.  PM = 1, 2, 3: p = PM;
+// 0: general p, with c = 2^(e2 log2 d^2 - ep), e2 = (p - 3) / 2 (nq = -e2).
+template <int PM>
+__device__ __forceinline__ void vjp_pair2(u64 xv, u64 yv, u64 zv, u64 av, u64 lv, u64 yx, u64 yy, u64 yz, u64 ah,
+                                          u64 nq, u64 (&C)[VJP_NC]) {
+  const u64 u = sub2(av, ah);
+  const u64 ep = fma2(u, u, lv);  // u^2 - L: the pose-free factor is 2^-ep
+  float e0, e1;
+  if (PM == 1) {
+    upk2(ep, e0, e1);
+    C[0] = add2(C[0], pk2(vjp_ex2_neg(e0), vjp_ex2_neg(e1)));
+    return;
+  }
+  const u64 rx = sub2(yx, xv), ry = sub2(yy, yv), rz = sub2(yz, zv);
+  u64 c;
+  if (PM == 3) {
+    upk2(ep, e0, e1);
+    c = pk2(vjp_ex2_neg(e0), vjp_ex2_neg(e1));
+  } else {
+    float q0, q1;
+    upk2(fma2(rz, rz, fma2(ry, ry, mul2(rx, rx))), q0, q1);
+    q0 = fmaxf(q0, VJP_D2_MIN);
+    q1 = fmaxf(q1, VJP_D2_MIN);
+    if (PM == 2) {
+      upk2(ep, e0, e1);
+      c = mul2(pk2(vjp_ex2_neg(e0), vjp_ex2_neg(e1)), pk2(vjp_rsqrt(q0), vjp_rsqrt(q1)));
+    } else {
+      upk2(fma2(nq, pk2(vjp_lg2(q0), vjp_lg2(q1)), ep), e0, e1);
+      c = pk2(vjp_ex2_neg(e0), vjp_ex2_neg(e1));
+    }
+  }
+  const u64 cx = mul2(c, rx), cy = mul2(c, ry), cz = mul2(c, rz);
+  C[0] = fma2(cx, rx, C[0]);
+  C[1] = fma2(cx, ry, C[1]);
+  C[2] = fma2(cx, rz, C[2]);
+  C[3] = fma2(cy, ry, C[3]);
+  C[4] = fma2(cy, rz, C[4]);
+  C[5] = fma2(cz, rz, C[5]);
+}
+
+// grad_i = -aY [sum_w v + (p - 1) C v] in float64.
+__device__ __forceinline__ void vjp_write(int i, const double (&C)[VJP_NC], double pm1, double ay,
+                                          const float* __restrict__ v, float* __restrict__ grad) {
+  const double W = pm1 == 0.0 ? C[0] : C[0] + C[3] + C[5];
+  const double vx = v[3 * (size_t)i], vy = v[3 * (size_t)i + 1], vz = v[3 * (size_t)i + 2];
+  double bx = 0.0, by = 0.0, bz = 0.0;
+  if (pm1 != 0.0) {
+    bx = pm1 * (C[0] * vx + C[1] * vy + C[2] * vz);
+    by = pm1 * (C[1] * vx + C[3] * vy + C[4] * vz);
+    bz = pm1 * (C[2] * vx + C[4] * vy + C[5] * vz);
+  }
+  grad[3 * (size_t)i] = (float)(-ay * (W * vx + bx));
+  grad[3 * (size_t)i + 1] = (float)(-ay * (W * vy + by));
+  grad[3 * (size_t)i + 2] = (float)(-ay * (W * vz + bz));
+}
+
+// Template points [blockIdx.x * P * VJP_TPB, ...) against the reference tiles
+// of split blockIdx.y.  One split: the gradient is written here; several: the
+// sums go to part[split][component][mpad] for vjp_combine_kernel.
+template <int P, int PM>
 __global__ void __launch_bounds__(VJP_TPB)
-    force_vjp_kernel(const float* __restrict__ Xr, const float* __restrict__ XA, int ntiles,
-                     const float4* __restrict__ Y0r, const double* __restrict__ aY64, int g_mode, int m,
+    force_vjp_kernel(const float* __restrict__ Xr, const float* __restrict__ XA, int ntiles, int tiles_per_split,
+                     const float4* __restrict__ Y0r, int mpad, const double* __restrict__ aY64, int g_mode, int m,
                      const DevPose* __restrict__ ps, double pm1, const float* __restrict__ v,
-                     float* __restrict__ grad) {
-  __shared__ float sT[6][VJP_TILE];
-  const int i = blockIdx.x * VJP_TPB + threadIdx.x;
+                     float* __restrict__ grad, float* __restrict__ part) {
+  constexpr int TJ = FORCE_TJ;
+  constexpr int Q4 = TJ / 4;
+  constexpr int NC = PM == 1 ? 1 : VJP_NC;
+  __shared__ __align__(16) float sT[5][TJ];
+  const int i0 = blockIdx.x * (P * VJP_TPB) + threadIdx.x;
   float A[9], b[3];
 #pragma unroll
   for (int q = 0; q < 9; ++q) A[q] = ps->A[q];
 #pragma unroll
   for (int q = 0; q < 3; ++q) b[q] = ps->b[q];
-  const float4 y0 = Y0r[i < m ? i : m - 1];
-  float yx, yy, yz;
-  tpoint(y0, A, b, yx, yy, yz);
-  const float ah = y0.w;
-  const float q = (float)(0.5 * pm1);           // d^(p-1) = (d^2)^q
-  double Ws = 0.0, B[6] = {0, 0, 0, 0, 0, 0};   // sum w, sum w (p-1) r r^T / d^2
-  for (int t = 0; t < ntiles; ++t) {
-    __syncthreads();
-    for (int u = threadIdx.x; u < 4 * VJP_TILE; u += VJP_TPB) (&sT[0][0])[u] = Xr[(size_t)t * 4 * VJP_TILE + u];
-    for (int u = threadIdx.x; u < 2 * VJP_TILE; u += VJP_TPB) (&sT[4][0])[u] = XA[(size_t)t * 2 * VJP_TILE + u];
-    __syncthreads();
-    float ws = 0.f, bb[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = 0; j < VJP_TILE; ++j) {
-      const float rx = yx - sT[0][j], ry = yy - sT[1][j], rz = yz - sT[2][j];
-      const float d2 = fmaf(rz, rz, fmaf(ry, ry, rx * rx));
-      const float uu = sT[4][j] - ah;
-      const float ep = fmaf(uu, uu, sT[5][j]);  // the weight is 2^-ep d^(p-1)
-      const float w = d2 > 0.f ? exp2f(fmaf(q, log2f(d2), -ep)) : (q == 0.f ? exp2f(-ep) : 0.f);
-      const float c = d2 > 0.f ? (float)pm1 * w / d2 : 0.f;
-      ws += w;
-      bb[0] = fmaf(c * rx, rx, bb[0]); bb[1] = fmaf(c * rx, ry, bb[1]); bb[2] = fmaf(c * rx, rz, bb[2]);
-      bb[3] = fmaf(c * ry, ry, bb[3]); bb[4] = fmaf(c * ry, rz, bb[4]); bb[5] = fmaf(c * rz, rz, bb[5]);
-    }
-    Ws += ws;
-    for (int u = 0; u < 6; ++u) B[u] += bb[u];
+  u64 yx[P], yy[P], yz[P], ah[P];
+#pragma unroll
+  for (int q = 0; q < P; ++q) {
+    const int i = i0 + q * VJP_TPB;
+    const float4 y0 = Y0r[i < m ? i : m - 1];
+    float x, y, z;
+    tpoint(y0, A, b, x, y, z);
+    yx[q] = pk2(x, x);
+    yy[q] = pk2(y, y);
+    yz[q] = pk2(z, z);
+    ah[q] = pk2(y0.w, y0.w);
   }
-  if (i >= m) return;
-  const double ay = g_mode == 1 ? aY64[i] : 1.0;
-  const double vx = v[3 * (size_t)i], vy = v[3 * (size_t)i + 1], vz = v[3 * (size_t)i + 2];
-  const double gx = -ay * (Ws * vx + B[0] * vx + B[1] * vy + B[2] * vz);
-  const double gy = -ay * (Ws * vy + B[1] * vx + B[3] * vy + B[4] * vz);
-  const double gz = -ay * (Ws * vz + B[2] * vx + B[4] * vy + B[5] * vz);
-  grad[3 * (size_t)i] = (float)gx;
-  grad[3 * (size_t)i + 1] = (float)gy;
-  grad[3 * (size_t)i + 2] = (float)gz;
+  const float e2 = (float)(0.5 * (pm1 - 2.0));
+  const u64 nq = pk2(-e2, -e2);
+  float h[P][NC], k[P][NC];
+#pragma unroll
+  for (int q = 0; q < P; ++q)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) h[q][c] = k[q][c] = 0.f;
+  const int t0 = blockIdx.y * tiles_per_split;
+  const int t1 = min(ntiles, t0 + tiles_per_split);
+  for (int t = t0; t < t1; ++t) {
+    __syncthreads();
+    const float4* g4 = reinterpret_cast<const float4*>(Xr + (size_t)t * 4 * TJ);  // x, y, z (and |X'|^2, not used)
+    const float4* a4 = reinterpret_cast<const float4*>(XA + (size_t)t * 2 * TJ);  // a_hat, -L
+#pragma unroll
+    for (int u = threadIdx.x; u < 5 * Q4; u += VJP_TPB)
+      *reinterpret_cast<float4*>(&sT[u / Q4][4 * (u % Q4)]) = u < 3 * Q4 ? g4[u] : a4[u - 3 * Q4];
+    __syncthreads();
+    u64 C[P][VJP_NC];
+#pragma unroll
+    for (int q = 0; q < P; ++q)
+#pragma unroll
+      for (int c = 0; c < VJP_NC; ++c) C[q][c] = 0ull;
+    constexpr int UNR = P == 1 ? 2 : 1;
+#pragma unroll UNR
+    for (int jq = 0; jq < TJ; jq += 4) {
+      const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(&sT[0][jq]);
+      const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(&sT[1][jq]);
+      const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(&sT[2][jq]);
+      const ulonglong2 Av = *reinterpret_cast<const ulonglong2*>(&sT[3][jq]);
+      const ulonglong2 Lv = *reinterpret_cast<const ulonglong2*>(&sT[4][jq]);
+#pragma unroll
+      for (int q = 0; q < P; ++q) {
+        vjp_pair2<PM>(X.x, Y.x, Z.x, Av.x, Lv.x, yx[q], yy[q], yz[q], ah[q], nq, C[q]);
+        vjp_pair2<PM>(X.y, Y.y, Z.y, Av.y, Lv.y, yx[q], yy[q], yz[q], ah[q], nq, C[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < P; ++q)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        float l0, l1;
+        upk2(C[q][c], l0, l1);
+        kahan_add(h[q][c], k[q][c], l0 + l1);
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < P; ++q) {
+    const int i = i0 + q * VJP_TPB;
+    if (i >= m) continue;
+    if (gridDim.y == 1) {
+      double C[VJP_NC];
+#pragma unroll
+      for (int c = 0; c < VJP_NC; ++c) C[c] = c < NC ? (double)h[q][c < NC ? c : 0] - (double)k[q][c < NC ? c : 0] : 0.0;
+      vjp_write(i, C, pm1, g_mode == 1 ? aY64[i] : 1.0, v, grad);
+    } else {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) part[((size_t)blockIdx.y * NC + c) * mpad + i] = h[q][c] - k[q][c];
+    }
+  }
 }
 
-cudaError_t launch_force_vjp(Launch L, const float4* Xr, const float2* XA, int ntiles, const float4* Y0r,
-                             const double* aY64, int g_mode, int m, const DevPose* ps, double p, const float* v,
-                             float* grad) {
-  if (m <= 0) return cudaSuccess;
-  force_vjp_kernel<<<(m + VJP_TPB - 1) / VJP_TPB, VJP_TPB, 0, L.stream>>>(
-      reinterpret_cast<const float*>(Xr), reinterpret_cast<const float*>(XA), ntiles, Y0r, aY64, g_mode, m, ps,
-      p - 1.0, v, grad);
+// The splits of one point added in order in float64, then its gradient.
+__global__ void __launch_bounds__(VJP_TPB)
+    vjp_combine_kernel(const float* __restrict__ part, int S, int nc, int mpad, const double* __restrict__ aY64,
+                       int g_mode, int m, double pm1, const float* __restrict__ v, float* __restrict__ grad) {
+  const int i = blockIdx.x * VJP_TPB + threadIdx.x;
+  if (i >= m) return;
+  double C[VJP_NC] = {0, 0, 0, 0, 0, 0};
+  for (int s = 0; s < S; ++s) {
+#pragma unroll
+    for (int c = 0; c < VJP_NC; ++c)
+      if (c < nc) C[c] += (double)part[((size_t)s * nc + c) * mpad + i];
+  }
+  vjp_write(i, C, pm1, g_mode == 1 ? aY64[i] : 1.0, v, grad);
+}
+
+// Splits of the reference range: enough blocks for about eight per SM (two
+// waves of the four to five that are resident), at least one tile each, and
+// at most what the scratch of `part_bytes` bytes holds (one split needs
+// none).  With few blocks even so, one template point per thread instead of
+// two.
+template <int PM>
+static void launch_vjp_pm(Launch L, const float* Xr, const float* XA, int ntiles, const float4* Y0r, int mpad,
+                          const double* aY64, int g_mode, int m, const DevPose* ps, double pm1, const float* v,
+                          float* grad, float* part, size_t part_bytes, int num_sms) {
+  constexpr int nc = PM == 1 ? 1 : VJP_NC;
+  const int64_t want = 8 * (int64_t)num_sms;
+  const int64_t cap = (int64_t)(part_bytes / ((size_t)nc * mpad * sizeof(float)));
+  const int64_t most = cap < ntiles ? (cap < 1 ? 1 : cap) : ntiles;
+  const int b2 = (m + 2 * VJP_TPB - 1) / (2 * VJP_TPB), b1 = (m + VJP_TPB - 1) / VJP_TPB;
+  const bool two = (int64_t)b2 * most >= want;
+  const int blocks = two ? b2 : b1;
+  int64_t S = (want + blocks - 1) / blocks;
+  if (S > most) S = most;
+  const int tps = (int)((ntiles + S - 1) / S);
+  const int splits = (ntiles + tps - 1) / tps;
+  const dim3 grid(blocks, splits);
+  if (two)
+    force_vjp_kernel<2, PM><<<grid, VJP_TPB, 0, L.stream>>>(Xr, XA, ntiles, tps, Y0r, mpad, aY64, g_mode, m, ps, pm1, v, grad, part);
+  else
+    force_vjp_kernel<1, PM><<<grid, VJP_TPB, 0, L.stream>>>(Xr, XA, ntiles, tps, Y0r, mpad, aY64, g_mode, m, ps, pm1, v, grad, part);
   if (L.counter) ++*L.counter;
+  if (splits > 1) {
+    vjp_combine_kernel<<<b1, VJP_TPB, 0, L.stream>>>(part, splits, nc, mpad, aY64, g_mode, m, pm1, v, grad);
+    if (L.counter) ++*L.counter;
+  }
+}
+
+cudaError_t launch_force_vjp(Launch L, const float4* Xr, const float2* XA, int ntiles, const float4* Y0r, int mpad,
+                             const double* aY64, int g_mode, int m, const DevPose* ps, double p, const float* v,
+                             float* grad, float* part, size_t part_bytes, int num_sms) {
+  if (m <= 0) return cudaSuccess;
+  const float* xr = reinterpret_cast<const float*>(Xr);
+  const float* xa = reinterpret_cast<const float*>(XA);
+  const auto launch = p == 1.0   ? launch_vjp_pm<1>
+                      : p == 2.0 ? launch_vjp_pm<2>
+                      : p == 3.0 ? launch_vjp_pm<3>
+                                 : launch_vjp_pm<0>;
+  launch(L, xr, xa, ntiles, Y0r, mpad, aY64, g_mode, m, ps, p - 1.0, v, grad, part, part_bytes, num_sms);
   return cudaGetLastError();
 }
 
