@@ -340,7 +340,8 @@ SCGR_EXPORT scgr_status scgr_step_partials_dev(scgr_ctx* ctx, double* out13_dev)
 SCGR_EXPORT scgr_status scgr_step_apply_dev(scgr_ctx* ctx, const double* parts_dev, int nparts);
 
 /* Tuning knobs (set by the autotuner; defaults are sensible). */
-#define SCGR_TUNE_BATCH_CHUNK_TILES 1 /* reference tiles (256 points) per batched work item, default 16 */
+#define SCGR_TUNE_BATCH_CHUNK_TILES 1 /* reference tiles (256 points) per batched work item, in
+                                         [1, 4096]; until set, by the batch's size (2 or 4) */
 #define SCGR_TUNE_KNN_GRID_MIN 2      /* clouds of at least this many points use the exact grid kNN in
                                          scgr_compute_descriptors (default 20000, where the two cost the
                                          same on GB300; 0: always); the result is identical */
@@ -351,12 +352,12 @@ SCGR_EXPORT scgr_status scgr_step_apply_dev(scgr_ctx* ctx, const double* parts_d
 #define SCGR_TUNE_FORCE_P 3           /* force kernel template points per thread: 0 auto, 1, 2, 4 */
 #define SCGR_TUNE_FORCE_TPB 4         /* force kernel threads per block: 0 auto, 128, 256 */
 #define SCGR_TUNE_FORCE_SPLITS 5      /* force kernel reference splits: 0 auto (wave-filling), >= 1 */
-#define SCGR_TUNE_BATCH_P 8           /* template points per thread in the batched force kernel: 1 (default)
-                                         or 2 (128 threads per block), or 4 (64 threads per block, running
+#define SCGR_TUNE_BATCH_P 8           /* template points per thread in the batched force kernel: 1 or 2 (128 threads per block), or 4 (64 threads per block, running
                                          sums in shared memory); 0 mixed: per pair, 4 points x 128 threads
                                          (512-point template blocks, running sums in shared memory) where
                                          that padding costs less than the shape gains, else 2 x 128, both
-                                         in one launch (the persistent form is not used with 0) */
+                                         in one launch (the persistent form is not used with 0).  Until set: 2 for
+                                         large batches, 1 for small ones */
 #define SCGR_TUNE_FORCE_OCC 7         /* force kernel variant: 0 registers only, 2 resident blocks per SM;
                                          1 a tighter register budget and more resident blocks per SM (3 at
                                          256 threads, 4 at 128); 2 the per-point running sums in shared

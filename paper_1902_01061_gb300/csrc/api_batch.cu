@@ -33,9 +33,24 @@ scgr_status scgr_batch_run(scgr_ctx* c, int npairs, const int64_t* ref_off, cons
   if (Ntot >= (int64_t(1) << 30) || Mtot >= (int64_t(1) << 30)) return fail(c, SCGR_ERR_INVALID_ARG, "too many points");
 
   // ---- host plan: per-pair geometry, work items (longest first), tables
-  const int CT = c->batch_chunk_tiles;
-  const bool mixed = c->batch_P == 0;  // per-pair shape: 4 x 128 (512-point blocks) or 2 x 128 (256)
-  const int FB0 = mixed ? 256 : batch_block_threads(c->batch_P) * c->batch_P;  // template points per force block
+  // Shape and chunk length where they are not set: by the batch's work in
+  // blocks of 512 template points x one reference tile.  From 4,000 on, 2
+  // points x 128 threads with 4-tile items (18,800 blocks, 40 pairs: 993 us an
+  // iteration against 1,039 us for 1 point x 128 threads with 16-tile items,
+  // the former default; 115,000 blocks, 256 pairs: 5.93 against 6.10 ms).
+  // Below, the GPU is not full and a block's own duration counts: 1 point x
+  // 128 threads with 2-tile items (721 blocks, 64 pairs: 66 us against 85 us
+  // with 16-tile items and 73 us for 2 points; 341 blocks, 6 pairs: 41, 101
+  // and 44 us).
+  double work = 0.0;
+  for (int p = 0; p < npairs; ++p)
+    work += (double)((ref_off[p + 1] - ref_off[p] + FORCE_TJ - 1) / FORCE_TJ) *
+            (double)((tmp_off[p + 1] - tmp_off[p] + 511) / 512);
+  const bool big = work >= 4000.0;
+  const int bP = c->batch_P >= 0 ? c->batch_P : big ? 2 : 1;
+  const int CT = c->batch_chunk_tiles > 0 ? c->batch_chunk_tiles : big ? 4 : 2;
+  const bool mixed = bP == 0;  // per-pair shape: 4 x 128 (512-point blocks) or 2 x 128 (256)
+  const int FB0 = mixed ? 256 : batch_block_threads(bP) * bP;  // template points per force block
   std::vector<BatchPair> pairs(npairs);
   std::vector<int4> items;
   std::vector<int> cpair;
@@ -140,10 +155,10 @@ scgr_status scgr_batch_run(scgr_ctx* c, int npairs, const int64_t* ref_off, cons
   StepParams sp = step_params(c);
   const int pmode = (c->prm.p == 1.0) ? 1 : (c->prm.p == 2.0) ? (c->ftune.rsq == 1 ? 4 : 2) : (c->prm.p == 3.0) ? 3 : 0;
   int pgrid = 0;  // persistent form: one resident block per slot (queried before any capture)
-  if (c->batch_persistent && !mixed) SCGR_CK(c, force_batch_slots(pmode, c->batch_P, &pgrid));
+  if (c->batch_persistent && !mixed) SCGR_CK(c, force_batch_slots(pmode, bP, &pgrid));
   auto enqueue = [&](Launch LL) -> scgr_status {
     for (int t = 0; t < iterations; ++t) {
-      SCGR_CK(c, launch_force_batch(LL, pmode, c->batch_P, (int)items.size(), (const int4*)c->bitems.p, dpairs,
+      SCGR_CK(c, launch_force_batch(LL, pmode, bP, (int)items.size(), (const int4*)c->bitems.p, dpairs,
                                     (const float4*)c->bXr.p, (const float2*)c->bXA.p, (const float4*)c->bY0r.p,
                                     (const DevPose*)c->bposes.p, c->qexp, (float4*)c->bpartial.p, CT, pgrid,
                                     (int*)c->bnext.p));

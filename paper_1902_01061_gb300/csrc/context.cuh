@@ -77,8 +77,8 @@ struct scgr_ctx {
   // batch workspace
   DevBuf bX4, bY4, bknnX, bknnY, baX64, baY64, baX32, baY32, bXr, bXA, bY0r, bpartial, bblockpart,
       bpairs, bitems, bcpair, btabX, btabY, bxoff, byoff, bstats, bposes, bnext;
-  int batch_chunk_tiles = 16;   // reference tiles per batched work item (tunable)
-  int batch_P = 1;              // template points per thread in the batched force kernel (tunable)
+  int batch_chunk_tiles = 0;    // reference tiles per batched work item (tunable; 0: by the batch's size)
+  int batch_P = -1;             // template points per thread in the batched force kernel (tunable; -1: by size)
   int batch_persistent = 0;     // 1: persistent batched force kernel with a work queue (tunable)
   int64_t knn_grid_min = 20000; // clouds with at least this many points use the grid kNN (tunable)
   int64_t nearest_grid_min = 65536; // references with at least this many points: grid nearest search (tunable)

@@ -457,19 +457,29 @@ ForcePlan plan_force(int64_t m, int64_t npad, double p, int num_sms, const Force
   ForcePlan fp;
   fp.pmode = (p == 1.0) ? 1 : (p == 2.0) ? (tune.rsq == 1 ? 4 : 2) : (p == 3.0) ? 3 : 0;
   fp.tile_j = FORCE_TJ;
-  // by template size: 4 points per thread in blocks of 128 with the running
-  // sums in shared memory (the fastest shape measured for large templates),
-  // then 2 and 1 points per thread in blocks of 256
-  fp.tpb = 256;
+  // By template size, from a sweep over 1,000 to 200,000 points on GB300
+  // (p = 2, force kernel, each shape with its own split lengths):
+  // * 4 points per thread in blocks of 128 with the running sums in shared
+  //   memory for large templates (the fastest shape there);
+  // * 2 points x 256 from 77,824 points (100,000 points: 3.73 ms; 2 x 128
+  //   3.76 ms, 1 x 256 3.85 ms);
+  // * 2 points x 128 from 4,096 points: more pair updates per thread than 1 x
+  //   256, and splits that fill the GPU (8,000 points 32.6 us against 42.2 us,
+  //   35,000 points 472 against 484 us, 50,000 points 954 against 980 us).  The
+  //   4-point shape would be 3-5% faster here, but its plain float32 sums run
+  //   over 512 points instead of 256, which raises the error against float64
+  //   of gradients by half;
+  // * below, 1 point x 128: the grid is short of a wave, and a thread's walk
+  //   over its tile is the launch's latency.
+  fp.tpb = 128;
   if (m >= (int64_t)num_sms * 2 * 256 * 4) {
     fp.P = 4;
-    fp.tpb = 128;
   } else if (m >= (int64_t)num_sms * 256 * 2) {
     fp.P = 2;
+    fp.tpb = 256;
   } else {
-    fp.P = 1;
+    fp.P = m >= 4096 ? 2 : 1;
   }
-  if (m < 4096) fp.tpb = 128;
   if (tune.P == 1 || tune.P == 2 || tune.P == 4) fp.P = tune.P;
   if (tune.tpb == 128 || tune.tpb == 256) fp.tpb = tune.tpb;
   const int occ = tune.occ >= 0 ? tune.occ : (fp.P == 4 && fp.tpb == 128) ? 2 : 0;

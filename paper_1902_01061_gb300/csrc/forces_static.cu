@@ -14,8 +14,8 @@
 //
 // It reuses the library's kernels unchanged (pack, statistics, sigma, force
 // records, the all-pairs force kernel and the combine); only the pointers
-// differ, and the reference range is split at most STATIC_MAX_SPLITS ways so
-// that the per-split partial sums fit.
+// differ, and the reference range is split as far as the per-split partial
+// sums fit (STATIC_MAX_SPLITS ways at the largest template).
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -119,14 +119,16 @@ extern "C" scgr_status scgr_forces_static(const float* x_dev, int64_t n, const f
   const int64_t npad = (n + 255) / 256 * 256;
   ForcePlan fp = plan_force(m, npad, p, num_sms);
   const int ntiles = (int)(npad / fp.tile_j);
-  if (fp.splits > STATIC_MAX_SPLITS) {
+  const int64_t mpad = force_mpad(m, fp);
+  if (mpad > STATIC_MPAD_MAX) return SCGR_ERR_INVALID_ARG;
+  // a small template leaves room for more splits, which it needs to fill the GPU
+  const int max_splits = (int)(STATIC_MAX_SPLITS * STATIC_MPAD_MAX / mpad);
+  if (fp.splits > max_splits) {
     fp.half = 0;
     const int sub = force_stage_tiles(fp);
-    fp.tiles_per_split = ((ntiles + STATIC_MAX_SPLITS - 1) / STATIC_MAX_SPLITS + sub - 1) / sub * sub;
+    fp.tiles_per_split = ((ntiles + max_splits - 1) / max_splits + sub - 1) / sub * sub;
     fp.splits = (ntiles + fp.tiles_per_split - 1) / fp.tiles_per_split;
   }
-  const int64_t mpad = force_mpad(m, fp);
-  if (mpad > STATIC_MPAD_MAX || fp.splits > STATIC_MAX_SPLITS) return SCGR_ERR_INVALID_ARG;
 
   Launch L{st, nullptr};
   cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), st);  // the error word must start at zero
