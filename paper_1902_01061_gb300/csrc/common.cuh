@@ -268,8 +268,9 @@ cudaError_t launch_nearest_grid(Launch L, const float4* sorted, const int* sorte
                                 const GridSpec& gs, const float* q3, int nq, int32_t* idx_out, float* key_out);
 cudaError_t launch_threshold(Launch L, const float* key, int nq, float thr2, uint8_t* mask, float* dist);
 cudaError_t launch_scale_double(Launch L, double* v, double f);
+size_t radius_scratch_bytes(int n, int num_sms);
 cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const double* e_dev, double scale2,
-                                    double* a64, float* a32, int* count_out);
+                                    const float* bb, int num_sms, double* part, double* a64, float* a32);
 cudaError_t launch_check_curvature(Launch L, const double* a64, int n, float* a32, int* err);
 cudaError_t launch_records(Launch L, const float4* X4, const double* aX64, int n, int npad,
                            const float4* Y4, const double* aY64, int m, int mpad, int g_mode,

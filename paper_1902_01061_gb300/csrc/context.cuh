@@ -85,7 +85,7 @@ struct scgr_ctx {
   ForceTuning ftune;            // force-plan overrides (tunable)
   int reuse_pose_free = 1;      // p = 1: one force pass per scgr_run (tunable)
   DevBuf gcell, gcount, gstart, gcursor, gblock, gsorted, gsidx, gbb, cd_key, cd_moved, wstore, wupart, wpartial,
-      mpart, mom;
+      mpart, mom, radpart;
   // the reference's grid for nearest-point queries, kept until the reference changes
   DevBuf rgstart, rgsorted, rgsidx, rcgstart, rcgsorted, rcgsidx;  // fine and coarse levels
   GridSpec rgspec{}, rcgspec{};

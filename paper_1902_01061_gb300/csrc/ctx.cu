@@ -260,8 +260,16 @@ scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_sca
   } else {
     c->prm.radius_scale = radius_scale;
     const double s2 = radius_scale * radius_scale;
-    SCGR_CK(c, launch_radius_curvature(L, X4, n, &st->eX, s2, (double*)c->aX64.p, (float*)c->aX32.p, nullptr));
-    SCGR_CK(c, launch_radius_curvature(L, Y4, m, &st->eY0, s2, (double*)c->aY64.p, (float*)c->aY32.p, nullptr));
+    const size_t bx = radius_scratch_bytes(n, c->num_sms), by = radius_scratch_bytes(m, c->num_sms);
+    SCGR_CK(c, ensure(c->radpart, bx > by ? bx : by));
+    SCGR_CK(c, ensure(c->gbb, sizeof(float) * (256 * 6 + 8)));
+    float* box = (float*)c->gbb.p;  // scratch, then the box
+    SCGR_CK(c, launch_bbox(L, X4, n, box, box + 256 * 6));
+    SCGR_CK(c, launch_radius_curvature(L, X4, n, &st->eX, s2, box + 256 * 6, c->num_sms, (double*)c->radpart.p,
+                                       (double*)c->aX64.p, (float*)c->aX32.p));
+    SCGR_CK(c, launch_bbox(L, Y4, m, box, box + 256 * 6));
+    SCGR_CK(c, launch_radius_curvature(L, Y4, m, &st->eY0, s2, box + 256 * 6, c->num_sms, (double*)c->radpart.p,
+                                       (double*)c->aY64.p, (float*)c->aY32.p));
   }
   const double user = c->prm.sigma > 0.0 ? c->prm.sigma * sigma_scale : 0.0;
   SCGR_CK(c, launch_sigma(L, (const double*)c->aX64.p, n, user, c->red, &st->sigma, &st->asum[0]));

@@ -309,85 +309,227 @@ cudaError_t launch_curvature(Launch L, const float4* P, const int32_t* nbr, int 
 // float32 key (dx*dx + dy*dy) + dz*dz, each operation rounded on its own,
 // is <= float32(scale^2 * e), e the largest eigenvalue of the cloud's 1/n
 // covariance (radius sqrt(e), Sec. IV).  Its 1/|N| covariance gives
-// a = lambda_min / trace.  Two passes over the cloud: the first finds the
-// neighbourhood's mean c (offsets summed in float32 per tile, float64
-// across tiles); the second accumulates the centred moments
-// sum (q - p - c) and sum (q - p - c)(q - p - c)^T in float64, so that a
-// near-planar neighbourhood keeps its small eigenvalue.
+// a = lambda_min / trace.
+//
+// One pass over the cloud sums the count, the offsets d = q - p and their
+// products, so accurately that the covariance S2/k - m m^T keeps a small
+// eigenvalue: a sum is a pair (acc, lo).  acc starts at c = 1.5 * 2^k, 2^k
+// above twice what a run of 32 points can add, so t = fma(x, y, acc) stays in
+// acc's binade, z = t - acc is exact, and so is acc's sum of the z; lo
+// collects fma(x, y, -z), the exact rest rounded once.  That is 4 float32
+// operations per sum and pair, with an error of 2^-42 of the bound on |d|^2
+// per pair; a float pair (two-sum) carries the totals from run to run.
+//
+// Bound: the FP32 pipe.  A pair costs 8 lane operations for the key, 4 for
+// the scaled offsets and the count and 36 for the nine sums: 2.6 pairs per
+// clock per SM, 8.3e11 pairs/s; a group of four points that no query of the
+// warp reaches costs only the keys.  (Before: two passes with 12 float64
+// operations per member, at 1/64 of the float32 rate.)
+//
+// Members' offsets are scaled by a power of two that brings the bound on
+// |d|^2 (the smaller of the squared radius and the box's squared diagonal)
+// near 1, so that no product overflows or underflows.
 constexpr int RAD_TPB = 128;
-constexpr int RAD_TILE = 512;
+constexpr int RAD_TILE = 256;
+constexpr int RAD_RUN = 32;
+constexpr int RAD_NS = 10;  // count, d (3), d d^T (6: xx xy xz yy yz zz)
 
-__device__ __forceinline__ bool radius_member(float4 q, float4 c, float r2, float& dx, float& dy, float& dz) {
-  dx = __fsub_rn(c.x, q.x);
-  dy = __fsub_rn(c.y, q.y);
-  dz = __fsub_rn(c.z, q.z);
-  const float key = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-  return key <= r2;
+struct RadiusScale {
+  float s;         // power of two applied to the offsets
+  float r2;        // squared radius (not scaled)
+  float c1, c2;    // acc's starting value for the offsets and for their products
+};
+__device__ __forceinline__ RadiusScale radius_scale_of(const double* e_dev, double scale2, const float* bb) {
+  const float r2 = (float)(scale2 * e_dev[0]);
+  const float dx = bb[3] - bb[0], dy = bb[4] - bb[1], dz = bb[5] - bb[2];
+  const float diag2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) * 1.0001f;
+  const float B = fmaxf(fminf(r2, diag2), 1e-36f);
+  const int h = min(60, max(-60, -(ilogbf(B) >> 1)));
+  RadiusScale o;
+  o.s = ldexpf(1.f, h);
+  o.r2 = r2;
+  const float Bs = (B * o.s) * o.s;
+  // Bs < 2^(ilogb + 1), sqrt(Bs) < 2^((ilogb >> 1) + 1): 2^(k - 1) >= the
+  // RAD_RUN / 2 = 16 terms of a lane
+  o.c2 = 1.5f * ldexpf(1.f, ilogbf(Bs) + 6);
+  o.c1 = 1.5f * ldexpf(1.f, (ilogbf(Bs) >> 1) + 6);
+  return o;
 }
 
+// (acc, lo) += x y in both lanes
+__device__ __forceinline__ void split_fma2(u64& acc, u64& lo, u64 x, u64 y) {
+  const u64 t = fma2(x, y, acc);
+  const u64 z = sub2(t, acc);
+  lo = add2(lo, fma2(x, y, sub2(0ull, z)));
+  acc = t;
+}
+__device__ __forceinline__ void split_add2(u64& acc, u64& lo, u64 x) {
+  const u64 t = add2(acc, x);
+  lo = add2(lo, sub2(x, sub2(t, acc)));
+  acc = t;
+}
+// (h, l) += x, h the rounded sum (two-sum)
+__device__ __forceinline__ void two_sum_add(float& h, float& l, float x) {
+  const float t = __fadd_rn(h, x);
+  const float bv = __fsub_rn(t, h);
+  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, bv)), __fsub_rn(x, bv)));
+  h = t;
+}
+
+__device__ __forceinline__ float member_mask(float key, float r2) {
+  float m;
+  asm("set.le.f32.f32 %0, %1, %2;" : "=f"(m) : "f"(key), "f"(r2));
+  return m;
+}
+
+// Query i's sums over the points of tiles [t0, t1) of split blockIdx.y, written
+// as doubles to part[split][sum][n] (in scaled coordinates).
 __global__ void __launch_bounds__(RAD_TPB)
-    radius_curvature_kernel(const float4* __restrict__ P, int n, const double* __restrict__ e_dev, double scale2,
-                            double* __restrict__ a64, float* __restrict__ a32, int* __restrict__ count_out) {
-  __shared__ float4 tile[RAD_TILE];
+    radius_sums_kernel(const float4* __restrict__ P, int n, const double* __restrict__ e_dev, double scale2,
+                       const float* __restrict__ bb, int tiles_per_split, double* __restrict__ part) {
+  __shared__ __align__(16) float tile[3][RAD_TILE];
   const int i = blockIdx.x * RAD_TPB + threadIdx.x;
-  const float4 q = P[i < n ? i : n - 1];
-  const float r2 = (float)(scale2 * e_dev[0]);
-  // pass 1: count and mean offset
-  double M[3] = {0, 0, 0};
-  int cnt = 0;
-  for (int base = 0; base < n; base += RAD_TILE) {
-    const int m = min(RAD_TILE, n - base);
+  const RadiusScale sc = radius_scale_of(e_dev, scale2, bb);
+  const float4 q4 = P[i < n ? i : n - 1];
+  const u64 q2x = pk2(q4.x, q4.x), q2y = pk2(q4.y, q4.y), q2z = pk2(q4.z, q4.z), s2 = pk2(sc.s, sc.s);
+  float H[RAD_NS], Lo[RAD_NS];
+#pragma unroll
+  for (int f = 0; f < RAD_NS; ++f) H[f] = Lo[f] = 0.f;
+  const int t0 = blockIdx.y * tiles_per_split * RAD_TILE;
+  const int t1 = min(n, t0 + tiles_per_split * RAD_TILE);
+  for (int base = t0; base < t1; base += RAD_TILE) {
     __syncthreads();
-    for (int t = threadIdx.x; t < m; t += RAD_TPB) tile[t] = P[base + t];
+#pragma unroll
+    for (int t = threadIdx.x; t < RAD_TILE; t += RAD_TPB) {
+      // past the end: a point at NaN, whose key is never <= r2
+      const float4 c = base + t < t1 ? P[base + t] : make_float4(NAN, NAN, NAN, 0.f);
+      tile[0][t] = c.x;
+      tile[1][t] = c.y;
+      tile[2][t] = c.z;
+    }
     __syncthreads();
-    float s[3] = {0, 0, 0};
-    for (int jj = 0; jj < m; ++jj) {
-      float dx, dy, dz;
-      if (radius_member(q, tile[jj], r2, dx, dy, dz)) {
-        ++cnt;
-        s[0] += dx; s[1] += dy; s[2] += dz;
+    u64 acc[RAD_NS], lo[RAD_NS];
+    acc[0] = 0ull;
+#pragma unroll
+    for (int f = 1; f < RAD_NS; ++f) lo[f] = 0ull;
+#pragma unroll 1
+    for (int run = 0; run < RAD_TILE; run += RAD_RUN) {
+#pragma unroll
+      for (int f = 1; f < RAD_NS; ++f) acc[f] = f < 4 ? pk2(sc.c1, sc.c1) : pk2(sc.c2, sc.c2);
+#pragma unroll 1
+      for (int j = run; j < run + RAD_RUN; j += 4) {
+        const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(&tile[0][j]);
+        const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(&tile[1][j]);
+        const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(&tile[2][j]);
+        u64 d[2][3], m[2];
+        d[0][0] = sub2(X.x, q2x); d[0][1] = sub2(Y.x, q2y); d[0][2] = sub2(Z.x, q2z);
+        d[1][0] = sub2(X.y, q2x); d[1][1] = sub2(Y.y, q2y); d[1][2] = sub2(Z.y, q2z);
+        bool any = false;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          // packed products, scalar sums: ptxas fuses a packed add with the
+          // packed product it adds, which would round the key once less
+          float x0, x1, y0, y1, z0, z1;
+          upk2(mul2(d[h][0], d[h][0]), x0, x1);
+          upk2(mul2(d[h][1], d[h][1]), y0, y1);
+          upk2(mul2(d[h][2], d[h][2]), z0, z1);
+          const float k0 = __fadd_rn(__fadd_rn(x0, y0), z0), k1 = __fadd_rn(__fadd_rn(x1, y1), z1);
+          any |= (k0 <= sc.r2) | (k1 <= sc.r2);
+          m[h] = pk2(member_mask(k0, sc.r2), member_mask(k1, sc.r2));
+        }
+        if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float m0, m1, x0, x1, y0, y1, z0, z1;
+          upk2(m[h], m0, m1);
+          upk2(d[h][0], x0, x1);
+          upk2(d[h][1], y0, y1);
+          upk2(d[h][2], z0, z1);
+          // a select before the product: a point past the end has NaN offsets
+          const u64 x = mul2(pk2(m0 != 0.f ? x0 : 0.f, m1 != 0.f ? x1 : 0.f), s2);
+          const u64 y = mul2(pk2(m0 != 0.f ? y0 : 0.f, m1 != 0.f ? y1 : 0.f), s2);
+          const u64 z = mul2(pk2(m0 != 0.f ? z0 : 0.f, m1 != 0.f ? z1 : 0.f), s2);
+          acc[0] = add2(acc[0], m[h]);
+          split_add2(acc[1], lo[1], x);
+          split_add2(acc[2], lo[2], y);
+          split_add2(acc[3], lo[3], z);
+          split_fma2(acc[4], lo[4], x, x);
+          split_fma2(acc[5], lo[5], x, y);
+          split_fma2(acc[6], lo[6], x, z);
+          split_fma2(acc[7], lo[7], y, y);
+          split_fma2(acc[8], lo[8], y, z);
+          split_fma2(acc[9], lo[9], z, z);
+        }
+      }
+#pragma unroll
+      for (int f = 1; f < RAD_NS; ++f) {
+        const float c = f < 4 ? sc.c1 : sc.c2;
+        float a0, a1;
+        upk2(acc[f], a0, a1);
+        two_sum_add(H[f], Lo[f], (a0 - c) + (a1 - c));  // exact: multiples of acc's last place
       }
     }
-    M[0] += s[0]; M[1] += s[1]; M[2] += s[2];
-  }
-  const double k = (double)cnt;
-  const double c[3] = {M[0] / k, M[1] / k, M[2] / k};
-  // pass 2: centred first and second moments in float64
-  double S[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  for (int base = 0; base < n; base += RAD_TILE) {
-    const int m = min(RAD_TILE, n - base);
-    __syncthreads();
-    for (int t = threadIdx.x; t < m; t += RAD_TPB) tile[t] = P[base + t];
-    __syncthreads();
-    for (int jj = 0; jj < m; ++jj) {
-      float dx, dy, dz;
-      if (radius_member(q, tile[jj], r2, dx, dy, dz)) {
-        const double ex = (double)dx - c[0], ey = (double)dy - c[1], ez = (double)dz - c[2];
-        S[0] += ex; S[1] += ey; S[2] += ez;
-        S[3] += ex * ex; S[4] += ex * ey; S[5] += ex * ez;
-        S[6] += ey * ey; S[7] += ey * ez; S[8] += ez * ez;
-      }
+    float b0, b1;
+    upk2(acc[0], b0, b1);
+    two_sum_add(H[0], Lo[0], b0 + b1);
+#pragma unroll
+    for (int f = 1; f < RAD_NS; ++f) {
+      upk2(lo[f], b0, b1);
+      two_sum_add(H[f], Lo[f], b0 + b1);
     }
   }
   if (i >= n) return;
-  const double mx = S[0] / k, my = S[1] / k, mz = S[2] / k;
+#pragma unroll
+  for (int f = 0; f < RAD_NS; ++f) part[((size_t)blockIdx.y * RAD_NS + f) * n + i] = (double)H[f] + (double)Lo[f];
+}
+
+// The splits' sums of a point added in order, its covariance (a power-of-two
+// scaling leaves a = lambda_min / trace unchanged) and its curvature.
+__global__ void __launch_bounds__(RAD_TPB)
+    radius_curvature_kernel(const double* __restrict__ part, int S, int n, double* __restrict__ a64,
+                            float* __restrict__ a32) {
+  const int i = blockIdx.x * RAD_TPB + threadIdx.x;
+  if (i >= n) return;
+  double v[RAD_NS];
+#pragma unroll
+  for (int f = 0; f < RAD_NS; ++f) v[f] = part[(size_t)f * n + i];
+  for (int s = 1; s < S; ++s) {
+#pragma unroll
+    for (int f = 0; f < RAD_NS; ++f) v[f] += part[((size_t)s * RAD_NS + f) * n + i];
+  }
+  const double ik = 1.0 / v[0];
+  const double mx = v[1] * ik, my = v[2] * ik, mz = v[3] * ik;
   double C[9];
-  C[0] = S[3] / k - mx * mx; C[1] = S[4] / k - mx * my; C[2] = S[5] / k - mx * mz;
-  C[4] = S[6] / k - my * my; C[5] = S[7] / k - my * mz; C[8] = S[8] / k - mz * mz;
+  C[0] = fma(v[4], ik, -mx * mx); C[1] = fma(v[5], ik, -mx * my); C[2] = fma(v[6], ik, -mx * mz);
+  C[4] = fma(v[7], ik, -my * my); C[5] = fma(v[8], ik, -my * mz); C[8] = fma(v[9], ik, -mz * mz);
   C[3] = C[1]; C[6] = C[2]; C[7] = C[5];
   const double lmin = sym3_min_eigenvalue(C);
   const double tr = C[0] + C[4] + C[8];
   const double a = tr > 0.0 ? fmax(lmin, 0.0) / tr : 0.0;
   a64[i] = a;
   a32[i] = (float)a;
-  if (count_out) count_out[i] = cnt;
 }
 
+// Splits of the cloud, so that a small one still gives every SM about eight
+// blocks (at least one tile each).
+int radius_splits(int n, int num_sms) {
+  const int blocks = (n + RAD_TPB - 1) / RAD_TPB, ntiles = (n + RAD_TILE - 1) / RAD_TILE;
+  int S = (8 * num_sms + blocks - 1) / blocks;
+  if (S > ntiles) S = ntiles;
+  const int tps = (ntiles + S - 1) / S;
+  return (ntiles + tps - 1) / tps;
+}
+size_t radius_scratch_bytes(int n, int num_sms) { return (size_t)radius_splits(n, num_sms) * RAD_NS * n * sizeof(double); }
+
+// bb: the cloud's bounding box (launch_bbox); part: radius_scratch_bytes.
 cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const double* e_dev, double scale2,
-                                    double* a64, float* a32, int* count_out) {
-  radius_curvature_kernel<<<(n + RAD_TPB - 1) / RAD_TPB, RAD_TPB, 0, L.stream>>>(P, n, e_dev, scale2, a64, a32,
-                                                                                 count_out);
-  return after_launch(L);
+                                    const float* bb, int num_sms, double* part, double* a64, float* a32) {
+  const int blocks = (n + RAD_TPB - 1) / RAD_TPB, ntiles = (n + RAD_TILE - 1) / RAD_TILE;
+  const int S = radius_splits(n, num_sms);
+  radius_sums_kernel<<<dim3(blocks, S), RAD_TPB, 0, L.stream>>>(P, n, e_dev, scale2, bb, (ntiles + S - 1) / S, part);
+  radius_curvature_kernel<<<blocks, RAD_TPB, 0, L.stream>>>(part, S, n, a64, a32);
+  if (L.counter) *L.counter += 2;
+  return cudaGetLastError();
 }
 
 // ---- fixed-order float64 reductions ------------------------------------
