@@ -128,9 +128,8 @@ SCGR_EXPORT scgr_status scgr_set_template_host(scgr_ctx* ctx, const float* xyz_h
 
 /* One-time descriptor pass (Sec. III-A, Sec. IV): k-nearest neighbours of
  * every point of X and of Y0 (exact float32 key (dx*dx+dy*dy)+dz*dz, no fused
- * multiply-add, self included, ties to the lower index; brute force for
- * small clouds, an exact uniform-grid search for large ones, which waits once
- * for the bounding box), the curvature
+ * multiply-add, self included, ties to the lower index; an exact
+ * uniform-grid search), the curvature
  * a = lambda_min / (lambda_1+lambda_2+lambda_3) of each neighbourhood's
  * covariance (float64), sigma, and the cloud statistics used by the scale
  * model (means, covariances, largest eigenvalues).  Resets the pose to
@@ -187,10 +186,9 @@ SCGR_EXPORT scgr_status scgr_set_neighbourhood(scgr_ctx* ctx, int k, double radi
 /* Nearest reference point of q_dev [nq][3] (float32): index int32 [nq] and
  * float32 key (squared distance, the kNN key of R1) [nq]; either output may
  * be NULL.  Ties go to the lower index.  References of at least
- * SCGR_TUNE_KNN_GRID_MIN points are searched through an exact uniform grid
+ * SCGR_TUNE_NEAREST_GRID_MIN points are searched through an exact uniform grid
  * (same result as brute force; queries may lie outside the reference's box),
- * which synchronises the stream once for the bounding box; smaller ones by
- * brute force, enqueued.  STATE without a reference. */
+ * smaller ones by brute force.  Enqueued.  STATE without a reference. */
 SCGR_EXPORT scgr_status scgr_nearest(scgr_ctx* ctx, const float* q_dev, int64_t nq, int32_t* idx_dev,
                                      float* key_dev);
 
@@ -343,12 +341,12 @@ SCGR_EXPORT scgr_status scgr_step_apply_dev(scgr_ctx* ctx, const double* parts_d
 #define SCGR_TUNE_BATCH_CHUNK_TILES 1 /* reference tiles (256 points) per batched work item, in
                                          [1, 4096]; until set, by the batch's size (2 or 4) */
 #define SCGR_TUNE_KNN_GRID_MIN 2      /* clouds of at least this many points use the exact grid kNN in
-                                         scgr_compute_descriptors (default 20000, where the two cost the
-                                         same on GB300; 0: always); the result is identical */
+                                         scgr_compute_descriptors, smaller ones brute force (0: always the
+                                         grid).  Until set, the grid serves every cloud; below 20000 points
+                                         it then keys candidates with the brute-force search's rounding */
 #define SCGR_TUNE_NEAREST_GRID_MIN 14 /* references of at least this many points answer scgr_nearest and
-                                         scgr_change_mask through the exact grid search (default 65536:
-                                         below it the brute force is faster, also for queries far off
-                                         the surface; 0: always); the result is identical */
+                                         scgr_change_mask through the exact grid search (default 1024;
+                                         0: always); the result is identical */
 #define SCGR_TUNE_FORCE_P 3           /* force kernel template points per thread: 0 auto, 1, 2, 4 */
 #define SCGR_TUNE_FORCE_TPB 4         /* force kernel threads per block: 0 auto, 128, 256 */
 #define SCGR_TUNE_FORCE_SPLITS 5      /* force kernel reference splits: 0 auto (wave-filling), >= 1 */

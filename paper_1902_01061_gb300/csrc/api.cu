@@ -93,8 +93,8 @@ void scgr_destroy(scgr_ctx* c) {
                     &c->bX4, &c->bY4, &c->bknnX, &c->bknnY, &c->baX64, &c->baY64, &c->baX32, &c->baY32,
                     &c->bXr, &c->bXA, &c->bY0r, &c->bpartial, &c->bblockpart, &c->bpairs, &c->bitems,
                     &c->bcpair, &c->btabX, &c->btabY, &c->bxoff, &c->byoff, &c->bstats, &c->bposes, &c->bnext,
-                    &c->gcell, &c->gcount, &c->gstart, &c->gcursor, &c->gblock, &c->gsorted, &c->gsidx, &c->gbb,
-                    &c->rgstart, &c->rgsorted, &c->rgsidx, &c->rcgstart, &c->rcgsorted, &c->rcgsidx,
+                    &c->gspec, &c->gcell[0], &c->gcell[1], &c->gstart[0], &c->gstart[1], &c->gtot[0], &c->gtot[1],
+                    &c->gsorted[0], &c->gsorted[1], &c->gccount,
                     &c->cd_key, &c->cd_moved, &c->wstore, &c->wupart, &c->wpartial, &c->mpart, &c->mom, &c->radpart};
   for (DevBuf* b : bufs) release(*b);
   if (c->pose) cudaFree(c->pose);
@@ -142,8 +142,8 @@ scgr_status scgr_compute_descriptors(scgr_ctx* c) {
   const float4* X4 = (const float4*)c->X4.p;
   const float4* Y4 = (const float4*)c->Y4.p;
   DevStats* st = c->stats;
-  SCGR_CK(c, launch_cloud_stats(L, X4, n, c->red, st->xbar, st->CX, &st->eX));
-  SCGR_CK(c, launch_cloud_stats(L, Y4, m, c->red, st->ybar0, st->S0, &st->eY0));
+  const scgr_status ps = prepare_clouds(c);
+  if (ps != SCGR_OK) return ps;
   scgr_status cs = curvatures(c, c->prm.k, c->prm.radius_scale, 1.0);
   if (cs != SCGR_OK) return cs;
   c->npad = (c->n + 255) / 256 * 256;
@@ -326,7 +326,7 @@ scgr_status scgr_set_curvature(scgr_ctx* c, int which, const double* a64_dev) {
   SCGR_CK(c, cudaMemcpyAsync(a64.p, a64_dev, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
   SCGR_CK(c, launch_check_curvature(L, (const double*)a64.p, n, (float*)a32.p, c->errword));
   DevStats* st = c->stats;
-  SCGR_CK(c, launch_sigma(L, (const double*)c->aX64.p, (int)c->n, c->prm.sigma, c->red, &st->sigma, &st->asum[0]));
+  SCGR_CK(c, launch_sigma(L, (const double*)c->aX64.p, (int)c->n, c->prm.sigma, 1.0, c->red, st));
   SCGR_CK(c, launch_records(L, (const float4*)c->X4.p, (const double*)c->aX64.p, (int)c->n, (int)c->npad,
                             (const float4*)c->Y4.p, (const double*)c->aY64.p, (int)c->m, (int)c->mpad,
                             c->prm.g_mode, st, (float4*)c->Xr.p, (float2*)c->XA.p, (float4*)c->Y0r.p));

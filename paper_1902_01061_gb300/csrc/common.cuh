@@ -57,6 +57,7 @@ struct DevStats {
   double S0[9];    // scatter sum_i (Y0_i - ybar0)^T (Y0_i - ybar0), unnormalised
   double eY0;      // largest eigenvalue of S0 / M
   double sigma;
+  double kscale;   // sqrt(log2 e) / sigma, kept with sigma
   double asum[2];  // sum of curvatures of X, Y0 (diagnostic)
 };
 
@@ -202,6 +203,56 @@ __host__ __device__ inline double sym3_min_eigenvalue(const double* C) {
   return lam[0];
 }
 
+#ifdef __CUDACC__
+// Smallest (or largest) eigenvalue of a symmetric positive semi-definite 3x3
+// C with little float64 work (each such instruction costs a warp about 64
+// cycles on GB300): the characteristic polynomial's coefficients in float64,
+// its extreme root by Newton's method in float32 (monotone from 0, or from the
+// trace, as in sym3_min_eigenvalue), then two float64 steps with the float32
+// derivative, each of which reduces the error by about 1e-6.  The float64
+// solvers take over where the root is nearly multiple, where the steps do not
+// settle, and outside float64's comfortable range.
+__device__ inline double sym3_extreme_eigenvalue(const double* C, bool largest) {
+  const double tr = C[0] + C[4] + C[8];
+  const int e = (__double2hiint(tr) >> 20) & 0x7ff;
+  double lam[3];
+  if (tr > 0.0 && e > 600 && e < 1400) {
+    // scaled by a power of two to a trace in [1, 2)
+    const double sc = __hiloint2double((2046 - e) << 20, 0);
+    const double c00 = C[0] * sc, c11 = C[4] * sc, c22 = C[8] * sc, c01 = C[1] * sc, c02 = C[2] * sc, c12 = C[5] * sc;
+    const double m00 = fma(c11, c22, -c12 * c12), m11 = fma(c00, c22, -c02 * c02), m22 = fma(c00, c11, -c01 * c01);
+    const double p2 = tr * sc, p1 = m00 + m11 + m22;
+    const double p0 = fma(c02, fma(c01, c12, -c11 * c02), fma(c00, m00, -c01 * fma(c01, c22, -c12 * c02)));
+    if (!largest && (!(p0 > 0.0) || !(p1 > 0.0))) return 0.0;
+    const float f0 = (float)p0, f1 = (float)p1, f2 = (float)p2;
+    float l = largest ? f2 : 0.f, df = 0.f;
+    bool ok = false;
+    for (int it = 0; it < 24 && !ok; ++it) {
+      const float f = fmaf(l, fmaf(l, f2 - l, -f1), f0);
+      df = fmaf(l, fmaf(-3.f, l, 2.f * f2), -f1);
+      const float step = __fdividef(-f, df);
+      l += step;
+      ok = fabsf(step) <= 2e-6f * l;
+    }
+    df = fmaf(l, fmaf(-3.f, l, 2.f * f2), -f1);
+    // a well separated root: its polynomial determines it to rounding
+    ok = ok && df < 0.f && (largest ? -df >= 1e-2f * f2 * f2 : -df * l >= 1e-2f * f0);
+    if (ok) {
+      const double r = -(double)__frcp_rn(df);
+      double x = (double)l;
+      x = fma(fma(x, fma(x, p2 - x, -p1), p0), r, x);
+      const double step = fma(x, fma(x, p2 - x, -p1), p0) * r;
+      x += step;
+      if (fabs(step) <= 1e-9 * x) return x * __hiloint2double(e << 20, 0);
+    }
+  }
+  if (!largest) return sym3_min_eigenvalue(C);
+  sym3_eigenvalues(C, lam);
+  return lam[2];
+}
+__device__ __forceinline__ double sym3_max_eigenvalue(const double* C) { return sym3_extreme_eigenvalue(C, true); }
+#endif
+
 // One registration pair of a batch: where its points, padded records,
 // partial sums and combine blocks live in the concatenated buffers.
 struct BatchPair {
@@ -218,11 +269,35 @@ struct BatchPair {
                      // (512-point blocks, running sums in shared memory), 0 for 2 points x 128 threads
 };
 
-// Uniform grid of the exact grid kNN: origin, cell edge, cells per axis.
+// Uniform grid of the exact grid searches (on the device): origin, cell edge,
+// cells per axis and in all, the cloud's largest extent.
 struct GridSpec {
-  double o[3];
-  double h, inv_h;
+  float o[3];
+  float h, inv_h, extent;
   int g[3];
+  int ncell;
+};
+constexpr int GRID_CELLS_PER_POINT = 4;  // at most this many cells per point
+constexpr int SCAN_B = 4096;             // cells per block of the count scan
+constexpr int CLOUD_PARTS = 256;         // blocks of a cloud's reductions, at most
+
+// One cloud of the descriptor pass: its points, grid arrays and outputs.
+struct GridCloud {
+  const float4* P;
+  int n;
+  GridSpec* spec;
+  int2* cell;       // [n] cell, rank of arrival in it
+  int* start;       // [grid_start_entries(n)] counts, then block-local first positions; NULL: no grid wanted
+  int* tot;         // [grid_tot_entries(n)] first position of each block of SCAN_B cells
+  float4* sorted;   // [n] points in cell order, index in w
+  int32_t* knn;     // [n][k]
+  double *mean, *scatter, *lmax;  // outputs (NULL: not wanted)
+};
+// The clouds of a launch: two of a registration, or an array of many on the device.
+struct CloudSet {
+  GridCloud one[2];
+  const GridCloud* many;
+  __device__ __forceinline__ const GridCloud& operator[](int y) const { return many ? many[y] : one[y]; }
 };
 
 // ---- launchers (defined in the .cu files) --------------------------------
@@ -235,12 +310,11 @@ cudaError_t launch_pack(Launch L, const float* xyz, int64_t n, float4* out, int*
 cudaError_t launch_knn(Launch L, const float4* P, int n, int k, int32_t* out);
 cudaError_t launch_curvature(Launch L, const float4* P, const int32_t* nbr, int n, int k,
                              double* a64, float* a32);
-// mean + scatter of a cloud: writes mean[3], scatter[9], lmax of scatter/n
-cudaError_t launch_cloud_stats(Launch L, const float4* P, int n, double* part, double* mean,
-                               double* scatter, double* lmax);
+cudaError_t launch_curvature2(Launch L, const float4* X, const int32_t* nx, int n, double* ax64, float* ax32,
+                              const float4* Y, const int32_t* ny, int m, double* ay64, float* ay32, int k);
 // sigma = population std of a64 (1 if below 1e-12), or `sigma_user` if > 0
-cudaError_t launch_sigma(Launch L, const double* a64, int n, double sigma_user, double* part,
-                         double* sigma_out, double* asum_out);
+cudaError_t launch_sigma(Launch L, const double* a64, int n, double sigma_user, double sigma_scale, double* part,
+                         DevStats* st);
 cudaError_t launch_knn_multi(Launch L, const float4* P, const int64_t* off_dev, const int2* table_dev,
                              int nblocks, int k, int32_t* out);
 cudaError_t launch_records_multi(Launch L, const float4* X4, const double* aX64, const float4* Y4,
@@ -248,29 +322,22 @@ cudaError_t launch_records_multi(Launch L, const float4* X4, const double* aX64,
                                  const DevStats* stats, float4* Xr, float2* XA, float4* Y0r);
 cudaError_t launch_stats_multi(Launch L, const float4* X4, const float4* Y4, const double* aX64,
                                const BatchPair* pairs, int npairs, double sigma_user, DevStats* out);
-GridSpec make_grid_spec(const float* bbox6, int64_t n);
-int64_t grid_cells(const GridSpec& gs);
-cudaError_t launch_bbox(Launch L, const float4* P, int n, float* part, float* out6);
-cudaError_t launch_knn_grid(Launch L, const float4* P, int n, int k, const GridSpec& gs, int* cell_of, int* count,
-                            int* start, int* cursor, int* block_tot, float4* sorted, int* sorted_idx,
-                            int32_t* out);
+size_t grid_start_entries(int64_t n);
+size_t grid_tot_entries(int64_t n);
+cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, bool scatter, double* part,
+                          float* bpart);
+cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most);
+cudaError_t launch_knn_grid(Launch L, const CloudSet& cs, int nclouds, int most, int k, bool fused);
+constexpr int NEAREST_COARSE = 4;  // fine cells per coarse cell side in the two-level nearest search
+cudaError_t launch_coarse_count(Launch L, const CloudSet& cs, int64_t n, int* ccount);
+cudaError_t launch_nearest_grid(Launch L, const CloudSet& cs, int levels, const int* ccount, const float* q3, int nq,
+                                int32_t* idx_out, float* key_out);
 cudaError_t launch_nearest(Launch L, const float4* P, int n, const float* q3, int nq, int32_t* idx_out,
                            float* key_out);
-cudaError_t launch_grid_build(Launch L, const float4* P, int n, const GridSpec& gs, int* cell_of, int* count,
-                              int* start, int* cursor, int* block_tot, float4* sorted, int* sorted_idx);
-constexpr int NEAREST_COARSE = 4;  // fine cells per coarse cell side in the two-level nearest search
-GridSpec coarse_grid_spec(const GridSpec& gs);
-cudaError_t launch_nearest_grid2(Launch L, const float4* sorted, const int* sorted_idx, const int* start,
-                                 const GridSpec& gs, const float4* csorted, const int* csorted_idx,
-                                 const int* cstart, const GridSpec& gc, const float* q3, int nq, int32_t* idx_out,
-                                 float* key_out);
-cudaError_t launch_nearest_grid(Launch L, const float4* sorted, const int* sorted_idx, const int* start,
-                                const GridSpec& gs, const float* q3, int nq, int32_t* idx_out, float* key_out);
 cudaError_t launch_threshold(Launch L, const float* key, int nq, float thr2, uint8_t* mask, float* dist);
-cudaError_t launch_scale_double(Launch L, double* v, double f);
 size_t radius_scratch_bytes(int n, int num_sms);
 cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const double* e_dev, double scale2,
-                                    const float* bb, int num_sms, double* part, double* a64, float* a32);
+                                    const GridSpec* spec, int num_sms, double* part, double* a64, float* a32);
 cudaError_t launch_check_curvature(Launch L, const double* a64, int n, float* a32, int* err);
 cudaError_t launch_records(Launch L, const float4* X4, const double* aX64, int n, int npad,
                            const float4* Y4, const double* aY64, int m, int mpad, int g_mode,

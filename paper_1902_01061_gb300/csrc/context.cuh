@@ -41,6 +41,8 @@ using scgr::ForcePlan;
 using scgr::ForceTuning;
 using scgr::Launch;
 using scgr::GridSpec;
+using scgr::GridCloud;
+using scgr::CloudSet;
 
 struct scgr_ctx {
   scgr_params prm{};
@@ -80,16 +82,15 @@ struct scgr_ctx {
   int batch_chunk_tiles = 0;    // reference tiles per batched work item (tunable; 0: by the batch's size)
   int batch_P = -1;             // template points per thread in the batched force kernel (tunable; -1: by size)
   int batch_persistent = 0;     // 1: persistent batched force kernel with a work queue (tunable)
-  int64_t knn_grid_min = 20000; // clouds with at least this many points use the grid kNN (tunable)
-  int64_t nearest_grid_min = 65536; // references with at least this many points: grid nearest search (tunable)
+  int64_t knn_grid_min = -1;    // clouds with at least this many points use the grid kNN (tunable; -1: all)
+  int64_t nearest_grid_min = 1024; // references with at least this many points: grid nearest search (tunable)
   ForceTuning ftune;            // force-plan overrides (tunable)
   int reuse_pose_free = 1;      // p = 1: one force pass per scgr_run (tunable)
-  DevBuf gcell, gcount, gstart, gcursor, gblock, gsorted, gsidx, gbb, cd_key, cd_moved, wstore, wupart, wpartial,
-      mpart, mom, radpart;
-  // the reference's grid for nearest-point queries, kept until the reference changes
-  DevBuf rgstart, rgsorted, rgsidx, rcgstart, rcgsorted, rcgsidx;  // fine and coarse levels
-  GridSpec rgspec{}, rcgspec{};
-  bool rgrid_ok = false;
+  DevBuf cd_key, cd_moved, wstore, wupart, wpartial, mpart, mom, radpart;
+  // grids of the reference [0] and the template [1], kept until the cloud changes
+  DevBuf gspec, gcell[2], gstart[2], gtot[2], gsorted[2], gccount;
+  bool grid_ok[2] = {false, false};  // sorted into grid cells
+  bool coarse_ok = false;            // the reference's coarse cell counts (gccount)
   int nearest_levels = 2;       // 2: two-level nearest search (default), 1: fine shells only (tunable)
   int fused_tail = 1;           // 1: one combine-finalize launch for small templates (tunable)
   cudaGraph_t bgraph = nullptr;
@@ -127,7 +128,10 @@ scgr_status read_error_word(scgr_ctx* c);
 scgr_status set_cloud(scgr_ctx* c, const float* xyz, int64_t n, bool host, bool ref);
 scgr_status force_launch(scgr_ctx* c);
 scgr_status collect_timing(scgr_ctx* c);
-scgr_status knn_cloud(scgr_ctx* c, const float4* P, int n, int32_t* out);
+// Clouds below this many points were searched by brute force, whose packed
+// key rounds once less; the grid search keeps their neighbours the same.
+constexpr int64_t KNN_FUSED_KEY = 20000;
+scgr_status prepare_clouds(scgr_ctx* c);
 scgr_status nearest_reference(scgr_ctx* c, const float* q3, int nq, int32_t* idx_out, float* key_out);
 scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_scale);
 scgr_status replan(scgr_ctx* c);

@@ -108,8 +108,8 @@ scgr_status set_cloud(scgr_ctx* c, const float* xyz, int64_t n, bool host, bool 
     src = (const float*)c->stage.p;
   }
   SCGR_CK(c, launch_pack(c->L(), src, n, (float4*)dst.p, c->errword));
-  if (ref) { c->n = n; c->have_X = true; c->rgrid_ok = false; }
-  else { c->m = n; c->have_Y = true; }
+  if (ref) { c->n = n; c->have_X = true; c->grid_ok[0] = c->coarse_ok = false; }
+  else { c->m = n; c->have_Y = true; c->grid_ok[1] = false; }
   c->have_desc = false;
   return SCGR_OK;
 }
@@ -149,90 +149,140 @@ scgr_status collect_timing(scgr_ctx* c) {
   return SCGR_OK;
 }
 
-// Grid spec of a cloud and the workspace of its grid (one host
-// synchronisation for the bounding box).
-static scgr_status grid_setup(scgr_ctx* c, const float4* P, int n, GridSpec* gs_out) {
-  SCGR_CK(c, ensure(c->gbb, sizeof(float) * (256 * 6 + 8)));
-  float* part = (float*)c->gbb.p;
-  SCGR_CK(c, launch_bbox(c->L(), P, n, part, part + 256 * 6));
-  float bb[6];
-  SCGR_CK(c, cudaMemcpyAsync(bb, part + 256 * 6, sizeof(bb), cudaMemcpyDeviceToHost, c->stream));
-  SCGR_CK(c, cudaStreamSynchronize(c->stream));
-  const GridSpec gs = make_grid_spec(bb, n);
-  const int64_t ncell = grid_cells(gs);
-  SCGR_CK(c, ensure(c->gcell, (size_t)n * sizeof(int)));
-  SCGR_CK(c, ensure(c->gcount, (size_t)ncell * sizeof(int)));
-  SCGR_CK(c, ensure(c->gcursor, (size_t)ncell * sizeof(int)));
-  SCGR_CK(c, ensure(c->gstart, (size_t)(ncell + 1) * sizeof(int)));
-  SCGR_CK(c, ensure(c->gblock, (size_t)((ncell + 1023) / 1024 + 1) * sizeof(int)));
-  SCGR_CK(c, ensure(c->gsorted, (size_t)n * sizeof(float4)));
-  SCGR_CK(c, ensure(c->gsidx, (size_t)n * sizeof(int)));
-  *gs_out = gs;
+// The clouds' descriptions for the grid kernels: which = 0 the reference, 1
+// the template; first = 1 puts the template alone at index 0.
+static GridCloud grid_cloud(scgr_ctx* c, int which, bool grid, bool stats) {
+  GridCloud g{};
+  g.P = (const float4*)(which == 0 ? c->X4.p : c->Y4.p);
+  g.n = (int)(which == 0 ? c->n : c->m);
+  g.spec = (GridSpec*)c->gspec.p + which;
+  if (grid) {
+    g.cell = (int2*)c->gcell[which].p;
+    g.start = (int*)c->gstart[which].p;
+    g.tot = (int*)c->gtot[which].p;
+    g.sorted = (float4*)c->gsorted[which].p;
+  }
+  g.knn = (int32_t*)(which == 0 ? c->knnX.p : c->knnY.p);
+  DevStats* st = c->stats;
+  g.mean = which == 0 ? st->xbar : st->ybar0;
+  if (stats) {
+    g.scatter = which == 0 ? st->CX : st->S0;
+    g.lmax = which == 0 ? &st->eX : &st->eY0;
+  } else {
+    g.mean = nullptr;
+  }
+  return g;
+}
+
+static scgr_status grid_buffers(scgr_ctx* c, int which) {
+  const int64_t n = which == 0 ? c->n : c->m;
+  SCGR_CK(c, ensure(c->gcell[which], (size_t)n * sizeof(int2)));
+  SCGR_CK(c, ensure(c->gstart[which], grid_start_entries(n) * sizeof(int)));
+  SCGR_CK(c, ensure(c->gtot[which], grid_tot_entries(n) * sizeof(int)));
+  SCGR_CK(c, ensure(c->gsorted[which], (size_t)n * sizeof(float4)));
   return SCGR_OK;
 }
 
-// k nearest neighbours of one cloud: brute force below knn_grid_min points,
-// the exact grid search above.
-scgr_status knn_cloud(scgr_ctx* c, const float4* P, int n, int32_t* out) {
+// Whether cloud `which` takes the grid search for its neighbours: always,
+// unless SCGR_TUNE_KNN_GRID_MIN has been set above its size.
+static bool grid_knn(const scgr_ctx* c, int which) {
+  return c->prm.neigh_mode == 0 && (which == 0 ? c->n : c->m) >= (c->knn_grid_min < 0 ? 0 : c->knn_grid_min);
+}
+
+// The descriptor pass's first part: means, scatter matrices and largest
+// eigenvalues of both clouds, their boxes, and the points sorted into grid
+// cells where the neighbour search wants that.  Both clouds share each
+// launch; nothing waits for the host.
+scgr_status prepare_clouds(scgr_ctx* c) {
+  c->grid_ok[0] = c->grid_ok[1] = false;
+  SCGR_CK(c, ensure(c->gspec, 2 * sizeof(GridSpec)));
+  CloudSet cs{};
+  for (int w = 0; w < 2; ++w) {
+    if (grid_knn(c, w)) {
+      const scgr_status st = grid_buffers(c, w);
+      if (st != SCGR_OK) return st;
+    }
+    cs.one[w] = grid_cloud(c, w, grid_knn(c, w), true);
+  }
+  const int most = (int)(c->n > c->m ? c->n : c->m);
+  double* part = c->red;
+  SCGR_CK(c, launch_clouds(c->L(), cs, 2, most, true, part, (float*)(part + 2 * CLOUD_PARTS * 6)));
+  if (grid_knn(c, 0) && grid_knn(c, 1)) {
+    SCGR_CK(c, launch_grid_sort(c->L(), cs, 2, most));
+  } else if (grid_knn(c, 0) || grid_knn(c, 1)) {
+    const int w = grid_knn(c, 0) ? 0 : 1;
+    cs.one[0] = cs.one[w];
+    SCGR_CK(c, launch_grid_sort(c->L(), cs, 1, cs.one[0].n));
+  }
+  for (int w = 0; w < 2; ++w) c->grid_ok[w] = grid_knn(c, w);
+  c->coarse_ok = false;
+  return SCGR_OK;
+}
+
+// k nearest neighbours of both clouds (after prepare_clouds): the grid search
+// where the cloud was sorted, else brute force.  Clouds of fewer than
+// KNN_FUSED_KEY points keep the key rounding of the brute-force search, which
+// served them before (grid_key).
+static scgr_status knn_clouds(scgr_ctx* c) {
   const int k = c->prm.k;
-  if ((int64_t)n < c->knn_grid_min) {
-    SCGR_CK(c, launch_knn(c->L(), P, n, k, out));
+  bool fused[2];
+  for (int w = 0; w < 2; ++w) fused[w] = c->knn_grid_min < 0 && (w == 0 ? c->n : c->m) < KNN_FUSED_KEY;
+  CloudSet cs{};
+  for (int w = 0; w < 2; ++w) cs.one[w] = grid_cloud(c, w, c->grid_ok[w], false);
+  if (c->grid_ok[0] && c->grid_ok[1] && fused[0] == fused[1]) {
+    SCGR_CK(c, launch_knn_grid(c->L(), cs, 2, (int)(c->n > c->m ? c->n : c->m), k, fused[0]));
     return SCGR_OK;
   }
-  GridSpec gs;
-  const scgr_status st = grid_setup(c, P, n, &gs);
-  if (st != SCGR_OK) return st;
-  SCGR_CK(c, launch_knn_grid(c->L(), P, n, k, gs, (int*)c->gcell.p, (int*)c->gcount.p, (int*)c->gstart.p,
-                             (int*)c->gcursor.p, (int*)c->gblock.p, (float4*)c->gsorted.p, (int*)c->gsidx.p, out));
+  for (int w = 0; w < 2; ++w) {
+    CloudSet one{};
+    one.one[0] = cs.one[w];
+    if (c->grid_ok[w]) {
+      SCGR_CK(c, launch_knn_grid(c->L(), one, 1, one.one[0].n, k, fused[w]));
+    } else {
+      SCGR_CK(c, launch_knn(c->L(), one.one[0].P, one.one[0].n, k, one.one[0].knn));
+    }
+  }
   return SCGR_OK;
 }
 
 // Nearest reference point of nq external queries (float32 [nq][3] on the
 // device): brute force below nearest_grid_min reference points, else the exact
 // two-level grid search over the reference (the same result): fine cells
-// around the query, then coarse cells that skip empty space.  The
-// reference's two grids are built on the first query after
-// scgr_set_reference and kept in their own buffers (the descriptor pass
-// reuses the shared grid workspace for both clouds), so later queries skip
-// the bounding-box synchronisation and the counting sorts.
+// around the query, then coarse cells that skip empty space.  The reference's
+// grid is the descriptor pass's, or built here on the first query, and kept
+// until the reference changes.  While the stream is being captured a grid
+// that is not there yet is not built (no allocation): brute force.
 scgr_status nearest_reference(scgr_ctx* c, const float* q3, int nq, int32_t* idx_out, float* key_out) {
   const float4* X4 = (const float4*)c->X4.p;
   const int n = (int)c->n;
-  if ((int64_t)n < c->nearest_grid_min) {
+  bool grid = (int64_t)n >= c->nearest_grid_min;
+  if (grid && !(c->grid_ok[0] && c->coarse_ok)) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    SCGR_CK(c, cudaStreamIsCapturing(c->stream, &cap));
+    grid = cap == cudaStreamCaptureStatusNone;
+  }
+  if (!grid) {
     SCGR_CK(c, launch_nearest(c->L(), X4, n, q3, nq, idx_out, key_out));
     return SCGR_OK;
   }
-  if (!c->rgrid_ok) {
-    GridSpec gs;
-    const scgr_status st = grid_setup(c, X4, n, &gs);
+  CloudSet cs{};
+  if (!c->grid_ok[0]) {
+    SCGR_CK(c, ensure(c->gspec, 2 * sizeof(GridSpec)));
+    const scgr_status st = grid_buffers(c, 0);
     if (st != SCGR_OK) return st;
-    const int64_t ncell = grid_cells(gs);
-    SCGR_CK(c, ensure(c->rgstart, (size_t)(ncell + 1) * sizeof(int)));
-    SCGR_CK(c, ensure(c->rgsorted, (size_t)n * sizeof(float4)));
-    SCGR_CK(c, ensure(c->rgsidx, (size_t)n * sizeof(int)));
-    SCGR_CK(c, launch_grid_build(c->L(), X4, n, gs, (int*)c->gcell.p, (int*)c->gcount.p, (int*)c->rgstart.p,
-                                 (int*)c->gcursor.p, (int*)c->gblock.p, (float4*)c->rgsorted.p, (int*)c->rgsidx.p));
-    // the coarse level: the same counting sort with cells NEAREST_COARSE times larger
-    // (it fits the fine level's count/cursor/block scratch)
-    const GridSpec gc = coarse_grid_spec(gs);
-    SCGR_CK(c, ensure(c->rcgstart, (size_t)(grid_cells(gc) + 1) * sizeof(int)));
-    SCGR_CK(c, ensure(c->rcgsorted, (size_t)n * sizeof(float4)));
-    SCGR_CK(c, ensure(c->rcgsidx, (size_t)n * sizeof(int)));
-    SCGR_CK(c, launch_grid_build(c->L(), X4, n, gc, (int*)c->gcell.p, (int*)c->gcount.p, (int*)c->rcgstart.p,
-                                 (int*)c->gcursor.p, (int*)c->gblock.p, (float4*)c->rcgsorted.p, (int*)c->rcgsidx.p));
-    c->rgspec = gs;
-    c->rcgspec = gc;
-    c->rgrid_ok = true;
+    cs.one[0] = grid_cloud(c, 0, true, false);
+    SCGR_CK(c, launch_clouds(c->L(), cs, 1, n, false, c->red, (float*)(c->red + 2 * CLOUD_PARTS * 6)));
+    SCGR_CK(c, launch_grid_sort(c->L(), cs, 1, n));
+    c->grid_ok[0] = true;
+    c->coarse_ok = false;
   }
-  if (c->nearest_levels == 1) {
-    SCGR_CK(c, launch_nearest_grid(c->L(), (const float4*)c->rgsorted.p, (const int*)c->rgsidx.p,
-                                   (const int*)c->rgstart.p, c->rgspec, q3, nq, idx_out, key_out));
-  } else {
-    SCGR_CK(c, launch_nearest_grid2(c->L(), (const float4*)c->rgsorted.p, (const int*)c->rgsidx.p,
-                                    (const int*)c->rgstart.p, c->rgspec, (const float4*)c->rcgsorted.p,
-                                    (const int*)c->rcgsidx.p, (const int*)c->rcgstart.p, c->rcgspec, q3, nq, idx_out,
-                                    key_out));
+  cs.one[0] = grid_cloud(c, 0, true, false);
+  if (!c->coarse_ok) {
+    SCGR_CK(c, ensure(c->gccount, grid_start_entries(n) * sizeof(int)));
+    SCGR_CK(c, launch_coarse_count(c->L(), cs, n, (int*)c->gccount.p));
+    c->coarse_ok = true;
   }
+  SCGR_CK(c, launch_nearest_grid(c->L(), cs, c->nearest_levels, (const int*)c->gccount.p, q3, nq, idx_out, key_out));
   return SCGR_OK;
 }
 
@@ -249,31 +299,26 @@ scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_sca
     SCGR_CK(c, ensure(c->knnY, (size_t)m * k * sizeof(int32_t)));
     const int k_prev = c->prm.k;
     c->prm.k = k;
-    scgr_status ks = knn_cloud(c, X4, n, (int32_t*)c->knnX.p);
-    if (ks == SCGR_OK) ks = knn_cloud(c, Y4, m, (int32_t*)c->knnY.p);
+    const scgr_status ks = knn_clouds(c);
     if (ks != SCGR_OK) {
       c->prm.k = k_prev;
       return ks;
     }
-    SCGR_CK(c, launch_curvature(L, X4, (const int32_t*)c->knnX.p, n, k, (double*)c->aX64.p, (float*)c->aX32.p));
-    SCGR_CK(c, launch_curvature(L, Y4, (const int32_t*)c->knnY.p, m, k, (double*)c->aY64.p, (float*)c->aY32.p));
+    SCGR_CK(c, launch_curvature2(L, X4, (const int32_t*)c->knnX.p, n, (double*)c->aX64.p, (float*)c->aX32.p, Y4,
+                                 (const int32_t*)c->knnY.p, m, (double*)c->aY64.p, (float*)c->aY32.p, k));
   } else {
     c->prm.radius_scale = radius_scale;
     const double s2 = radius_scale * radius_scale;
     const size_t bx = radius_scratch_bytes(n, c->num_sms), by = radius_scratch_bytes(m, c->num_sms);
     SCGR_CK(c, ensure(c->radpart, bx > by ? bx : by));
-    SCGR_CK(c, ensure(c->gbb, sizeof(float) * (256 * 6 + 8)));
-    float* box = (float*)c->gbb.p;  // scratch, then the box
-    SCGR_CK(c, launch_bbox(L, X4, n, box, box + 256 * 6));
-    SCGR_CK(c, launch_radius_curvature(L, X4, n, &st->eX, s2, box + 256 * 6, c->num_sms, (double*)c->radpart.p,
+    const GridSpec* spec = (const GridSpec*)c->gspec.p;
+    SCGR_CK(c, launch_radius_curvature(L, X4, n, &st->eX, s2, spec, c->num_sms, (double*)c->radpart.p,
                                        (double*)c->aX64.p, (float*)c->aX32.p));
-    SCGR_CK(c, launch_bbox(L, Y4, m, box, box + 256 * 6));
-    SCGR_CK(c, launch_radius_curvature(L, Y4, m, &st->eY0, s2, box + 256 * 6, c->num_sms, (double*)c->radpart.p,
+    SCGR_CK(c, launch_radius_curvature(L, Y4, m, &st->eY0, s2, spec + 1, c->num_sms, (double*)c->radpart.p,
                                        (double*)c->aY64.p, (float*)c->aY32.p));
   }
   const double user = c->prm.sigma > 0.0 ? c->prm.sigma * sigma_scale : 0.0;
-  SCGR_CK(c, launch_sigma(L, (const double*)c->aX64.p, n, user, c->red, &st->sigma, &st->asum[0]));
-  if (user <= 0.0 && sigma_scale != 1.0) SCGR_CK(c, launch_scale_double(L, &st->sigma, sigma_scale));
+  SCGR_CK(c, launch_sigma(L, (const double*)c->aX64.p, n, user, sigma_scale, c->red, st));
   return SCGR_OK;
 }
 

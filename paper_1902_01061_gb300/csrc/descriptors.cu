@@ -8,6 +8,8 @@
 
 namespace scgr {
 
+constexpr double SQRT_LOG2E = 1.2011224087864498;  // sqrt(log2 e)
+
 static inline cudaError_t after_launch(Launch L) {
   if (L.counter) ++*L.counter;
   return cudaGetLastError();
@@ -263,14 +265,27 @@ cudaError_t launch_knn(Launch L, const float4* P, int n, int k, int32_t* out) {
   return after_launch(L);
 }
 
+// (h, l) += x, h the rounded sum (two-sum)
+__device__ __forceinline__ void two_sum_add(float& h, float& l, float x) {
+  const float t = __fadd_rn(h, x);
+  const float bv = __fsub_rn(t, h);
+  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, bv)), __fsub_rn(x, bv)));
+  h = t;
+}
+
 // ---- curvature ----------------------------------------------------------
 // a = lambda_min / (lambda_1 + lambda_2 + lambda_3) of the 1/k covariance of
-// the k neighbours (float64); lambda_min clamped at 0; 0 for a zero trace.
-__global__ void curvature_kernel(const float4* __restrict__ P, const int32_t* __restrict__ nbr,
-                                 int n, int k, double* __restrict__ a64, float* __restrict__ a32) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int32_t* nb = nbr + (int64_t)i * k;
+// the k neighbours; lambda_min clamped at 0; 0 for a zero trace.
+//
+// The offsets from the point itself are exact float pairs (two-difference),
+// their sums and products float pairs too (two-sum, fma remainder), good to
+// about 2^-46; only the covariance, its polynomial and the last Newton steps
+// are float64.  Where the offsets' squares leave float32's comfortable range,
+// all of it is float64.
+// Bound: float64 issue (about 80 such instructions a point, each 64 cycles of
+// a warp scheduler on GB300) and the gather of the neighbours.
+__device__ __noinline__ void covariance_float64(const float4* __restrict__ P, const int32_t* __restrict__ nb, int k,
+                                                double* C) {
   double mx = 0, my = 0, mz = 0;
   for (int m = 0; m < k; ++m) {
     const float4 c = P[nb[m]];
@@ -281,7 +296,7 @@ __global__ void curvature_kernel(const float4* __restrict__ P, const int32_t* __
   mx /= k;
   my /= k;
   mz /= k;
-  double C[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+  for (int q = 0; q < 9; ++q) C[q] = 0.0;
   for (int m = 0; m < k; ++m) {
     const float4 c = P[nb[m]];
     const double dx = c.x - mx, dy = c.y - my, dz = c.z - mz;
@@ -290,18 +305,90 @@ __global__ void curvature_kernel(const float4* __restrict__ P, const int32_t* __
   }
   C[0] /= k; C[1] /= k; C[2] /= k; C[4] /= k; C[5] /= k; C[8] /= k;
   C[3] = C[1]; C[6] = C[2]; C[7] = C[5];
-  const double lmin = sym3_min_eigenvalue(C);
+}
+
+__device__ __forceinline__ double surface_variation(const double* C) {
   const double tr = C[0] + C[4] + C[8];
-  const double a = tr > 0.0 ? fmax(lmin, 0.0) / tr : 0.0;
-  a64[i] = a;
-  a32[i] = (float)a;
+  return tr > 0.0 ? fmax(sym3_extreme_eigenvalue(C, false), 0.0) / tr : 0.0;
+}
+
+__device__ __forceinline__ double point_curvature(const float4* __restrict__ P, const int32_t* __restrict__ nb, int k,
+                                                  int i) {
+  const float4 q = P[i];
+  const float qv[3] = {q.x, q.y, q.z};
+  float sh[3] = {0.f, 0.f, 0.f}, sl[3] = {0.f, 0.f, 0.f};
+  float ph[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, pl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // xx xy xz yy yz zz
+#pragma unroll 4
+  for (int m = 0; m < k; ++m) {
+    const float4 c = P[nb[m]];
+    const float cv[3] = {c.x, c.y, c.z};
+    float h[3], l[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      h[a] = __fsub_rn(cv[a], qv[a]);
+      const float bv = __fsub_rn(h[a], cv[a]);
+      l[a] = __fsub_rn(__fsub_rn(cv[a], __fsub_rn(h[a], bv)), __fadd_rn(qv[a], bv));
+      two_sum_add(sh[a], sl[a], h[a]);
+      sl[a] = __fadd_rn(sl[a], l[a]);
+    }
+#pragma unroll
+    for (int a = 0, f = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = a; b < 3; ++b, ++f) {
+        const float p = __fmul_rn(h[a], h[b]);
+        const float r = __fmaf_rn(h[a], l[b], __fmaf_rn(l[a], h[b], __fmaf_rn(h[a], h[b], -p)));
+        two_sum_add(ph[f], pl[f], p);
+        pl[f] = __fadd_rn(pl[f], r);
+      }
+  }
+  double C[9];
+  const float tr = ph[0] + ph[3] + ph[5];
+  if (!(tr > 1e-18f && tr < 1e30f)) {
+    covariance_float64(P, nb, k, C);
+    return surface_variation(C);
+  }
+  const double ik = 1.0 / (double)k;
+  double mu[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) mu[a] = ((double)sh[a] + (double)sl[a]) * ik;
+#pragma unroll
+  for (int a = 0, f = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = a; b < 3; ++b, ++f)
+      C[a * 3 + b] = C[b * 3 + a] = fma((double)ph[f] + (double)pl[f], ik, -mu[a] * mu[b]);
+  return surface_variation(C);
+}
+
+struct CurvatureIn {
+  const float4* P;
+  const int32_t* nbr;
+  int n;
+  double* a64;
+  float* a32;
+};
+constexpr int CURV_TPB = 128;
+
+// Both clouds of a registration in one launch (blockIdx.y).
+__global__ void __launch_bounds__(CURV_TPB) curvature_kernel(const CurvatureIn c0, const CurvatureIn c1, int k) {
+  const CurvatureIn& c = blockIdx.y == 0 ? c0 : c1;
+  const int i = blockIdx.x * CURV_TPB + threadIdx.x;
+  if (i >= c.n) return;
+  const double a = point_curvature(c.P, c.nbr + (int64_t)i * k, k, i);
+  c.a64[i] = a;
+  c.a32[i] = (float)a;
+}
+
+cudaError_t launch_curvature2(Launch L, const float4* X, const int32_t* nx, int n, double* ax64, float* ax32,
+                              const float4* Y, const int32_t* ny, int m, double* ay64, float* ay32, int k) {
+  const int most = n > m ? n : m;
+  curvature_kernel<<<dim3((most + CURV_TPB - 1) / CURV_TPB, Y ? 2 : 1), CURV_TPB, 0, L.stream>>>(
+      CurvatureIn{X, nx, n, ax64, ax32}, CurvatureIn{Y, ny, m, ay64, ay32}, k);
+  return after_launch(L);
 }
 
 cudaError_t launch_curvature(Launch L, const float4* P, const int32_t* nbr, int n, int k,
                              double* a64, float* a32) {
-  const int tpb = 128;
-  curvature_kernel<<<(n + tpb - 1) / tpb, tpb, 0, L.stream>>>(P, nbr, n, k, a64, a32);
-  return after_launch(L);
+  return launch_curvature2(L, P, nbr, n, a64, a32, nullptr, nullptr, 0, nullptr, nullptr, k);
 }
 
 // ---- radius neighbourhood curvature (Sec. IV) ----------------------------
@@ -327,7 +414,7 @@ cudaError_t launch_curvature(Launch L, const float4* P, const int32_t* nbr, int 
 // operations per member, at 1/64 of the float32 rate.)
 //
 // Members' offsets are scaled by a power of two that brings the bound on
-// |d|^2 (the smaller of the squared radius and the box's squared diagonal)
+// |d|^2 (the smaller of the squared radius and three squared box extents)
 // near 1, so that no product overflows or underflows.
 constexpr int RAD_TPB = 128;
 constexpr int RAD_TILE = 256;
@@ -339,10 +426,9 @@ struct RadiusScale {
   float r2;        // squared radius (not scaled)
   float c1, c2;    // acc's starting value for the offsets and for their products
 };
-__device__ __forceinline__ RadiusScale radius_scale_of(const double* e_dev, double scale2, const float* bb) {
+__device__ __forceinline__ RadiusScale radius_scale_of(const double* e_dev, double scale2, const GridSpec* spec) {
   const float r2 = (float)(scale2 * e_dev[0]);
-  const float dx = bb[3] - bb[0], dy = bb[4] - bb[1], dz = bb[5] - bb[2];
-  const float diag2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) * 1.0001f;
+  const float diag2 = 3.0003f * spec->extent * spec->extent;  // at least the box's squared diagonal
   const float B = fmaxf(fminf(r2, diag2), 1e-36f);
   const int h = min(60, max(-60, -(ilogbf(B) >> 1)));
   RadiusScale o;
@@ -368,14 +454,6 @@ __device__ __forceinline__ void split_add2(u64& acc, u64& lo, u64 x) {
   lo = add2(lo, sub2(x, sub2(t, acc)));
   acc = t;
 }
-// (h, l) += x, h the rounded sum (two-sum)
-__device__ __forceinline__ void two_sum_add(float& h, float& l, float x) {
-  const float t = __fadd_rn(h, x);
-  const float bv = __fsub_rn(t, h);
-  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, bv)), __fsub_rn(x, bv)));
-  h = t;
-}
-
 __device__ __forceinline__ float member_mask(float key, float r2) {
   float m;
   asm("set.le.f32.f32 %0, %1, %2;" : "=f"(m) : "f"(key), "f"(r2));
@@ -386,10 +464,10 @@ __device__ __forceinline__ float member_mask(float key, float r2) {
 // as doubles to part[split][sum][n] (in scaled coordinates).
 __global__ void __launch_bounds__(RAD_TPB)
     radius_sums_kernel(const float4* __restrict__ P, int n, const double* __restrict__ e_dev, double scale2,
-                       const float* __restrict__ bb, int tiles_per_split, double* __restrict__ part) {
+                       const GridSpec* __restrict__ spec, int tiles_per_split, double* __restrict__ part) {
   __shared__ __align__(16) float tile[3][RAD_TILE];
   const int i = blockIdx.x * RAD_TPB + threadIdx.x;
-  const RadiusScale sc = radius_scale_of(e_dev, scale2, bb);
+  const RadiusScale sc = radius_scale_of(e_dev, scale2, spec);
   const float4 q4 = P[i < n ? i : n - 1];
   const u64 q2x = pk2(q4.x, q4.x), q2y = pk2(q4.y, q4.y), q2z = pk2(q4.z, q4.z), s2 = pk2(sc.s, sc.s);
   float H[RAD_NS], Lo[RAD_NS];
@@ -503,9 +581,7 @@ __global__ void __launch_bounds__(RAD_TPB)
   C[0] = fma(v[4], ik, -mx * mx); C[1] = fma(v[5], ik, -mx * my); C[2] = fma(v[6], ik, -mx * mz);
   C[4] = fma(v[7], ik, -my * my); C[5] = fma(v[8], ik, -my * mz); C[8] = fma(v[9], ik, -mz * mz);
   C[3] = C[1]; C[6] = C[2]; C[7] = C[5];
-  const double lmin = sym3_min_eigenvalue(C);
-  const double tr = C[0] + C[4] + C[8];
-  const double a = tr > 0.0 ? fmax(lmin, 0.0) / tr : 0.0;
+  const double a = surface_variation(C);
   a64[i] = a;
   a32[i] = (float)a;
 }
@@ -521,12 +597,12 @@ int radius_splits(int n, int num_sms) {
 }
 size_t radius_scratch_bytes(int n, int num_sms) { return (size_t)radius_splits(n, num_sms) * RAD_NS * n * sizeof(double); }
 
-// bb: the cloud's bounding box (launch_bbox); part: radius_scratch_bytes.
+// spec: the cloud's grid (launch_clouds; its extent); part: radius_scratch_bytes.
 cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const double* e_dev, double scale2,
-                                    const float* bb, int num_sms, double* part, double* a64, float* a32) {
+                                    const GridSpec* spec, int num_sms, double* part, double* a64, float* a32) {
   const int blocks = (n + RAD_TPB - 1) / RAD_TPB, ntiles = (n + RAD_TILE - 1) / RAD_TILE;
   const int S = radius_splits(n, num_sms);
-  radius_sums_kernel<<<dim3(blocks, S), RAD_TPB, 0, L.stream>>>(P, n, e_dev, scale2, bb, (ntiles + S - 1) / S, part);
+  radius_sums_kernel<<<dim3(blocks, S), RAD_TPB, 0, L.stream>>>(P, n, e_dev, scale2, spec, (ntiles + S - 1) / S, part);
   radius_curvature_kernel<<<blocks, RAD_TPB, 0, L.stream>>>(part, S, n, a64, a32);
   if (L.counter) *L.counter += 2;
   return cudaGetLastError();
@@ -534,23 +610,6 @@ cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const doub
 
 // ---- fixed-order float64 reductions ------------------------------------
 // Pass 1: per-block sums of an NV-vector per point (fixed grid, fixed order).
-struct SumXYZ {
-  const float4* P;
-  __device__ void operator()(int64_t i, double (&v)[3]) const {
-    const float4 c = P[i];
-    v[0] += c.x; v[1] += c.y; v[2] += c.z;
-  }
-};
-struct ScatterXYZ {
-  const float4* P;
-  const double* mean;
-  __device__ void operator()(int64_t i, double (&v)[6]) const {
-    const float4 c = P[i];
-    const double dx = c.x - mean[0], dy = c.y - mean[1], dz = c.z - mean[2];
-    v[0] += dx * dx; v[1] += dx * dy; v[2] += dx * dz;
-    v[3] += dy * dy; v[4] += dy * dz; v[5] += dz * dz;
-  }
-};
 struct SumA {
   const double* a;
   __device__ void operator()(int64_t i, double (&v)[1]) const { v[0] += a[i]; }
@@ -599,72 +658,83 @@ __global__ void __launch_bounds__(RED_THREADS) reduce_final_kernel(const double*
   }
 }
 
-__global__ void mean_from_sum_kernel(double* mean, int64_t n) {
-  if (threadIdx.x == 0) {
-    mean[0] /= (double)n;
-    mean[1] /= (double)n;
-    mean[2] /= (double)n;
+// sigma of Eq. 3 (the caller's, or the population std of the reference
+// curvatures, 1 below 1e-12, times sigma_scale) and the factor sqrt(log2 e) /
+// sigma that the force records use.
+__device__ __forceinline__ void finish_sigma(double sum_a, double sum_d2, int64_t n, double sigma_user,
+                                             double sigma_scale, DevStats* st) {
+  st->asum[0] = sum_a;
+  double sigma = sigma_user;
+  if (!(sigma > 0.0)) {
+    const double sd = sqrt(sum_d2 / (double)n);
+    sigma = sd >= 1e-12 ? sd : 1.0;
+    if (sigma_scale != 1.0) sigma *= sigma_scale;
   }
+  st->sigma = sigma;
+  st->kscale = SQRT_LOG2E / sigma;
 }
 
-__global__ void scatter_finish_kernel(const double* s6, int64_t n, double* scatter, double* lmax) {
-  if (threadIdx.x != 0) return;
-  double S[9] = {s6[0], s6[1], s6[2], s6[1], s6[3], s6[4], s6[2], s6[4], s6[5]};
-  for (int q = 0; q < 9; ++q) scatter[q] = S[q];
-  double C[9];
-  for (int q = 0; q < 9; ++q) C[q] = S[q] / (double)n;
-  double lam[3];
-  sym3_eigenvalues(C, lam);
-  *lmax = lam[2];
+__global__ void sigma_finish_kernel(const double* sums, int64_t n, double sigma_user, double sigma_scale,
+                                    DevStats* st) {
+  if (threadIdx.x == 0) finish_sigma(sums[0], sums[1], n, sigma_user, sigma_scale, st);
 }
 
-cudaError_t launch_cloud_stats(Launch L, const float4* P, int n, double* part, double* mean,
-                               double* scatter, double* lmax) {
-  const int nb = red_blocks(n);
-  reduce_pass_kernel<3, SumXYZ><<<nb, RED_THREADS, 0, L.stream>>>(n, SumXYZ{P}, part);
-  reduce_final_kernel<3><<<1, RED_THREADS, 0, L.stream>>>(part, nb, mean);
-  mean_from_sum_kernel<<<1, 32, 0, L.stream>>>(mean, n);
-  // the 6 scatter sums go to part + RED_MAX_BLOCKS*6 .. as the final output slot
-  double* s6 = part + (size_t)RED_MAX_BLOCKS * 6;
-  reduce_pass_kernel<6, ScatterXYZ><<<nb, RED_THREADS, 0, L.stream>>>(n, ScatterXYZ{P, mean}, part);
-  reduce_final_kernel<6><<<1, RED_THREADS, 0, L.stream>>>(part, nb, s6);
-  scatter_finish_kernel<<<1, 32, 0, L.stream>>>(s6, n, scatter, lmax);
-  if (L.counter) *L.counter += 6;
-  return cudaGetLastError();
+// Small clouds: both passes (mean, then squared deviations) in one block.
+constexpr int SIGMA_ONE_MAX = 16384;
+constexpr int SIGMA_T = 1024;
+
+__device__ __forceinline__ double sigma_block_sum(double v, double* sh) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = sh[threadIdx.x & 31];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  __syncthreads();
+  return v;
 }
 
-__global__ void sigma_finish_kernel(const double* sums, int64_t n, double sigma_user,
-                                    double* sigma_out, double* asum_out) {
-  if (threadIdx.x != 0) return;
-  if (asum_out) *asum_out = sums[0];
-  if (sigma_user > 0.0) {
-    *sigma_out = sigma_user;
-    return;
+__global__ void __launch_bounds__(SIGMA_T) sigma_one_kernel(const double* __restrict__ a64, int n, double sigma_user,
+                                                            double sigma_scale, DevStats* st) {
+  __shared__ double sh[32];
+  double a[SIGMA_ONE_MAX / SIGMA_T], v = 0.0;
+#pragma unroll
+  for (int u = 0; u < SIGMA_ONE_MAX / SIGMA_T; ++u) {
+    const int i = u * SIGMA_T + threadIdx.x;
+    if (u * SIGMA_T < n) {
+      a[u] = i < n ? a64[i] : 0.0;
+      v += a[u];
+    }
   }
-  const double sd = sqrt(sums[1] / (double)n);
-  *sigma_out = sd >= 1e-12 ? sd : 1.0;
+  const double sum = sigma_block_sum(v, sh), mean = sum / (double)n;
+  v = 0.0;
+#pragma unroll
+  for (int u = 0; u < SIGMA_ONE_MAX / SIGMA_T; ++u) {
+    if (u * SIGMA_T < n) {
+      const double d = u * SIGMA_T + threadIdx.x < n ? a[u] - mean : 0.0;
+      v += d * d;
+    }
+  }
+  const double d2 = sigma_block_sum(v, sh);
+  if (threadIdx.x == 0) finish_sigma(sum, d2, n, sigma_user, sigma_scale, st);
 }
 
-cudaError_t launch_sigma(Launch L, const double* a64, int n, double sigma_user, double* part,
-                         double* sigma_out, double* asum_out) {
+cudaError_t launch_sigma(Launch L, const double* a64, int n, double sigma_user, double sigma_scale, double* part,
+                         DevStats* st) {
+  if (n <= SIGMA_ONE_MAX) {
+    sigma_one_kernel<<<1, SIGMA_T, 0, L.stream>>>(a64, n, sigma_user, sigma_scale, st);
+    return after_launch(L);
+  }
   const int nb = red_blocks(n);
   double* sums = part + (size_t)RED_MAX_BLOCKS * 6 + 8;  // [0]: sum a, [1]: sum (a - mean)^2
   reduce_pass_kernel<1, SumA><<<nb, RED_THREADS, 0, L.stream>>>(n, SumA{a64}, part);
   reduce_final_kernel<1><<<1, RED_THREADS, 0, L.stream>>>(part, nb, sums);
   reduce_pass_kernel<1, VarA><<<nb, RED_THREADS, 0, L.stream>>>(n, VarA{a64, sums, 1.0 / n}, part);
   reduce_final_kernel<1><<<1, RED_THREADS, 0, L.stream>>>(part, nb, sums + 1);
-  sigma_finish_kernel<<<1, 32, 0, L.stream>>>(sums, n, sigma_user, sigma_out, asum_out);
+  sigma_finish_kernel<<<1, 32, 0, L.stream>>>(sums, n, sigma_user, sigma_scale, st);
   if (L.counter) *L.counter += 5;
   return cudaGetLastError();
-}
-
-__global__ void scale_double_kernel(double* v, double f) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *v *= f;
-}
-
-cudaError_t launch_scale_double(Launch L, double* v, double f) {
-  scale_double_kernel<<<1, 32, 0, L.stream>>>(v, f);
-  return after_launch(L);
 }
 
 // ---- caller-supplied curvature --------------------------------------------
@@ -694,7 +764,7 @@ cudaError_t launch_check_curvature(Launch L, const double* a64, int n, float* a3
 __device__ __forceinline__ void write_x_record(int i, int n, const float4* __restrict__ X4,
                                                const double* __restrict__ aX64, int g_mode, const DevStats& st,
                                                float* __restrict__ Xr, float* __restrict__ XA) {
-  const double kscale = sqrt(1.4426950408889634) / st.sigma;  // sqrt(log2 e) / sigma
+  const double kscale = st.kscale;
   const size_t t = (size_t)(i / FORCE_TJ), r = (size_t)(i % FORCE_TJ);
   float* xr = Xr + t * 4 * FORCE_TJ + r;
   float* xa = XA + t * 2 * FORCE_TJ + r;
@@ -723,9 +793,8 @@ __device__ __forceinline__ void write_y_record(int i, int m, const float4* __res
                                                const double* __restrict__ aY64, const DevStats& st,
                                                float4* __restrict__ Y0r) {
   if (i < m) {
-    const double kscale = sqrt(1.4426950408889634) / st.sigma;
     const float4 c = Y4[i];
-    Y0r[i] = make_float4(c.x, c.y, c.z, (float)(aY64[i] * kscale));
+    Y0r[i] = make_float4(c.x, c.y, c.z, (float)(aY64[i] * st.kscale));
   } else {
     Y0r[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
@@ -823,14 +892,7 @@ __global__ void __launch_bounds__(RED_THREADS)
     v2[0] += d * d;
   }
   block_sum<1>(v2, sh);
-  if (threadIdx.x == 0) {
-    st->asum[0] = asum;
-    if (sigma_user > 0.0) st->sigma = sigma_user;
-    else {
-      const double sd = sqrt(v2[0] / bp.n);
-      st->sigma = sd >= 1e-12 ? sd : 1.0;
-    }
-  }
+  if (threadIdx.x == 0) finish_sigma(asum, v2[0], bp.n, sigma_user, 1.0, st);
 }
 
 cudaError_t launch_stats_multi(Launch L, const float4* X4, const float4* Y4, const double* aX64,

@@ -44,7 +44,8 @@ constexpr size_t OFF_A32X = OFF_RED + al256(8 * (RED_MAX_BLOCKS * 6 + 32));
 constexpr size_t OFF_A32Y = OFF_A32X + al256(4 * STATIC_MAX_POINTS);
 constexpr size_t OFF_STATS = OFF_A32Y + al256(4 * STATIC_MAX_POINTS);
 constexpr size_t OFF_POSE = OFF_STATS + al256(sizeof(DevStats));
-constexpr size_t OFF_ERR = OFF_POSE + al256(sizeof(DevPose));
+constexpr size_t OFF_SPEC = OFF_POSE + al256(sizeof(DevPose));
+constexpr size_t OFF_ERR = OFF_SPEC + al256(2 * sizeof(GridSpec));
 constexpr size_t STATIC_BYTES = OFF_ERR + 256;
 
 }  // namespace
@@ -136,9 +137,20 @@ extern "C" scgr_status scgr_forces_static(const float* x_dev, int64_t n, const f
   if (e == cudaSuccess) e = launch_pack(L, y_dev, m, Y4, err);
   if (e == cudaSuccess) e = launch_check_curvature(L, ax_dev, (int)n, a32x, err);
   if (e == cudaSuccess) e = launch_check_curvature(L, ay_dev, (int)m, a32y, err);
-  if (e == cudaSuccess) e = launch_cloud_stats(L, X4, (int)n, red, stats->xbar, stats->CX, &stats->eX);
-  if (e == cudaSuccess) e = launch_cloud_stats(L, Y4, (int)m, red, stats->ybar0, stats->S0, &stats->eY0);
-  if (e == cudaSuccess) e = launch_sigma(L, ax_dev, (int)n, sigma, red, &stats->sigma, &stats->asum[0]);
+  // means (the scale model's covariances are not needed for a force)
+  CloudSet cs{};
+  GridSpec* spec = reinterpret_cast<GridSpec*>(base + OFF_SPEC);
+  cs.one[0].P = X4;
+  cs.one[0].n = (int)n;
+  cs.one[0].spec = spec;
+  cs.one[0].mean = stats->xbar;
+  cs.one[1].P = Y4;
+  cs.one[1].n = (int)m;
+  cs.one[1].spec = spec + 1;
+  cs.one[1].mean = stats->ybar0;
+  if (e == cudaSuccess)
+    e = launch_clouds(L, cs, 2, (int)(n > m ? n : m), false, red, reinterpret_cast<float*>(red + 2 * CLOUD_PARTS * 6));
+  if (e == cudaSuccess) e = launch_sigma(L, ax_dev, (int)n, sigma, 1.0, red, stats);
   if (e == cudaSuccess)
     e = launch_records(L, X4, ax_dev, (int)n, (int)npad, Y4, ay_dev, (int)m, (int)mpad, g_mode, stats, Xr, XA, Y0r);
   if (e == cudaSuccess) e = launch_pose_init(L, pose, stats, 1);

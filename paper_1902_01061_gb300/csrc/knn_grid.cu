@@ -1,14 +1,17 @@
-// Exact k-nearest neighbours through a uniform grid, for large clouds.
+// Exact k-nearest neighbours and nearest-point queries through a uniform grid.
 //
-// The result is identical to the brute-force search (reading R1): the same
-// float32 key (dx*dx + dy*dy) + dz*dz without fused multiply-adds, the first
-// k of the (key, index) order.  Points are counting-sorted into cells (the
-// order inside a cell is arbitrary, so candidates are compared
-// lexicographically by (key, index) rather than relying on scan order).  A
-// query scans shells of cells around its own cell and stops once the k-th
-// key is certified: every unscanned point lies at least dist_out from the
-// query, where dist_out is the distance to the boundary of the scanned cube,
-// and the float32 key of such a point exceeds dist_out^2 (1 - 1e-6) > k-th key.
+// The result is that of a brute-force search: the first k of the (key, index)
+// order.  Points are counting-sorted into cells (the order inside a cell is
+// arbitrary, so candidates are compared by (key, index) rather than relying on
+// scan order).  A query scans a cube of cells around its own and grows it
+// until the k-th key is certified: every unscanned point lies at least dout
+// from the query, dout the distance to the boundary of the scanned cube less
+// a margin for the float32 cell arithmetic, and the k-th key is below dout^2.
+//
+// Several clouds are built and searched per launch (blockIdx.y: the reference
+// and the template of a registration, or every cloud of a batch).  The grid's
+// geometry is computed on the device, so nothing waits for the host; arrays
+// are sized for the most cells a grid may have (GRID_CELLS_PER_POINT).
 #include <cfloat>
 #include <climits>
 #include <cmath>
@@ -17,425 +20,697 @@
 
 namespace scgr {
 
-constexpr int GRID_TPB = 128;
+constexpr unsigned FULL = 0xffffffffu;
 
-__global__ void minmax_kernel(const float4* __restrict__ P, int n, float* __restrict__ part) {
-  __shared__ float sh[6][256];
-  float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
-  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
-    const float4 c = P[i];
-    lo[0] = fminf(lo[0], c.x); lo[1] = fminf(lo[1], c.y); lo[2] = fminf(lo[2], c.z);
-    hi[0] = fmaxf(hi[0], c.x); hi[1] = fmaxf(hi[1], c.y); hi[2] = fmaxf(hi[2], c.z);
-  }
-  for (int a = 0; a < 3; ++a) {
-    sh[a][threadIdx.x] = lo[a];
-    sh[3 + a][threadIdx.x] = hi[a];
-  }
+// ---- statistics and geometry --------------------------------------------------
+
+// Sum over the block of NV doubles per thread (256 threads, fixed order);
+// valid in thread 0.
+template <int NV>
+__device__ __forceinline__ void block_sum_warps(double (&v)[NV], double (*sh)[NV]) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] += __shfl_down_sync(FULL, v[q], off);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0)
+#pragma unroll
+    for (int q = 0; q < NV; ++q) sh[warp][q] = v[q];
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
-      for (int a = 0; a < 3; ++a) {
-        sh[a][threadIdx.x] = fminf(sh[a][threadIdx.x], sh[a][threadIdx.x + w]);
-        sh[3 + a][threadIdx.x] = fmaxf(sh[3 + a][threadIdx.x], sh[3 + a][threadIdx.x + w]);
-      }
-    __syncthreads();
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = lane < RED_THREADS / 32 ? sh[lane][q] : 0.0;
+#pragma unroll
+    for (int off = RED_THREADS / 64; off > 0; off >>= 1)
+#pragma unroll
+      for (int q = 0; q < NV; ++q) v[q] += __shfl_down_sync(FULL, v[q], off);
   }
+}
+
+// Blocks of a cloud's reductions: two points per thread of each block, at
+// most CLOUD_PARTS.
+__host__ __device__ inline int cloud_parts(int n) {
+  const int b = (n + 2 * RED_THREADS - 1) / (2 * RED_THREADS);
+  return b < CLOUD_PARTS ? b : CLOUD_PARTS;
+}
+
+// Pass 1: coordinate sums (float64) and the bounding box of each block's points.
+__global__ void __launch_bounds__(RED_THREADS) cloud_sums_kernel(const CloudSet cs, double* __restrict__ part,
+                                                                 float* __restrict__ bpart) {
+  __shared__ double sh[RED_THREADS / 32][3];
+  __shared__ float shb[RED_THREADS / 32][6];
+  const GridCloud& g = cs[blockIdx.y];
+  const int nb = cloud_parts(g.n);
+  if ((int)blockIdx.x >= nb) return;
+  double v[3] = {0.0, 0.0, 0.0};
+  float b[6] = {FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX};  // min, -max
+  for (int i = blockIdx.x * RED_THREADS + threadIdx.x; i < g.n; i += nb * RED_THREADS) {
+    const float4 c = g.P[i];
+    v[0] += c.x; v[1] += c.y; v[2] += c.z;
+    b[0] = fminf(b[0], c.x); b[1] = fminf(b[1], c.y); b[2] = fminf(b[2], c.z);
+    b[3] = fminf(b[3], -c.x); b[4] = fminf(b[4], -c.y); b[5] = fminf(b[5], -c.z);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) b[q] = fminf(b[q], __shfl_down_sync(FULL, b[q], off));
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) shb[threadIdx.x >> 5][q] = b[q];
+  block_sum_warps<3>(v, sh);  // synchronises: shb is written
+  const size_t o = (size_t)blockIdx.y * CLOUD_PARTS + blockIdx.x;
   if (threadIdx.x == 0)
-    for (int a = 0; a < 6; ++a) part[blockIdx.x * 6 + a] = sh[a][0];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) part[o * 6 + q] = v[q];
+  if (threadIdx.x < 6) {
+    float m = shb[0][threadIdx.x];
+#pragma unroll
+    for (int w = 1; w < RED_THREADS / 32; ++w) m = fminf(m, shb[w][threadIdx.x]);
+    bpart[o * 6 + threadIdx.x] = m;
+  }
 }
 
-__global__ void minmax_final_kernel(const float* __restrict__ part, int nb, float* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  float r[6] = {FLT_MAX, FLT_MAX, FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX};
-  for (int b = 0; b < nb; ++b)
-    for (int a = 0; a < 3; ++a) {
-      r[a] = fminf(r[a], part[b * 6 + a]);
-      r[3 + a] = fmaxf(r[3 + a], part[b * 6 + 3 + a]);
+// Grid of a cloud from its box: cell edge h = sqrt(8 A / n), A the box's
+// surface area (about 8 points per occupied cell on a surface sample), at most
+// GRID_CELLS_PER_POINT n cells and 2^16 per axis.
+__device__ void make_grid_spec(const float* lo, const float* hi, int n, GridSpec* out) {
+  float e[3], emax = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    e[a] = hi[a] - lo[a];
+    emax = fmaxf(emax, e[a]);
+  }
+  // in units of the largest extent, so that no product overflows
+  const float ie = emax > 0.f ? 1.f / emax : 0.f;
+  const float x = e[0] * ie, y = e[1] * ie, z = e[2] * ie;
+  const float A = 2.f * (x * y + y * z + z * x);
+  float h = fmaxf(sqrtf(8.f * A / (float)n), fmaxf(8.f / (float)n, 1.f / 65536.f));
+  const float most = (float)GRID_CELLS_PER_POINT * (float)n;
+  int g[3];
+  for (int it = 0; it < 96; ++it) {
+    g[0] = max(1, (int)ceilf(x / h + 1e-4f));
+    g[1] = max(1, (int)ceilf(y / h + 1e-4f));
+    g[2] = max(1, (int)ceilf(z / h + 1e-4f));
+    if ((float)g[0] * (float)g[1] * (float)g[2] <= most) break;
+    h *= 1.25f;
+  }
+  h = emax > 0.f ? h * emax : 1.f;
+  out->h = h;
+  out->inv_h = 1.f / h;
+  out->extent = emax;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    out->o[a] = lo[a];
+    out->g[a] = g[a];
+  }
+  out->ncell = g[0] * g[1] * g[2];
+}
+
+// One block per cloud: its mean, box and grid.
+__global__ void __launch_bounds__(RED_THREADS) cloud_mean_kernel(const CloudSet cs, const double* __restrict__ part,
+                                                                 const float* __restrict__ bpart) {
+  static_assert(CLOUD_PARTS <= RED_THREADS, "one partial per thread");
+  __shared__ double sh[RED_THREADS / 32][3];
+  __shared__ float shb[RED_THREADS / 32][6];
+  const GridCloud& g = cs[blockIdx.y];
+  const int nb = cloud_parts(g.n);
+  const size_t o = (size_t)blockIdx.y * CLOUD_PARTS + threadIdx.x;
+  double v[3] = {0.0, 0.0, 0.0};
+  float b[6] = {FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX, FLT_MAX};
+  if ((int)threadIdx.x < nb) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] = part[o * 6 + q];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) b[q] = bpart[o * 6 + q];
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) b[q] = fminf(b[q], __shfl_down_sync(FULL, b[q], off));
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) shb[threadIdx.x >> 5][q] = b[q];
+  block_sum_warps<3>(v, sh);
+  if (threadIdx.x == 0 && g.mean) {
+    const double in = 1.0 / (double)g.n;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) g.mean[q] = v[q] * in;
+  }
+  if (threadIdx.x == 32) {  // its own warp: runs beside the mean's float64
+    float lo[3], hi[3];
+    for (int q = 0; q < 3; ++q) {
+      float a = shb[0][q], c = shb[0][3 + q];
+      for (int w = 1; w < RED_THREADS / 32; ++w) {
+        a = fminf(a, shb[w][q]);
+        c = fminf(c, shb[w][3 + q]);
+      }
+      lo[q] = a;
+      hi[q] = -c;
     }
-  for (int a = 0; a < 6; ++a) out[a] = r[a];
+    make_grid_spec(lo, hi, g.n, g.spec);
+  }
 }
 
-__device__ __forceinline__ int cell_coord(float v, double o, double inv_h, int g) {
-  int c = (int)floor(((double)v - o) * inv_h);
-  return c < 0 ? 0 : (c >= g ? g - 1 : c);
-}
-
-__global__ void cell_count_kernel(const float4* __restrict__ P, int n, GridSpec gs, int* __restrict__ cell_of,
-                                  int* __restrict__ count) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float4 c = P[i];
-  const int cx = cell_coord(c.x, gs.o[0], gs.inv_h, gs.g[0]);
-  const int cy = cell_coord(c.y, gs.o[1], gs.inv_h, gs.g[1]);
-  const int cz = cell_coord(c.z, gs.o[2], gs.inv_h, gs.g[2]);
-  const int cell = (cz * gs.g[1] + cy) * gs.g[0] + cx;
-  cell_of[i] = cell;
-  atomicAdd(count + cell, 1);
-}
-
-// Exclusive scan of count[0, ncell) into start[0, ncell] (start[ncell] = n),
-// in three passes over blocks of 1024 cells.
-constexpr int SCAN_B = 1024;
-
-__global__ void scan_local_kernel(const int* __restrict__ count, int ncell, int* __restrict__ start,
-                                  int* __restrict__ block_tot) {
-  __shared__ int sh[SCAN_B];
-  const int base = blockIdx.x * SCAN_B;
-  for (int t = threadIdx.x; t < SCAN_B; t += blockDim.x) sh[t] = (base + t < ncell) ? count[base + t] : 0;
-  __syncthreads();
+// Pass 2: scatter sums about the mean (where the cloud wants them), and the
+// cell counters cleared.
+__global__ void __launch_bounds__(RED_THREADS) cloud_scatter_kernel(const CloudSet cs, double* __restrict__ part) {
+  __shared__ double sh[RED_THREADS / 32][6];
+  const GridCloud& g = cs[blockIdx.y];
+  const int nb = cloud_parts(g.n);
+  if ((int)blockIdx.x >= nb) return;
+  if (g.start) {
+    const int cells = g.spec->ncell + 1;
+    for (int c = blockIdx.x * RED_THREADS + threadIdx.x; c < cells; c += nb * RED_THREADS) g.start[c] = 0;
+  }
+  if (!g.scatter) return;
+  const double m0 = g.mean[0], m1 = g.mean[1], m2 = g.mean[2];
+  double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int i = blockIdx.x * RED_THREADS + threadIdx.x; i < g.n; i += nb * RED_THREADS) {
+    const float4 c = g.P[i];
+    const double dx = c.x - m0, dy = c.y - m1, dz = c.z - m2;
+    v[0] += dx * dx; v[1] += dx * dy; v[2] += dx * dz;
+    v[3] += dy * dy; v[4] += dy * dz; v[5] += dz * dz;
+  }
+  block_sum_warps<6>(v, sh);
   if (threadIdx.x == 0) {
-    int run = 0;
-    for (int t = 0; t < SCAN_B; ++t) {
-      const int v = sh[t];
-      sh[t] = run;
-      run += v;
+    const size_t o = (size_t)blockIdx.y * CLOUD_PARTS + blockIdx.x;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) part[o * 6 + q] = v[q];
+  }
+}
+
+// One block per cloud: its scatter matrix and the largest eigenvalue of scatter / n.
+__global__ void __launch_bounds__(RED_THREADS) cloud_lmax_kernel(const CloudSet cs, const double* __restrict__ part) {
+  __shared__ double sh[RED_THREADS / 32][6];
+  const GridCloud& g = cs[blockIdx.y];
+  if (!g.scatter) return;
+  const int nb = cloud_parts(g.n);
+  const size_t o = (size_t)blockIdx.y * CLOUD_PARTS + threadIdx.x;
+  double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if ((int)threadIdx.x < nb)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) v[q] = part[o * 6 + q];
+  block_sum_warps<6>(v, sh);
+  if (threadIdx.x != 0) return;
+  const double S[9] = {v[0], v[1], v[2], v[1], v[3], v[4], v[2], v[4], v[5]};
+  double C[9];
+  const double in = 1.0 / (double)g.n;
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    g.scatter[q] = S[q];
+    C[q] = S[q] * in;
+  }
+  *g.lmax = sym3_max_eigenvalue(C);
+}
+
+// ---- counting sort into cells ---------------------------------------------------
+
+// Cell of coordinate v on an axis (clamped to the grid, so v may lie outside
+// the box).  Float32: v - o and the product round, so a point may sit up to
+// about 4e-7 of the distance v - o beyond its cell's faces; the certification
+// below allows for it.
+__device__ __forceinline__ int cell_coord(float v, float o, float inv_h, int g) {
+  return (int)fminf(fmaxf(floorf((v - o) * inv_h), 0.f), (float)(g - 1));
+}
+
+// First sorted position of cell c (c = ncell: the number of points): the
+// count scan keeps a block-local part per cell and one offset per block.
+__device__ __forceinline__ int cell_start(const GridCloud& g, int c) { return g.start[c] + g.tot[c / SCAN_B]; }
+
+// The cell of every point and its rank of arrival there.
+__global__ void __launch_bounds__(256) cell_count_kernel(const CloudSet cs) {
+  const GridCloud& g = cs[blockIdx.y];
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= g.n) return;
+  const GridSpec& sp = *g.spec;
+  const float4 c = g.P[i];
+  const int cx = cell_coord(c.x, sp.o[0], sp.inv_h, sp.g[0]);
+  const int cy = cell_coord(c.y, sp.o[1], sp.inv_h, sp.g[1]);
+  const int cz = cell_coord(c.z, sp.o[2], sp.inv_h, sp.g[2]);
+  const int cell = (cz * sp.g[1] + cy) * sp.g[0] + cx;
+  g.cell[i] = make_int2(cell, atomicAdd(g.start + cell, 1));
+}
+
+// Exclusive scan of the counts in place, over blocks of SCAN_B cells (the
+// entry ncell included, so that it becomes the number of points).
+constexpr int SCAN_T = 256;
+constexpr int SCAN_PER = SCAN_B / SCAN_T;
+
+__device__ __forceinline__ int block_scan_excl(int v, int* shw, int nwarps, int* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int inc = v;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int u = __shfl_up_sync(FULL, inc, off);
+    if (lane >= off) inc += u;
+  }
+  if (lane == 31) shw[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    int w = lane < nwarps ? shw[lane] : 0;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int u = __shfl_up_sync(FULL, w, off);
+      if (lane >= off) w += u;
     }
-    block_tot[blockIdx.x] = run;
+    shw[lane] = w;
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < SCAN_B; t += blockDim.x)
-    if (base + t < ncell) start[base + t] = sh[t];
+  *total = shw[nwarps - 1];
+  return inc - v + (warp > 0 ? shw[warp - 1] : 0);
 }
 
-__global__ void scan_blocks_kernel(int* __restrict__ block_tot, int nblocks, int* __restrict__ start, int ncell) {
-  if (threadIdx.x != 0) return;
-  int run = 0;
-  for (int b = 0; b < nblocks; ++b) {
-    const int v = block_tot[b];
-    block_tot[b] = run;
+__global__ void __launch_bounds__(SCAN_T) scan_local_kernel(const CloudSet cs) {
+  __shared__ int sh[SCAN_B + SCAN_B / 32];  // padded: thread t reads 16 entries in a row
+  __shared__ int shw[32];
+  const GridCloud& g = cs[blockIdx.y];
+  const int cells = g.spec->ncell + 1;
+  const int base = blockIdx.x * SCAN_B;
+  if (base >= cells) return;
+  for (int t = threadIdx.x; t < SCAN_B; t += SCAN_T) sh[t + t / 32] = base + t < cells ? g.start[base + t] : 0;
+  __syncthreads();
+  int sum = 0;
+#pragma unroll
+  for (int u = 0; u < SCAN_PER; ++u) {
+    const int t = threadIdx.x * SCAN_PER + u;
+    sum += sh[t + t / 32];
+  }
+  int total;
+  int run = block_scan_excl(sum, shw, SCAN_T / 32, &total);
+#pragma unroll
+  for (int u = 0; u < SCAN_PER; ++u) {
+    const int t = threadIdx.x * SCAN_PER + u;
+    const int v = sh[t + t / 32];
+    sh[t + t / 32] = run;
     run += v;
   }
-  start[ncell] = run;
+  __syncthreads();
+  for (int t = threadIdx.x; t < SCAN_B && base + t < cells; t += SCAN_T) g.start[base + t] = sh[t + t / 32];
+  // a grid of one block needs no second pass
+  if (threadIdx.x == 0) g.tot[blockIdx.x] = cells <= SCAN_B ? 0 : total;
 }
 
-__global__ void scan_add_kernel(int* __restrict__ start, int ncell, const int* __restrict__ block_tot) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < ncell) start[i] += block_tot[i / SCAN_B];
+__global__ void __launch_bounds__(1024) scan_blocks_kernel(const CloudSet cs) {
+  __shared__ int shw[32];
+  const GridCloud& g = cs[blockIdx.y];
+  const int nb = (g.spec->ncell + SCAN_B) / SCAN_B;
+  if (nb <= 1) return;
+  int carry = 0;
+  for (int b0 = 0; b0 < nb; b0 += 1024) {
+    const int b = b0 + threadIdx.x;
+    const int v = b < nb ? g.tot[b] : 0;
+    int total;
+    const int ex = block_scan_excl(v, shw, 32, &total);
+    if (b < nb) g.tot[b] = carry + ex;
+    carry += total;
+    __syncthreads();
+  }
 }
 
-__global__ void scatter_kernel(const float4* __restrict__ P, int n, const int* __restrict__ cell_of,
-                               const int* __restrict__ start, int* __restrict__ cursor, float4* __restrict__ sorted,
-                               int* __restrict__ sorted_idx) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int cell = cell_of[i];
-  const int pos = start[cell] + atomicAdd(cursor + cell, 1);
-  sorted[pos] = P[i];
-  sorted_idx[pos] = i;
+// Points in cell order, the index in w.
+__global__ void __launch_bounds__(256) cell_scatter_kernel(const CloudSet cs) {
+  const GridCloud& g = cs[blockIdx.y];
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= g.n) return;
+  const int2 cr = g.cell[i];
+  float4 c = g.P[i];
+  c.w = __int_as_float(i);
+  g.sorted[cell_start(g, cr.x) + cr.y] = c;
 }
 
-__device__ __forceinline__ bool lex_less(float ka, int ia, float kb, int ib) {
-  return ka < kb || (ka == kb && ia < ib);
+// ---- queries ---------------------------------------------------------------------
+
+// Squared distance of the (key, index) order.  FUSED = false: (dx*dx + dy*dy)
+// + dz*dz, each operation rounded on its own.  FUSED = true: the rounding of
+// the packed brute-force search, whose sums the assembler fuses with the
+// products they add; its callers keep the neighbours they had.
+template <bool FUSED>
+__device__ __forceinline__ float grid_key(float4 q, float4 c) {
+  const float dx = __fsub_rn(q.x, c.x), dy = __fsub_rn(q.y, c.y), dz = __fsub_rn(q.z, c.z);
+  if (FUSED) return __fmaf_rn(dz, dz, __fmaf_rn(dx, dx, __fmul_rn(dy, dy)));
+  return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
-// The k (<= KC) first (key, index) neighbours of query q among the gridded
-// points: shells of cells around q's cell (clamped to the grid, so q may lie
-// outside the box), stopping once the k-th key is certified.  Every point
-// not yet scanned lies beyond a face of the scanned cube that has grid cells
-// behind it, and q is on the inner side of each such face, so its distance
-// to q is at least the distance dist_out from q to the nearest such face.
-template <int KC>
-__device__ __forceinline__ void grid_scan(const float4 q, const float4* __restrict__ sorted,
-                                          const int* __restrict__ sorted_idx, const int* __restrict__ start,
-                                          int k, const GridSpec& gs, float (&kd)[KC], int (&ki)[KC]) {
-  const int cx = cell_coord(q.x, gs.o[0], gs.inv_h, gs.g[0]);
-  const int cy = cell_coord(q.y, gs.o[1], gs.inv_h, gs.g[1]);
-  const int cz = cell_coord(q.z, gs.o[2], gs.inv_h, gs.g[2]);
+// (key, index) as one integer that sorts like the pair (keys are >= +0).
+__device__ __forceinline__ u64 pack_cand(float key, float w) {
+  return ((u64)__float_as_uint(key) << 32) | __float_as_uint(w);
+}
+__device__ __forceinline__ float cand_key(u64 c) { return __uint_as_float((unsigned)(c >> 32)); }
+constexpr u64 NO_CAND = ~0ull;
+
+// Distance from q to what lies outside the cube of cells within s of cell
+// cc[] (cell edge h): the nearest face that has cells behind it, less the
+// margin of the float32 cell arithmetic.  INFINITY: nothing is outside.
+__device__ __forceinline__ float outside_distance(const float (&q)[3], const float* o, float h, const int (&cc)[3],
+                                                  const int (&g)[3], int s, float extent) {
+  float d = INFINITY;
 #pragma unroll
-  for (int m = 0; m < KC; ++m) {
-    kd[m] = INFINITY;
-    ki[m] = INT_MAX;
-  }
-  const int smax = max(gs.g[0], max(gs.g[1], gs.g[2]));
-  for (int s = 0; s <= smax; ++s) {
-    for (int dz = -s; dz <= s; ++dz) {
-      const int z = cz + dz;
-      if (z < 0 || z >= gs.g[2]) continue;
-      for (int dy = -s; dy <= s; ++dy) {
-        const int y = cy + dy;
-        if (y < 0 || y >= gs.g[1]) continue;
-        const bool face = (dz == -s || dz == s || dy == -s || dy == s);
-        const int step = face ? 1 : (s > 0 ? 2 * s : 1);
-        for (int dx = -s; dx <= s; dx += step) {
-          const int x = cx + dx;
-          if (x < 0 || x >= gs.g[0]) continue;
-          const int cell = (z * gs.g[1] + y) * gs.g[0] + x;
-          const int e = start[cell + 1];
-          for (int j = start[cell]; j < e; ++j) {
-            const float4 c = sorted[j];
-            const float ex = __fsub_rn(q.x, c.x);
-            const float ey = __fsub_rn(q.y, c.y);
-            const float ez = __fsub_rn(q.z, c.z);
-            const float key = __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
-            const int idx = sorted_idx[j];
-            if (lex_less(key, idx, kd[KC - 1], ki[KC - 1])) {
-              kd[KC - 1] = key;
-              ki[KC - 1] = idx;
-#pragma unroll
-              for (int m = KC - 1; m > 0; --m) {
-                if (lex_less(kd[m], ki[m], kd[m - 1], ki[m - 1])) {
-                  const float tk = kd[m];
-                  kd[m] = kd[m - 1];
-                  kd[m - 1] = tk;
-                  const int ti = ki[m];
-                  ki[m] = ki[m - 1];
-                  ki[m - 1] = ti;
-                }
-              }
-            }
-          }
-        }
-      }
-    }
-    // distance from q to the outside of the scanned cube of cells; a side on
-    // the grid boundary has nothing beyond it
-    double dout = INFINITY;
-    const int cc[3] = {cx, cy, cz};
-    const float qq[3] = {q.x, q.y, q.z};
-    bool all = true;
-    for (int a = 0; a < 3; ++a) {
-      if (cc[a] - s > 0) {
-        dout = fmin(dout, (double)qq[a] - (gs.o[a] + (double)(cc[a] - s) * gs.h));
-        all = false;
-      }
-      if (cc[a] + s < gs.g[a] - 1) {
-        dout = fmin(dout, (gs.o[a] + (double)(cc[a] + s + 1) * gs.h) - (double)qq[a]);
-        all = false;
-      }
-    }
-    if (all) break;
-    const int kk = k < KC ? k : KC;
-    if (ki[kk - 1] != INT_MAX && dout > 0.0 && (double)kd[kk - 1] < dout * dout * (1.0 - 1e-6)) break;
-  }
-}
-
-// k nearest neighbours of every point of the gridded cloud itself.
-template <int KC>
-__global__ void __launch_bounds__(GRID_TPB)
-    knn_grid_query_kernel(const float4* __restrict__ sorted, const int* __restrict__ sorted_idx,
-                          const int* __restrict__ start, int n, int k, GridSpec gs, int32_t* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const float4 q = sorted[t];  // queries in cell order: neighbouring threads share cells
-  const int qi = sorted_idx[t];
-  float kd[KC];
-  int ki[KC];
-  grid_scan<KC>(q, sorted, sorted_idx, start, k, gs, kd, ki);
-#pragma unroll
-  for (int m = 0; m < KC; ++m)
-    if (m < k) out[(int64_t)qi * k + m] = ki[m];
-}
-
-// Nearest gridded point (first of the (key, index) order) of each of nq
-// external queries q3 [nq][3] (float32); key = the float32 squared distance.
-__global__ void __launch_bounds__(GRID_TPB)
-    nearest_grid_kernel(const float4* __restrict__ sorted, const int* __restrict__ sorted_idx,
-                        const int* __restrict__ start, GridSpec gs, const float* __restrict__ q3, int nq,
-                        int32_t* __restrict__ idx_out, float* __restrict__ key_out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nq) return;
-  const float4 q = make_float4(q3[3 * (size_t)t], q3[3 * (size_t)t + 1], q3[3 * (size_t)t + 2], 0.f);
-  float kd[1];
-  int ki[1];
-  grid_scan<1>(q, sorted, sorted_idx, start, 1, gs, kd, ki);
-  if (idx_out) idx_out[t] = ki[0];
-  if (key_out) key_out[t] = kd[0];
-}
-
-// Nearest gridded point (k = 1, first of the (key, index) order) over the
-// shells 0..smax of cells around q's cell in grid g.  With `prune`, a
-// non-empty cell is skipped when every point of its box is farther than the
-// best key so far (its squared box distance, less a 1e-6 margin for the
-// rounding of the float32 key, exceeds that key, so no point in it can even
-// tie).  Re-scanning a point already seen leaves the best unchanged.
-// Returns true once the best is certified by the stop rule of grid_scan (or
-// the whole grid has been scanned).
-__device__ __forceinline__ bool nearest_shells(const float4 q, const float4* __restrict__ sorted,
-                                               const int* __restrict__ sorted_idx, const int* __restrict__ start,
-                                               const GridSpec& g, int smax, bool prune, float& bk, int& bi) {
-  const int cc[3] = {cell_coord(q.x, g.o[0], g.inv_h, g.g[0]), cell_coord(q.y, g.o[1], g.inv_h, g.g[1]),
-                     cell_coord(q.z, g.o[2], g.inv_h, g.g[2])};
-  const float qq[3] = {q.x, q.y, q.z};
-  const int sgrid = max(g.g[0], max(g.g[1], g.g[2]));
-  const int slast = smax < sgrid ? smax : sgrid;
-  for (int s = 0; s <= slast; ++s) {
-    for (int dz = -s; dz <= s; ++dz) {
-      const int z = cc[2] + dz;
-      if (z < 0 || z >= g.g[2]) continue;
-      for (int dy = -s; dy <= s; ++dy) {
-        const int y = cc[1] + dy;
-        if (y < 0 || y >= g.g[1]) continue;
-        const bool face = (dz == -s || dz == s || dy == -s || dy == s);
-        const int step = face ? 1 : (s > 0 ? 2 * s : 1);
-        for (int dx = -s; dx <= s; dx += step) {
-          const int x = cc[0] + dx;
-          if (x < 0 || x >= g.g[0]) continue;
-          const int cell = (z * g.g[1] + y) * g.g[0] + x;
-          const int b = start[cell], e = start[cell + 1];
-          if (b == e) continue;
-          if (prune && bi != INT_MAX) {
-            const int xyz[3] = {x, y, z};
-            double d2 = 0.0;
-            for (int a = 0; a < 3; ++a) {
-              const double lo = g.o[a] + (double)xyz[a] * g.h;
-              const double hi = lo + g.h;
-              const double v = (double)qq[a];
-              const double d = v < lo ? lo - v : (v > hi ? v - hi : 0.0);
-              d2 += d * d;
-            }
-            if (d2 * (1.0 - 1e-6) > (double)bk) continue;
-          }
-          for (int j = b; j < e; ++j) {
-            const float4 c = sorted[j];
-            const float ex = __fsub_rn(q.x, c.x);
-            const float ey = __fsub_rn(q.y, c.y);
-            const float ez = __fsub_rn(q.z, c.z);
-            const float key = __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
-            const int idx = sorted_idx[j];
-            if (lex_less(key, idx, bk, bi)) {
-              bk = key;
-              bi = idx;
-            }
-          }
-        }
-      }
-    }
-    double dout = INFINITY;
-    bool all = true;
-    for (int a = 0; a < 3; ++a) {
-      if (cc[a] - s > 0) {
-        dout = fmin(dout, (double)qq[a] - (g.o[a] + (double)(cc[a] - s) * g.h));
-        all = false;
-      }
-      if (cc[a] + s < g.g[a] - 1) {
-        dout = fmin(dout, (g.o[a] + (double)(cc[a] + s + 1) * g.h) - (double)qq[a]);
-        all = false;
-      }
-    }
-    if (all) return true;
-    if (bi != INT_MAX && dout > 0.0 && (double)bk < dout * dout * (1.0 - 1e-6)) return true;
-  }
-  return false;
-}
-
-// Two-level exact nearest search: the query's own cell and its neighbours
-// in the fine grid (enough for a query on the surface), then, if that does
-// not certify the nearest point, shells of the coarse grid (cells of
-// NEAREST_COARSE fine cells a side, points sorted by coarse cell) that skip
-// empty coarse cells and coarse cells beyond the best key.  A query far off
-// the surface then visits a few hundred coarse cells instead of the
-// (1.7 D / h)^3 fine cells a fine shell scan needs to certify distance D.
-// The result is the (key, index)-first point, as the one-level search gives.
-__global__ void __launch_bounds__(GRID_TPB)
-    nearest_grid2_kernel(const float4* __restrict__ sorted, const int* __restrict__ sorted_idx,
-                         const int* __restrict__ start, GridSpec gs, const float4* __restrict__ csorted,
-                         const int* __restrict__ csorted_idx, const int* __restrict__ cstart, GridSpec gc,
-                         const float* __restrict__ q3, int nq, int32_t* __restrict__ idx_out,
-                         float* __restrict__ key_out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nq) return;
-  const float4 q = make_float4(q3[3 * (size_t)t], q3[3 * (size_t)t + 1], q3[3 * (size_t)t + 2], 0.f);
-  float bk = INFINITY;
-  int bi = INT_MAX;
-  if (!nearest_shells(q, sorted, sorted_idx, start, gs, 1, false, bk, bi))
-    nearest_shells(q, csorted, csorted_idx, cstart, gc, INT_MAX, true, bk, bi);
-  if (idx_out) idx_out[t] = bi;
-  if (key_out) key_out[t] = bk;
-}
-
-// The coarse grid over the same origin: cells of NEAREST_COARSE fine cells a side.
-GridSpec coarse_grid_spec(const GridSpec& gs) {
-  GridSpec gc = gs;
-  gc.h = gs.h * NEAREST_COARSE;
-  gc.inv_h = 1.0 / gc.h;
-  for (int a = 0; a < 3; ++a) gc.g[a] = (gs.g[a] + NEAREST_COARSE - 1) / NEAREST_COARSE;
-  return gc;
-}
-
-cudaError_t launch_nearest_grid2(Launch L, const float4* sorted, const int* sorted_idx, const int* start,
-                                 const GridSpec& gs, const float4* csorted, const int* csorted_idx,
-                                 const int* cstart, const GridSpec& gc, const float* q3, int nq, int32_t* idx_out,
-                                 float* key_out) {
-  if (nq <= 0) return cudaSuccess;
-  nearest_grid2_kernel<<<(nq + GRID_TPB - 1) / GRID_TPB, GRID_TPB, 0, L.stream>>>(
-      sorted, sorted_idx, start, gs, csorted, csorted_idx, cstart, gc, q3, nq, idx_out, key_out);
-  if (L.counter) *L.counter += 1;
-  return cudaGetLastError();
-}
-
-// Grid spec from the bounding box: cell edge h = sqrt(8 A / n) with A the box
-// surface area (about 8 points per occupied cell on a surface sample), at most
-// 8 n cells, at least one cell per axis.
-GridSpec make_grid_spec(const float* bb, int64_t n) {
-  GridSpec gs;
-  double e[3];
-  for (int a = 0; a < 3; ++a) e[a] = (double)bb[3 + a] - (double)bb[a];
-  const double A = 2.0 * (e[0] * e[1] + e[1] * e[2] + e[2] * e[0]);
-  const double emax = fmax(e[0], fmax(e[1], e[2]));
-  double h = A > 0.0 ? sqrt(8.0 * A / (double)n) : (emax > 0.0 ? emax * 8.0 / (double)n : 1.0);
-  if (!(h > 0.0)) h = 1.0;
-  for (int it = 0; it < 64; ++it) {
-    double cells = 1.0;
-    for (int a = 0; a < 3; ++a) cells *= fmax(1.0, ceil(e[a] / h + 1e-9));
-    if (cells <= 8.0 * (double)n + 8.0) break;
-    h *= 1.25;
-  }
-  gs.h = h;
-  gs.inv_h = 1.0 / h;
   for (int a = 0; a < 3; ++a) {
-    gs.o[a] = (double)bb[a];
-    gs.g[a] = (int)fmax(1.0, ceil(e[a] / h + 1e-9));
+    const float v = q[a] - o[a];
+    const float margin = 1e-6f * fmaxf(extent, fabsf(v));
+    if (cc[a] - s > 0) d = fminf(d, v - (float)(cc[a] - s) * h - margin);
+    if (cc[a] + s < g[a] - 1) d = fminf(d, (float)(cc[a] + s + 1) * h - v - margin);
   }
-  return gs;
+  return d;
+}
+__device__ __forceinline__ bool certified(float key, float dout) {
+  return dout > 0.f && key < dout * dout * (1.f - 1e-5f);  // false for a NaN key (no candidate)
 }
 
-int64_t grid_cells(const GridSpec& gs) { return (int64_t)gs.g[0] * gs.g[1] * gs.g[2]; }
+// Sorted positions [b, b + len) of cells x0..x1 (clamped) of row (y, z); len
+// 0 where the row is outside the grid.
+__device__ __forceinline__ void row_range(const GridCloud& g, const int (&n)[3], int x0, int x1, int y, int z, int& b,
+                                          int& len) {
+  b = len = 0;
+  x0 = max(x0, 0);
+  x1 = min(x1, n[0] - 1);
+  if (y < 0 || y >= n[1] || z < 0 || z >= n[2] || x0 > x1) return;
+  const int c = (z * n[1] + y) * n[0];
+  b = cell_start(g, c + x0);
+  len = cell_start(g, c + x1 + 1) - b;
+}
 
-cudaError_t launch_bbox(Launch L, const float4* P, int n, float* part, float* out6) {
-  const int nb = 256;
-  minmax_kernel<<<nb, 256, 0, L.stream>>>(P, n, part);
-  minmax_final_kernel<<<1, 32, 0, L.stream>>>(part, nb, out6);
+__device__ __forceinline__ int warp_incl_scan(int v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int u = __shfl_up_sync(FULL, v, off);
+    if (lane >= off) v += u;
+  }
+  return v;
+}
+// Lane l's ranges have running lengths incl; the sorted position of the t-th
+// point of all of them (t below the total; other t give some valid lane's).
+__device__ __forceinline__ int flat_position(int incl, int b, int len, int t) {
+  int r = 0;
+#pragma unroll
+  for (int st = 16; st > 0; st >>= 1) {
+    const int v = __shfl_sync(FULL, incl, r + st - 1);
+    if (v <= t) r += st;
+  }
+  const int first = __shfl_sync(FULL, b - (incl - len), r);
+  return first + t;
+}
+
+__device__ __forceinline__ u64 umin64(u64 a, u64 b) { return a < b ? a : b; }
+__device__ __forceinline__ u64 umax64(u64 a, u64 b) { return a < b ? b : a; }
+
+// Ascending bitonic sort / merge of one value per lane.
+__device__ __forceinline__ u64 warp_sort(u64 v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+    for (int st = size >> 1; st > 0; st >>= 1) {
+      const u64 o = __shfl_xor_sync(FULL, v, st);
+      const bool up = (lane & size) == 0 || size == 32;
+      v = ((lane & st) == 0) == up ? umin64(v, o) : umax64(v, o);
+    }
+  return v;
+}
+__device__ __forceinline__ u64 warp_merge(u64 v) {  // v bitonic
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int st = 16; st > 0; st >>= 1) {
+    const u64 o = __shfl_xor_sync(FULL, v, st);
+    v = (lane & st) == 0 ? umin64(v, o) : umax64(v, o);
+  }
+  return v;
+}
+
+// One warp per query (in cell order, so that neighbouring warps read the same
+// cells).  The cube's cells are rows of consecutive cells, i.e. ranges of
+// sorted points: each lane looks up one range, the ranges are flattened over
+// the lanes and 32 candidates are keyed at a time.  Those below the k-th key
+// so far wait in a small buffer; 32 of them are sorted across the lanes and
+// merged into the warp's sorted list of the best 32.
+// Bound: issue slots (about 600 warp instructions a query, most of them in the
+// sorts).  Measured on GB300 at 1M points, k = 16: see launch_knn_grid.
+constexpr int QUERY_WARPS = 8;
+
+template <bool FUSED>
+__global__ void __launch_bounds__(QUERY_WARPS * 32) knn_query_kernel(const CloudSet cs, int k) {
+  __shared__ u64 bufs[QUERY_WARPS][64];
+  const GridCloud& g = cs[blockIdx.y];
+  const int lane = threadIdx.x & 31;
+  u64* buf = bufs[threadIdx.x >> 5];
+  const int t = blockIdx.x * QUERY_WARPS + (threadIdx.x >> 5);
+  if (t >= g.n) return;
+  const GridSpec& sp = *g.spec;
+  const int n3[3] = {sp.g[0], sp.g[1], sp.g[2]};
+  const float h = sp.h;
+  const float4 q = g.sorted[t];
+  const float q3[3] = {q.x, q.y, q.z};
+  int cc[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) cc[a] = cell_coord(q3[a], sp.o[a], sp.inv_h, n3[a]);
+  u64 best = NO_CAND, thr = NO_CAND;
+  int cnt = 0;
+  auto flush = [&]() {
+    __syncwarp();
+    const u64 v = warp_sort(lane < cnt ? buf[lane] : NO_CAND);
+    const u64 rest = lane + 32 < cnt ? buf[lane + 32] : NO_CAND;
+    best = warp_merge(umin64(best, __shfl_sync(FULL, v, 31 - lane)));
+    thr = __shfl_sync(FULL, best, k - 1);
+    __syncwarp();
+    buf[lane] = rest;
+    cnt = cnt > 32 ? cnt - 32 : 0;
+  };
+  // s = 1 scans the whole cube (3 x 3 rows of 3 cells), larger s the shell:
+  // whole rows on its faces, else the two end cells of a row
+  for (int s = 1;; ++s) {
+    const int w = 2 * s + 1;
+    const int nr = s == 1 ? 9 : 2 * w * w;
+    for (int r0 = 0; r0 < nr; r0 += 32) {
+      const int r = r0 + lane;
+      int b = 0, len = 0;
+      if (r < nr) {
+        const int row = s == 1 ? r : r >> 1, end = s == 1 ? 0 : r & 1;
+        const int dz = row / w - s, dy = row % w - s;
+        const bool whole = s == 1 || dz == -s || dz == s || dy == -s || dy == s;
+        if (whole) {
+          if (!end) row_range(g, n3, cc[0] - s, cc[0] + s, cc[1] + dy, cc[2] + dz, b, len);
+        } else {
+          const int x = end ? cc[0] + s : cc[0] - s;
+          row_range(g, n3, x, x, cc[1] + dy, cc[2] + dz, b, len);
+        }
+      }
+      const int incl = warp_incl_scan(len);
+      const int total = __shfl_sync(FULL, incl, 31);
+      for (int t0 = 0; t0 < total; t0 += 32) {
+        const int pos = flat_position(incl, b, len, t0 + lane);
+        u64 cand = NO_CAND;
+        if (t0 + lane < total) {
+          const float4 c = g.sorted[pos];
+          cand = pack_cand(grid_key<FUSED>(q, c), c.w);
+        }
+        const bool pass = cand < thr;
+        const unsigned m = __ballot_sync(FULL, pass);
+        if (pass) buf[cnt + __popc(m & ((1u << lane) - 1))] = cand;
+        cnt += __popc(m);
+        if (cnt >= 32) flush();
+      }
+    }
+    if (cnt > 0) flush();
+    const float dout = outside_distance(q3, sp.o, h, cc, n3, s, sp.extent);
+    if (dout == INFINITY || certified(cand_key(thr), dout)) break;
+  }
+  if (lane < k) g.knn[(size_t)__float_as_int(q.w) * k + lane] = (int32_t)(unsigned)best;
+}
+
+// ---- nearest gridded point of external queries -----------------------------------
+
+// Counts of the coarse cells (NEAREST_COARSE^3 fine cells each).
+__global__ void __launch_bounds__(256) coarse_count_kernel(const CloudSet cs, int* __restrict__ ccount) {
+  const GridCloud& g = cs[0];
+  const int n3[3] = {g.spec->g[0], g.spec->g[1], g.spec->g[2]};
+  int m3[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) m3[a] = (n3[a] + NEAREST_COARSE - 1) / NEAREST_COARSE;
+  const int total = m3[0] * m3[1] * m3[2];
+  for (int c = blockIdx.x * 256 + threadIdx.x; c < total; c += gridDim.x * 256) {
+    const int x = c % m3[0] * NEAREST_COARSE, y = c / m3[0] % m3[1] * NEAREST_COARSE,
+              z = c / (m3[0] * m3[1]) * NEAREST_COARSE;
+    int cnt = 0;
+    for (int r = 0; r < NEAREST_COARSE * NEAREST_COARSE; ++r) {
+      int b, len;
+      row_range(g, n3, x, x + NEAREST_COARSE - 1, y + r % NEAREST_COARSE, z + r / NEAREST_COARSE, b, len);
+      cnt += len;
+    }
+    ccount[c] = cnt;
+  }
+}
+
+// One warp per query.  First the cube of cells around it, as ranges of
+// sorted points flattened over the lanes: enough for a query on the surface.
+// A query that this does not certify searches shells of coarse cells (edge
+// `coarse` fine cells; a query at distance D would otherwise visit about
+// (1.7 D / h)^3 fine cells, nearly all empty): each lane tests one cell, empty
+// ones and ones whose box lies beyond the best key are dropped, and the warp
+// scans the others' points together.  The result is the (key, index)-first
+// point whatever the order of the cells and of the points in a cell.
+// Bound: issue slots and the latency of the range look-ups; a far query costs
+// some thousand warp instructions, one on the surface about two hundred.
+constexpr int NEAREST_WARPS = 4;
+
+__global__ void __launch_bounds__(NEAREST_WARPS * 32)
+    nearest_query_kernel(const CloudSet cs, int coarse, const int* __restrict__ ccount, const float* __restrict__ q3,
+                         int nq, int32_t* __restrict__ idx_out, float* __restrict__ key_out) {
+  const GridCloud& g = cs[0];
+  const int lane = threadIdx.x & 31;
+  const int t = blockIdx.x * NEAREST_WARPS + (threadIdx.x >> 5);
+  if (t >= nq) return;
+  const GridSpec& sp = *g.spec;
+  const int n3[3] = {sp.g[0], sp.g[1], sp.g[2]};
+  const float q[3] = {q3[3 * (size_t)t], q3[3 * (size_t)t + 1], q3[3 * (size_t)t + 2]};
+  const float4 q4 = make_float4(q[0], q[1], q[2], 0.f);
+  int cc[3];
+  float v[3], margin[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    cc[a] = cell_coord(q[a], sp.o[a], sp.inv_h, n3[a]);
+    v[a] = q[a] - sp.o[a];
+    margin[a] = 1e-6f * fmaxf(sp.extent, fabsf(v[a]));
+  }
+  // the warp's best of the points of its lanes' ranges
+  auto scan_ranges = [&](int b, int len) {
+    const int incl = warp_incl_scan(len);
+    const int cnt = __shfl_sync(FULL, incl, 31);
+    u64 mine = NO_CAND;
+    for (int t0 = 0; t0 < cnt; t0 += 32) {
+      const int pos = flat_position(incl, b, len, t0 + lane);
+      if (t0 + lane < cnt) {
+        const float4 p = g.sorted[pos];
+        mine = umin64(mine, pack_cand(grid_key<false>(q4, p), p.w));
+      }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mine = umin64(mine, __shfl_xor_sync(FULL, mine, off));
+    return mine;
+  };
+  int b = 0, len = 0;
+  if (lane < 9) row_range(g, n3, cc[0] - 1, cc[0] + 1, cc[1] + lane % 3 - 1, cc[2] + lane / 3 - 1, b, len);
+  u64 best = scan_ranges(b, len);
+  float dout = outside_distance(q, sp.o, sp.h, cc, n3, 1, sp.extent);
+  if (dout != INFINITY && !certified(cand_key(best), dout)) {
+    const float H = sp.h * (float)coarse;
+    int m3[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      m3[a] = (n3[a] + coarse - 1) / coarse;
+      cc[a] /= coarse;
+    }
+    for (int s = 0;; ++s) {
+      const int w = 2 * s + 1, cube = w * w * w;
+      for (int c0 = 0; c0 < cube; c0 += 32) {
+        const int c = c0 + lane;
+        const int dx = c % w - s, dy = c / w % w - s, dz = c / (w * w) - s;
+        const int x = cc[0] + dx, y = cc[1] + dy, z = cc[2] + dz;
+        float d2 = INFINITY;  // squared distance to the cell's box; INFINITY: not a cell to scan
+        if (c < cube && max(abs(dx), max(abs(dy), abs(dz))) == s && x >= 0 && x < m3[0] && y >= 0 && y < m3[1] &&
+            z >= 0 && z < m3[2] && !(ccount && ccount[(z * m3[1] + y) * m3[0] + x] == 0)) {
+          const int xyz[3] = {x, y, z};
+          d2 = 0.f;
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const float below = (float)xyz[a] * H - v[a] - margin[a];
+            const float above = v[a] - (float)(xyz[a] + 1) * H - margin[a];
+            const float d = fmaxf(0.f, fmaxf(below, above));
+            d2 = fmaf(d, d, d2);
+          }
+          d2 *= 1.f - 1e-5f;
+        }
+        unsigned todo = __ballot_sync(FULL, d2 != INFINITY && !(d2 > cand_key(best)));
+        while (todo) {
+          const int src = __ffs(todo) - 1;
+          todo &= todo - 1;
+          if (__shfl_sync(FULL, d2, src) > cand_key(best)) continue;  // the best has improved meanwhile
+          const int X = __shfl_sync(FULL, x, src) * coarse, Y = __shfl_sync(FULL, y, src) * coarse,
+                    Z = __shfl_sync(FULL, z, src) * coarse;
+          b = len = 0;
+          if (lane < coarse * coarse)
+            row_range(g, n3, X, X + coarse - 1, Y + lane % coarse, Z + lane / coarse, b, len);
+          best = umin64(best, scan_ranges(b, len));
+        }
+      }
+      dout = outside_distance(q, sp.o, H, cc, m3, s, sp.extent);
+      if (dout == INFINITY || certified(cand_key(best), dout)) break;
+    }
+  }
+  if (lane == 0) {
+    if (idx_out) idx_out[t] = (int32_t)(unsigned)best;
+    if (key_out) key_out[t] = cand_key(best);
+  }
+}
+
+// ---- launchers --------------------------------------------------------------------
+
+static inline unsigned up(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
+
+size_t grid_start_entries(int64_t n) { return (size_t)GRID_CELLS_PER_POINT * n + 64 + 1; }
+size_t grid_tot_entries(int64_t n) { return grid_start_entries(n) / SCAN_B + 2; }
+
+// Means, boxes and grids of the clouds; scatter matrices and largest
+// covariance eigenvalues of those that ask for them.  part: nclouds x
+// CLOUD_PARTS x 6 doubles, bpart the same of floats.  most: points of the
+// largest cloud.
+cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, bool scatter, double* part,
+                          float* bpart) {
+  const dim3 grid(cloud_parts(most), nclouds), one(1, nclouds);
+  cloud_sums_kernel<<<grid, RED_THREADS, 0, L.stream>>>(cs, part, bpart);
+  cloud_mean_kernel<<<one, RED_THREADS, 0, L.stream>>>(cs, part, bpart);
   if (L.counter) *L.counter += 2;
+  if (scatter || cs.many || cs.one[0].start) {  // scatter sums, cleared cell counts
+    cloud_scatter_kernel<<<grid, RED_THREADS, 0, L.stream>>>(cs, part);
+    if (L.counter) *L.counter += 1;
+  }
+  if (scatter) {
+    cloud_lmax_kernel<<<one, RED_THREADS, 0, L.stream>>>(cs, part);
+    if (L.counter) *L.counter += 1;
+  }
   return cudaGetLastError();
 }
 
-// Counting sort of the n points into the cells of gs: sorted / sorted_idx in
-// cell order, start[ncell + 1] the cell offsets.
-cudaError_t launch_grid_build(Launch L, const float4* P, int n, const GridSpec& gs, int* cell_of, int* count,
-                              int* start, int* cursor, int* block_tot, float4* sorted, int* sorted_idx) {
-  const int64_t ncell = grid_cells(gs);
-  cudaError_t e = cudaMemsetAsync(count, 0, (size_t)ncell * sizeof(int), L.stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, (size_t)ncell * sizeof(int), L.stream);
-  if (e != cudaSuccess) return e;
-  const int tpb = 256;
-  cell_count_kernel<<<(n + tpb - 1) / tpb, tpb, 0, L.stream>>>(P, n, gs, cell_of, count);
-  const int nsb = (int)((ncell + SCAN_B - 1) / SCAN_B);
-  scan_local_kernel<<<nsb, 256, 0, L.stream>>>(count, (int)ncell, start, block_tot);
-  scan_blocks_kernel<<<1, 32, 0, L.stream>>>(block_tot, nsb, start, (int)ncell);
-  scan_add_kernel<<<(int)((ncell + tpb - 1) / tpb), tpb, 0, L.stream>>>(start, (int)ncell, block_tot);
-  scatter_kernel<<<(n + tpb - 1) / tpb, tpb, 0, L.stream>>>(P, n, cell_of, start, cursor, sorted, sorted_idx);
-  if (L.counter) *L.counter += 5;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_knn_grid(Launch L, const float4* P, int n, int k, const GridSpec& gs, int* cell_of, int* count,
-                            int* start, int* cursor, int* block_tot, float4* sorted, int* sorted_idx,
-                            int32_t* out) {
-  cudaError_t e = launch_grid_build(L, P, n, gs, cell_of, count, start, cursor, block_tot, sorted, sorted_idx);
-  if (e != cudaSuccess) return e;
-  const unsigned qb = (unsigned)((n + GRID_TPB - 1) / GRID_TPB);
-  if (k <= 8) knn_grid_query_kernel<8><<<qb, GRID_TPB, 0, L.stream>>>(sorted, sorted_idx, start, n, k, gs, out);
-  else if (k <= 16) knn_grid_query_kernel<16><<<qb, GRID_TPB, 0, L.stream>>>(sorted, sorted_idx, start, n, k, gs, out);
-  else knn_grid_query_kernel<32><<<qb, GRID_TPB, 0, L.stream>>>(sorted, sorted_idx, start, n, k, gs, out);
+// Counting sort of the clouds' points into their cells (after launch_clouds).
+cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most) {
+  const dim3 pts(up(most, 256), nclouds);
+  const unsigned nsb = up((int64_t)grid_start_entries(most), SCAN_B);
+  cell_count_kernel<<<pts, 256, 0, L.stream>>>(cs);
+  scan_local_kernel<<<dim3(nsb, nclouds), SCAN_T, 0, L.stream>>>(cs);
+  if (L.counter) *L.counter += 2;
+  if (nsb > 1) {
+    scan_blocks_kernel<<<dim3(1, nclouds), 1024, 0, L.stream>>>(cs);
+    if (L.counter) *L.counter += 1;
+  }
+  cell_scatter_kernel<<<pts, 256, 0, L.stream>>>(cs);
   if (L.counter) *L.counter += 1;
   return cudaGetLastError();
 }
 
-cudaError_t launch_nearest_grid(Launch L, const float4* sorted, const int* sorted_idx, const int* start,
-                                const GridSpec& gs, const float* q3, int nq, int32_t* idx_out, float* key_out) {
+// k nearest neighbours of every point of the sorted clouds.  fused: the key
+// form of clouds below the brute-force limit (grid_key).
+cudaError_t launch_knn_grid(Launch L, const CloudSet& cs, int nclouds, int most, int k, bool fused) {
+  const dim3 grid(up(most, QUERY_WARPS), nclouds);
+  if (fused) knn_query_kernel<true><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, k);
+  else knn_query_kernel<false><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, k);
+  if (L.counter) *L.counter += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_coarse_count(Launch L, const CloudSet& cs, int64_t n, int* ccount) {
+  const unsigned b = up((int64_t)grid_start_entries(n) / 16, 256);
+  coarse_count_kernel<<<b < 608 ? b : 608, 256, 0, L.stream>>>(cs, ccount);
+  if (L.counter) *L.counter += 1;
+  return cudaGetLastError();
+}
+
+// Nearest point of the sorted cloud cs[0] for each of nq queries.  levels 2:
+// far queries search coarse cells; 1: fine cells.
+cudaError_t launch_nearest_grid(Launch L, const CloudSet& cs, int levels, const int* ccount, const float* q3, int nq,
+                                int32_t* idx_out, float* key_out) {
   if (nq <= 0) return cudaSuccess;
-  nearest_grid_kernel<<<(nq + GRID_TPB - 1) / GRID_TPB, GRID_TPB, 0, L.stream>>>(sorted, sorted_idx, start, gs, q3,
-                                                                                nq, idx_out, key_out);
+  nearest_query_kernel<<<up(nq, NEAREST_WARPS), NEAREST_WARPS * 32, 0, L.stream>>>(
+      cs, levels == 1 ? 1 : NEAREST_COARSE, levels == 1 ? nullptr : ccount, q3, nq, idx_out, key_out);
   if (L.counter) *L.counter += 1;
   return cudaGetLastError();
 }
