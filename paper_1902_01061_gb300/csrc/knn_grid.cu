@@ -439,31 +439,31 @@ __device__ __forceinline__ u64 warp_merge(u64 v) {  // v bitonic
 }
 
 // One warp per query (in cell order, so that neighbouring warps read the same
-// cells).  The cube's cells are rows of consecutive cells, i.e. ranges of
+// cells).  A cube's cells are rows of consecutive cells, i.e. ranges of
 // sorted points: each lane looks up one range, the ranges are flattened over
-// the lanes and 32 candidates are keyed at a time.  Those below the k-th key
-// so far wait in a small buffer; 32 of them are sorted across the lanes and
-// merged into the warp's sorted list of the best 32.
-// Bound: issue slots (about 600 warp instructions a query, most of them in the
-// sorts).  Measured on GB300 at 1M points, k = 16: see launch_knn_grid.
+// the lanes and 32 candidates are keyed at a time.
+//
+// Only candidates closer than what the cube certifies (dout) can settle the
+// query, so the others are dropped at once.  If at least k remain they hold
+// the answer: a threshold near the wanted count cuts them to a warp's width
+// (their number grows like the threshold, an area, so interpolation finds it
+// in one or two steps) and each candidate's rank is the number of smaller
+// ones.  If fewer than k remain the cube grows.  A cube with more candidates
+// than the buffer holds goes to knn_stream.
+// Bound: issue slots.  Measured on GB300 at 1M + 1M points, k = 16: see
+// launch_knn_grid.
 constexpr int QUERY_WARPS = 8;
+constexpr int QUERY_CAP = 256;  // candidates a warp keeps
+constexpr int QUERY_PER = QUERY_CAP / 32;
 
+// The search without a limit on the candidates: those below the k-th key so
+// far wait in the buffer, 32 of them are sorted across the lanes and merged
+// into the warp's sorted list of the best 32.  The cube grows by shells.
 template <bool FUSED>
-__global__ void __launch_bounds__(QUERY_WARPS * 32) knn_query_kernel(const CloudSet cs, int k) {
-  __shared__ u64 bufs[QUERY_WARPS][64];
-  const GridCloud& g = cs[blockIdx.y];
+__device__ __noinline__ void knn_stream(const GridCloud& g, float4 q, const float (&q3)[3], const int (&cc)[3],
+                                        const int (&n3)[3], int k, u64* buf) {
   const int lane = threadIdx.x & 31;
-  u64* buf = bufs[threadIdx.x >> 5];
-  const int t = blockIdx.x * QUERY_WARPS + (threadIdx.x >> 5);
-  if (t >= g.n) return;
   const GridSpec& sp = *g.spec;
-  const int n3[3] = {sp.g[0], sp.g[1], sp.g[2]};
-  const float h = sp.h;
-  const float4 q = g.sorted[t];
-  const float q3[3] = {q.x, q.y, q.z};
-  int cc[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) cc[a] = cell_coord(q3[a], sp.o[a], sp.inv_h, n3[a]);
   u64 best = NO_CAND, thr = NO_CAND;
   int cnt = 0;
   auto flush = [&]() {
@@ -512,10 +512,132 @@ __global__ void __launch_bounds__(QUERY_WARPS * 32) knn_query_kernel(const Cloud
       }
     }
     if (cnt > 0) flush();
-    const float dout = outside_distance(q3, sp.o, h, cc, n3, s, sp.extent);
+    const float dout = outside_distance(q3, sp.o, sp.h, cc, n3, s, sp.extent);
     if (dout == INFINITY || certified(cand_key(thr), dout)) break;
   }
   if (lane < k) g.knn[(size_t)__float_as_int(q.w) * k + lane] = (int32_t)(unsigned)best;
+}
+
+template <bool FUSED>
+__global__ void __launch_bounds__(QUERY_WARPS * 32, 5) knn_query_kernel(const CloudSet cs, int k) {
+  __shared__ __align__(16) u64 bufs[QUERY_WARPS][QUERY_CAP];
+  const GridCloud& g = cs[blockIdx.y];
+  const int lane = threadIdx.x & 31;
+  u64* buf = bufs[threadIdx.x >> 5];
+  const int t = blockIdx.x * QUERY_WARPS + (threadIdx.x >> 5);
+  if (t >= g.n) return;
+  const GridSpec& sp = *g.spec;
+  const int n3[3] = {sp.g[0], sp.g[1], sp.g[2]};
+  const float4 q = g.sorted[t];
+  const float q3[3] = {q.x, q.y, q.z};
+  int cc[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) cc[a] = cell_coord(q3[a], sp.o[a], sp.inv_h, n3[a]);
+  const int keep = k <= 24 ? 32 : 64;  // candidates to rank, at most
+  for (int s = 1; s <= 32; s += s < 4 ? 1 : s >> 1) {
+    const float dout = outside_distance(q3, sp.o, sp.h, cc, n3, s, sp.extent);
+    float lim = dout > 0.f ? dout * dout * (1.f - 1e-5f) : 0.f;  // INFINITY where the cube covers the grid
+    const int w = 2 * s + 1, rows = w * w;
+    int cnt = 0;
+    __syncwarp();
+    for (int r0 = 0; r0 < rows && cnt <= QUERY_CAP; r0 += 32) {
+      const int r = r0 + lane;
+      int b = 0, len = 0;
+      if (r < rows) row_range(g, n3, cc[0] - s, cc[0] + s, cc[1] + r % w - s, cc[2] + r / w - s, b, len);
+      const int incl = warp_incl_scan(len);
+      const int total = __shfl_sync(FULL, incl, 31);
+      for (int t0 = 0; t0 < total && cnt <= QUERY_CAP; t0 += 32) {
+        const int pos = flat_position(incl, b, len, t0 + lane);
+        float key = INFINITY, id = 0.f;
+        if (t0 + lane < total) {
+          const float4 c = g.sorted[pos];
+          key = grid_key<FUSED>(q, c);
+          id = c.w;
+        }
+        const unsigned m = __ballot_sync(FULL, key < lim);
+        const int at = cnt + __popc(m & ((1u << lane) - 1));
+        if (key < lim && at < QUERY_CAP) buf[at] = pack_cand(key, id);
+        cnt += __popc(m);
+      }
+    }
+    if (cnt > QUERY_CAP) break;
+    if (cnt < k) {
+      if (lim == INFINITY) break;
+      continue;
+    }
+    __syncwarp();
+    if (cnt > keep) {
+      u64 c[QUERY_PER];
+      float top = 0.f;
+#pragma unroll
+      for (int j = 0; j < QUERY_PER; ++j) {
+        c[j] = j * 32 + lane < cnt ? buf[j * 32 + lane] : NO_CAND;
+        if (j * 32 + lane < cnt) top = fmaxf(top, cand_key(c[j]));
+      }
+      if (lim == INFINITY) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(FULL, top, off));
+        lim = top;
+      }
+      // a threshold below which k to `keep` candidates lie
+      float lo = 0.f, hi = lim, nlo = 0.f, nhi = (float)cnt;
+      const float want = 0.5f * (float)(k + keep);
+      bool found = false;
+      for (int it = 0; it < 24; ++it) {
+        const float f = fminf(fmaxf(__fdividef(want - nlo, nhi - nlo), 0.1f), 0.9f);
+        const float mid = fmaf(hi - lo, f, lo);
+        int below = 0;
+#pragma unroll
+        for (int j = 0; j < QUERY_PER; ++j)
+          if (j * 32 < cnt) below += __popc(__ballot_sync(FULL, cand_key(c[j]) < mid));  // NO_CAND: NaN, not below
+        if (below < k) {
+          lo = mid;
+          nlo = (float)below;
+        } else if (below > keep) {
+          hi = mid;
+          nhi = (float)below;
+        } else {
+          lim = mid;
+          found = true;
+          break;
+        }
+      }
+      if (!found) break;
+      __syncwarp();
+      cnt = 0;
+#pragma unroll
+      for (int j = 0; j < QUERY_PER; ++j) {
+        const bool in = cand_key(c[j]) < lim;
+        const unsigned m = __ballot_sync(FULL, in);
+        if (in) buf[cnt + __popc(m & ((1u << lane) - 1))] = c[j];
+        cnt += __popc(m);
+      }
+      __syncwarp();
+    }
+    // ranks in the (key, index) order: the number of smaller candidates
+    int32_t* out = g.knn + (size_t)__float_as_int(q.w) * k;
+    if (lane == 0) buf[cnt] = NO_CAND;  // read in pairs (cnt <= QUERY_CAP - 1 here: keep < QUERY_CAP)
+    __syncwarp();
+    const u64 c0 = lane < cnt ? buf[lane] : NO_CAND;
+    int r0 = 0;
+    for (int j = 0; j < cnt; j += 2) {
+      const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(buf + j);
+      r0 += (o.x < c0 ? 1 : 0) + (o.y < c0 ? 1 : 0);
+    }
+    if (lane < cnt && r0 < k) out[r0] = (int32_t)(unsigned)c0;
+    if (cnt > 32) {
+      const u64 c1 = lane + 32 < cnt ? buf[lane + 32] : NO_CAND;
+      int r1 = 0;
+      for (int j = 0; j < cnt; j += 2) {
+        const ulonglong2 o = *reinterpret_cast<const ulonglong2*>(buf + j);
+        r1 += (o.x < c1 ? 1 : 0) + (o.y < c1 ? 1 : 0);
+      }
+      if (lane + 32 < cnt && r1 < k) out[r1] = (int32_t)(unsigned)c1;
+    }
+    return;
+  }
+  __syncwarp();
+  knn_stream<FUSED>(g, q, q3, cc, n3, k, buf);
 }
 
 // ---- nearest gridded point of external queries -----------------------------------
