@@ -58,7 +58,7 @@ scgr_status scgr_create(const scgr_params* params, void* cuda_stream, scgr_ctx**
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->pose_eval, sizeof(DevPose));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->aux, sizeof(double) * 64);
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->errword, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->red, sizeof(double) * (RED_MAX_BLOCKS * 6 + 32));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->red, sizeof(double) * CLOUD_SCRATCH_DOUBLES);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->errword, 0, sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->pose, 0, sizeof(DevPose), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->stats, 0, sizeof(DevStats), c->stream);
@@ -95,7 +95,7 @@ void scgr_destroy(scgr_ctx* c) {
                     &c->bcpair, &c->btabX, &c->btabY, &c->bxoff, &c->byoff, &c->bstats, &c->bposes, &c->bnext,
                     &c->gspec, &c->gcell[0], &c->gcell[1], &c->gstart[0], &c->gstart[1], &c->gtot[0], &c->gtot[1],
                     &c->gsorted[0], &c->gsorted[1], &c->gccount,
-                    &c->cd_key, &c->cd_moved, &c->wstore, &c->wupart, &c->wpartial, &c->mpart, &c->mom, &c->radpart};
+                    &c->cd_key, &c->cd_moved, &c->wstore, &c->wupart, &c->wpartial, &c->mpart, &c->mom, &c->radpart, &c->sigpart};
   for (DevBuf* b : bufs) release(*b);
   if (c->pose) cudaFree(c->pose);
   if (c->pose_eval) cudaFree(c->pose_eval);
@@ -326,7 +326,7 @@ scgr_status scgr_set_curvature(scgr_ctx* c, int which, const double* a64_dev) {
   SCGR_CK(c, cudaMemcpyAsync(a64.p, a64_dev, (size_t)n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
   SCGR_CK(c, launch_check_curvature(L, (const double*)a64.p, n, (float*)a32.p, c->errword));
   DevStats* st = c->stats;
-  SCGR_CK(c, launch_sigma(L, (const double*)c->aX64.p, (int)c->n, c->prm.sigma, 1.0, c->red, st));
+  SCGR_CK(c, launch_sigma(L, (const double*)c->aX64.p, (int)c->n, c->prm.sigma, 1.0, (double*)c->sigpart.p, st));
   SCGR_CK(c, launch_records(L, (const float4*)c->X4.p, (const double*)c->aX64.p, (int)c->n, (int)c->npad,
                             (const float4*)c->Y4.p, (const double*)c->aY64.p, (int)c->m, (int)c->mpad,
                             c->prm.g_mode, st, (float4*)c->Xr.p, (float2*)c->XA.p, (float4*)c->Y0r.p));

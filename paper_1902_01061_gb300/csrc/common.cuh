@@ -70,15 +70,6 @@ struct StepParams {
 
 // ---- fixed-order float64 reductions ------------------------------------
 constexpr int RED_THREADS = 256;
-constexpr int RED_MAX_BLOCKS = 1024;
-
-inline int red_blocks(int64_t n) {
-  int64_t b = (n + RED_THREADS - 1) / RED_THREADS;
-  if (b < 1) b = 1;
-  if (b > RED_MAX_BLOCKS) b = RED_MAX_BLOCKS;
-  return (int)b;
-}
-
 // Sum v[0..NV) over the block in a fixed tree order; thread 0 gets the result.
 template <int NV>
 __device__ __forceinline__ void block_sum(double (&v)[NV], double (*sh)[RED_THREADS]) {
@@ -280,6 +271,8 @@ struct GridSpec {
 constexpr int GRID_CELLS_PER_POINT = 4;  // at most this many cells per point
 constexpr int SCAN_B = 4096;             // cells per block of the count scan
 constexpr int CLOUD_PARTS = 256;         // blocks of a cloud's reductions, at most
+// scratch of launch_clouds for two clouds: 6 doubles, then 6 floats a part
+constexpr int CLOUD_SCRATCH_DOUBLES = 2 * CLOUD_PARTS * 9;
 
 // One cloud of the descriptor pass: its points, grid arrays and outputs.
 struct GridCloud {
@@ -311,7 +304,11 @@ cudaError_t launch_knn(Launch L, const float4* P, int n, int k, int32_t* out);
 cudaError_t launch_curvature(Launch L, const float4* P, const int32_t* nbr, int n, int k,
                              double* a64, float* a32);
 cudaError_t launch_curvature2(Launch L, const float4* X, const int32_t* nx, int n, double* ax64, float* ax32,
-                              const float4* Y, const int32_t* ny, int m, double* ay64, float* ay32, int k);
+                              double* xpart, const float4* Y, const int32_t* ny, int m, double* ay64, float* ay32,
+                              int k);
+size_t sigma_part_bytes(int64_t n);
+cudaError_t launch_sigma_finish(Launch L, const double* part, int n, double sigma_user, double sigma_scale,
+                                DevStats* st);
 // sigma = population std of a64 (1 if below 1e-12), or `sigma_user` if > 0
 cudaError_t launch_sigma(Launch L, const double* a64, int n, double sigma_user, double sigma_scale, double* part,
                          DevStats* st);
@@ -324,9 +321,9 @@ cudaError_t launch_stats_multi(Launch L, const float4* X4, const float4* Y4, con
                                const BatchPair* pairs, int npairs, double sigma_user, DevStats* out);
 size_t grid_start_entries(int64_t n);
 size_t grid_tot_entries(int64_t n);
-cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, bool scatter, double* part,
+cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, bool scatter, bool sorted, double* part,
                           float* bpart);
-cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most);
+cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most, const double* part);
 cudaError_t launch_knn_grid(Launch L, const CloudSet& cs, int nclouds, int most, int k, bool fused);
 constexpr int NEAREST_COARSE = 4;  // fine cells per coarse cell side in the two-level nearest search
 cudaError_t launch_coarse_count(Launch L, const CloudSet& cs, int64_t n, int* ccount);
@@ -337,7 +334,8 @@ cudaError_t launch_nearest(Launch L, const float4* P, int n, const float* q3, in
 cudaError_t launch_threshold(Launch L, const float* key, int nq, float thr2, uint8_t* mask, float* dist);
 size_t radius_scratch_bytes(int n, int num_sms);
 cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const double* e_dev, double scale2,
-                                    const GridSpec* spec, int num_sms, double* part, double* a64, float* a32);
+                                    const GridSpec* spec, int num_sms, double* part, double* a64, float* a32,
+                                    double* sigma_out);
 cudaError_t launch_check_curvature(Launch L, const double* a64, int n, float* a32, int* err);
 cudaError_t launch_records(Launch L, const float4* X4, const double* aX64, int n, int npad,
                            const float4* Y4, const double* aY64, int m, int mpad, int g_mode,

@@ -205,14 +205,16 @@ scgr_status prepare_clouds(scgr_ctx* c) {
     cs.one[w] = grid_cloud(c, w, grid_knn(c, w), true);
   }
   const int most = (int)(c->n > c->m ? c->n : c->m);
-  double* part = c->red;
-  SCGR_CK(c, launch_clouds(c->L(), cs, 2, most, true, part, (float*)(part + 2 * CLOUD_PARTS * 6)));
+  double* part = c->red;  // CLOUD_SCRATCH_DOUBLES
+  SCGR_CK(c, launch_clouds(c->L(), cs, 2, most, true, grid_knn(c, 0) && grid_knn(c, 1), part,
+                           (float*)(part + 2 * CLOUD_PARTS * 6)));
   if (grid_knn(c, 0) && grid_knn(c, 1)) {
-    SCGR_CK(c, launch_grid_sort(c->L(), cs, 2, most));
+    SCGR_CK(c, launch_grid_sort(c->L(), cs, 2, most, part));
   } else if (grid_knn(c, 0) || grid_knn(c, 1)) {
     const int w = grid_knn(c, 0) ? 0 : 1;
     cs.one[0] = cs.one[w];
-    SCGR_CK(c, launch_grid_sort(c->L(), cs, 1, cs.one[0].n));
+    cs.one[0].scatter = nullptr;  // finished above
+    SCGR_CK(c, launch_grid_sort(c->L(), cs, 1, cs.one[0].n, part));
   }
   for (int w = 0; w < 2; ++w) c->grid_ok[w] = grid_knn(c, w);
   c->coarse_ok = false;
@@ -271,8 +273,8 @@ scgr_status nearest_reference(scgr_ctx* c, const float* q3, int nq, int32_t* idx
     const scgr_status st = grid_buffers(c, 0);
     if (st != SCGR_OK) return st;
     cs.one[0] = grid_cloud(c, 0, true, false);
-    SCGR_CK(c, launch_clouds(c->L(), cs, 1, n, false, c->red, (float*)(c->red + 2 * CLOUD_PARTS * 6)));
-    SCGR_CK(c, launch_grid_sort(c->L(), cs, 1, n));
+    SCGR_CK(c, launch_clouds(c->L(), cs, 1, n, false, false, c->red, (float*)(c->red + 2 * CLOUD_PARTS * 6)));
+    SCGR_CK(c, launch_grid_sort(c->L(), cs, 1, n, c->red));
     c->grid_ok[0] = true;
     c->coarse_ok = false;
   }
@@ -294,6 +296,7 @@ scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_sca
   const float4* X4 = (const float4*)c->X4.p;
   const float4* Y4 = (const float4*)c->Y4.p;
   DevStats* st = c->stats;
+  SCGR_CK(c, ensure(c->sigpart, sigma_part_bytes(n)));
   if (c->prm.neigh_mode == 0) {
     SCGR_CK(c, ensure(c->knnX, (size_t)n * k * sizeof(int32_t)));
     SCGR_CK(c, ensure(c->knnY, (size_t)m * k * sizeof(int32_t)));
@@ -304,8 +307,8 @@ scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_sca
       c->prm.k = k_prev;
       return ks;
     }
-    SCGR_CK(c, launch_curvature2(L, X4, (const int32_t*)c->knnX.p, n, (double*)c->aX64.p, (float*)c->aX32.p, Y4,
-                                 (const int32_t*)c->knnY.p, m, (double*)c->aY64.p, (float*)c->aY32.p, k));
+    SCGR_CK(c, launch_curvature2(L, X4, (const int32_t*)c->knnX.p, n, (double*)c->aX64.p, (float*)c->aX32.p,
+                                 (double*)c->sigpart.p, Y4, (const int32_t*)c->knnY.p, m, (double*)c->aY64.p, (float*)c->aY32.p, k));
   } else {
     c->prm.radius_scale = radius_scale;
     const double s2 = radius_scale * radius_scale;
@@ -313,12 +316,12 @@ scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_sca
     SCGR_CK(c, ensure(c->radpart, bx > by ? bx : by));
     const GridSpec* spec = (const GridSpec*)c->gspec.p;
     SCGR_CK(c, launch_radius_curvature(L, X4, n, &st->eX, s2, spec, c->num_sms, (double*)c->radpart.p,
-                                       (double*)c->aX64.p, (float*)c->aX32.p));
+                                       (double*)c->aX64.p, (float*)c->aX32.p, (double*)c->sigpart.p));
     SCGR_CK(c, launch_radius_curvature(L, Y4, m, &st->eY0, s2, spec + 1, c->num_sms, (double*)c->radpart.p,
-                                       (double*)c->aY64.p, (float*)c->aY32.p));
+                                       (double*)c->aY64.p, (float*)c->aY32.p, nullptr));
   }
   const double user = c->prm.sigma > 0.0 ? c->prm.sigma * sigma_scale : 0.0;
-  SCGR_CK(c, launch_sigma(L, (const double*)c->aX64.p, n, user, sigma_scale, c->red, st));
+  SCGR_CK(c, launch_sigma_finish(L, (const double*)c->sigpart.p, n, user, sigma_scale, st));
   return SCGR_OK;
 }
 

@@ -265,6 +265,108 @@ cudaError_t launch_knn(Launch L, const float4* P, int n, int k, int32_t* out) {
   return after_launch(L);
 }
 
+constexpr int CURV_TPB = 128;  // points per block of the curvature kernels
+
+// ---- sigma of Eq. 3 ----------------------------------------------------------
+// The population std of the reference curvatures from per-block sums and
+// squared deviations about the block's own mean (sigma_part), merged in a fixed
+// order: M2 = sum_b [M2_b + n_b (mean_b - mean)^2], as accurate as a second pass
+// over the points without reading them again.
+__device__ __forceinline__ void sigma_part(double a, bool live, int n_block, double* __restrict__ part) {
+  __shared__ double sh[2][CURV_TPB / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double v = live ? a : 0.0;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if (lane == 0) sh[0][warp] = v;
+  __syncthreads();
+  double sum = sh[0][0];
+#pragma unroll
+  for (int w = 1; w < CURV_TPB / 32; ++w) sum += sh[0][w];
+  const double d = live ? a - sum / (double)n_block : 0.0;
+  v = d * d;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if (lane == 0) sh[1][warp] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double m2 = sh[1][0];
+#pragma unroll
+    for (int w = 1; w < CURV_TPB / 32; ++w) m2 += sh[1][w];
+    part[2 * (size_t)blockIdx.x] = sum;
+    part[2 * (size_t)blockIdx.x + 1] = m2;
+  }
+}
+
+__global__ void __launch_bounds__(CURV_TPB) sigma_parts_kernel(const double* __restrict__ a64, int n,
+                                                              double* __restrict__ part) {
+  const int i = blockIdx.x * CURV_TPB + threadIdx.x;
+  sigma_part(i < n ? a64[i] : 0.0, i < n, min(CURV_TPB, n - (int)blockIdx.x * CURV_TPB), part);
+}
+
+// sigma (the caller's, or the std, 1 below 1e-12, times sigma_scale) and the
+// factor sqrt(log2 e) / sigma that the force records use.
+__device__ __forceinline__ void finish_sigma(double sum_a, double sum_d2, int64_t n, double sigma_user,
+                                             double sigma_scale, DevStats* st) {
+  st->asum[0] = sum_a;
+  double sigma = sigma_user;
+  if (!(sigma > 0.0)) {
+    const double sd = sqrt(sum_d2 / (double)n);
+    sigma = sd >= 1e-12 ? sd : 1.0;
+    if (sigma_scale != 1.0) sigma *= sigma_scale;
+  }
+  st->sigma = sigma;
+  st->kscale = SQRT_LOG2E / sigma;
+}
+
+constexpr int SIGMA_T = 256;
+
+__device__ __forceinline__ double sigma_block_sum(double v, double* sh) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = sh[0];
+#pragma unroll
+  for (int w = 1; w < SIGMA_T / 32; ++w) v += sh[w];
+  __syncthreads();
+  return v;
+}
+
+__global__ void __launch_bounds__(SIGMA_T) sigma_finish_kernel(const double* __restrict__ part, int n,
+                                                              double sigma_user, double sigma_scale, DevStats* st) {
+  __shared__ double sh[SIGMA_T / 32];
+  const int nb = (n + CURV_TPB - 1) / CURV_TPB;
+  double v = 0.0;
+  for (int b = threadIdx.x; b < nb; b += SIGMA_T) v += part[2 * (size_t)b];
+  const double sum = sigma_block_sum(v, sh), mean = sum / (double)n;
+  v = 0.0;
+  for (int b = threadIdx.x; b < nb; b += SIGMA_T) {
+    const double nbk = (double)min(CURV_TPB, n - b * CURV_TPB);
+    const double d = part[2 * (size_t)b] - nbk * mean;  // n_b (mean_b - mean)
+    v += fma(d * d, b < nb - 1 ? 1.0 / CURV_TPB : 1.0 / nbk, part[2 * (size_t)b + 1]);
+  }
+  const double d2 = sigma_block_sum(v, sh);
+  if (threadIdx.x == 0) finish_sigma(sum, d2, n, sigma_user, sigma_scale, st);
+}
+
+size_t sigma_part_bytes(int64_t n) { return (size_t)((n + CURV_TPB - 1) / CURV_TPB) * 2 * sizeof(double); }
+
+// From the parts that the curvature kernels wrote.
+cudaError_t launch_sigma_finish(Launch L, const double* part, int n, double sigma_user, double sigma_scale,
+                                DevStats* st) {
+  sigma_finish_kernel<<<1, SIGMA_T, 0, L.stream>>>(part, n, sigma_user, sigma_scale, st);
+  return after_launch(L);
+}
+
+// From curvatures of any origin.
+cudaError_t launch_sigma(Launch L, const double* a64, int n, double sigma_user, double sigma_scale, double* part,
+                         DevStats* st) {
+  sigma_parts_kernel<<<(n + CURV_TPB - 1) / CURV_TPB, CURV_TPB, 0, L.stream>>>(a64, n, part);
+  if (L.counter) ++*L.counter;
+  return launch_sigma_finish(L, part, n, sigma_user, sigma_scale, st);
+}
+
 // (h, l) += x, h the rounded sum (two-sum)
 __device__ __forceinline__ void two_sum_add(float& h, float& l, float x) {
   const float t = __fadd_rn(h, x);
@@ -365,30 +467,35 @@ struct CurvatureIn {
   int n;
   double* a64;
   float* a32;
+  double* part;  // sigma_part's output (NULL: not wanted)
 };
-constexpr int CURV_TPB = 128;
 
 // Both clouds of a registration in one launch (blockIdx.y).
 __global__ void __launch_bounds__(CURV_TPB) curvature_kernel(const CurvatureIn c0, const CurvatureIn c1, int k) {
   const CurvatureIn& c = blockIdx.y == 0 ? c0 : c1;
   const int i = blockIdx.x * CURV_TPB + threadIdx.x;
-  if (i >= c.n) return;
-  const double a = point_curvature(c.P, c.nbr + (int64_t)i * k, k, i);
-  c.a64[i] = a;
-  c.a32[i] = (float)a;
+  if ((int)blockIdx.x * CURV_TPB >= c.n) return;
+  double a = 0.0;
+  if (i < c.n) {
+    a = point_curvature(c.P, c.nbr + (int64_t)i * k, k, i);
+    c.a64[i] = a;
+    c.a32[i] = (float)a;
+  }
+  if (c.part) sigma_part(a, i < c.n, min(CURV_TPB, c.n - (int)blockIdx.x * CURV_TPB), c.part);
 }
 
 cudaError_t launch_curvature2(Launch L, const float4* X, const int32_t* nx, int n, double* ax64, float* ax32,
-                              const float4* Y, const int32_t* ny, int m, double* ay64, float* ay32, int k) {
+                              double* xpart, const float4* Y, const int32_t* ny, int m, double* ay64, float* ay32,
+                              int k) {
   const int most = n > m ? n : m;
   curvature_kernel<<<dim3((most + CURV_TPB - 1) / CURV_TPB, Y ? 2 : 1), CURV_TPB, 0, L.stream>>>(
-      CurvatureIn{X, nx, n, ax64, ax32}, CurvatureIn{Y, ny, m, ay64, ay32}, k);
+      CurvatureIn{X, nx, n, ax64, ax32, xpart}, CurvatureIn{Y, ny, m, ay64, ay32, nullptr}, k);
   return after_launch(L);
 }
 
 cudaError_t launch_curvature(Launch L, const float4* P, const int32_t* nbr, int n, int k,
                              double* a64, float* a32) {
-  return launch_curvature2(L, P, nbr, n, a64, a32, nullptr, nullptr, 0, nullptr, nullptr, k);
+  return launch_curvature2(L, P, nbr, n, a64, a32, nullptr, nullptr, nullptr, 0, nullptr, nullptr, k);
 }
 
 // ---- radius neighbourhood curvature (Sec. IV) ----------------------------
@@ -563,11 +670,11 @@ __global__ void __launch_bounds__(RAD_TPB)
 
 // The splits' sums of a point added in order, its covariance (a power-of-two
 // scaling leaves a = lambda_min / trace unchanged) and its curvature.
-__global__ void __launch_bounds__(RAD_TPB)
+__global__ void __launch_bounds__(CURV_TPB)
     radius_curvature_kernel(const double* __restrict__ part, int S, int n, double* __restrict__ a64,
-                            float* __restrict__ a32) {
-  const int i = blockIdx.x * RAD_TPB + threadIdx.x;
-  if (i >= n) return;
+                            float* __restrict__ a32, double* __restrict__ sigma_out) {
+  const int i0 = blockIdx.x * CURV_TPB + threadIdx.x;
+  const int i = min(i0, n - 1);
   double v[RAD_NS];
 #pragma unroll
   for (int f = 0; f < RAD_NS; ++f) v[f] = part[(size_t)f * n + i];
@@ -582,8 +689,11 @@ __global__ void __launch_bounds__(RAD_TPB)
   C[4] = fma(v[7], ik, -my * my); C[5] = fma(v[8], ik, -my * mz); C[8] = fma(v[9], ik, -mz * mz);
   C[3] = C[1]; C[6] = C[2]; C[7] = C[5];
   const double a = surface_variation(C);
-  a64[i] = a;
-  a32[i] = (float)a;
+  if (i0 < n) {
+    a64[i] = a;
+    a32[i] = (float)a;
+  }
+  if (sigma_out) sigma_part(a, i0 < n, min(CURV_TPB, n - (int)blockIdx.x * CURV_TPB), sigma_out);
 }
 
 // Splits of the cloud, so that a small one still gives every SM about eight
@@ -597,143 +707,16 @@ int radius_splits(int n, int num_sms) {
 }
 size_t radius_scratch_bytes(int n, int num_sms) { return (size_t)radius_splits(n, num_sms) * RAD_NS * n * sizeof(double); }
 
-// spec: the cloud's grid (launch_clouds; its extent); part: radius_scratch_bytes.
+// spec: the cloud's grid (launch_clouds; its extent); part: radius_scratch_bytes;
+// sigma_out: sigma_part's output (NULL: not wanted).
 cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const double* e_dev, double scale2,
-                                    const GridSpec* spec, int num_sms, double* part, double* a64, float* a32) {
+                                    const GridSpec* spec, int num_sms, double* part, double* a64, float* a32,
+                                    double* sigma_out) {
   const int blocks = (n + RAD_TPB - 1) / RAD_TPB, ntiles = (n + RAD_TILE - 1) / RAD_TILE;
   const int S = radius_splits(n, num_sms);
   radius_sums_kernel<<<dim3(blocks, S), RAD_TPB, 0, L.stream>>>(P, n, e_dev, scale2, spec, (ntiles + S - 1) / S, part);
-  radius_curvature_kernel<<<blocks, RAD_TPB, 0, L.stream>>>(part, S, n, a64, a32);
+  radius_curvature_kernel<<<(n + CURV_TPB - 1) / CURV_TPB, CURV_TPB, 0, L.stream>>>(part, S, n, a64, a32, sigma_out);
   if (L.counter) *L.counter += 2;
-  return cudaGetLastError();
-}
-
-// ---- fixed-order float64 reductions ------------------------------------
-// Pass 1: per-block sums of an NV-vector per point (fixed grid, fixed order).
-struct SumA {
-  const double* a;
-  __device__ void operator()(int64_t i, double (&v)[1]) const { v[0] += a[i]; }
-};
-struct VarA {
-  const double* a;
-  const double* mean_sum;  // sum of a; mean = sum / n
-  double inv_n;
-  __device__ void operator()(int64_t i, double (&v)[1]) const {
-    const double d = a[i] - mean_sum[0] * inv_n;
-    v[0] += d * d;
-  }
-};
-
-template <int NV, class Fn>
-__global__ void __launch_bounds__(RED_THREADS) reduce_pass_kernel(int64_t n, Fn fn, double* part) {
-  __shared__ double sh[NV][RED_THREADS];
-  double v[NV];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = 0.0;
-  const int64_t stride = (int64_t)gridDim.x * RED_THREADS;
-  for (int64_t i = blockIdx.x * (int64_t)RED_THREADS + threadIdx.x; i < n; i += stride) fn(i, v);
-  block_sum<NV>(v, sh);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) part[blockIdx.x * NV + q] = v[q];
-  }
-}
-
-// Pass 2: one block sums the per-block partials in fixed order into out[NV].
-template <int NV>
-__global__ void __launch_bounds__(RED_THREADS) reduce_final_kernel(const double* part, int nb,
-                                                                   double* out) {
-  __shared__ double sh[NV][RED_THREADS];
-  double v[NV];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = 0.0;
-  for (int b = threadIdx.x; b < nb; b += RED_THREADS) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) v[q] += part[b * NV + q];
-  }
-  block_sum<NV>(v, sh);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) out[q] = v[q];
-  }
-}
-
-// sigma of Eq. 3 (the caller's, or the population std of the reference
-// curvatures, 1 below 1e-12, times sigma_scale) and the factor sqrt(log2 e) /
-// sigma that the force records use.
-__device__ __forceinline__ void finish_sigma(double sum_a, double sum_d2, int64_t n, double sigma_user,
-                                             double sigma_scale, DevStats* st) {
-  st->asum[0] = sum_a;
-  double sigma = sigma_user;
-  if (!(sigma > 0.0)) {
-    const double sd = sqrt(sum_d2 / (double)n);
-    sigma = sd >= 1e-12 ? sd : 1.0;
-    if (sigma_scale != 1.0) sigma *= sigma_scale;
-  }
-  st->sigma = sigma;
-  st->kscale = SQRT_LOG2E / sigma;
-}
-
-__global__ void sigma_finish_kernel(const double* sums, int64_t n, double sigma_user, double sigma_scale,
-                                    DevStats* st) {
-  if (threadIdx.x == 0) finish_sigma(sums[0], sums[1], n, sigma_user, sigma_scale, st);
-}
-
-// Small clouds: both passes (mean, then squared deviations) in one block.
-constexpr int SIGMA_ONE_MAX = 16384;
-constexpr int SIGMA_T = 1024;
-
-__device__ __forceinline__ double sigma_block_sum(double v, double* sh) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  v = sh[threadIdx.x & 31];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  __syncthreads();
-  return v;
-}
-
-__global__ void __launch_bounds__(SIGMA_T) sigma_one_kernel(const double* __restrict__ a64, int n, double sigma_user,
-                                                            double sigma_scale, DevStats* st) {
-  __shared__ double sh[32];
-  double a[SIGMA_ONE_MAX / SIGMA_T], v = 0.0;
-#pragma unroll
-  for (int u = 0; u < SIGMA_ONE_MAX / SIGMA_T; ++u) {
-    const int i = u * SIGMA_T + threadIdx.x;
-    if (u * SIGMA_T < n) {
-      a[u] = i < n ? a64[i] : 0.0;
-      v += a[u];
-    }
-  }
-  const double sum = sigma_block_sum(v, sh), mean = sum / (double)n;
-  v = 0.0;
-#pragma unroll
-  for (int u = 0; u < SIGMA_ONE_MAX / SIGMA_T; ++u) {
-    if (u * SIGMA_T < n) {
-      const double d = u * SIGMA_T + threadIdx.x < n ? a[u] - mean : 0.0;
-      v += d * d;
-    }
-  }
-  const double d2 = sigma_block_sum(v, sh);
-  if (threadIdx.x == 0) finish_sigma(sum, d2, n, sigma_user, sigma_scale, st);
-}
-
-cudaError_t launch_sigma(Launch L, const double* a64, int n, double sigma_user, double sigma_scale, double* part,
-                         DevStats* st) {
-  if (n <= SIGMA_ONE_MAX) {
-    sigma_one_kernel<<<1, SIGMA_T, 0, L.stream>>>(a64, n, sigma_user, sigma_scale, st);
-    return after_launch(L);
-  }
-  const int nb = red_blocks(n);
-  double* sums = part + (size_t)RED_MAX_BLOCKS * 6 + 8;  // [0]: sum a, [1]: sum (a - mean)^2
-  reduce_pass_kernel<1, SumA><<<nb, RED_THREADS, 0, L.stream>>>(n, SumA{a64}, part);
-  reduce_final_kernel<1><<<1, RED_THREADS, 0, L.stream>>>(part, nb, sums);
-  reduce_pass_kernel<1, VarA><<<nb, RED_THREADS, 0, L.stream>>>(n, VarA{a64, sums, 1.0 / n}, part);
-  reduce_final_kernel<1><<<1, RED_THREADS, 0, L.stream>>>(part, nb, sums + 1);
-  sigma_finish_kernel<<<1, 32, 0, L.stream>>>(sums, n, sigma_user, sigma_scale, st);
-  if (L.counter) *L.counter += 5;
   return cudaGetLastError();
 }
 

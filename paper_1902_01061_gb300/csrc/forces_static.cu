@@ -40,9 +40,10 @@ constexpr size_t OFF_Y0R = OFF_XA + al256(8 * STATIC_MAX_POINTS);
 constexpr size_t OFF_PART = OFF_Y0R + al256(16 * STATIC_MPAD_MAX);
 constexpr size_t OFF_BLK = OFF_PART + al256(16 * STATIC_MAX_SPLITS * STATIC_MPAD_MAX);
 constexpr size_t OFF_RED = OFF_BLK + al256(8 * 13 * (STATIC_MPAD_MAX / 256 + 1));
-constexpr size_t OFF_A32X = OFF_RED + al256(8 * (RED_MAX_BLOCKS * 6 + 32));
+constexpr size_t OFF_A32X = OFF_RED + al256(8 * CLOUD_SCRATCH_DOUBLES);
 constexpr size_t OFF_A32Y = OFF_A32X + al256(4 * STATIC_MAX_POINTS);
-constexpr size_t OFF_STATS = OFF_A32Y + al256(4 * STATIC_MAX_POINTS);
+constexpr size_t OFF_SIG = OFF_A32Y + al256(4 * STATIC_MAX_POINTS);
+constexpr size_t OFF_STATS = OFF_SIG + al256(16 * (STATIC_MAX_POINTS / 128 + 1));
 constexpr size_t OFF_POSE = OFF_STATS + al256(sizeof(DevStats));
 constexpr size_t OFF_SPEC = OFF_POSE + al256(sizeof(DevPose));
 constexpr size_t OFF_ERR = OFF_SPEC + al256(2 * sizeof(GridSpec));
@@ -149,8 +150,8 @@ extern "C" scgr_status scgr_forces_static(const float* x_dev, int64_t n, const f
   cs.one[1].spec = spec + 1;
   cs.one[1].mean = stats->ybar0;
   if (e == cudaSuccess)
-    e = launch_clouds(L, cs, 2, (int)(n > m ? n : m), false, red, reinterpret_cast<float*>(red + 2 * CLOUD_PARTS * 6));
-  if (e == cudaSuccess) e = launch_sigma(L, ax_dev, (int)n, sigma, 1.0, red, stats);
+    e = launch_clouds(L, cs, 2, (int)(n > m ? n : m), false, false, red, reinterpret_cast<float*>(red + 2 * CLOUD_PARTS * 6));
+  if (e == cudaSuccess) e = launch_sigma(L, ax_dev, (int)n, sigma, 1.0, reinterpret_cast<double*>(base + OFF_SIG), stats);
   if (e == cudaSuccess)
     e = launch_records(L, X4, ax_dev, (int)n, (int)npad, Y4, ay_dev, (int)m, (int)mpad, g_mode, stats, Xr, XA, Y0r);
   if (e == cudaSuccess) e = launch_pose_init(L, pose, stats, 1);

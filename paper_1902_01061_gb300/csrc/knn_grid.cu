@@ -199,13 +199,12 @@ __global__ void __launch_bounds__(RED_THREADS) cloud_scatter_kernel(const CloudS
   }
 }
 
-// One block per cloud: its scatter matrix and the largest eigenvalue of scatter / n.
-__global__ void __launch_bounds__(RED_THREADS) cloud_lmax_kernel(const CloudSet cs, const double* __restrict__ part) {
+// One block: cloud y's scatter matrix and the largest eigenvalue of scatter / n.
+__device__ void cloud_lmax(const GridCloud& g, int y, const double* __restrict__ part) {
   __shared__ double sh[RED_THREADS / 32][6];
-  const GridCloud& g = cs[blockIdx.y];
   if (!g.scatter) return;
   const int nb = cloud_parts(g.n);
-  const size_t o = (size_t)blockIdx.y * CLOUD_PARTS + threadIdx.x;
+  const size_t o = (size_t)y * CLOUD_PARTS + threadIdx.x;
   double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   if ((int)threadIdx.x < nb)
 #pragma unroll
@@ -222,6 +221,9 @@ __global__ void __launch_bounds__(RED_THREADS) cloud_lmax_kernel(const CloudSet 
   }
   *g.lmax = sym3_max_eigenvalue(C);
 }
+__global__ void __launch_bounds__(RED_THREADS) cloud_lmax_kernel(const CloudSet cs, const double* __restrict__ part) {
+  cloud_lmax(cs[blockIdx.y], blockIdx.y, part);
+}
 
 // ---- counting sort into cells ---------------------------------------------------
 
@@ -237,10 +239,16 @@ __device__ __forceinline__ int cell_coord(float v, float o, float inv_h, int g) 
 // count scan keeps a block-local part per cell and one offset per block.
 __device__ __forceinline__ int cell_start(const GridCloud& g, int c) { return g.start[c] + g.tot[c / SCAN_B]; }
 
-// The cell of every point and its rank of arrival there.
-__global__ void __launch_bounds__(256) cell_count_kernel(const CloudSet cs) {
+// The cell of every point and its rank of arrival there.  Block 0 of a cloud
+// finishes the cloud's statistics meanwhile (a float64 latency chain).
+__global__ void __launch_bounds__(256) cell_count_kernel(const CloudSet cs, const double* __restrict__ part) {
+  static_assert(RED_THREADS == 256, "cloud_lmax runs in one of these blocks");
   const GridCloud& g = cs[blockIdx.y];
-  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (blockIdx.x == 0) {
+    cloud_lmax(g, blockIdx.y, part);
+    return;
+  }
+  const int i = (blockIdx.x - 1) * 256 + threadIdx.x;
   if (i >= g.n) return;
   const GridSpec& sp = *g.spec;
   const float4 c = g.P[i];
@@ -776,7 +784,9 @@ size_t grid_tot_entries(int64_t n) { return grid_start_entries(n) / SCAN_B + 2; 
 // covariance eigenvalues of those that ask for them.  part: nclouds x
 // CLOUD_PARTS x 6 doubles, bpart the same of floats.  most: points of the
 // largest cloud.
-cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, bool scatter, double* part,
+// sorted: launch_grid_sort of the same clouds and part follows, which finishes
+// the scatter matrices.
+cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, bool scatter, bool sorted, double* part,
                           float* bpart) {
   const dim3 grid(cloud_parts(most), nclouds), one(1, nclouds);
   cloud_sums_kernel<<<grid, RED_THREADS, 0, L.stream>>>(cs, part, bpart);
@@ -786,7 +796,7 @@ cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, b
     cloud_scatter_kernel<<<grid, RED_THREADS, 0, L.stream>>>(cs, part);
     if (L.counter) *L.counter += 1;
   }
-  if (scatter) {
+  if (scatter && !sorted) {
     cloud_lmax_kernel<<<one, RED_THREADS, 0, L.stream>>>(cs, part);
     if (L.counter) *L.counter += 1;
   }
@@ -794,10 +804,10 @@ cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, b
 }
 
 // Counting sort of the clouds' points into their cells (after launch_clouds).
-cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most) {
+cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most, const double* part) {
   const dim3 pts(up(most, 256), nclouds);
   const unsigned nsb = up((int64_t)grid_start_entries(most), SCAN_B);
-  cell_count_kernel<<<pts, 256, 0, L.stream>>>(cs);
+  cell_count_kernel<<<dim3(pts.x + 1, nclouds), 256, 0, L.stream>>>(cs, part);
   scan_local_kernel<<<dim3(nsb, nclouds), SCAN_T, 0, L.stream>>>(cs);
   if (L.counter) *L.counter += 2;
   if (nsb > 1) {
