@@ -315,27 +315,32 @@ __device__ bool polar_float_refined_warp(double A, Lane3 L, double& Q) {
   float mine = x[0];
 #pragma unroll
   for (int k = 1; k < 9; ++k) mine = (q == k) ? x[k] : mine;
-  double Qd = (double)mine;
+  // lanes 0..8 own Q^T Q, lanes 16..24 Q^T A: the two products share their
+  // float64 instructions
+  const int half = threadIdx.x & 16, e = min((int)(threadIdx.x & 15), 8), r = e / 3, c = e % 3;
+  double Qd = (double)__shfl_sync(WFULL, mine, e);
   // A scaled by a power of two near 1 / ||A|| (exact), so that the 3x3
   // quantities below stay near unit size
   int e2 = 0;
   frexpf(sqrtf(n2), &e2);
-  const double As = A * __longlong_as_double((long long)(1023 - e2) << 52);
-  const double I = (L.r == L.c) ? 1.0 : 0.0;
+  const double As = wget(A, e) * __longlong_as_double((long long)(1023 - e2) << 52);
+  const double I = (r == c) ? 1.0 : 0.0;
   for (int step = 0; step < 2; ++step) {
-    const double E = wmul_ta(Qd, Qd, L) - I;
-    const double B = wmul_ta(Qd, As, L);
-    const double K = B - wget(B, L.c * 3 + L.r);
-    const float ef = (float)E, bf = (float)B, kf = (float)K;
+    const double Z = half ? As : Qd;
+    double prod = wget(Qd, r) * wget(Z, half + c);
+    prod = fma(wget(Qd, 3 + r), wget(Z, half + 3 + c), prod);
+    prod = fma(wget(Qd, 6 + r), wget(Z, half + 6 + c), prod);
+    const double tB = wget(prod, 16 + c * 3 + r);  // B^T, B = Q^T A
+    const float of = (float)(prod - (half ? tB : I)), bf = (float)prod;  // E = Q^T Q - I, or K = B - B^T; B
     float sm[9], bm[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      sm[k] = 0.5f * __shfl_sync(WFULL, ef, k);
-      bm[k] = __shfl_sync(WFULL, bf, k);
+      sm[k] = 0.5f * __shfl_sync(WFULL, of, k);
+      bm[k] = __shfl_sync(WFULL, bf, 16 + k);
     }
-    const float k21 = __shfl_sync(WFULL, kf, 7), k02 = __shfl_sync(WFULL, kf, 2), k10 = __shfl_sync(WFULL, kf, 3);
+    const float k21 = __shfl_sync(WFULL, of, 23), k02 = __shfl_sync(WFULL, of, 18), k10 = __shfl_sync(WFULL, of, 19);
     // entries of S B for its skew part
-    auto sb = [&](int r, int c) { return fmaf(sm[r * 3 + 2], bm[6 + c], fmaf(sm[r * 3 + 1], bm[3 + c], sm[r * 3] * bm[c])); };
+    auto sb = [&](int rr, int cc) { return fmaf(sm[rr * 3 + 2], bm[6 + cc], fmaf(sm[rr * 3 + 1], bm[3 + cc], sm[rr * 3] * bm[cc])); };
     const float kp0 = k21 - (sb(2, 1) - sb(1, 2));
     const float kp1 = k02 - (sb(0, 2) - sb(2, 0));
     const float kp2 = k10 - (sb(1, 0) - sb(0, 1));
@@ -361,19 +366,19 @@ __device__ bool polar_float_refined_warp(double A, Lane3 L, double& Q) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
       const float xd = fmaf(x[(k / 3) * 3 + 2], d[6 + k % 3], fmaf(x[(k / 3) * 3 + 1], d[3 + k % 3], x[(k / 3) * 3] * d[k % 3]));
-      p = (q == k) ? xd : p;
+      p = (e == k) ? xd : p;
     }
     Qd += (double)p;
   }
+  Qd = wget(Qd, q);
   Q = Qd;
   return true;
 }
 
-// Warp form of reorthonormalise for the product of the pose's rotation and
-// the increment, both orthogonal to float64 rounding: one Newton-Schulz step
-// brings R^T R - I back to rounding (a second changes nothing above it);
-// false (the caller takes the SVD route) when R^T R is further than 1e-6
-// from I.
+// The pose's rotation is a product of increments that are orthogonal to
+// float64 rounding; one Newton-Schulz step on it before the next product
+// keeps R^T R - I at rounding (a second changes nothing above it).  False (the
+// caller takes the SVD route) when R^T R is further than 1e-6 from I.
 __device__ bool reorth_warp(double R, Lane3 L, double& out) {
   const double I = (L.r == L.c) ? 1.0 : 0.0;
   const double e = wmul_ta(R, R, L) - I;
@@ -390,54 +395,114 @@ __device__ bool reorth_warp(double R, Lane3 L, double& out) {
 // * up to FINALIZE_SPLIT_ROWS, each of the 8 warps adds every 8th row (warp
 //   w: rows w, w + 8, ...) and warp 0 adds the 8 warp sums in order, a chain
 //   of rows / 8 + 8 additions instead of rows;
-// * beyond that, each thread adds its rows and a block-wide tree follows
-//   (about 150 float64 instructions however many rows there are).
+// * beyond that, each thread adds its rows, and each warp two of the 13
+//   columns of thread sums.
 constexpr int FINALIZE_WARP_ROWS = 16;
 constexpr int FINALIZE_SPLIT_ROWS = 512;
 
-// Warp 0 forms the update from the 13 totals v (the same in every lane of
-// warp 0; F[3], W, T[3][3]); lane (r, c) owns entry (r, c) of each 3x3.
-// sh is scratch (at least 64 doubles).
-__device__ void finalize_update(const double (&v)[13], DevPose* ps, const DevStats* __restrict__ st,
-                                StepParams sp, int* err, double (*sh)[RED_THREADS]) {
+// The update in two halves.  What does not depend on this iteration's totals
+// (the schedule of Eq. 12, the scale factor, s^2 R^T S0 R, the template mean, the
+// re-orthonormalised R) is formed by four warps, on the SM's four schedulers,
+// while other warps still add the totals; warp 0 then forms the rest.  All of
+// it is float64 latency (see warp-parallel 3x3 algebra), so the split takes
+// two thirds of the instructions off the critical path.
+struct PosePre {
+  double R[9];      // the pose's rotation, re-orthonormalised
+  double SRR[9];    // s^2 R^T S0 R
+  double yb[3];     // template mean at the pose
+  double tmy[3];    // t - yb
+  double ybx[3];    // yb - xbar
+  double sched;     // step_mode 0: eta0 G / G1; 1: G time^2
+  double s, sn, cs; // scale, next scale, their ratio
+  double scr[64];   // scratch of the SVD routes
+};
+constexpr int POSE_PRE_WARPS = 4;
+
+// Part `role` of the first half (one warp each; all 32 lanes).
+__device__ void pose_pre(int role, const DevPose* ps, const DevStats* __restrict__ st, StepParams sp, PosePre& o) {
   const Lane3 L = lane3();
-  const int lane = threadIdx.x;
-  const double W = v[3];
-  const double Tq = v[4 + L.q];  // T[a][b] = sum_i f_i[a] (Y_i - ybar)[b]
-  const int it = ps->it;
-  const double E = (double)ps->E;
-  // Eq. 12, 0-based iteration index: G / G1 = 0.1 + 0.9 / (1 + e), written
-  // over one division (each float64 division is a chain of about ten
-  // float64 instructions, about 65 cycles each on GB300)
-  const double e1 = 1.0 + exp(-((double)it - E / 2.0));
-  const double gnum = fma(0.1, e1, 0.9);  // (G / G1) (1 + e)
-  double kappa, dq;                       // dc = dq v_c
-  bool bad = false;
-  if (sp.step_mode == 0) {
-    // kappa = eta0 (G / G1) M / W, and Eq. 5.5's d = kappa v / M needs no M
-    if (!(W > 0.0) || !isfinite(W)) bad = true;
-    dq = bad ? 0.0 : sp.eta0 * gnum / (e1 * W);
-    kappa = dq * (double)sp.M;
+  const int lane = threadIdx.x & 31;
+  if (role == 0) {
+    // Eq. 12, 0-based iteration index: G / G1 = 0.1 + 0.9 / (1 + e), written
+    // over one division (each float64 division is a chain of about ten
+    // float64 instructions, about 65 cycles each on GB300)
+    const double e1 = 1.0 + exp(-((double)ps->it - (double)ps->E / 2.0));
+    const double g = fma(0.1, e1, 0.9) / e1;
+    if (lane == 0) o.sched = sp.step_mode == 0 ? sp.eta0 * g : sp.G1 * g * sp.time * sp.time;
+  } else if (role == 1) {
+    // scale model (Sec. III-B): c from the largest covariance eigenvalues
+    const double s = ps->s;
+    const double eY = s * s * st->eY0;
+    double cs = 1.0;
+    if (sp.scale_mode == 0) cs = sqrt(st->eX / eY);
+    else if (sp.scale_mode == 1) cs = st->eX / eY;
+    if (lane == 0) {
+      o.s = s;
+      o.cs = cs;
+      o.sn = cs * s;
+    }
+  } else if (role == 2) {
+    const double s = ps->s, R = ps->R[L.q];
+    const double SR = wmul(st->S0[L.q], R, L);
+    const double v = s * s * wmul_ta(R, SR, L);
+    if (lane < 9) o.SRR[lane] = v;
   } else {
-    kappa = sp.G1 * gnum / e1 * sp.time * sp.time;
-    dq = kappa / (double)sp.M;
+    const double s = ps->s, R = ps->R[L.q], tc = ps->t[L.c];
+    const double yb =
+        fma(s, fma(st->ybar0[2], ps->R[6 + L.c], fma(st->ybar0[1], ps->R[3 + L.c], st->ybar0[0] * ps->R[L.c])), tc);
+    const double tmy = tc - yb, ybx = yb - st->xbar[L.c];
+    if (lane < 3) {
+      o.yb[lane] = yb;
+      o.tmy[lane] = tmy;
+      o.ybx[lane] = ybx;
+    }
+    double Rn;
+    if (!reorth_warp(R, L, Rn)) {
+      if (lane < 9) o.scr[32 + lane] = R;
+      __syncwarp();
+      if (lane == 0) polar3(o.scr + 32, o.scr + 48);
+      __syncwarp();
+      Rn = o.scr[48 + L.q];
+    }
+    if (lane < 9) o.R[lane] = Rn;
   }
-  const double s = ps->s;
-  const double Rq = ps->R[L.q];
-  // template mean at this pose, component L.c in each lane, and t - ybar
-  const double tc = ps->t[L.c];
-  const double ybc =
-      fma(s, fma(st->ybar0[2], ps->R[6 + L.c], fma(st->ybar0[1], ps->R[3 + L.c], st->ybar0[0] * ps->R[L.c])), tc);
-  const double tmy = tc - ybc;
-  const double dc = dq * v[L.c];  // Eq. 5.5, unit masses, v = 0 (component c)
-  // C^ = Y_D^T Y_c = s^2 R^T S0 R + kappa T   (Eq. 6 with the displaced cloud)
-  const double SR = wmul(st->S0[L.q], Rq, L);
-  const double Ch = fma(kappa, Tq, s * s * wmul_ta(Rq, SR, L));
+}
+
+// Eq. 5.5's d_c = dq F_c and kappa = dq M from the totals (every lane).
+__device__ __forceinline__ bool pose_step(const double* tot, const StepParams& sp, const PosePre& o, double& dq,
+                                          double& kappa) {
+  if (sp.step_mode == 0) {
+    // kappa = eta0 (G / G1) M / W, and Eq. 5.5's d = kappa F / M needs no M
+    const double W = tot[3];
+    const bool ok = W > 0.0 && isfinite(W);
+    dq = !ok ? 0.0 : (W > 1e-30 && W < 1e30) ? o.sched * wrcp(W) : o.sched / W;
+    kappa = dq * (double)sp.M;
+    return ok;
+  }
+  kappa = o.sched;
+  dq = kappa / (double)sp.M;
+  return true;
+}
+
+// Second half, by one warp: the step from the 13 totals tot (F[3], W, T[3][3]),
+// the Kabsch rotation and the composed pose, written to *ps.  Lane (r, c) owns
+// entry (r, c) of each 3x3; lanes 9..11 carry the translation as a fourth row.
+__device__ void pose_post(const double* tot, DevPose* ps, const DevStats* __restrict__ st, const StepParams& sp,
+                          PosePre& o, int* err) {
+  const Lane3 L = lane3();
+  const int lane = threadIdx.x & 31;
+  const int row = min(lane / 3, 3), col = lane < 12 ? lane % 3 : 2;
+  double dq, kappa;
+  bool bad = !pose_step(tot, sp, o, dq, kappa);
+  const double dc = dq * tot[col];
+  // C^ = Y_D^T Y_c = s^2 R^T S0 R + kappa T   (Eq. 6 with the displaced cloud;
+  // T[a][b] = sum_i f_i[a] (Y_i - ybar)[b])
+  const double Ch = fma(kappa, tot[4 + L.q], o.SRR[L.q]);
   bad = bad || !isfinite(Ch) || !isfinite(dc);
   if (__any_sync(WFULL, bad)) {
     if (lane == 0) {
       atomicOr(err, ERR_NUMERIC);
-      ps->it = it + 1;
+      ps->it += 1;
     }
     return;
   }
@@ -446,11 +511,9 @@ __device__ void finalize_update(const double (&v)[13], DevPose* ps, const DevSta
   // (C^ = (U V^T)(V S V^T)), taken by Newton's iteration (in float32 with
   // float64 corrections, else all in float64); the SVD handles det C^ <= 0,
   // near-singular C^ and the degenerate case.
-  double Rinc, Qp;
-  if (polar_float_refined_warp(Ch, L, Qp) || polar_newton_warp(Ch, L, Qp)) {
-    Rinc = wget(Qp, L.c * 3 + L.r);
-  } else {
-    double* scr = &sh[0][0];
+  double Q;  // R_inc^T
+  if (!polar_float_refined_warp(Ch, L, Q) && !polar_newton_warp(Ch, L, Q)) {
+    double* scr = o.scr;
     if (lane < 9) scr[lane] = Ch;
     __syncwarp();
     if (lane == 0) {
@@ -470,97 +533,101 @@ __device__ void finalize_update(const double (&v)[13], DevPose* ps, const DevSta
       for (int q = 0; q < 9; ++q) scr[16 + q] = Ri[q];
     }
     __syncwarp();
-    Rinc = scr[16 + L.q];
+    Q = scr[16 + L.c * 3 + L.r];
   }
-  // scale model (Sec. III-B): c from the largest covariance eigenvalues
-  const double eY = s * s * st->eY0;
-  double cs = 1.0;
-  if (sp.scale_mode == 0) cs = sqrt(st->eX / eY);
-  else if (sp.scale_mode == 1) cs = st->eX / eY;
-  // Eq. 8, Eq. 9: Y(t+1) = c (Y - ybar) R_inc + ybar + d, composed into the pose
-  // (lanes 0, 1, 2 hold t - ybar of components 0, 1, 2)
-  double acc = wget(tmy, 0) * wget(Rinc, L.c);
-  acc = fma(wget(tmy, 1), wget(Rinc, 3 + L.c), acc);
-  acc = fma(wget(tmy, 2), wget(Rinc, 6 + L.c), acc);
-  const double tn = fma(cs, acc, ybc + dc);  // component c
-  const double RR = wmul(Rq, Rinc, L);
-  double Rn;
-  if (!reorth_warp(RR, L, Rn)) {
-    double* scr = &sh[0][0];
-    if (lane < 9) scr[32 + lane] = RR;
-    __syncwarp();
-    if (lane == 0) polar3(scr + 32, scr + 48);
-    __syncwarp();
-    Rn = scr[48 + L.q];
-  }
-  const bool ok = isfinite(cs) && isfinite(Rn) && isfinite(tn);
-  if (!__all_sync(WFULL, ok)) {
+  // Eq. 8, Eq. 9: Y(t+1) = c (Y - ybar) R_inc + ybar + d, composed into the pose:
+  // rows 0..2 of [R; t - ybar] R_inc are the next rotation, row 3 its translation
+  const double x = lane < 9 ? o.R[lane] : o.tmy[col];
+  double y = wget(x, row * 3) * wget(Q, col * 3);
+  y = fma(wget(x, row * 3 + 1), wget(Q, col * 3 + 1), y);
+  y = fma(wget(x, row * 3 + 2), wget(Q, col * 3 + 2), y);
+  if (row == 3) y = fma(o.cs, y, o.yb[col] + dc);
+  if (!__all_sync(WFULL, isfinite(o.cs) && isfinite(y))) {
     if (lane == 0) {
       atomicOr(err, ERR_NUMERIC);
-      ps->it = it + 1;
+      ps->it += 1;
     }
     return;
   }
-  // new pose and its derived float32 map (the warp form of refresh_pose)
-  const double sn = cs * s;
-  const double ybs = fma(sn, fma(st->ybar0[2], wget(Rn, 6 + L.c), fma(st->ybar0[1], wget(Rn, 3 + L.c),
-                                                                         st->ybar0[0] * wget(Rn, L.c))),
-                         tn) - st->xbar[L.c];
+  // the new pose and its float32 map: A = s R, b = t - xbar
+  const float f = (float)fma(lane < 9 ? o.sn : 1.0, y, lane < 9 ? 0.0 : -st->xbar[col]);
   if (lane < 9) {
-    ps->R[lane] = Rn;
-    ps->A[lane] = (float)(sn * Rn);
+    ps->R[lane] = y;
+    ps->A[lane] = f;
+  } else if (lane < 12) {
+    ps->t[col] = y;
+    ps->b[col] = f;
   }
-  if (lane < 3) {
-    ps->t[lane] = tn;
-    ps->b[lane] = (float)(tn - st->xbar[lane]);
-    set_ybs(ps, lane, ybs);
+  if (lane == 12) {
+    ps->s = o.sn;
+    ps->it += 1;
   }
-  if (lane == 0) {
-    ps->s = sn;
-    ps->it = it + 1;
-  }
+  // the mean moves by d exactly (Eq. 9)
+  const double ybs = o.ybx[col] + dc;
+  if (lane < 3) set_ybs(ps, lane, ybs);
 }
 
-// Totals of nblocks rows of 13 partials (fixed order), then the update.
+// Totals of nblocks rows of 13 partials (fixed order) by warps 0..7 while
+// warps 8..11 form the update's first half, then the second half.
+constexpr int FINALIZE_THREADS = RED_THREADS + 32 * POSE_PRE_WARPS;
+
+struct FinalizeShared {
+  double sh[13][RED_THREADS];
+  double tot[13];
+  PosePre pre;
+};
+
 __device__ void finalize_body(const double* __restrict__ blockpart, int nblocks, DevPose* ps,
-                              const DevStats* __restrict__ st, StepParams sp, int* err,
-                              double (*sh)[RED_THREADS]) {
-  double v[13];
-  if (nblocks <= FINALIZE_WARP_ROWS) {
-    if (threadIdx.x >= 32) return;
-    const int lane = threadIdx.x;
-    double col = 0.0;
-    if (lane < 13)
-      for (int b = 0; b < nblocks; ++b) col += blockpart[(size_t)b * 13 + lane];
-#pragma unroll
-    for (int q = 0; q < 13; ++q) v[q] = __shfl_sync(WFULL, col, q);
-  } else if (nblocks <= FINALIZE_SPLIT_ROWS) {
-    constexpr int NW = RED_THREADS / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double col = 0.0;
-    if (lane < 13)
-      for (int b = warp; b < nblocks; b += NW) col += blockpart[(size_t)b * 13 + lane];
-    if (lane < 13) sh[lane][warp] = col;
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    double tot = 0.0;
-    if (lane < 13)
-      for (int k = 0; k < NW; ++k) tot += sh[lane][k];
-    __syncwarp();  // every lane has read its sums: sh is scratch from here on
-#pragma unroll
-    for (int q = 0; q < 13; ++q) v[q] = __shfl_sync(WFULL, tot, q);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 13; ++q) v[q] = 0.0;
-    for (int bidx = threadIdx.x; bidx < nblocks; bidx += RED_THREADS) {
-#pragma unroll
-      for (int q = 0; q < 13; ++q) v[q] += blockpart[(size_t)bidx * 13 + q];
+                              const DevStats* __restrict__ st, StepParams sp, int* err, FinalizeShared& F) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int NW = RED_THREADS / 32;
+  if (nblocks <= FINALIZE_SPLIT_ROWS) {
+    // rows in turn by one warp, or every 8th row by each of 8 (FINALIZE_WARP_ROWS)
+    const int nw = nblocks <= FINALIZE_WARP_ROWS ? 1 : NW;
+    if (warp >= NW) {
+      pose_pre(warp - NW, ps, st, sp, F.pre);
+    } else if (warp < nw && lane < 13) {
+      double col = 0.0;
+      for (int b = warp; b < nblocks; b += nw) col += blockpart[(size_t)b * 13 + lane];
+      F.sh[lane][warp] = col;
     }
-    block_sum<13>(v, sh);
-    __syncthreads();  // every thread has read the totals: sh is scratch from here on
-    if (threadIdx.x >= 32) return;
+    __syncthreads();
+    if (warp != 0) return;
+    if (lane < 13) {
+      double tot = F.sh[lane][0];
+      for (int k = 1; k < nw; ++k) tot += F.sh[lane][k];
+      F.tot[lane] = tot;
+    }
+    __syncwarp();
+  } else {
+    if (warp >= NW) {
+      pose_pre(warp - NW, ps, st, sp, F.pre);
+    } else {
+      double v[13];
+#pragma unroll
+      for (int q = 0; q < 13; ++q) v[q] = 0.0;
+      for (int b = threadIdx.x; b < nblocks; b += RED_THREADS) {
+#pragma unroll
+        for (int q = 0; q < 13; ++q) v[q] += blockpart[(size_t)b * 13 + q];
+      }
+#pragma unroll
+      for (int q = 0; q < 13; ++q) F.sh[q][threadIdx.x] = v[q];
+    }
+    // each warp adds the threads' sums of columns w, w + 8
+    __syncthreads();
+    if (warp < NW)
+      for (int q = warp; q < 13; q += NW) {
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < RED_THREADS / 32; ++k) t += F.sh[q][k * 32 + lane];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(WFULL, t, off);
+        if (lane == 0) F.tot[q] = t;
+      }
+    __syncthreads();
+    if (warp != 0) return;
   }
-  finalize_update(v, ps, st, sp, err, sh);
+  pose_post(F.tot, ps, st, sp, F.pre, err);
 }
 
 // Combine and finalize in one block, for templates of at most
@@ -581,43 +648,43 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1)
     combine_finalize_kernel(const float4* __restrict__ partial, int S, int mpad, int m,
                             const float4* __restrict__ Y0r, const float* __restrict__ aY32, int g_mode,
                             DevPose* ps, const DevStats* __restrict__ st, StepParams sp, int* err) {
-  // (f, W_i) per point in steps 1-2; the float64 sums and scratch from step 3
-  __shared__ __align__(16) unsigned char smem[FUSED_MAX_SLOTS * sizeof(float4)];
-  static_assert(FUSED_MAX_SLOTS * sizeof(float4) >= sizeof(double) * 13 * RED_THREADS, "scratch too small");
-  float4* fws = reinterpret_cast<float4*>(smem);
-  double(*sh)[RED_THREADS] = reinterpret_cast<double(*)[RED_THREADS]>(smem);
+  __shared__ __align__(16) float4 fws[FUSED_MAX_SLOTS];  // (f, W_i) per point
+  __shared__ double sh[13][RED_THREADS / 32];
+  __shared__ double tot[13];
+  __shared__ PosePre pre;
+  static_assert(FUSED_THREADS >= FINALIZE_THREADS, "warps for the update's first half");
   const PointFrame fr(ps);
   for (int i = threadIdx.x; i < m; i += FUSED_THREADS)
     fws[i] = point_fw(partial, (size_t)mpad, S, i, Y0r[i], g_mode == 1 ? aY32[i] : 1.f, fr);
   __syncthreads();
-  if (threadIdx.x >= RED_THREADS) return;  // all of ps read
-  float acc[13];
-#pragma unroll
-  for (int q = 0; q < 13; ++q) acc[q] = 0.f;
-  for (int i = threadIdx.x; i < m; i += RED_THREADS) point_acc(fws[i], Y0r[i], fr, acc);
-  double w[16];
-#pragma unroll
-  for (int q = 0; q < 13; ++q) w[q] = (double)acc[q];
-  w[13] = w[14] = w[15] = 0.0;
-  warp_reduce16(w);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __syncthreads();  // every (f, W_i) read: smem holds the float64 sums from here
-  // even lanes hold quantities 0..15 after the reduction; 13..15 are padding
-  // and have no row in sh
-  if ((lane & 1) == 0) {
-    const int q = warp_reduce16_slot(lane);
-    if (q < 13) sh[q][warp] = w[0];
-  }
-  __syncthreads();  // all of ps and sh read/written: warp 0 updates the pose from here
-  if (warp != 0) return;
-  double col = 0.0;
-  if (lane < 13)
-    for (int k = 0; k < RED_THREADS / 32; ++k) col += sh[lane][k];
-  __syncwarp();
-  double v[13];
+  if (threadIdx.x >= RED_THREADS) {
+    if (warp < FINALIZE_THREADS / 32) pose_pre(warp - RED_THREADS / 32, ps, st, sp, pre);
+  } else {
+    float acc[13];
 #pragma unroll
-  for (int q = 0; q < 13; ++q) v[q] = __shfl_sync(WFULL, col, q);
-  finalize_update(v, ps, st, sp, err, sh);
+    for (int q = 0; q < 13; ++q) acc[q] = 0.f;
+    for (int i = threadIdx.x; i < m; i += RED_THREADS) point_acc(fws[i], Y0r[i], fr, acc);
+    double w[16];
+#pragma unroll
+    for (int q = 0; q < 13; ++q) w[q] = (double)acc[q];
+    w[13] = w[14] = w[15] = 0.0;
+    warp_reduce16(w);
+    // even lanes hold quantities 0..15 after the reduction; 13..15 are padding
+    if ((lane & 1) == 0) {
+      const int q = warp_reduce16_slot(lane);
+      if (q < 13) sh[q][warp] = w[0];
+    }
+  }
+  __syncthreads();  // all of ps read: warp 0 updates the pose from here
+  if (warp != 0) return;
+  if (lane < 13) {
+    double col = 0.0;
+    for (int k = 0; k < RED_THREADS / 32; ++k) col += sh[lane][k];
+    tot[lane] = col;
+  }
+  __syncwarp();
+  pose_post(tot, ps, st, sp, pre, err);
 }
 
 cudaError_t launch_combine_finalize(Launch L, const float4* partial, int S, int mpad, int m, const float4* Y0r,
@@ -629,27 +696,27 @@ cudaError_t launch_combine_finalize(Launch L, const float4* partial, int S, int 
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(RED_THREADS)
+__global__ void __launch_bounds__(FINALIZE_THREADS)
     finalize_kernel(const double* __restrict__ blockpart, int nblocks, DevPose* ps,
                     const DevStats* __restrict__ st, StepParams sp, int* err) {
-  __shared__ double sh[13][RED_THREADS];
-  finalize_body(blockpart, nblocks, ps, st, sp, err, sh);
+  __shared__ FinalizeShared F;
+  finalize_body(blockpart, nblocks, ps, st, sp, err, F);
 }
 
 // One block per pair of a batch.
-__global__ void __launch_bounds__(RED_THREADS)
+__global__ void __launch_bounds__(FINALIZE_THREADS)
     finalize_multi_kernel(const double* __restrict__ blockpart, const BatchPair* __restrict__ pairs,
                           DevPose* poses, const DevStats* __restrict__ stats, StepParams sp, int* err) {
-  __shared__ double sh[13][RED_THREADS];
+  __shared__ FinalizeShared F;
   const BatchPair& bp = pairs[blockIdx.x];
   StepParams spp = sp;
   spp.M = (int)bp.m;
-  finalize_body(blockpart + (size_t)bp.cblk0 * 13, bp.ncblk, poses + blockIdx.x, stats + blockIdx.x, spp, err, sh);
+  finalize_body(blockpart + (size_t)bp.cblk0 * 13, bp.ncblk, poses + blockIdx.x, stats + blockIdx.x, spp, err, F);
 }
 
 cudaError_t launch_finalize_multi(Launch L, const double* blockpart, const BatchPair* pairs, int npairs,
                                   DevPose* poses, const DevStats* stats, StepParams sp, int* err) {
-  finalize_multi_kernel<<<npairs, RED_THREADS, 0, L.stream>>>(blockpart, pairs, poses, stats, sp, err);
+  finalize_multi_kernel<<<npairs, FINALIZE_THREADS, 0, L.stream>>>(blockpart, pairs, poses, stats, sp, err);
   if (L.counter) ++*L.counter;
   return cudaGetLastError();
 }
@@ -675,7 +742,7 @@ cudaError_t launch_pose_init_multi(Launch L, DevPose* poses, const DevStats* sta
 
 cudaError_t launch_finalize(Launch L, const double* blockpart, int nblocks, DevPose* pose,
                             const DevStats* stats, StepParams sp, int* err) {
-  finalize_kernel<<<1, RED_THREADS, 0, L.stream>>>(blockpart, nblocks, pose, stats, sp, err);
+  finalize_kernel<<<1, FINALIZE_THREADS, 0, L.stream>>>(blockpart, nblocks, pose, stats, sp, err);
   if (L.counter) ++*L.counter;
   return cudaGetLastError();
 }
