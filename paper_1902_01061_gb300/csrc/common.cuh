@@ -393,6 +393,16 @@ constexpr int FUSED_MAX_SLOTS = 2048;  // templates up to this many padded slots
 cudaError_t launch_combine_finalize(Launch L, const float4* partial, int S, int mpad, int m, const float4* Y0r,
                                     const float* aY32, int g_mode, DevPose* pose, const DevStats* stats,
                                     StepParams sp, int* err);
+constexpr int SMALL_MAX_POINTS = 8192;  // padded reference points that fit a block's shared memory
+bool small_run_available();
+cudaError_t launch_small_run(Launch L, int pmode, const float4* Xr, const float2* XA, int npad, const float4* Y0r,
+                             const float* aY32, int g_mode, int m, DevPose* pose, const DevStats* stats,
+                             StepParams sp, float qexp, int iters, int* err);
+size_t fixed_part_bytes(int num_sms);
+cudaError_t launch_fixed_moments(Launch L, const float4* partial, int S, int mpad, int m, const float4* Y0r,
+                                 const double* aY64, int g_mode, const DevStats* stats, int num_sms, double* part);
+cudaError_t launch_fixed_run(Launch L, const double* part, int m, int num_sms, DevPose* pose, const DevStats* stats,
+                             StepParams sp, int iters, int* err);
 cudaError_t launch_finalize(Launch L, const double* blockpart, int nblocks, DevPose* pose,
                             const DevStats* stats, StepParams sp, int* err);
 cudaError_t launch_apply(Launch L, const float4* Y4, int m, const DevPose* pose, float* out);

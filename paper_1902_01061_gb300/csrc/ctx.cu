@@ -344,11 +344,19 @@ scgr_status replan(scgr_ctx* c) {
 
 // Odd integer p needs no all-pairs pass per iteration.  For p = 1 the pair
 // weight aX s_ij d^0 does not depend on the pose, so the force kernel's
-// per-split sums (sum w, sum w X') are the same in every iteration: the first
-// iteration of a run computes them and the others reuse them (bit-identical).
+// per-split sums (sum w, sum w X') are the same in every iteration: they are
+// computed once.  Templates of the fused tail's size then combine them in
+// every iteration (bit-identical to recomputing them); for larger ones the
+// iteration's totals come from 22 moments of the sums, and one launch runs all
+// iterations (launch_fixed_run; equal up to rounding): 35,000 x 30,800, 200
+// iterations 4.6 -> 1.2 ms.
 // For p = 3 the sums are a quadratic form in the template point over 14
 // pose-free moments of g (computed once per run; an exact re-association, so
 // equal to the direct pass up to rounding).
+// Small problems of the other exponents run all iterations in one launch of
+// a thread-block cluster (launch_small_run) unless the force launches are to be
+// timed.  The cluster's 16 SMs bound its pair rate (2.8e11/s), so from 5e6
+// pairs on the whole GPU is faster, launches and all.
 scgr_status enqueue_iterations(scgr_ctx* c, int iters) {
   const int nb = combine_blocks(c->mpad);
   const StepParams sp = step_params(c);
@@ -363,6 +371,24 @@ scgr_status enqueue_iterations(scgr_ctx* c, int iters) {
     SCGR_CK(c, launch_moments(c->L(), (const float4*)c->Xr.p, (const float2*)c->XA.p, ntiles, (const float4*)c->Y0r.p,
                               (int)c->mpad, mloc, S, (double*)c->mpart.p, (double*)c->mom.p));
   }
+  const bool fused = c->fused_tail && c->mpad <= FUSED_MAX_SLOTS;
+  if (pose_free && !fused && iters > 0) {
+    const scgr_status fs = force_launch(c);
+    if (fs != SCGR_OK) return fs;
+    SCGR_CK(c, launch_fixed_moments(c->L(), (const float4*)c->partial.p, c->fp.splits, (int)c->mpad, mloc,
+                                    (const float4*)c->Y0r.p, (const double*)c->aY64.p, c->prm.g_mode, c->stats,
+                                    c->num_sms, (double*)c->fixpart.p));
+    SCGR_CK(c, launch_fixed_run(c->L(), (const double*)c->fixpart.p, mloc, c->num_sms, c->pose, c->stats, sp, iters,
+                                c->errword));
+    return SCGR_OK;
+  }
+  if (fused && c->small_ok && !c->timing && !moments && c->fp.pmode != 1 && c->npad <= SMALL_MAX_POINTS &&
+      c->n * c->m <= 5000000 && iters > 0) {
+    SCGR_CK(c, launch_small_run(c->L(), c->fp.pmode, (const float4*)c->Xr.p, (const float2*)c->XA.p, (int)c->npad,
+                                (const float4*)c->Y0r.p, (const float*)c->aY32.p, c->prm.g_mode, (int)c->m, c->pose,
+                                c->stats, sp, c->qexp, iters, c->errword));
+    return SCGR_OK;
+  }
   for (int t = 0; t < iters; ++t) {
     if (moments) {
       SCGR_CK(c, launch_combine_moments(c->L(), (const double*)c->mom.p, mloc, (int)c->mpad, (const float4*)c->Y0r.p,
@@ -375,7 +401,7 @@ scgr_status enqueue_iterations(scgr_ctx* c, int iters) {
       scgr_status fs = force_launch(c);
       if (fs != SCGR_OK) return fs;
     }
-    if (c->fused_tail && c->mpad <= FUSED_MAX_SLOTS) {
+    if (fused) {
       // small templates: combine and finalize in one block (one launch less per iteration)
       SCGR_CK(c, launch_combine_finalize(c->L(), (const float4*)c->partial.p, c->fp.splits, (int)c->mpad, (int)c->m,
                                          (const float4*)c->Y0r.p, (const float*)c->aY32.p, c->prm.g_mode, c->pose,

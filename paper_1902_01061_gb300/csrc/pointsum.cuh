@@ -39,14 +39,13 @@ struct PointFrame {
   }
 };
 
-// Force on template slot i from its S split partials (sum_j w X', sum_j w)
-// at stride pstride: the splits added in order with Kahan compensation, then
-// f = aY (S - Y' W) from an exact product and an exact two-sum, so f is as
-// accurate as float allows even when S and Y' W nearly cancel; W_i = aY W.
-// Returns (f, W_i).
-__device__ __forceinline__ float4 point_fw(const float4* __restrict__ pbase, size_t pstride, int S, int i,
-                                           const float4 y0, float ay, const PointFrame& fr) {
-  float Wh = 0.f, Wc = 0.f, Sh[3] = {0.f, 0.f, 0.f}, Sc[3] = {0.f, 0.f, 0.f};
+// Sums of template slot i over its S split partials (sum_j w, sum_j w X') at
+// stride pstride, added in order with Kahan compensation: value h - c.
+struct PointSums {
+  float Wh, Wc, Sh[3], Sc[3];
+};
+__device__ __forceinline__ PointSums point_sums(const float4* __restrict__ pbase, size_t pstride, int S, int i) {
+  PointSums r{0.f, 0.f, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
   // splits in order, eight loads in flight per step (small templates leave
   // few threads per SM, so the pass over the splits is load-latency bound)
   for (int s = 0; s < S; s += 8) {
@@ -57,13 +56,25 @@ __device__ __forceinline__ float4 point_fw(const float4* __restrict__ pbase, siz
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       if (s + u < S) {
-        kahan_add(Wh, Wc, pp[u].x);
-        kahan_add(Sh[0], Sc[0], pp[u].y);
-        kahan_add(Sh[1], Sc[1], pp[u].z);
-        kahan_add(Sh[2], Sc[2], pp[u].w);
+        kahan_add(r.Wh, r.Wc, pp[u].x);
+        kahan_add(r.Sh[0], r.Sc[0], pp[u].y);
+        kahan_add(r.Sh[1], r.Sc[1], pp[u].z);
+        kahan_add(r.Sh[2], r.Sc[2], pp[u].w);
       }
     }
   }
+  return r;
+}
+
+// Force on template slot i from its split partials (point_sums), then
+// f = aY (S - Y' W) from an exact product and an exact two-sum, so f is as
+// accurate as float allows even when S and Y' W nearly cancel; W_i = aY W.
+// Returns (f, W_i).
+__device__ __forceinline__ float4 point_fw(const float4* __restrict__ pbase, size_t pstride, int S, int i,
+                                           const float4 y0, float ay, const PointFrame& fr) {
+  const PointSums r = point_sums(pbase, pstride, S, i);
+  const float Wh = r.Wh, Wc = r.Wc;
+  const float (&Sh)[3] = r.Sh, (&Sc)[3] = r.Sc;
   float y[3];
   template_point(y0, fr.A, fr.b, y[0], y[1], y[2]);
   float f[3];
