@@ -311,8 +311,12 @@ __global__ void __launch_bounds__(FIXED_RUN_THREADS)
     if (warp == 2) pose_pre(2, &ps, &st, sp, pre, now);
     if (warp == 3) pose_pre(3, &ps, &st, sp, pre, now);
     if (warp == 1) {
-      const double A = ps.s * ps.R[lane3().q];  // entry (r, c) in lanes 0..8
-      double v = fma(-U, ps.ybs[col], N);
+      const double R = ps.R[lane3().q];  // entry (r, c) in lanes 0..8
+      const double A = ps.s * R;
+      const double ybs =
+          fma(ps.s, fma(st.ybar0[2], ps.R[6 + col], fma(st.ybar0[1], ps.R[3 + col], st.ybar0[0] * ps.R[col])), ps.t[col]) -
+          st.xbar[col];
+      double v = fma(-U, ybs, N);
 #pragma unroll
       for (int k = 0; k < 3; ++k) v = fma(-P[k], wget(A, k * 3 + col), v);
       // T[a][b] = sum_c K[c][a] A[c][b]: lane (a, b) in 0..8
@@ -325,7 +329,7 @@ __global__ void __launch_bounds__(FIXED_RUN_THREADS)
     }
     __syncthreads();
     if (warp == 0) {
-      const bool moved = pose_post(tot, &ps, &st, sp, pre, now, err);
+      const bool moved = pose_post(tot, &ps, &st, sp, pre, now, err, false);
       if (lane == 0) ok = moved;
     } else if (warp == 5) {
       pose_schedule(it0 + it + 1, E, sp, next);
@@ -338,6 +342,8 @@ __global__ void __launch_bounds__(FIXED_RUN_THREADS)
       __syncthreads();
     }
   }
+  if (threadIdx.x == 0) refresh_pose(&ps, &st);
+  __syncthreads();
   if (threadIdx.x < sizeof(DevPose) / 4) reinterpret_cast<int*>(pose)[threadIdx.x] = reinterpret_cast<const int*>(&ps)[threadIdx.x];
 }
 

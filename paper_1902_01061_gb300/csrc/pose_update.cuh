@@ -202,6 +202,32 @@ __device__ inline bool polar_newton_warp(double A, Lane3 L, double& Q) {
   return true;
 }
 
+__device__ __forceinline__ float fsqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// Sum of squares of nine values in a chain of three.
+__device__ __forceinline__ float sq9(const float (&v)[9]) {
+  const float p = fmaf(v[2], v[2], fmaf(v[1], v[1], v[0] * v[0]));
+  const float q = fmaf(v[5], v[5], fmaf(v[4], v[4], v[3] * v[3]));
+  const float r = fmaf(v[8], v[8], fmaf(v[7], v[7], v[6] * v[6]));
+  return (p + q) + r;
+}
+
+// Float64 tests on the integer pipe (a float64 comparison costs as much as an
+// addition): finite; positive and within [2^-100, 2^100); times 2^k for a
+// normal value whose exponent stays in range (0 for zero).
+__device__ __forceinline__ bool finite64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool moderate64(double v) {
+  const int h = __double2hiint(v);
+  return h >= ((1023 - 100) << 20) && h < ((1023 + 100) << 20);
+}
+__device__ __forceinline__ double scale64(double v, int k) {
+  const int h = __double2hiint(v);
+  return (h & 0x7ff00000) == 0 ? 0.0 : __hiloint2double(h + (k << 20), __double2loint(v));
+}
+
 // Polar factor of A (lane-owned) with most of the work in float32.  On
 // GB300 a float64 instruction costs about 65 cycles whatever the number of
 // active lanes, and consecutive ones do not overlap, so the float64 work is
@@ -225,10 +251,8 @@ __device__ inline bool polar_float_refined_warp(double A, Lane3 L, double& Q) {
   float x[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) x[k] = __shfl_sync(WFULL, fa, k);
-  float n2 = 0.f;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) n2 = fmaf(x[k], x[k], n2);
-  if (!(n2 > 0.f) || !isfinite(n2)) return false;
+  const float n2 = sq9(x);
+  if (!(n2 > 1e-30f) || !isfinite(n2)) return false;
   const float inv = rsqrtf(n2);
 #pragma unroll
   for (int k = 0; k < 9; ++k) x[k] *= inv;
@@ -246,26 +270,26 @@ __device__ inline bool polar_float_refined_warp(double A, Lane3 L, double& Q) {
     c[8] = x[0] * x[4] - x[1] * x[3];
     const float det = fmaf(x[2], c[2], fmaf(x[1], c[1], x[0] * c[0]));
     if (!(det > 1e-20f) || !isfinite(det)) return false;
-    const float rd = __frcp_rn(det);
-    float nx = 0.f, ny = 0.f;
+    const float rd = __fdividef(1.f, det);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      c[k] *= rd;
-      nx = fmaf(x[k], x[k], nx);
-      ny = fmaf(c[k], c[k], ny);
+    for (int k = 0; k < 9; ++k) c[k] *= rd;
+    float a = 0.5f, b = 0.5f;
+    if (scale) {
+      const float nx = sq9(x), ny = sq9(c);
+      if (it == 0 && !(nx * ny <= 1e6f)) return false;
+      // any positive weights keep the polar factor: an approximate fourth root
+      const float g = fsqrt_approx(fsqrt_approx(__fdividef(ny, nx)));
+      a = 0.5f * g;
+      b = __fdividef(0.5f, g);
     }
-    if (it == 0 && !(nx * ny <= 1e6f)) return false;
-    const float g = scale ? sqrtf(sqrtf(__fdividef(ny, nx))) : 1.f;
-    const float a = 0.5f * g, b = __fdividef(0.5f, g);
-    float dd = 0.f, nn = 0.f;
+    float d[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
       const float xn = fmaf(a, x[k], b * c[k]);
-      const float d = xn - x[k];
-      dd = fmaf(d, d, dd);
-      nn = fmaf(xn, xn, nn);
+      d[k] = xn - x[k];
       x[k] = xn;
     }
+    const float dd = sq9(d), nn = sq9(x);
     done = dd <= 1e-10f * nn;
     scale = dd > 1e-4f * nn;
   }
@@ -282,7 +306,7 @@ __device__ inline bool polar_float_refined_warp(double A, Lane3 L, double& Q) {
   // quantities below stay near unit size
   int e2 = 0;
   frexpf(sqrtf(n2), &e2);
-  const double As = wget(A, e) * __longlong_as_double((long long)(1023 - e2) << 52);
+  const double As = scale64(wget(A, e), -e2);
   const double I = (r == c) ? 1.0 : 0.0;
   for (int step = 0; step < 2; ++step) {
     const double Z = half ? As : Qd;
@@ -429,8 +453,13 @@ __device__ __forceinline__ bool pose_step(const double* tot, const StepParams& s
   if (sp.step_mode == 0) {
     // kappa = eta0 (G / G1) M / W, and Eq. 5.5's d = kappa F / M needs no M
     const double W = tot[3];
-    const bool ok = W > 0.0 && isfinite(W);
-    dq = !ok ? 0.0 : (W > 1e-30 && W < 1e30) ? o.sched * wrcp(W) : o.sched / W;
+    bool ok = true;
+    if (moderate64(W)) {
+      dq = o.sched * wrcp(W);
+    } else {
+      ok = W > 0.0 && isfinite(W);
+      dq = ok ? o.sched / W : 0.0;
+    }
     kappa = dq * (double)sp.M;
     return ok;
   }
@@ -443,8 +472,9 @@ __device__ __forceinline__ bool pose_step(const double* tot, const StepParams& s
 // the Kabsch rotation and the composed pose, written to *ps.  Lane (r, c) owns
 // entry (r, c) of each 3x3; lanes 9..11 carry the translation as a fourth row.
 // False (every lane) where the step is not finite and the pose is kept.
+// set_mean = false leaves ybs and its float pair to the caller.
 __device__ inline bool pose_post(const double* tot, DevPose* ps, const DevStats* __restrict__ st, const StepParams& sp,
-                                 PosePre& o, const PoseRate& rate, int* err) {
+                                 PosePre& o, const PoseRate& rate, int* err, bool set_mean = true) {
   const Lane3 L = lane3();
   const int lane = threadIdx.x & 31;
   const int row = min(lane / 3, 3), col = lane < 12 ? lane % 3 : 2;
@@ -454,7 +484,7 @@ __device__ inline bool pose_post(const double* tot, DevPose* ps, const DevStats*
   // C^ = Y_D^T Y_c = s^2 R^T S0 R + kappa T   (Eq. 6 with the displaced cloud;
   // T[a][b] = sum_i f_i[a] (Y_i - ybar)[b])
   const double Ch = fma(kappa, tot[4 + L.q], o.SRR[L.q]);
-  bad = bad || !isfinite(Ch) || !isfinite(dc);
+  bad = bad || !finite64(Ch) || !finite64(dc);
   if (__any_sync(WFULL, bad)) {
     if (lane == 0) {
       atomicOr(err, ERR_NUMERIC);
@@ -498,7 +528,7 @@ __device__ inline bool pose_post(const double* tot, DevPose* ps, const DevStats*
   y = fma(wget(x, row * 3 + 1), wget(Q, col * 3 + 1), y);
   y = fma(wget(x, row * 3 + 2), wget(Q, col * 3 + 2), y);
   if (row == 3) y = fma(rate.cs, y, o.yb[col] + dc);
-  if (!__all_sync(WFULL, isfinite(rate.cs) && isfinite(y))) {
+  if (!__all_sync(WFULL, finite64(rate.cs) && finite64(y))) {
     if (lane == 0) {
       atomicOr(err, ERR_NUMERIC);
       ps->it += 1;
@@ -518,6 +548,7 @@ __device__ inline bool pose_post(const double* tot, DevPose* ps, const DevStats*
     ps->s = rate.sn;
     ps->it += 1;
   }
+  if (!set_mean) return true;
   // the template mean at the new pose, as refresh_pose forms it
   const double mean = fma(rate.sn, fma(st->ybar0[2], wget(y, 6 + col), fma(st->ybar0[1], wget(y, 3 + col), st->ybar0[0] * wget(y, col))),
                           wget(y, 9 + col));
