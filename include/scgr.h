@@ -394,7 +394,9 @@ SCGR_EXPORT scgr_status scgr_step_apply_dev(scgr_ctx* ctx, const double* parts_d
 #define SCGR_TUNE_REUSE_POSE_FREE 6   /* 1 (default): odd integer p skips the per-iteration all-pairs pass.
                                          p = 1: the pair weights do not depend on the pose, so scgr_run
                                          computes the force sums once per call and reuses them
-                                         (bit-identical).  p = 3: the sums are a quadratic form in the
+                                         (templates of the fused tail's size: bit-identical; larger ones: the
+                                         totals of every iteration come from 22 float64 moments of the sums,
+                                         equal up to rounding).  p = 3: the sums are a quadratic form in the
                                          template point over 14 moments of the similarity weights,
                                          computed once per call (equal up to rounding).  0: the all-pairs
                                          pass in every iteration */

@@ -393,7 +393,7 @@ constexpr int FUSED_MAX_SLOTS = 2048;  // templates up to this many padded slots
 cudaError_t launch_combine_finalize(Launch L, const float4* partial, int S, int mpad, int m, const float4* Y0r,
                                     const float* aY32, int g_mode, DevPose* pose, const DevStats* stats,
                                     StepParams sp, int* err);
-constexpr int SMALL_MAX_POINTS = 8192;  // padded reference points that fit a block's shared memory
+constexpr int SMALL_MAX_POINTS = 7680;  // padded reference points that fit a block's shared memory
 bool small_run_available();
 cudaError_t launch_small_run(Launch L, int pmode, const float4* Xr, const float2* XA, int npad, const float4* Y0r,
                              const float* aY32, int g_mode, int m, DevPose* pose, const DevStats* stats,

@@ -349,14 +349,17 @@ scgr_status replan(scgr_ctx* c) {
 // every iteration (bit-identical to recomputing them); for larger ones the
 // iteration's totals come from 22 moments of the sums, and one launch runs all
 // iterations (launch_fixed_run; equal up to rounding): 35,000 x 30,800, 200
-// iterations 4.6 -> 1.2 ms.
+// iterations 4.6 -> 1.3 ms.
 // For p = 3 the sums are a quadratic form in the template point over 14
 // pose-free moments of g (computed once per run; an exact re-association, so
 // equal to the direct pass up to rounding).
 // Small problems of the other exponents run all iterations in one launch of
 // a thread-block cluster (launch_small_run) unless the force launches are to be
-// timed.  The cluster's 16 SMs bound its pair rate (2.8e11/s), so from 5e6
-// pairs on the whole GPU is faster, launches and all.
+// timed.  The cluster's 16 SMs bound its pair rate, so from SMALL_MAX_PAIRS on
+// the whole GPU is faster, launches and all (an iteration, cluster against
+// launches: 500 x 500 7.6 and 20.9 us, 1,000 x 1,000 11.0 and 22.7, 2,000 x
+// 2,000 26.4 and 28.4, 3,000 x 1,600 35.8 and 31.7).
+constexpr int64_t SMALL_MAX_PAIRS = 4200000;
 scgr_status enqueue_iterations(scgr_ctx* c, int iters) {
   const int nb = combine_blocks(c->mpad);
   const StepParams sp = step_params(c);
@@ -383,7 +386,7 @@ scgr_status enqueue_iterations(scgr_ctx* c, int iters) {
     return SCGR_OK;
   }
   if (fused && c->small_ok && !c->timing && !moments && c->fp.pmode != 1 && c->npad <= SMALL_MAX_POINTS &&
-      c->n * c->m <= 5000000 && iters > 0) {
+      c->n * c->m <= SMALL_MAX_PAIRS && iters > 0) {
     SCGR_CK(c, launch_small_run(c->L(), c->fp.pmode, (const float4*)c->Xr.p, (const float2*)c->XA.p, (int)c->npad,
                                 (const float4*)c->Y0r.p, (const float*)c->aY32.p, c->prm.g_mode, (int)c->m, c->pose,
                                 c->stats, sp, c->qexp, iters, c->errword));

@@ -20,36 +20,38 @@ namespace cg = cooperative_groups;
 
 namespace scgr {
 
-constexpr int SMALL_FORCE = 512;                                // threads on the pairs
-constexpr int SMALL_THREADS = SMALL_FORCE + 32 * POSE_PRE_WARPS;  // and the update's first half (leader)
+constexpr int SMALL_THREADS = 512;
+constexpr int SMALL_WARPS = SMALL_THREADS / 32;  // slices of the reference, one per warp
 constexpr int SMALL_CLUSTER = 16;
 constexpr int SMALL_RUN = 128;  // reference points per plain float32 sum (as the half-tile force pass)
-constexpr int SMALL_MAX_ROWS = 64;  // sums that meet in the leader: one per warp of points and block
+constexpr int SMALL_MAX_P = 4;
 
 struct SmallShared {
   DevPose ps;          // the leader's pose; the other blocks use its float32 map
   DevStats st;
   PosePre pre;
-  PoseRate rate;
-  double rows[SMALL_MAX_ROWS][13];
-  double cols[8][13];
+  PoseRate rate[2];
+  double rows[SMALL_CLUSTER * SMALL_MAX_P][13];  // one per warp of points and block
+  double cols[4][13];
   double tot[13];
-  float4 part[SMALL_FORCE];
+  bool ok;
 };
 
-// pc: template points per block (32, 64 or 128), so SMALL_FORCE / pc slices of
-// the reference per point; a warp shares its slice (broadcast reads).
-template <int PM>
+// P template points per lane: a block owns 32 P points, and each of its warps
+// takes them against one slice of the reference (broadcast reads).
+template <int PM, int P>
 __global__ void __launch_bounds__(SMALL_THREADS, 1)
     small_run_kernel(const float* __restrict__ Xr, const float* __restrict__ XA, int npad,
-                     const float4* __restrict__ Y0r, const float* __restrict__ aY32, int g_mode, int m, int pc,
-                     DevPose* pose, const DevStats* __restrict__ stats, StepParams sp, float qexp, int iters, int* err) {
-  extern __shared__ __align__(16) float sX[];  // [6][npad]
+                     const float4* __restrict__ Y0r, const float* __restrict__ aY32, int g_mode, int m, DevPose* pose,
+                     const DevStats* __restrict__ stats, StepParams sp, float qexp, int iters, int* err) {
+  constexpr int PC = 32 * P;
+  extern __shared__ __align__(16) float sX[];  // [6][npad], then the slices' sums [SMALL_WARPS][PC]
   __shared__ SmallShared S;
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank(), nblk = (int)cluster.num_blocks();
+  const int rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool leader = rank == 0;
+  float4* part = reinterpret_cast<float4*>(sX + (size_t)6 * npad);
 
   for (int t = tid; t < npad / FORCE_TJ * 6 * (FORCE_TJ / 4); t += SMALL_THREADS) {
     const int tile = t / (6 * (FORCE_TJ / 4)), r = t / (FORCE_TJ / 4) % 6, j = t % (FORCE_TJ / 4);
@@ -58,123 +60,159 @@ __global__ void __launch_bounds__(SMALL_THREADS, 1)
   }
   if (tid < (int)(sizeof(DevPose) / 4)) reinterpret_cast<int*>(&S.ps)[tid] = reinterpret_cast<const int*>(pose)[tid];
   if (tid < (int)(sizeof(DevStats) / 4)) reinterpret_cast<int*>(&S.st)[tid] = reinterpret_cast<const int*>(stats)[tid];
-  const int p = tid % pc, sl = tid / pc, i = rank * pc + p;
-  const float4 y0 = i < m ? Y0r[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-  const float ay = i < m && g_mode == 1 ? aY32[i] : 1.f;
-  const int len = npad / (SMALL_FORCE / pc);
+  float4 y0[P];
+#pragma unroll
+  for (int q = 0; q < P; ++q) {
+    const int i = rank * PC + q * 32 + lane;
+    y0[q] = i < m ? Y0r[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  const int len = npad / SMALL_WARPS;
   cluster.sync();
+  const int it0 = S.ps.it, E = S.ps.E;
+  if (leader && warp == 1) pose_schedule(it0, E, sp, S.rate[0]);
+  if (leader && warp == 2) pose_scale(S.ps.s, &S.st, sp, S.rate[0]);
 
   for (int it = 0; it < iters; ++it) {
-    if (tid >= SMALL_FORCE) {
-      if (leader) pose_pre(warp - SMALL_FORCE / 32, &S.ps, &S.st, sp, S.pre, S.rate);
-    } else {
-      const PointFrame fr(&S.ps);
-      {
+    PoseRate& now = S.rate[it & 1];
+    PoseRate& next = S.rate[(it + 1) & 1];
+    const PointFrame fr(&S.ps);
+    if (leader && warp >= SMALL_WARPS - 2) pose_pre(2 + (warp & 1), &S.ps, &S.st, sp, S.pre, now);
+    {
+      u64 mx[P], my[P], mz[P], ny[P], ah[P];
+      float h[P][4], c[P][4];
+#pragma unroll
+      for (int q = 0; q < P; ++q) {
         float yx, yy, yz;
-        template_point(y0, fr.A, fr.b, yx, yy, yz);
+        template_point(y0[q], fr.A, fr.b, yx, yy, yz);
         const float n = fmaf(yz, yz, fmaf(yy, yy, yx * yx));
-        const u64 mx = pk2(-2.f * yx, -2.f * yx), my = pk2(-2.f * yy, -2.f * yy), mz = pk2(-2.f * yz, -2.f * yz);
-        const u64 ny = pk2(n, n), ah = pk2(y0.w, y0.w), nq = pk2(-qexp, -qexp);
-        float h[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
-        const float* x0 = sX + sl * len;
-        for (int j0 = 0; j0 < len; j0 += SMALL_RUN) {
-          u64 a[2][4];
+        mx[q] = pk2(-2.f * yx, -2.f * yx);
+        my[q] = pk2(-2.f * yy, -2.f * yy);
+        mz[q] = pk2(-2.f * yz, -2.f * yz);
+        ny[q] = pk2(n, n);
+        ah[q] = pk2(y0[q].w, y0[q].w);
 #pragma unroll
-          for (int u = 0; u < 2; ++u)
+        for (int v = 0; v < 4; ++v) h[q][v] = c[q][v] = 0.f;
+      }
+      const u64 nq = pk2(-qexp, -qexp);
+      const float* x0 = sX + warp * len;
+      for (int j0 = 0; j0 < len; j0 += SMALL_RUN) {
+        u64 a[P][4];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) a[u][v] = 0ull;
-          const int j1 = min(len, j0 + SMALL_RUN);
-#pragma unroll 2
-          for (int j = j0; j < j1; j += 4) {
-            const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(x0 + j);
-            const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(x0 + npad + j);
-            const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(x0 + 2 * npad + j);
-            const ulonglong2 N = *reinterpret_cast<const ulonglong2*>(x0 + 3 * npad + j);
-            const ulonglong2 Av = *reinterpret_cast<const ulonglong2*>(x0 + 4 * npad + j);
-            const ulonglong2 Lv = *reinterpret_cast<const ulonglong2*>(x0 + 5 * npad + j);
-            pair2<PM>(X.x, Y.x, Z.x, N.x, Av.x, Lv.x, mx, my, mz, ny, ah, nq, a[0][0], a[0][1], a[0][2], a[0][3]);
-            pair2<PM>(X.y, Y.y, Z.y, N.y, Av.y, Lv.y, mx, my, mz, ny, ah, nq, a[1][0], a[1][1], a[1][2], a[1][3]);
-          }
+        for (int q = 0; q < P; ++q)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) a[q][v] = 0ull;
+        const int j1 = min(len, j0 + SMALL_RUN);
+        constexpr int UNR = P >= 4 ? 1 : P == 2 ? 2 : 4;
+#pragma unroll UNR
+        for (int j = j0; j < j1; j += 4) {
+          const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(x0 + j);
+          const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(x0 + npad + j);
+          const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(x0 + 2 * npad + j);
+          const ulonglong2 N = *reinterpret_cast<const ulonglong2*>(x0 + 3 * npad + j);
+          const ulonglong2 Av = *reinterpret_cast<const ulonglong2*>(x0 + 4 * npad + j);
+          const ulonglong2 Lv = *reinterpret_cast<const ulonglong2*>(x0 + 5 * npad + j);
+#pragma unroll
+          for (int q = 0; q < P; ++q)
+            pair2<PM>(X.x, Y.x, Z.x, N.x, Av.x, Lv.x, mx[q], my[q], mz[q], ny[q], ah[q], nq, a[q][0], a[q][1], a[q][2], a[q][3]);
+#pragma unroll
+          for (int q = 0; q < P; ++q)
+            pair2<PM>(X.y, Y.y, Z.y, N.y, Av.y, Lv.y, mx[q], my[q], mz[q], ny[q], ah[q], nq, a[q][0], a[q][1], a[q][2], a[q][3]);
+        }
+#pragma unroll
+        for (int q = 0; q < P; ++q)
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
             float l0, l1;
-            upk2(add2(a[0][v], a[1][v]), l0, l1);
-            kahan_add(h[v], c[v], l0 + l1);
+            upk2(a[q][v], l0, l1);
+            kahan_add(h[q][v], c[q][v], l0 + l1);
           }
-        }
-        S.part[sl * pc + p] = make_float4(h[0] - c[0], h[1] - c[1], h[2] - c[2], h[3] - c[3]);
       }
-      asm volatile("bar.sync 1, %0;" ::"n"(SMALL_FORCE) : "memory");
-      if (tid < pc) {  // whole warps
-        float acc[13];
 #pragma unroll
-        for (int q = 0; q < 13; ++q) acc[q] = 0.f;
-        const float4 fw = point_fw(S.part, (size_t)pc, SMALL_FORCE / pc, p, y0, ay, fr);
-        if (i < m) point_acc(fw, y0, fr, acc);
-        double w[16];
+      for (int q = 0; q < P; ++q)
+        part[warp * PC + q * 32 + lane] =
+            make_float4(h[q][0] - c[q][0], h[q][1] - c[q][1], h[q][2] - c[q][2], h[q][3] - c[q][3]);
+    }
+    __syncthreads();
+    if (warp < P) {  // point `tid` of the block
+      const int i = rank * PC + tid;
+      const float4 y = i < m ? Y0r[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      float acc[13];
 #pragma unroll
-        for (int q = 0; q < 13; ++q) w[q] = (double)acc[q];
-        w[13] = w[14] = w[15] = 0.0;
-        warp_reduce16(w);
-        const int q = warp_reduce16_slot(lane);
-        double* row = cluster.map_shared_rank(&S.rows[0][0], 0) + (rank * (pc / 32) + warp) * 13;
-        if ((lane & 1) == 0 && q < 13) row[q] = w[0];
+      for (int q = 0; q < 13; ++q) acc[q] = 0.f;
+      if (i < m) {
+        const float4 fw = point_fw(part, (size_t)PC, SMALL_WARPS, tid, y, g_mode == 1 ? aY32[i] : 1.f, fr);
+        point_acc(fw, y, fr, acc);
       }
+      double w[16];
+#pragma unroll
+      for (int q = 0; q < 13; ++q) w[q] = (double)acc[q];
+      w[13] = w[14] = w[15] = 0.0;
+      warp_reduce16(w);
+      const int q = warp_reduce16_slot(lane);
+      double* row = cluster.map_shared_rank(&S.rows[0][0], 0) + (rank * P + warp) * 13;
+      if ((lane & 1) == 0 && q < 13) row[q] = w[0];
     }
     cluster.sync();  // the rows are in the leader, every block has read its map
     if (leader) {
-      const int rows = nblk * (pc / 32);
-      if (warp < 8 && lane < 13) {
+      constexpr int ROWS = SMALL_CLUSTER * P;
+      // column sums: 8 chains (4 warps x 2 half warps) of ROWS / 8, then across
+      if (warp < 4) {
+        const int half = lane >> 4, q = lane & 15;
         double v = 0.0;
-        for (int r = warp; r < rows; r += 8) v += S.rows[r][lane];
-        S.cols[warp][lane] = v;
+        if (q < 13)
+#pragma unroll
+          for (int r = 0; r < ROWS / 8; ++r) v += S.rows[r * 8 + warp * 2 + half][q];
+        v += __shfl_xor_sync(WFULL, v, 16);
+        if (lane < 13) S.cols[warp][lane] = v;
       }
       __syncthreads();
       if (warp == 0) {
-        if (lane < 13) {
-          double v = S.cols[0][lane];
-#pragma unroll
-          for (int k = 1; k < 8; ++k) v += S.cols[k][lane];
-          S.tot[lane] = v;
-        }
+        if (lane < 13) S.tot[lane] = ((S.cols[0][lane] + S.cols[1][lane]) + S.cols[2][lane]) + S.cols[3][lane];
         __syncwarp();
-        pose_post(S.tot, &S.ps, &S.st, sp, S.pre, S.rate, err);
+        const bool moved = pose_post(S.tot, &S.ps, &S.st, sp, S.pre, now, err);
+        if (lane == 0) S.ok = moved;
         __syncwarp();
         // the float32 map (A, b, ych, ycl: 18 consecutive floats) to the other blocks
         constexpr int MAP = 18;
         static_assert(sizeof(((DevPose*)0)->A) + sizeof(((DevPose*)0)->b) + sizeof(((DevPose*)0)->ych) +
                               sizeof(((DevPose*)0)->ycl) == MAP * 4, "map layout");
-        for (int e = lane; e < (nblk - 1) * MAP; e += 32)
+        for (int e = lane; e < (SMALL_CLUSTER - 1) * MAP; e += 32)
           cluster.map_shared_rank(S.ps.A, 1 + e / MAP)[e % MAP] = S.ps.A[e % MAP];
+      } else if (warp == 1) {  // beside it: the next iteration's schedule and scale
+        pose_schedule(it0 + it + 1, E, sp, next);
+      } else if (warp == 2) {
+        pose_scale(now.sn, &S.st, sp, next);
       }
     }
     cluster.sync();
+    if (leader && !S.ok) {  // the pose was kept, and so is its scale
+      if (warp == 2) pose_scale(S.ps.s, &S.st, sp, next);
+      __syncthreads();
+    }
   }
   if (leader && tid < (int)(sizeof(DevPose) / 4)) reinterpret_cast<int*>(pose)[tid] = reinterpret_cast<const int*>(&S.ps)[tid];
 }
 
-static int small_points(int m) {
-  const int per = (m + SMALL_CLUSTER - 1) / SMALL_CLUSTER;
-  return per <= 32 ? 32 : per <= 64 ? 64 : 128;
+static size_t small_smem(int npad, int P) {
+  return (size_t)npad * 6 * sizeof(float) + (size_t)SMALL_WARPS * 32 * P * sizeof(float4);
 }
 
-template <int PM>
+template <int PM, int P>
 static cudaError_t small_config(int npad, int* clusters, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at) {
-  const size_t smem = (size_t)npad * 6 * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(small_run_kernel<PM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       SMALL_MAX_POINTS * 6 * (int)sizeof(float));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(small_run_kernel<PM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = cudaFuncSetAttribute(small_run_kernel<PM, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)small_smem(SMALL_MAX_POINTS, P));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(small_run_kernel<PM, P>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3(SMALL_CLUSTER);
   cfg->blockDim = dim3(SMALL_THREADS);
-  cfg->dynamicSmemBytes = smem;
+  cfg->dynamicSmemBytes = small_smem(npad, P);
   at->id = cudaLaunchAttributeClusterDimension;
   at->val.clusterDim.x = SMALL_CLUSTER;
   at->val.clusterDim.y = at->val.clusterDim.z = 1;
   cfg->attrs = at;
   cfg->numAttrs = 1;
-  return clusters ? cudaOccupancyMaxActiveClusters(clusters, small_run_kernel<PM>, cfg) : cudaSuccess;
+  return clusters ? cudaOccupancyMaxActiveClusters(clusters, small_run_kernel<PM, P>, cfg) : cudaSuccess;
 }
 
 // Whether the device runs a cluster of this kernel (asked once per context).
@@ -182,25 +220,35 @@ bool small_run_available() {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
   int clusters = 0;
-  if (small_config<2>(SMALL_MAX_POINTS, &clusters, &cfg, at) != cudaSuccess) {
+  if (small_config<2, SMALL_MAX_P>(SMALL_MAX_POINTS, &clusters, &cfg, at) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   return clusters > 0;
 }
 
+template <int PM, int P>
+static cudaError_t launch_small_p(Launch L, const float* Xr, const float* XA, int npad, const float4* Y0r,
+                                  const float* aY32, int g_mode, int m, DevPose* pose, const DevStats* stats,
+                                  StepParams sp, float qexp, int iters, int* err) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  cudaError_t e = small_config<PM, P>(npad, nullptr, &cfg, at);
+  if (e != cudaSuccess) return e;
+  cfg.stream = L.stream;
+  if (L.counter) ++*L.counter;
+  return cudaLaunchKernelEx(&cfg, small_run_kernel<PM, P>, Xr, XA, npad, Y0r, aY32, g_mode, m, pose, stats, sp, qexp,
+                            iters, err);
+}
+
 template <int PM>
 static cudaError_t launch_small_pm(Launch L, const float* Xr, const float* XA, int npad, const float4* Y0r,
                                    const float* aY32, int g_mode, int m, DevPose* pose, const DevStats* stats,
                                    StepParams sp, float qexp, int iters, int* err) {
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute at[1];
-  cudaError_t e = small_config<PM>(npad, nullptr, &cfg, at);
-  if (e != cudaSuccess) return e;
-  cfg.stream = L.stream;
-  if (L.counter) ++*L.counter;
-  return cudaLaunchKernelEx(&cfg, small_run_kernel<PM>, Xr, XA, npad, Y0r, aY32, g_mode, m, small_points(m), pose,
-                            stats, sp, qexp, iters, err);
+  const auto launch = m <= SMALL_CLUSTER * 32   ? launch_small_p<PM, 1>
+                      : m <= SMALL_CLUSTER * 64 ? launch_small_p<PM, 2>
+                                                : launch_small_p<PM, 4>;
+  return launch(L, Xr, XA, npad, Y0r, aY32, g_mode, m, pose, stats, sp, qexp, iters, err);
 }
 
 cudaError_t launch_small_run(Launch L, int pmode, const float4* Xr, const float2* XA, int npad, const float4* Y0r,
