@@ -96,7 +96,7 @@ void scgr_destroy(scgr_ctx* c) {
                     &c->bcpair, &c->btabX, &c->btabY, &c->bxoff, &c->byoff, &c->bstats, &c->bposes, &c->bnext,
                     &c->gspec, &c->gcell[0], &c->gcell[1], &c->gstart[0], &c->gstart[1], &c->gtot[0], &c->gtot[1],
                     &c->gsorted[0], &c->gsorted[1], &c->gccount,
-                    &c->cd_key, &c->cd_moved, &c->wstore, &c->wupart, &c->wpartial, &c->mpart, &c->mom, &c->radpart, &c->sigpart, &c->fixpart};
+                    &c->cd_key, &c->cd_moved, &c->wstore, &c->wupart, &c->wpartial, &c->mpart, &c->mom, &c->radpart, &c->sigpart, &c->fixpart, &c->upart};
   for (DevBuf* b : bufs) release(*b);
   if (c->pose) cudaFree(c->pose);
   if (c->pose_eval) cudaFree(c->pose_eval);
@@ -149,14 +149,10 @@ scgr_status scgr_compute_descriptors(scgr_ctx* c) {
   if (cs != SCGR_OK) return cs;
   c->npad = (c->n + 255) / 256 * 256;
   const int64_t mloc = c->rows >= 0 ? c->rows : c->m;
-  c->fp = plan_force(mloc, c->npad, c->prm.p, c->num_sms, c->ftune);
-  c->mpad = force_mpad(mloc, c->fp);
+  const scgr_status bs = plan_buffers(c);
+  if (bs != SCGR_OK) return bs;
   SCGR_CK(c, ensure(c->Xr, (size_t)c->npad * sizeof(float4)));
   SCGR_CK(c, ensure(c->XA, (size_t)c->npad * sizeof(float2)));
-  SCGR_CK(c, ensure(c->Y0r, (size_t)c->mpad * sizeof(float4)));
-  SCGR_CK(c, ensure(c->partial, (size_t)c->fp.splits * c->mpad * sizeof(float4)));
-  SCGR_CK(c, ensure(c->blockpart, (size_t)combine_blocks(c->mpad) * 13 * sizeof(double)));
-  SCGR_CK(c, ensure(c->fixpart, fixed_part_bytes(c->num_sms)));
   SCGR_CK(c, launch_records(L, X4, (const double*)c->aX64.p, n, (int)c->npad, Y4 + c->row0,
                             (const double*)c->aY64.p + c->row0, (int)mloc, (int)c->mpad, c->prm.g_mode, st,
                             (float4*)c->Xr.p, (float2*)c->XA.p, (float4*)c->Y0r.p));

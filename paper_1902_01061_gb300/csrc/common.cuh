@@ -435,16 +435,23 @@ cudaError_t launch_force_vjp(Launch L, const float4* Xr, const float2* XA, int n
 // length of the records, a multiple of 256).
 cudaError_t launch_store_pairs(Launch L, const float2* XA, const float4* Xr, int npad, const float4* Y0r,
                                const double* aY64, int g_mode, int m, const DevPose* ps, float qexp, float* Wst,
-                               double* Upart, double* Uout);
+                               double* Upart);
 cudaError_t launch_stored_rows(Launch L, const float* Wst, int npad, int m, const float4* Xr, float4* partial);
 int store_pairs_columns(int npad);   // grid columns of the store pass
 int store_pairs_row_blocks(int m);   // grid rows of the store pass
-cudaError_t launch_pose_from7(Launch L, const double* pose7_dev, DevPose* ps, const DevStats* st);
+// A pose formed on the host (row-vector convention).
+struct HostPose {
+  double R[9], t[3], s;
+};
+cudaError_t launch_pose_from_host(Launch L, const HostPose& hp, DevPose* ps, const DevStats* st);
+cudaError_t launch_potential(Launch L, const ForcePlan& fp, bool grad, const float4* Xr, const float2* XA, int ntiles,
+                             const float4* Y0r, int mpad, int m, const float* aY32, int g_mode, const DevPose* ps,
+                             float qexp, float4* partial, double* upart);
+cudaError_t launch_potential_finish(Launch L, const double* upart, int64_t nu, const double* blockpart, int nb,
+                                    const int* err, double* out);
 cudaError_t launch_adjoint_combine(Launch L, const float4* partial, int S, int mpad, int m, const float4* Y0r,
                                    const double* aY64, int g_mode, const DevPose* ps, float* grad_xyz,
                                    double* blockpart);
 cudaError_t launch_column_sum13(Launch L, const double* part, int nb, double* out);
-cudaError_t launch_adjoint_finish(Launch L, const double* tot, const double* pose7_dev, const DevPose* ps,
-                                  double* grad7);
 
 }  // namespace scgr

@@ -57,13 +57,14 @@ struct scgr_ctx {
   int iterations = 0;      // iterations enqueued since the descriptors
   int64_t launches = 0;
   ForcePlan fp{};
+  ForcePlan fpot{};        // the potential's pair pass
   float qexp = 0.f;        // (p - 1) / 2, exponent of d^2 in the weight
 
   DevBuf X4, Y4, stage, knnX, knnY, aX64, aY64, aX32, aY32, Xr, XA, Y0r, partial, blockpart,
       moved_stage;
   DevPose* pose = nullptr;
   DevPose* pose_eval = nullptr;  // pose of a potential / gradient evaluation
-  double* aux = nullptr;         // [0,13) forward sums, [16,29) adjoint sums, [32,39) grad7, [48,55) pose7
+  double* aux = nullptr;         // sums on their way to or from the host (64 doubles)
   DevStats* stats = nullptr;
   int* errword = nullptr;
   double* red = nullptr;   // reduction scratch
@@ -86,7 +87,7 @@ struct scgr_ctx {
   int64_t nearest_grid_min = 1024; // references with at least this many points: grid nearest search (tunable)
   ForceTuning ftune;            // force-plan overrides (tunable)
   int reuse_pose_free = 1;      // p = 1: one force pass per scgr_run (tunable)
-  DevBuf cd_key, cd_moved, wstore, wupart, wpartial, mpart, mom, radpart, sigpart, fixpart;
+  DevBuf cd_key, cd_moved, wstore, wupart, wpartial, mpart, mom, radpart, sigpart, fixpart, upart;
   // grids of the reference [0] and the template [1], kept until the cloud changes
   DevBuf gspec, gcell[2], gstart[2], gtot[2], gsorted[2], gccount;
   bool grid_ok[2] = {false, false};  // sorted into grid cells
@@ -135,6 +136,7 @@ constexpr int64_t KNN_FUSED_KEY = 20000;
 scgr_status prepare_clouds(scgr_ctx* c);
 scgr_status nearest_reference(scgr_ctx* c, const float* q3, int nq, int32_t* idx_out, float* key_out);
 scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_scale);
+scgr_status plan_buffers(scgr_ctx* c);
 scgr_status replan(scgr_ctx* c);
 scgr_status enqueue_iterations(scgr_ctx* c, int iters);
 void drop_graph(scgr_ctx* c);

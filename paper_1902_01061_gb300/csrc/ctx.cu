@@ -325,15 +325,41 @@ scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_sca
   return SCGR_OK;
 }
 
+// The force plan of the context's template rows, the potential's plan beside
+// it, and the buffers whose size they set.  The potential runs 1 or 2 points x
+// 128 threads (the shapes its kernel has) in splits that fit the force pass's
+// partials.
+scgr_status plan_buffers(scgr_ctx* c) {
+  const int64_t mloc = c->rows >= 0 ? c->rows : c->m;
+  c->fp = plan_force(mloc, c->npad, c->prm.p, c->num_sms, c->ftune);
+  c->mpad = force_mpad(mloc, c->fp);
+  ForceTuning t;
+  t.P = mloc >= 4096 ? 2 : 1;
+  t.tpb = 128;
+  t.occ = 0;
+  ForcePlan& fu = c->fpot;
+  fu = plan_force(mloc, c->npad, c->prm.p, c->num_sms, t);
+  const int64_t ntiles = c->npad / FORCE_TJ, cap = (int64_t)c->fp.splits;
+  if (fu.half || fu.splits > cap) {
+    const int64_t S = fu.half ? (cap < ntiles ? cap : ntiles) : cap;
+    fu.half = 0;
+    fu.tiles_per_split = (int)((ntiles + S - 1) / S);
+    fu.splits = (int)((ntiles + fu.tiles_per_split - 1) / fu.tiles_per_split);
+  }
+  SCGR_CK(c, ensure(c->Y0r, (size_t)c->mpad * sizeof(float4)));
+  SCGR_CK(c, ensure(c->partial, (size_t)c->fp.splits * c->mpad * sizeof(float4)));
+  SCGR_CK(c, ensure(c->blockpart, (size_t)combine_blocks(c->mpad) * 13 * sizeof(double)));
+  SCGR_CK(c, ensure(c->fixpart, fixed_part_bytes(c->num_sms)));
+  SCGR_CK(c, ensure(c->upart, (size_t)fu.splits * fu.iblocks * sizeof(double)));
+  return SCGR_OK;
+}
+
 // Recompute the force plan (after a tuning change) and the buffers and
 // template records that depend on it; descriptors and pose are kept.
 scgr_status replan(scgr_ctx* c) {
   const int64_t mloc = c->rows >= 0 ? c->rows : c->m;
-  c->fp = plan_force(mloc, c->npad, c->prm.p, c->num_sms, c->ftune);
-  c->mpad = force_mpad(mloc, c->fp);
-  SCGR_CK(c, ensure(c->Y0r, (size_t)c->mpad * sizeof(float4)));
-  SCGR_CK(c, ensure(c->partial, (size_t)c->fp.splits * c->mpad * sizeof(float4)));
-  SCGR_CK(c, ensure(c->blockpart, (size_t)combine_blocks(c->mpad) * 13 * sizeof(double)));
+  const scgr_status ps = plan_buffers(c);
+  if (ps != SCGR_OK) return ps;
   SCGR_CK(c, launch_records(c->L(), (const float4*)c->X4.p, (const double*)c->aX64.p, (int)c->n, (int)c->npad,
                             (const float4*)c->Y4.p + c->row0, (const double*)c->aY64.p + c->row0, (int)mloc,
                             (int)c->mpad, c->prm.g_mode, c->stats, (float4*)c->Xr.p, (float2*)c->XA.p,

@@ -11,122 +11,304 @@
 // dU/domega = J_r(omega)^T w, where w is the axial vector of the skew part of
 // B = (dU/dR) R_col (w_c = sum_ab eps_abc B_ab).
 //
-// The forward pass is the force kernel with the distance exponent raised by
-// two (it accumulates sum_j g d^(p+1)); the adjoint pass re-runs the force
-// kernel at the same pose (tile recomputation: no N x M storage) and reduces
-// the chain-rule terms in float64 in a fixed order.
+// U and the adjoint's per-point sums come from one pass over the pairs:
+// w_ij = g d^(p-1) gives both w d^2 = g d^(p+1) for U and the sums of the force
+// kernel (sum w, sum w X') for G_i; without gradients only U is summed.  Tiles
+// are recomputed (no N x M storage), the chain-rule terms reduced in float64 in
+// a fixed order.  The 3x3 algebra of the pose (Rodrigues' formula, J_r) is done
+// by the host, which has pose7 and reads the totals anyway.
 #include <cmath>
 
 #include "common.cuh"
+#include "pair.cuh"
 #include "pointsum.cuh"
 
 namespace scgr {
 
-// Template point in the frame centred on the reference mean (identical
-// arithmetic to the force kernel's).
 __device__ __forceinline__ void tpoint(const float4 y0, const float* A, const float* b, float& yx,
                                        float& yy, float& yz) {
-  yx = fmaf(y0.z, A[6], fmaf(y0.y, A[3], fmaf(y0.x, A[0], b[0])));
-  yy = fmaf(y0.z, A[7], fmaf(y0.y, A[4], fmaf(y0.x, A[1], b[1])));
-  yz = fmaf(y0.z, A[8], fmaf(y0.y, A[5], fmaf(y0.x, A[2], b[2])));
+  template_point(y0, A, b, yx, yy, yz);
 }
 
-// Row-vector rotation R = exp([w]_x)^T by the Rodrigues formula.
-__device__ void rotation_from_axis_angle(const double* w, double* R) {
-  const double th2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
-  double a, bq;  // exp([w]x) = I + a K + bq K^2
-  if (th2 < 1e-16) {
-    a = 1.0 - th2 / 6.0;
-    bq = 0.5 - th2 / 24.0;
+// The pose of an evaluation and its float32 map (one warp).
+__global__ void pose_from_host_kernel(const HostPose hp, DevPose* ps, const DevStats* __restrict__ st) {
+  const int l = threadIdx.x;
+  if (l < 9) {
+    ps->R[l] = hp.R[l];
+    ps->A[l] = (float)(hp.s * hp.R[l]);
+  }
+  if (l < 3) {
+    ps->t[l] = hp.t[l];
+    ps->b[l] = (float)(hp.t[l] - st->xbar[l]);
+    const double yb = hp.s * (st->ybar0[0] * hp.R[l] + st->ybar0[1] * hp.R[3 + l] + st->ybar0[2] * hp.R[6 + l]) + hp.t[l];
+    set_ybs(ps, l, yb - st->xbar[l]);
+  }
+  if (l == 0) {
+    ps->s = hp.s;
+    ps->it = 0;
+    ps->E = 1;
+    ps->degenerate = 0;
+  }
+}
+
+// ---- the pair pass -----------------------------------------------------------
+
+// Reference points (j, j+1) against one template point: U += w d^2, and with
+// GRAD W += w, S += w X'.
+template <int PM, bool GRAD>
+__device__ __forceinline__ void potential_pair2(u64 xv, u64 yv, u64 zv, u64 nv, u64 av, u64 lv, u64 mx, u64 my, u64 mz,
+                                                u64 ny, u64 ah, u64 nq, u64& U, u64& W, u64& Sx, u64& Sy, u64& Sz) {
+  u64 d2 = add2(nv, ny);
+  d2 = fma2(xv, mx, d2);
+  d2 = fma2(yv, my, d2);
+  d2 = fma2(zv, mz, d2);
+  const u64 u = sub2(av, ah);
+  const u64 ep = fma2(u, u, lv);
+  float e0, e1, q0, q1;
+  u64 w;
+  if (PM == 0) {
+    upk2(d2, q0, q1);
+    upk2(fma2(nq, pk2(lg2_approx(fabsf(q0)), lg2_approx(fabsf(q1))), ep), e0, e1);
+    w = pk2(ex2_neg(e0), ex2_neg(e1));
   } else {
-    const double th = sqrt(th2);
-    a = sin(th) / th;
-    bq = (1.0 - cos(th)) / th2;
-  }
-  const double K[9] = {0.0, -w[2], w[1], w[2], 0.0, -w[0], -w[1], w[0], 0.0};
-  for (int r = 0; r < 3; ++r)
-    for (int c = 0; c < 3; ++c) {
-      double k2 = 0.0;
-      for (int q = 0; q < 3; ++q) k2 += K[r * 3 + q] * K[q * 3 + c];
-      const double rc = (r == c ? 1.0 : 0.0) + a * K[r * 3 + c] + bq * k2;
-      R[c * 3 + r] = rc;  // transpose: row-vector convention
+    upk2(ep, e0, e1);
+    w = pk2(ex2_neg(e0), ex2_neg(e1));
+    if (PM == 2) {
+      upk2(d2, q0, q1);
+      w = mul2(w, pk2(sqrt_approx(fabsf(q0)), sqrt_approx(fabsf(q1))));
+    } else if (PM == 3) {
+      w = mul2(w, d2);
     }
-}
-
-__global__ void pose_from7_kernel(const double* __restrict__ pose7, DevPose* ps, const DevStats* st) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  rotation_from_axis_angle(pose7, ps->R);
-  for (int c = 0; c < 3; ++c) ps->t[c] = pose7[3 + c];
-  ps->s = pose7[6];
-  for (int q = 0; q < 9; ++q) ps->A[q] = (float)(ps->s * ps->R[q]);
-  for (int c = 0; c < 3; ++c) {
-    ps->b[c] = (float)(ps->t[c] - st->xbar[c]);
-    const double yb = ps->s * (st->ybar0[0] * ps->R[c] + st->ybar0[1] * ps->R[3 + c] +
-                               st->ybar0[2] * ps->R[6 + c]) + ps->t[c];
-    set_ybs(ps, c, yb - st->xbar[c]);
   }
-  ps->it = 0;
-  ps->E = 1;
-  ps->degenerate = 0;
+  U = fma2(w, d2, U);
+  if (GRAD) {
+    W = add2(W, w);
+    Sx = fma2(w, xv, Sx);
+    Sy = fma2(w, yv, Sy);
+    Sz = fma2(w, zv, Sz);
+  }
 }
 
-// Per point: G_i = -f_i from the split partials; the template-coordinate
-// gradient s G_i R^T; per-block chain-rule sums (sum G, sum G.(Y0 R),
-// sum Y0^T G).
+// Template points [blockIdx.x * P * POT_TPB, ...) against the reference tiles
+// of split blockIdx.y, at pose *ps.  The block's sum of aY U goes to upart in
+// float64; with GRAD the points' (sum w, sum w X') to partial[split][mpad].
+// Bound and layout are the force kernel's: ex2 and sqrt on the special-function
+// unit (10.6 pairs per clock per SM), 12 FP32 lane operations a pair with
+// gradients, 8 without; packed pairs, broadcast tiles, Kahan sums across tiles.
+constexpr int POT_TPB = 128;
+
+template <int P, int PM, bool GRAD>
+__global__ void __launch_bounds__(POT_TPB)
+    potential_tile_kernel(const float* __restrict__ Xr, const float* __restrict__ XA, int ntiles, int tiles_per_split,
+                          const float4* __restrict__ Y0r, int mpad, int m, const float* __restrict__ aY32, int g_mode,
+                          const DevPose* __restrict__ ps, float qexp, float4* __restrict__ partial,
+                          double* __restrict__ upart) {
+  constexpr int TJ = FORCE_TJ, Q4 = TJ / 4, NV = GRAD ? 5 : 1;
+  __shared__ __align__(16) float sT[6][TJ];
+  __shared__ double shu[POT_TPB / 32];
+  const int i0 = blockIdx.x * (P * POT_TPB) + threadIdx.x;
+  float A[9], b[3];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) A[q] = ps->A[q];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) b[q] = ps->b[q];
+  u64 mx[P], my[P], mz[P], ny[P], ah[P];
+  float h[P][NV], c[P][NV];
+#pragma unroll
+  for (int q = 0; q < P; ++q) {
+    const float4 y0 = Y0r[i0 + q * POT_TPB];
+    float x, y, z;
+    tpoint(y0, A, b, x, y, z);
+    const float n = fmaf(z, z, fmaf(y, y, x * x));
+    mx[q] = pk2(-2.f * x, -2.f * x);
+    my[q] = pk2(-2.f * y, -2.f * y);
+    mz[q] = pk2(-2.f * z, -2.f * z);
+    ny[q] = pk2(n, n);
+    ah[q] = pk2(y0.w, y0.w);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) h[q][v] = c[q][v] = 0.f;
+  }
+  const u64 nq = pk2(-qexp, -qexp);
+  const int t0 = blockIdx.y * tiles_per_split, t1 = min(ntiles, t0 + tiles_per_split);
+  for (int t = t0; t < t1; ++t) {
+    __syncthreads();
+    const float4* g4 = reinterpret_cast<const float4*>(Xr + (size_t)t * 4 * TJ);
+    const float4* a4 = reinterpret_cast<const float4*>(XA + (size_t)t * 2 * TJ);
+#pragma unroll
+    for (int u = threadIdx.x; u < 6 * Q4; u += POT_TPB)
+      *reinterpret_cast<float4*>(&sT[u / Q4][4 * (u % Q4)]) = u < 4 * Q4 ? g4[u] : a4[u - 4 * Q4];
+    __syncthreads();
+    u64 acc[P][5];
+#pragma unroll
+    for (int q = 0; q < P; ++q)
+#pragma unroll
+      for (int v = 0; v < 5; ++v) acc[q][v] = 0ull;
+#pragma unroll 2
+    for (int jq = 0; jq < TJ; jq += 4) {
+      const ulonglong2 X = *reinterpret_cast<const ulonglong2*>(&sT[0][jq]);
+      const ulonglong2 Y = *reinterpret_cast<const ulonglong2*>(&sT[1][jq]);
+      const ulonglong2 Z = *reinterpret_cast<const ulonglong2*>(&sT[2][jq]);
+      const ulonglong2 N = *reinterpret_cast<const ulonglong2*>(&sT[3][jq]);
+      const ulonglong2 Av = *reinterpret_cast<const ulonglong2*>(&sT[4][jq]);
+      const ulonglong2 Lv = *reinterpret_cast<const ulonglong2*>(&sT[5][jq]);
+#pragma unroll
+      for (int q = 0; q < P; ++q)
+        potential_pair2<PM, GRAD>(X.x, Y.x, Z.x, N.x, Av.x, Lv.x, mx[q], my[q], mz[q], ny[q], ah[q], nq, acc[q][0],
+                                  acc[q][1], acc[q][2], acc[q][3], acc[q][4]);
+#pragma unroll
+      for (int q = 0; q < P; ++q)
+        potential_pair2<PM, GRAD>(X.y, Y.y, Z.y, N.y, Av.y, Lv.y, mx[q], my[q], mz[q], ny[q], ah[q], nq, acc[q][0],
+                                  acc[q][1], acc[q][2], acc[q][3], acc[q][4]);
+    }
+#pragma unroll
+    for (int q = 0; q < P; ++q)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        float l0, l1;
+        upk2(acc[q][v], l0, l1);
+        kahan_add(h[q][v], c[q][v], l0 + l1);
+      }
+  }
+  double u = 0.0;
+#pragma unroll
+  for (int q = 0; q < P; ++q) {
+    const int i = i0 + q * POT_TPB;
+    if (i < m) u += (g_mode == 1 ? (double)aY32[i] : 1.0) * ((double)h[q][0] - (double)c[q][0]);
+    if constexpr (GRAD)
+      partial[(size_t)blockIdx.y * mpad + i] =
+          make_float4(h[q][1] - c[q][1], h[q][2] - c[q][2], h[q][3] - c[q][3], h[q][4] - c[q][4]);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) u += __shfl_down_sync(0xffffffffu, u, off);
+  if ((threadIdx.x & 31) == 0) shu[threadIdx.x >> 5] = u;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = shu[0];
+#pragma unroll
+    for (int w = 1; w < POT_TPB / 32; ++w) t += shu[w];
+    upart[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
+  }
+}
+
+template <int PM>
+static void launch_potential_pm(Launch L, const ForcePlan& fp, bool grad, const float* Xr, const float* XA, int ntiles,
+                                const float4* Y0r, int mpad, int m, const float* aY32, int g_mode, const DevPose* ps,
+                                float qexp, float4* partial, double* upart) {
+  const dim3 grid(fp.iblocks, fp.splits);
+  const auto k = fp.P == 2 ? (grad ? potential_tile_kernel<2, PM, true> : potential_tile_kernel<2, PM, false>)
+                           : (grad ? potential_tile_kernel<1, PM, true> : potential_tile_kernel<1, PM, false>);
+  k<<<grid, POT_TPB, 0, L.stream>>>(Xr, XA, ntiles, fp.tiles_per_split, Y0r, mpad, m, aY32, g_mode, ps, qexp, partial,
+                                    upart);
+}
+
+// The pair pass of the potential under plan fp (1 or 2 points x 128 threads).
+cudaError_t launch_potential(Launch L, const ForcePlan& fp, bool grad, const float4* Xr, const float2* XA, int ntiles,
+                             const float4* Y0r, int mpad, int m, const float* aY32, int g_mode, const DevPose* ps,
+                             float qexp, float4* partial, double* upart) {
+  const float* xr = reinterpret_cast<const float*>(Xr);
+  const float* xa = reinterpret_cast<const float*>(XA);
+  const auto launch = fp.pmode == 1   ? launch_potential_pm<1>
+                      : fp.pmode == 3 ? launch_potential_pm<3>
+                      : fp.pmode == 0 ? launch_potential_pm<0>
+                                      : launch_potential_pm<2>;
+  launch(L, fp, grad, xr, xa, ntiles, Y0r, mpad, m, aY32, g_mode, ps, qexp, partial, upart);
+  if (L.counter) ++*L.counter;
+  return cudaGetLastError();
+}
+
+// Per point: G_i = -f_i from the split partials (added with Kahan
+// compensation, the rest in float64); the template-coordinate gradient s G_i R^T;
+// per-block chain-rule sums (sum G, sum G.(Y0 R), sum Y0^T G).
 __global__ void __launch_bounds__(RED_THREADS)
     adjoint_combine_kernel(const float4* __restrict__ partial, int S, int mpad, int m,
                            const float4* __restrict__ Y0r, const double* __restrict__ aY64,
                            int g_mode, const DevPose* __restrict__ ps, float* __restrict__ grad_xyz,
                            double* __restrict__ blockpart) {
-  __shared__ double sh[13][RED_THREADS];
+  __shared__ double sh[RED_THREADS / 32][16];
   const int i = blockIdx.x * RED_THREADS + threadIdx.x;
-  double v[13];
+  double v[16];
 #pragma unroll
-  for (int q = 0; q < 13; ++q) v[q] = 0.0;
+  for (int q = 0; q < 16; ++q) v[q] = 0.0;
   if (i < m) {
-    double W = 0, Sx = 0, Sy = 0, Sz = 0;
-    for (int s = 0; s < S; ++s) {
-      const float4 pp = partial[(size_t)s * mpad + i];
-      W += pp.x;
-      Sx += pp.y;
-      Sy += pp.z;
-      Sz += pp.w;
-    }
+    const PointSums r = point_sums(partial, (size_t)mpad, S, i);
+    const double W = (double)r.Wh - (double)r.Wc;
     float A[9], b[3];
 #pragma unroll
     for (int q = 0; q < 9; ++q) A[q] = ps->A[q];
 #pragma unroll
     for (int q = 0; q < 3; ++q) b[q] = ps->b[q];
     const float4 y0 = Y0r[i];
-    float yx, yy, yz;
-    tpoint(y0, A, b, yx, yy, yz);
+    float y[3];
+    tpoint(y0, A, b, y[0], y[1], y[2]);
     const double ay = g_mode == 1 ? aY64[i] : 1.0;
-    // G = dU/dY = -f = aY (Y' sum w - sum w X')
-    const double G[3] = {ay * ((double)yx * W - Sx), ay * ((double)yy * W - Sy), ay * ((double)yz * W - Sz)};
     const double Y0d[3] = {(double)y0.x, (double)y0.y, (double)y0.z};
-    double y0R[3];
-    for (int c = 0; c < 3; ++c)
-      y0R[c] = Y0d[0] * ps->R[c] + Y0d[1] * ps->R[3 + c] + Y0d[2] * ps->R[6 + c];
-    v[0] = G[0];
-    v[1] = G[1];
-    v[2] = G[2];
-    v[3] = G[0] * y0R[0] + G[1] * y0R[1] + G[2] * y0R[2];
+    double R[9], G[3];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) R[q] = ps->R[q];
+    // G = dU/dY = -f = aY (Y' sum w - sum w X')
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      G[c] = ay * fma((double)y[c], W, (double)r.Sc[c] - (double)r.Sh[c]);
+      v[c] = G[c];
+    }
+    double gY[3];  // G R^T: dU/dY0 = s gY, and G.(Y0 R) = Y0 . gY
+#pragma unroll
+    for (int a = 0; a < 3; ++a) gY[a] = fma(G[2], R[a * 3 + 2], fma(G[1], R[a * 3 + 1], G[0] * R[a * 3]));
+    v[3] = fma(Y0d[2], gY[2], fma(Y0d[1], gY[1], Y0d[0] * gY[0]));
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
       for (int bb = 0; bb < 3; ++bb) v[4 + 3 * a + bb] = Y0d[a] * G[bb];
     if (grad_xyz) {
-      for (int a = 0; a < 3; ++a) {
-        const double gr = ps->s * (G[0] * ps->R[a * 3] + G[1] * ps->R[a * 3 + 1] + G[2] * ps->R[a * 3 + 2]);
-        grad_xyz[(size_t)i * 3 + a] = (float)gr;
-      }
+      const double s = ps->s;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) grad_xyz[(size_t)i * 3 + a] = (float)(s * gY[a]);
     }
   }
-  block_sum<13>(v, sh);
-  if (threadIdx.x == 0) {
+  warp_reduce16(v);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if ((lane & 1) == 0) sh[warp][warp_reduce16_slot(lane)] = v[0];
+  __syncthreads();
+  if (threadIdx.x < 13) {
+    double t = sh[0][threadIdx.x];
 #pragma unroll
-    for (int q = 0; q < 13; ++q) blockpart[(size_t)blockIdx.x * 13 + q] = v[q];
+    for (int w = 1; w < RED_THREADS / 32; ++w) t += sh[w][threadIdx.x];
+    blockpart[(size_t)blockIdx.x * 13 + threadIdx.x] = t;
   }
+}
+
+// One block: out[0] = sum of nu doubles of upart, out[1 .. 13] = column sums of
+// nb rows of blockpart (nb = 0: none), out[14] = the device error word; all in
+// a fixed order.
+constexpr int PF_T = 512;
+__global__ void __launch_bounds__(PF_T)
+    potential_finish_kernel(const double* __restrict__ upart, int64_t nu, const double* __restrict__ blockpart, int nb,
+                            const int* __restrict__ err, double* __restrict__ out) {
+  __shared__ double sh[PF_T / 32][14];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double u = 0.0;
+  for (int64_t q = threadIdx.x; q < nu; q += PF_T) u += upart[q];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) u += __shfl_xor_sync(0xffffffffu, u, off);
+  double col = 0.0;
+  if (lane < 13)
+    for (int b = warp; b < nb; b += PF_T / 32) col += blockpart[(size_t)b * 13 + lane];
+  if (lane < 13) sh[warp][1 + lane] = col;
+  if (lane == 0) sh[warp][0] = u;
+  __syncthreads();
+  if (threadIdx.x < 14) {
+    double t = sh[0][threadIdx.x];
+    for (int w = 1; w < PF_T / 32; ++w) t += sh[w][threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+  if (threadIdx.x == 32) out[14] = (double)*err;
+}
+
+cudaError_t launch_potential_finish(Launch L, const double* upart, int64_t nu, const double* blockpart, int nb,
+                                    const int* err, double* out) {
+  potential_finish_kernel<<<1, PF_T, 0, L.stream>>>(upart, nu, blockpart, nb, err, out);
+  if (L.counter) ++*L.counter;
+  return cudaGetLastError();
 }
 
 // One block: fixed-order column sums of [nb][13] partials.
@@ -145,46 +327,6 @@ __global__ void __launch_bounds__(RED_THREADS) column_sum13_kernel(const double*
 #pragma unroll
     for (int q = 0; q < 13; ++q) out[q] = v[q];
   }
-}
-
-// grad7 = (dU/domega, dU/dt, dU/ds) from the chain-rule sums.
-__global__ void adjoint_finish_kernel(const double* __restrict__ tot, const double* __restrict__ pose7,
-                                      const DevPose* __restrict__ ps, double* __restrict__ grad7) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const double s = ps->s;
-  double M[9];  // dU/dR
-  for (int q = 0; q < 9; ++q) M[q] = s * tot[4 + q];
-  // B = M R_col, R_col = R^T
-  double B[9];
-  for (int a = 0; a < 3; ++a)
-    for (int c = 0; c < 3; ++c) {
-      double acc = 0.0;
-      for (int q = 0; q < 3; ++q) acc += M[a * 3 + q] * ps->R[c * 3 + q];
-      B[a * 3 + c] = acc;
-    }
-  const double w[3] = {B[5] - B[7], B[6] - B[2], B[1] - B[3]};
-  const double* om = pose7;
-  const double th2 = om[0] * om[0] + om[1] * om[1] + om[2] * om[2];
-  double c1, c2;  // J_r = I - c1 K + c2 K^2
-  if (th2 < 1e-12) {
-    c1 = 0.5 - th2 / 24.0;
-    c2 = 1.0 / 6.0 - th2 / 120.0;
-  } else {
-    const double th = sqrt(th2);
-    c1 = (1.0 - cos(th)) / th2;
-    c2 = (th - sin(th)) / (th2 * th);
-  }
-  const double K[9] = {0.0, -om[2], om[1], om[2], 0.0, -om[0], -om[1], om[0], 0.0};
-  double J[9];
-  for (int r = 0; r < 3; ++r)
-    for (int c = 0; c < 3; ++c) {
-      double k2 = 0.0;
-      for (int q = 0; q < 3; ++q) k2 += K[r * 3 + q] * K[q * 3 + c];
-      J[r * 3 + c] = (r == c ? 1.0 : 0.0) - c1 * K[r * 3 + c] + c2 * k2;
-    }
-  for (int k = 0; k < 3; ++k) grad7[k] = J[0 * 3 + k] * w[0] + J[1 * 3 + k] * w[1] + J[2 * 3 + k] * w[2];
-  for (int c = 0; c < 3; ++c) grad7[3 + c] = tot[c];
-  grad7[6] = tot[3];
 }
 
 // ---- vector-Jacobian product of the force field ---------------------------
@@ -214,22 +356,6 @@ constexpr int VJP_TPB = 128;
 constexpr int VJP_NC = 6;                 // C: xx xy xz yy yz zz
 constexpr float VJP_D2_MIN = 1e-37f;      // keeps rsqrt and lg2 of d^2 = 0 finite (the products with r are 0)
 
-__device__ __forceinline__ float vjp_ex2_neg(float x) {
-  float y;
-  asm("{ .reg .f32 t; neg.f32 t, %1; ex2.approx.ftz.f32 %0, t; }" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float vjp_rsqrt(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float vjp_lg2(float x) {
-  float y;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Reference points (j, j+1) against one template point.  PM = 1, 2, 3: p = PM;
 // 0: general p, with c = 2^(e2 log2 d^2 - ep), e2 = (p - 3) / 2 (nq = -e2).
 template <int PM>
@@ -240,14 +366,14 @@ __device__ __forceinline__ void vjp_pair2(u64 xv, u64 yv, u64 zv, u64 av, u64 lv
   float e0, e1;
   if (PM == 1) {
     upk2(ep, e0, e1);
-    C[0] = add2(C[0], pk2(vjp_ex2_neg(e0), vjp_ex2_neg(e1)));
+    C[0] = add2(C[0], pk2(ex2_neg(e0), ex2_neg(e1)));
     return;
   }
   const u64 rx = sub2(yx, xv), ry = sub2(yy, yv), rz = sub2(yz, zv);
   u64 c;
   if (PM == 3) {
     upk2(ep, e0, e1);
-    c = pk2(vjp_ex2_neg(e0), vjp_ex2_neg(e1));
+    c = pk2(ex2_neg(e0), ex2_neg(e1));
   } else {
     float q0, q1;
     upk2(fma2(rz, rz, fma2(ry, ry, mul2(rx, rx))), q0, q1);
@@ -255,10 +381,10 @@ __device__ __forceinline__ void vjp_pair2(u64 xv, u64 yv, u64 zv, u64 av, u64 lv
     q1 = fmaxf(q1, VJP_D2_MIN);
     if (PM == 2) {
       upk2(ep, e0, e1);
-      c = mul2(pk2(vjp_ex2_neg(e0), vjp_ex2_neg(e1)), pk2(vjp_rsqrt(q0), vjp_rsqrt(q1)));
+      c = mul2(pk2(ex2_neg(e0), ex2_neg(e1)), pk2(rsqrt_approx(q0), rsqrt_approx(q1)));
     } else {
-      upk2(fma2(nq, pk2(vjp_lg2(q0), vjp_lg2(q1)), ep), e0, e1);
-      c = pk2(vjp_ex2_neg(e0), vjp_ex2_neg(e1));
+      upk2(fma2(nq, pk2(lg2_approx(q0), lg2_approx(q1)), ep), e0, e1);
+      c = pk2(ex2_neg(e0), ex2_neg(e1));
     }
   }
   const u64 cx = mul2(c, rx), cy = mul2(c, ry), cz = mul2(c, rz);
@@ -589,25 +715,15 @@ __global__ void __launch_bounds__(ST_TPB, 2)
                                             (float)red[0][threadIdx.x * 4 + 2], (float)red[0][threadIdx.x * 4 + 3]);
 }
 
-__global__ void __launch_bounds__(RED_THREADS) sum_rows_kernel(const double* __restrict__ part, int64_t count,
-                                                               double* __restrict__ out) {
-  __shared__ double sh[1][RED_THREADS];
-  double v[1] = {0.0};
-  for (int64_t q = threadIdx.x; q < count; q += RED_THREADS) v[0] += part[q];
-  block_sum<1>(v, sh);
-  if (threadIdx.x == 0) out[0] = v[0];
-}
-
 cudaError_t launch_store_pairs(Launch L, const float2* XA, const float4* Xr, int npad, const float4* Y0r,
                                const double* aY64, int g_mode, int m, const DevPose* ps, float qexp, float* Wst,
-                               double* Upart, double* Uout) {
+                               double* Upart) {
   const int nb = store_pairs_columns(npad);
   const int ib = (m + ST_ROWS - 1) / ST_ROWS;
   store_pairs_kernel<<<dim3(ib, nb), ST_TPB, 0, L.stream>>>(reinterpret_cast<const float*>(Xr),
                                                            reinterpret_cast<const float*>(XA), npad, m, Y0r, aY64,
                                                            g_mode, ps, qexp, Wst, Upart);
-  sum_rows_kernel<<<1, RED_THREADS, 0, L.stream>>>(Upart, (int64_t)nb * ib, Uout);
-  if (L.counter) *L.counter += 2;
+  if (L.counter) *L.counter += 1;
   return cudaGetLastError();
 }
 
@@ -621,8 +737,8 @@ cudaError_t launch_stored_rows(Launch L, const float* Wst, int npad, int m, cons
   return cudaGetLastError();
 }
 
-cudaError_t launch_pose_from7(Launch L, const double* pose7_dev, DevPose* ps, const DevStats* st) {
-  pose_from7_kernel<<<1, 32, 0, L.stream>>>(pose7_dev, ps, st);
+cudaError_t launch_pose_from_host(Launch L, const HostPose& hp, DevPose* ps, const DevStats* st) {
+  pose_from_host_kernel<<<1, 32, 0, L.stream>>>(hp, ps, st);
   if (L.counter) ++*L.counter;
   return cudaGetLastError();
 }
@@ -638,13 +754,6 @@ cudaError_t launch_adjoint_combine(Launch L, const float4* partial, int S, int m
 
 cudaError_t launch_column_sum13(Launch L, const double* part, int nb, double* out) {
   column_sum13_kernel<<<1, RED_THREADS, 0, L.stream>>>(part, nb, out);
-  if (L.counter) ++*L.counter;
-  return cudaGetLastError();
-}
-
-cudaError_t launch_adjoint_finish(Launch L, const double* tot, const double* pose7_dev, const DevPose* ps,
-                                  double* grad7) {
-  adjoint_finish_kernel<<<1, 32, 0, L.stream>>>(tot, pose7_dev, ps, grad7);
   if (L.counter) ++*L.counter;
   return cudaGetLastError();
 }
