@@ -93,7 +93,8 @@ void scgr_destroy(scgr_ctx* c) {
                     &c->aY32, &c->Xr, &c->XA, &c->Y0r, &c->partial, &c->blockpart, &c->moved_stage,
                     &c->bX4, &c->bY4, &c->bknnX, &c->bknnY, &c->baX64, &c->baY64, &c->baX32, &c->baY32,
                     &c->bXr, &c->bXA, &c->bY0r, &c->bpartial, &c->bblockpart, &c->bpairs, &c->bitems,
-                    &c->bcpair, &c->btabX, &c->btabY, &c->bxoff, &c->byoff, &c->bstats, &c->bposes, &c->bnext,
+                    &c->bcpair, &c->btab, &c->bstats, &c->bposes, &c->bnext,
+                    &c->bgclouds, &c->bgspec, &c->bgcell, &c->bgsorted, &c->bgstart, &c->bgtot, &c->bgpart,
                     &c->gspec, &c->gcell[0], &c->gcell[1], &c->gstart[0], &c->gstart[1], &c->gtot[0], &c->gtot[1],
                     &c->gsorted[0], &c->gsorted[1], &c->gccount,
                     &c->cd_key, &c->cd_moved, &c->wstore, &c->wupart, &c->wpartial, &c->mpart, &c->mom, &c->radpart, &c->sigpart, &c->fixpart, &c->upart};

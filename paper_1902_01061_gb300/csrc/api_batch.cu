@@ -54,7 +54,7 @@ scgr_status scgr_batch_run(scgr_ctx* c, int npairs, const int64_t* ref_off, cons
   std::vector<BatchPair> pairs(npairs);
   std::vector<int4> items;
   std::vector<int> cpair;
-  std::vector<int2> tabX, tabY;
+  std::vector<int2> tab;  // kNN queries: (cloud, first), references then templates
   int64_t xt = 0, yb = 0, pb = 0;
   int cb = 0;
   for (int p = 0; p < npairs; ++p) {
@@ -86,15 +86,27 @@ scgr_status scgr_batch_run(scgr_ctx* c, int npairs, const int64_t* ref_off, cons
         const int pts = (int)std::min<int64_t>(FB, bp.m - (int64_t)b * FB);
         items.push_back(make_int4(p, b, ch, tiles * pts));
       }
-    for (int64_t q0 = 0; q0 < bp.n; q0 += 128) tabX.push_back(make_int2(p, (int)q0));
-    for (int64_t q0 = 0; q0 < bp.m; q0 += 128) tabY.push_back(make_int2(p, (int)q0));
+    for (int64_t q0 = 0; q0 < bp.n; q0 += KNN_TABLE_CHUNK) tab.push_back(make_int2(p, (int)q0));
+    for (int64_t q0 = 0; q0 < bp.m; q0 += KNN_TABLE_CHUNK) tab.push_back(make_int2(npairs + p, (int)q0));
   }
   std::stable_sort(items.begin(), items.end(), [](const int4& a, const int4& b) { return a.w > b.w; });
-  // kNN blocks scan their whole cloud: biggest clouds first, so the small
-  // ones fill the last wave
-  std::stable_sort(tabX.begin(), tabX.end(), [&](const int2& a, const int2& b) { return pairs[a.x].n > pairs[b.x].n; });
-  std::stable_sort(tabY.begin(), tabY.end(), [&](const int2& a, const int2& b) { return pairs[a.x].m > pairs[b.x].m; });
-  std::vector<int64_t> xoff(ref_off, ref_off + npairs + 1), yoff(tmp_off, tmp_off + npairs + 1);
+  // the clouds' grids: references 0..npairs-1, templates npairs..2 npairs-1
+  const int nclouds = 2 * npairs;
+  std::vector<GridCloud> clouds(nclouds);
+  int64_t most = 0;
+  size_t gstart = 0, gtot = 0;
+  std::vector<size_t> start_off(nclouds), tot_off(nclouds);
+  for (int q = 0; q < nclouds; ++q) {
+    const BatchPair& bp = pairs[q % npairs];
+    const int64_t n = q < npairs ? bp.n : bp.m;
+    clouds[q].n = (int)n;
+    clouds[q].base = (int)(q < npairs ? bp.x0 : bp.y0);
+    most = std::max(most, n);
+    start_off[q] = gstart;
+    tot_off[q] = gtot;
+    gstart += grid_start_entries(n);
+    gtot += grid_tot_entries(n);
+  }
 
   // ---- device buffers
   SCGR_CK(c, ensure(c->bX4, (size_t)Ntot * sizeof(float4)));
@@ -113,37 +125,63 @@ scgr_status scgr_batch_run(scgr_ctx* c, int npairs, const int64_t* ref_off, cons
   SCGR_CK(c, ensure(c->bpairs, pairs.size() * sizeof(BatchPair)));
   SCGR_CK(c, ensure(c->bitems, items.size() * sizeof(int4)));
   SCGR_CK(c, ensure(c->bcpair, cpair.size() * sizeof(int)));
-  SCGR_CK(c, ensure(c->btabX, tabX.size() * sizeof(int2)));
-  SCGR_CK(c, ensure(c->btabY, tabY.size() * sizeof(int2)));
-  SCGR_CK(c, ensure(c->bxoff, xoff.size() * sizeof(int64_t)));
-  SCGR_CK(c, ensure(c->byoff, yoff.size() * sizeof(int64_t)));
+  SCGR_CK(c, ensure(c->btab, tab.size() * sizeof(int2)));
+  SCGR_CK(c, ensure(c->bgclouds, (size_t)nclouds * sizeof(GridCloud)));
+  SCGR_CK(c, ensure(c->bgspec, (size_t)nclouds * sizeof(GridSpec)));
+  SCGR_CK(c, ensure(c->bgcell, (size_t)(Ntot + Mtot) * sizeof(int2)));
+  SCGR_CK(c, ensure(c->bgsorted, (size_t)(Ntot + Mtot) * sizeof(float4)));
+  SCGR_CK(c, ensure(c->bgstart, gstart * sizeof(int)));
+  SCGR_CK(c, ensure(c->bgtot, gtot * sizeof(int)));
+  SCGR_CK(c, ensure(c->bgpart, (size_t)nclouds * CLOUD_PARTS * 6 * (sizeof(double) + sizeof(float))));
   SCGR_CK(c, ensure(c->bstats, (size_t)npairs * sizeof(DevStats)));
   SCGR_CK(c, ensure(c->bposes, (size_t)npairs * sizeof(DevPose)));
   SCGR_CK(c, ensure(c->bnext, sizeof(int)));
+  DevStats* bst = (DevStats*)c->bstats.p;
+  for (int q = 0; q < nclouds; ++q) {
+    const bool ref = q < npairs;
+    const int p = q % npairs;
+    const size_t at = (ref ? 0 : (size_t)Ntot) + clouds[q].base;
+    GridCloud& g = clouds[q];
+    g.P = (const float4*)(ref ? c->bX4.p : c->bY4.p) + g.base;
+    g.spec = (GridSpec*)c->bgspec.p + q;
+    g.cell = (int2*)c->bgcell.p + at;
+    g.sorted = (float4*)c->bgsorted.p + at;
+    g.start = (int*)c->bgstart.p + start_off[q];
+    g.tot = (int*)c->bgtot.p + tot_off[q];
+    g.knn = (int32_t*)(ref ? c->bknnX.p : c->bknnY.p);
+    // addresses on the device, not read here
+    g.mean = ref ? bst[p].xbar : bst[p].ybar0;
+    g.scatter = ref ? bst[p].CX : bst[p].S0;
+    g.lmax = ref ? &bst[p].eX : &bst[p].eY0;
+  }
   cudaStream_t st = c->stream;
   SCGR_CK(c, cudaMemcpyAsync(c->bpairs.p, pairs.data(), pairs.size() * sizeof(BatchPair), cudaMemcpyHostToDevice, st));
   SCGR_CK(c, cudaMemcpyAsync(c->bitems.p, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
   SCGR_CK(c, cudaMemcpyAsync(c->bcpair.p, cpair.data(), cpair.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  SCGR_CK(c, cudaMemcpyAsync(c->btabX.p, tabX.data(), tabX.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
-  SCGR_CK(c, cudaMemcpyAsync(c->btabY.p, tabY.data(), tabY.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
-  SCGR_CK(c, cudaMemcpyAsync(c->bxoff.p, xoff.data(), xoff.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-  SCGR_CK(c, cudaMemcpyAsync(c->byoff.p, yoff.data(), yoff.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st));
+  SCGR_CK(c, cudaMemcpyAsync(c->btab.p, tab.data(), tab.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+  SCGR_CK(c, cudaMemcpyAsync(c->bgclouds.p, clouds.data(), clouds.size() * sizeof(GridCloud), cudaMemcpyHostToDevice, st));
 
   // ---- descriptors for every cloud, in one launch per stage
   Launch L = c->L();
   const BatchPair* dpairs = (const BatchPair*)c->bpairs.p;
   SCGR_CK(c, launch_pack(L, ref_xyz_dev, Ntot, (float4*)c->bX4.p, c->errword));
   SCGR_CK(c, launch_pack(L, tmp_xyz_dev, Mtot, (float4*)c->bY4.p, c->errword));
-  SCGR_CK(c, launch_knn_multi(L, (const float4*)c->bX4.p, (const int64_t*)c->bxoff.p, (const int2*)c->btabX.p,
-                              (int)tabX.size(), k, (int32_t*)c->bknnX.p));
-  SCGR_CK(c, launch_knn_multi(L, (const float4*)c->bY4.p, (const int64_t*)c->byoff.p, (const int2*)c->btabY.p,
-                              (int)tabY.size(), k, (int32_t*)c->bknnY.p));
-  SCGR_CK(c, launch_curvature(L, (const float4*)c->bX4.p, (const int32_t*)c->bknnX.p, (int)Ntot, k,
-                              (double*)c->baX64.p, (float*)c->baX32.p));
-  SCGR_CK(c, launch_curvature(L, (const float4*)c->bY4.p, (const int32_t*)c->bknnY.p, (int)Mtot, k,
-                              (double*)c->baY64.p, (float*)c->baY32.p));
-  SCGR_CK(c, launch_stats_multi(L, (const float4*)c->bX4.p, (const float4*)c->bY4.p, (const double*)c->baX64.p,
-                                dpairs, npairs, c->prm.sigma, (DevStats*)c->bstats.p));
+  // grids and statistics of all clouds (65,535 a launch, the grid's y limit)
+  const GridCloud* dclouds = (const GridCloud*)c->bgclouds.p;
+  for (int q0 = 0; q0 < nclouds; q0 += 65535) {
+    const int nq = std::min(65535, nclouds - q0);
+    CloudSet cs{};
+    cs.many = dclouds + q0;
+    double* part = (double*)c->bgpart.p + (size_t)q0 * CLOUD_PARTS * 6;
+    float* bpart = (float*)((double*)c->bgpart.p + (size_t)nclouds * CLOUD_PARTS * 6) + (size_t)q0 * CLOUD_PARTS * 6;
+    SCGR_CK(c, launch_clouds(L, cs, nq, (int)most, true, true, part, bpart));
+    SCGR_CK(c, launch_grid_sort(L, cs, nq, (int)most, part));
+  }
+  SCGR_CK(c, launch_knn_grid_table(L, dclouds, (const int2*)c->btab.p, (int)tab.size(), k));
+  SCGR_CK(c, launch_curvature2(L, (const float4*)c->bX4.p, (const int32_t*)c->bknnX.p, (int)Ntot,
+                               (double*)c->baX64.p, (float*)c->baX32.p, nullptr, (const float4*)c->bY4.p,
+                               (const int32_t*)c->bknnY.p, (int)Mtot, (double*)c->baY64.p, (float*)c->baY32.p, k));
+  SCGR_CK(c, launch_sigma_multi(L, (const double*)c->baX64.p, dpairs, npairs, c->prm.sigma, bst));
   SCGR_CK(c, launch_records_multi(L, (const float4*)c->bX4.p, (const double*)c->baX64.p, (const float4*)c->bY4.p,
                                   (const double*)c->baY64.p, dpairs, npairs, c->prm.g_mode,
                                   (const DevStats*)c->bstats.p, (float4*)c->bXr.p, (float2*)c->bXA.p,

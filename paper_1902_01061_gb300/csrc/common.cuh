@@ -278,6 +278,7 @@ constexpr int CLOUD_SCRATCH_DOUBLES = 2 * CLOUD_PARTS * 9;
 struct GridCloud {
   const float4* P;
   int n;
+  int base;         // index of the first point in knn and in its lists (a batch's clouds share arrays)
   GridSpec* spec;
   int2* cell;       // [n] cell, rank of arrival in it
   int* start;       // [grid_start_entries(n)] counts, then block-local first positions; NULL: no grid wanted
@@ -289,7 +290,7 @@ struct GridCloud {
 // The clouds of a launch: two of a registration, or an array of many on the device.
 struct CloudSet {
   GridCloud one[2];
-  const GridCloud* many;
+  const GridCloud* many = nullptr;
   __device__ __forceinline__ const GridCloud& operator[](int y) const { return many ? many[y] : one[y]; }
 };
 
@@ -312,19 +313,19 @@ cudaError_t launch_sigma_finish(Launch L, const double* part, int n, double sigm
 // sigma = population std of a64 (1 if below 1e-12), or `sigma_user` if > 0
 cudaError_t launch_sigma(Launch L, const double* a64, int n, double sigma_user, double sigma_scale, double* part,
                          DevStats* st);
-cudaError_t launch_knn_multi(Launch L, const float4* P, const int64_t* off_dev, const int2* table_dev,
-                             int nblocks, int k, int32_t* out);
 cudaError_t launch_records_multi(Launch L, const float4* X4, const double* aX64, const float4* Y4,
                                  const double* aY64, const BatchPair* pairs, int npairs, int g_mode,
                                  const DevStats* stats, float4* Xr, float2* XA, float4* Y0r);
-cudaError_t launch_stats_multi(Launch L, const float4* X4, const float4* Y4, const double* aX64,
-                               const BatchPair* pairs, int npairs, double sigma_user, DevStats* out);
+cudaError_t launch_sigma_multi(Launch L, const double* aX64, const BatchPair* pairs, int npairs, double sigma_user,
+                               DevStats* out);
 size_t grid_start_entries(int64_t n);
 size_t grid_tot_entries(int64_t n);
 cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, bool scatter, bool sorted, double* part,
                           float* bpart);
 cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most, const double* part);
 cudaError_t launch_knn_grid(Launch L, const CloudSet& cs, int nclouds, int most, int k, bool fused);
+cudaError_t launch_knn_grid_table(Launch L, const GridCloud* many, const int2* table, int nblocks, int k);
+constexpr int KNN_TABLE_CHUNK = 128;  // queries per table entry
 constexpr int NEAREST_COARSE = 4;  // fine cells per coarse cell side in the two-level nearest search
 cudaError_t launch_coarse_count(Launch L, const CloudSet& cs, int64_t n, int* ccount);
 cudaError_t launch_nearest_grid(Launch L, const CloudSet& cs, int levels, const int* ccount, const float* q3, int nq,

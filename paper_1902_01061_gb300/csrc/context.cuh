@@ -79,7 +79,7 @@ struct scgr_ctx {
 
   // batch workspace
   DevBuf bX4, bY4, bknnX, bknnY, baX64, baY64, baX32, baY32, bXr, bXA, bY0r, bpartial, bblockpart,
-      bpairs, bitems, bcpair, btabX, btabY, bxoff, byoff, bstats, bposes, bnext;
+      bpairs, bitems, bcpair, btab, bstats, bposes, bnext, bgclouds, bgspec, bgcell, bgsorted, bgstart, bgtot, bgpart;
   int batch_chunk_tiles = 0;    // reference tiles per batched work item (tunable; 0: by the batch's size)
   int batch_P = -1;             // template points per thread in the batched force kernel (tunable; -1: by size)
   int batch_persistent = 0;     // 1: persistent batched force kernel with a work queue (tunable)

@@ -183,31 +183,6 @@ __global__ void __launch_bounds__(KNN_TPB, KC > 16 ? 2 : 4) knn_brute_kernel(con
   }
 }
 
-// Many clouds in one launch: block b handles queries [q0, q0 + KNN_TPB) of
-// cloud c = table[b].x (q0 = table[b].y), each against its own cloud only.
-template <int KC>
-__global__ void __launch_bounds__(KNN_TPB, KC > 16 ? 2 : 4) knn_brute_multi_kernel(const float4* __restrict__ P,
-                                                                  const int64_t* __restrict__ off,
-                                                                  const int2* __restrict__ table, int k,
-                                                                  int32_t* __restrict__ out) {
-  __shared__ __align__(16) float tile[3 * KNN_TILE];
-  __shared__ float qks[KNN_QL * KNN_TPB];
-  __shared__ int qis[KNN_QL * KNN_TPB];
-  const int2 e = table[blockIdx.x];
-  const int64_t base = off[e.x];
-  const int n = (int)(off[e.x + 1] - base);
-  const int ql = e.y + threadIdx.x;
-  const float4 q = P[base + (ql < n ? ql : n - 1)];
-  float kd[KC];
-  int ki[KC];
-  knn_scan<KC>(P, base, n, q, kd, ki, tile, qks, qis);
-  if (ql < n) {
-#pragma unroll
-    for (int m = 0; m < KC; ++m)
-      if (m < k) out[(base + ql) * k + m] = ki[m];
-  }
-}
-
 // Nearest reference point of arbitrary query points (change detection):
 // the same exact key and (key, index) order as the kNN, k = 1.
 __global__ void __launch_bounds__(KNN_TPB) nearest_kernel(const float4* __restrict__ P, int n,
@@ -245,15 +220,6 @@ __global__ void threshold_kernel(const float* __restrict__ key, int nq, float th
 cudaError_t launch_threshold(Launch L, const float* key, int nq, float thr2, uint8_t* mask, float* dist) {
   if (nq <= 0) return cudaSuccess;
   threshold_kernel<<<(nq + 255) / 256, 256, 0, L.stream>>>(key, nq, thr2, mask, dist);
-  return after_launch(L);
-}
-
-cudaError_t launch_knn_multi(Launch L, const float4* P, const int64_t* off_dev, const int2* table_dev,
-                             int nblocks, int k, int32_t* out) {
-  if (nblocks <= 0) return cudaSuccess;
-  if (k <= 8) knn_brute_multi_kernel<8><<<nblocks, KNN_TPB, 0, L.stream>>>(P, off_dev, table_dev, k, out);
-  else if (k <= 16) knn_brute_multi_kernel<16><<<nblocks, KNN_TPB, 0, L.stream>>>(P, off_dev, table_dev, k, out);
-  else knn_brute_multi_kernel<32><<<nblocks, KNN_TPB, 0, L.stream>>>(P, off_dev, table_dev, k, out);
   return after_launch(L);
 }
 
@@ -820,67 +786,29 @@ cudaError_t launch_records_multi(Launch L, const float4* X4, const double* aX64,
   return after_launch(L);
 }
 
-// Batched statistics: block p computes, in a fixed order, the reference and
-// template means, scatters and largest eigenvalues of pair p, and sigma
-// (population std of its reference curvatures, or sigma_user if > 0).
-__global__ void __launch_bounds__(RED_THREADS)
-    stats_multi_kernel(const float4* __restrict__ X4, const float4* __restrict__ Y4,
-                       const double* __restrict__ aX64, const BatchPair* __restrict__ pairs,
-                       double sigma_user, DevStats* __restrict__ out) {
-  __shared__ double sh[6][RED_THREADS];
-  const BatchPair bp = pairs[blockIdx.x];
-  DevStats* st = out + blockIdx.x;
-  for (int side = 0; side < 2; ++side) {
-    const float4* P = side == 0 ? X4 + bp.x0 : Y4 + bp.y0;
-    const int64_t n = side == 0 ? bp.n : bp.m;
-    double v3[3] = {0, 0, 0};
-    for (int64_t i = threadIdx.x; i < n; i += RED_THREADS) {
-      const float4 c = P[i];
-      v3[0] += c.x; v3[1] += c.y; v3[2] += c.z;
-    }
-    block_sum<3>(v3, sh);
-    const double mean[3] = {v3[0] / n, v3[1] / n, v3[2] / n};
-    __syncthreads();
-    double v6[6] = {0, 0, 0, 0, 0, 0};
-    for (int64_t i = threadIdx.x; i < n; i += RED_THREADS) {
-      const float4 c = P[i];
-      const double dx = c.x - mean[0], dy = c.y - mean[1], dz = c.z - mean[2];
-      v6[0] += dx * dx; v6[1] += dx * dy; v6[2] += dx * dz;
-      v6[3] += dy * dy; v6[4] += dy * dz; v6[5] += dz * dz;
-    }
-    block_sum<6>(v6, sh);
-    if (threadIdx.x == 0) {
-      const double S[9] = {v6[0], v6[1], v6[2], v6[1], v6[3], v6[4], v6[2], v6[4], v6[5]};
-      double C[9], lam[3];
-      for (int q = 0; q < 9; ++q) C[q] = S[q] / (double)n;
-      sym3_eigenvalues(C, lam);
-      double* mo = side == 0 ? st->xbar : st->ybar0;
-      double* so = side == 0 ? st->CX : st->S0;
-      for (int q = 0; q < 3; ++q) mo[q] = mean[q];
-      for (int q = 0; q < 9; ++q) so[q] = S[q];
-      if (side == 0) st->eX = lam[2];
-      else st->eY0 = lam[2];
-    }
-    __syncthreads();
+// sigma of every pair of a batch: block p takes pair p's reference curvatures
+// (mean, then squared deviations, in a fixed order).
+__global__ void __launch_bounds__(SIGMA_T)
+    sigma_multi_kernel(const double* __restrict__ aX64, const BatchPair* __restrict__ pairs, double sigma_user,
+                       DevStats* __restrict__ out) {
+  __shared__ double sh[SIGMA_T / 32];
+  const BatchPair& bp = pairs[blockIdx.x];
+  const double* a = aX64 + bp.x0;
+  double v = 0.0;
+  for (int64_t i = threadIdx.x; i < bp.n; i += SIGMA_T) v += a[i];
+  const double sum = sigma_block_sum(v, sh), mean = sum / (double)bp.n;
+  v = 0.0;
+  for (int64_t i = threadIdx.x; i < bp.n; i += SIGMA_T) {
+    const double d = a[i] - mean;
+    v = fma(d, d, v);
   }
-  double v1[1] = {0};
-  for (int64_t i = threadIdx.x; i < bp.n; i += RED_THREADS) v1[0] += aX64[bp.x0 + i];
-  block_sum<1>(v1, sh);
-  const double amean = v1[0] / bp.n;
-  const double asum = v1[0];
-  __syncthreads();
-  double v2[1] = {0};
-  for (int64_t i = threadIdx.x; i < bp.n; i += RED_THREADS) {
-    const double d = aX64[bp.x0 + i] - amean;
-    v2[0] += d * d;
-  }
-  block_sum<1>(v2, sh);
-  if (threadIdx.x == 0) finish_sigma(asum, v2[0], bp.n, sigma_user, 1.0, st);
+  const double d2 = sigma_block_sum(v, sh);
+  if (threadIdx.x == 0) finish_sigma(sum, d2, bp.n, sigma_user, 1.0, out + blockIdx.x);
 }
 
-cudaError_t launch_stats_multi(Launch L, const float4* X4, const float4* Y4, const double* aX64,
-                               const BatchPair* pairs, int npairs, double sigma_user, DevStats* out) {
-  stats_multi_kernel<<<npairs, RED_THREADS, 0, L.stream>>>(X4, Y4, aX64, pairs, sigma_user, out);
+cudaError_t launch_sigma_multi(Launch L, const double* aX64, const BatchPair* pairs, int npairs, double sigma_user,
+                               DevStats* out) {
+  sigma_multi_kernel<<<npairs, SIGMA_T, 0, L.stream>>>(aX64, pairs, sigma_user, out);
   return after_launch(L);
 }
 

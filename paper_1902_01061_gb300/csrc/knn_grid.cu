@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(256) cell_scatter_kernel(const CloudSet cs) {
   if (i >= g.n) return;
   const int2 cr = g.cell[i];
   float4 c = g.P[i];
-  c.w = __int_as_float(i);
+  c.w = __int_as_float(g.base + i);
   g.sorted[cell_start(g, cr.x) + cr.y] = c;
 }
 
@@ -527,13 +527,8 @@ __device__ __noinline__ void knn_stream(const GridCloud& g, float4 q, const floa
 }
 
 template <bool FUSED>
-__global__ void __launch_bounds__(QUERY_WARPS * 32, 5) knn_query_kernel(const CloudSet cs, int k) {
-  __shared__ __align__(16) u64 bufs[QUERY_WARPS][QUERY_CAP];
-  const GridCloud& g = cs[blockIdx.y];
+__device__ __forceinline__ void knn_query(const GridCloud& g, int t, int k, u64* buf) {
   const int lane = threadIdx.x & 31;
-  u64* buf = bufs[threadIdx.x >> 5];
-  const int t = blockIdx.x * QUERY_WARPS + (threadIdx.x >> 5);
-  if (t >= g.n) return;
   const GridSpec& sp = *g.spec;
   const int n3[3] = {sp.g[0], sp.g[1], sp.g[2]};
   const float4 q = g.sorted[t];
@@ -646,6 +641,28 @@ __global__ void __launch_bounds__(QUERY_WARPS * 32, 5) knn_query_kernel(const Cl
   }
   __syncwarp();
   knn_stream<FUSED>(g, q, q3, cc, n3, k, buf);
+}
+
+// Cloud blockIdx.y, one query per warp; or (a batch, whose clouds differ in
+// size) the KNN_TABLE_CHUNK queries from table[b].y of cloud table[b].x.
+template <bool FUSED>
+__global__ void __launch_bounds__(QUERY_WARPS * 32, 5)
+    knn_query_kernel(const CloudSet cs, const int2* __restrict__ table, int k) {
+  __shared__ __align__(16) u64 bufs[QUERY_WARPS][QUERY_CAP];
+  const int warp = threadIdx.x >> 5;
+  if (!table) {
+    const GridCloud& g = cs[blockIdx.y];
+    const int t = blockIdx.x * QUERY_WARPS + warp;
+    if (t < g.n) knn_query<FUSED>(g, t, k, bufs[warp]);
+    return;
+  }
+  const int2 e = table[blockIdx.x];
+  const GridCloud& g = cs[e.x];
+  const int end = min(g.n, e.y + KNN_TABLE_CHUNK);
+  for (int t = e.y + warp; t < end; t += QUERY_WARPS) {
+    knn_query<FUSED>(g, t, k, bufs[warp]);
+    __syncwarp();
+  }
 }
 
 // ---- nearest gridded point of external queries -----------------------------------
@@ -823,8 +840,19 @@ cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most
 // form of clouds below the brute-force limit (grid_key).
 cudaError_t launch_knn_grid(Launch L, const CloudSet& cs, int nclouds, int most, int k, bool fused) {
   const dim3 grid(up(most, QUERY_WARPS), nclouds);
-  if (fused) knn_query_kernel<true><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, k);
-  else knn_query_kernel<false><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, k);
+  if (fused) knn_query_kernel<true><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, nullptr, k);
+  else knn_query_kernel<false><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, nullptr, k);
+  if (L.counter) *L.counter += 1;
+  return cudaGetLastError();
+}
+
+// The same for a batch's clouds (device array), in the order of a table of
+// (cloud, first query).  Batches keep the key rounding they had (grid_key).
+cudaError_t launch_knn_grid_table(Launch L, const GridCloud* many, const int2* table, int nblocks, int k) {
+  if (nblocks <= 0) return cudaSuccess;
+  CloudSet cs{};
+  cs.many = many;
+  knn_query_kernel<true><<<nblocks, QUERY_WARPS * 32, 0, L.stream>>>(cs, table, k);
   if (L.counter) *L.counter += 1;
   return cudaGetLastError();
 }
