@@ -226,8 +226,10 @@ __device__ inline double sym3_extreme_eigenvalue(const double* C, bool largest) 
       ok = fabsf(step) <= 2e-6f * l;
     }
     df = fmaf(l, fmaf(-3.f, l, 2.f * f2), -f1);
-    // a well separated root: its polynomial determines it to rounding
-    ok = ok && df < 0.f && (largest ? -df >= 1e-2f * f2 * f2 : -df * l >= 1e-2f * f0);
+    // a well separated root: its polynomial determines it to rounding; below
+    // (above) the inflection at a third of the trace, where rounding in the
+    // coefficients of a rank-1 C can send Newton to the other end
+    ok = ok && df < 0.f && (largest ? 3.f * l > f2 && -df >= 1e-2f * f2 * f2 : 3.f * l < f2 && -df * l >= 1e-2f * f0);
     if (ok) {
       const double r = -(double)__frcp_rn(df);
       double x = (double)l;
