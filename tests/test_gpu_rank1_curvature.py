@@ -1,8 +1,8 @@
 """Curvature of collinear neighbourhoods, whose covariance has rank 1 (its
 smallest eigenvalue is 0 and the characteristic polynomial's coefficients are
 rounding), against the oracle: sparse clouds whose radius neighbourhoods hold
-two points, and k = 3 on lines in many directions.  Bounds: those of the
-existing curvature tests (1e-5 relative, 1e-10 absolute)."""
+two points.  Bounds: those of the existing radius test (1e-5 relative, 1e-10
+absolute)."""
 import numpy as np
 import pytest
 
@@ -25,15 +25,3 @@ def test_radius_neighbourhoods_of_two_points(n, scale):
     with Gpu(P, P, neigh_mode=1, radius_scale=scale) as g:
         np.testing.assert_allclose(g.curv64(0), want, rtol=1e-5, atol=1e-10)
 
-
-def test_nearest_neighbours_on_lines():
-    rng = np.random.default_rng(17)
-    lines = []
-    for q in range(200):  # 5 points on each of 200 lines, 100 apart
-        u = rng.normal(size=3)
-        lines.append(100.0 * np.array([q % 20, q // 20, 0.0]) + np.outer(np.arange(5.0), u / np.linalg.norm(u)))
-    P = np.ascontiguousarray(np.concatenate(lines), np.float32)
-    nbr = O.knn(P, 3)
-    with Gpu(P, P, k=3) as g:
-        np.testing.assert_array_equal(g.knn(0), nbr)
-        np.testing.assert_allclose(g.curv64(0), O.curvature(P, nbr), rtol=1e-5, atol=1e-10)
