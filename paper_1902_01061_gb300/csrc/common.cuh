@@ -304,8 +304,6 @@ struct Launch {
 
 cudaError_t launch_pack(Launch L, const float* xyz, int64_t n, float4* out, int* err);
 cudaError_t launch_knn(Launch L, const float4* P, int n, int k, int32_t* out);
-cudaError_t launch_curvature(Launch L, const float4* P, const int32_t* nbr, int n, int k,
-                             double* a64, float* a32);
 cudaError_t launch_curvature2(Launch L, const float4* X, const int32_t* nx, int n, double* ax64, float* ax32,
                               double* xpart, const float4* Y, const int32_t* ny, int m, double* ay64, float* ay32,
                               int k);
@@ -335,10 +333,27 @@ cudaError_t launch_nearest_grid(Launch L, const CloudSet& cs, int levels, const 
 cudaError_t launch_nearest(Launch L, const float4* P, int n, const float* q3, int nq, int32_t* idx_out,
                            float* key_out);
 cudaError_t launch_threshold(Launch L, const float* key, int nq, float thr2, uint8_t* mask, float* dist);
-size_t radius_scratch_bytes(int n, int num_sms);
-cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const double* e_dev, double scale2,
-                                    const GridSpec* spec, int num_sms, double* part, double* a64, float* a32,
-                                    double* sigma_out);
+size_t radius_scratch_bytes(int n, int num_sms, bool ordered);
+// A cloud in Morton order (order.cu).
+struct OrderCloud {
+  const float4* P;
+  const GridSpec* spec;      // the cloud's box
+  int n;
+  float4* sorted;            // [n] points in order, index in w
+  float* box;                // [ceil(n / 32)][6] min, -max of each run of 32
+  unsigned short* key[2];    // [n]
+  int* perm[2];              // [n]; perm[1] is the order
+  int* count;                // 256 counts a block
+};
+struct OrderClouds {
+  OrderCloud c[2];
+};
+size_t order_bytes(int64_t n);
+OrderCloud order_cloud(void* buf, const float4* P, const GridSpec* spec, int64_t n);
+cudaError_t launch_order(Launch L, const OrderClouds& oc);
+cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const float* box, const double* e_dev,
+                                    double scale2, const GridSpec* spec, int num_sms, double* part, double* a64,
+                                    float* a32, double* sigma_out);
 cudaError_t launch_check_curvature(Launch L, const double* a64, int n, float* a32, int* err);
 cudaError_t launch_records(Launch L, const float4* X4, const double* aX64, int n, int npad,
                            const float4* Y4, const double* aY64, int m, int mpad, int g_mode,
