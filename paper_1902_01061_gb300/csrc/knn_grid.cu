@@ -458,8 +458,9 @@ __device__ __forceinline__ u64 warp_merge(u64 v) {  // v bitonic
 // in one or two steps) and each candidate's rank is the number of smaller
 // ones.  If fewer than k remain the cube grows.  A cube with more candidates
 // than the buffer holds goes to knn_stream.
-// Bound: issue slots.  Measured on GB300 at 1M + 1M points, k = 16: see
-// launch_knn_grid.
+// Bound: issue slots and the look-ups' latency.  1M + 1M points, k = 16: 2.5 ms
+// for both clouds (12.2 ms with a sorted list of 16 per query that every
+// candidate was inserted into); 5,003 + 4,801 points: 43 us (brute force: 350).
 constexpr int QUERY_WARPS = 8;
 constexpr int QUERY_CAP = 256;  // candidates a warp keeps
 constexpr int QUERY_PER = QUERY_CAP / 32;
@@ -667,7 +668,7 @@ __global__ void __launch_bounds__(QUERY_WARPS * 32, 5)
 
 // ---- nearest gridded point of external queries -----------------------------------
 
-// Counts of the coarse cells (NEAREST_COARSE^3 fine cells each).
+// Whether each coarse cell (NEAREST_COARSE^3 fine cells) holds a point: counts.
 __global__ void __launch_bounds__(256) coarse_count_kernel(const CloudSet cs, int* __restrict__ ccount) {
   const GridCloud& g = cs[0];
   const int n3[3] = {g.spec->g[0], g.spec->g[1], g.spec->g[2]};
@@ -688,16 +689,45 @@ __global__ void __launch_bounds__(256) coarse_count_kernel(const CloudSet cs, in
   }
 }
 
+// Counts of the cells of the next level (NEAREST_COARSE^3 coarse cells each),
+// behind the coarse ones.
+__global__ void __launch_bounds__(256) super_count_kernel(const CloudSet cs, int* __restrict__ ccount) {
+  const GridCloud& g = cs[0];
+  int m3[3], s3[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    m3[a] = (g.spec->g[a] + NEAREST_COARSE - 1) / NEAREST_COARSE;
+    s3[a] = (m3[a] + NEAREST_COARSE - 1) / NEAREST_COARSE;
+  }
+  const int coarse = m3[0] * m3[1] * m3[2], total = s3[0] * s3[1] * s3[2];
+  for (int c = blockIdx.x * 256 + threadIdx.x; c < total; c += gridDim.x * 256) {
+    const int x0 = c % s3[0] * NEAREST_COARSE, y0 = c / s3[0] % s3[1] * NEAREST_COARSE,
+              z0 = c / (s3[0] * s3[1]) * NEAREST_COARSE;
+    int cnt = 0;
+    for (int z = z0; z < min(z0 + NEAREST_COARSE, m3[2]); ++z)
+      for (int y = y0; y < min(y0 + NEAREST_COARSE, m3[1]); ++y)
+        for (int x = x0; x < min(x0 + NEAREST_COARSE, m3[0]); ++x) cnt += ccount[(z * m3[1] + y) * m3[0] + x];
+    ccount[coarse + c] = cnt;
+  }
+}
+
 // One warp per query.  First the cube of cells around it, as ranges of
 // sorted points flattened over the lanes: enough for a query on the surface.
-// A query that this does not certify searches shells of coarse cells (edge
-// `coarse` fine cells; a query at distance D would otherwise visit about
+// A query that this does not certify searches shells of large cells (edge
+// 4 * `coarse` fine cells; a query at distance D would otherwise visit about
 // (1.7 D / h)^3 fine cells, nearly all empty): each lane tests one cell, empty
 // ones and ones whose box lies beyond the best key are dropped, and the warp
-// scans the others' points together.  The result is the (key, index)-first
-// point whatever the order of the cells and of the points in a cell.
-// Bound: issue slots and the latency of the range look-ups; a far query costs
-// some thousand warp instructions, one on the surface about two hundred.
+// takes the others nearest first: of a large cell's 4^3 coarse cells it
+// scans, again nearest first and two at a time, the rows of fine cells that the
+// best key does not rule out (a far query is a chain of dependent look-ups: the
+// fewer links, the shorter).  The
+// result is the (key, index)-first point whatever the order of the cells and
+// of the points in a cell.
+// Bound: issue slots and the latency of the range look-ups; a query on the
+// surface costs about two hundred warp instructions.  (Shells of coarse cells,
+// interiors enumerated, 300,000 reference points, 250,007 queries: 823 us;
+// now 566 us: 154 for the 231,563 queries within a cell edge of the surface, the rest for 18,444
+// farther ones, 20 to 200 us of chain each.)
 constexpr int NEAREST_WARPS = 4;
 
 __global__ void __launch_bounds__(NEAREST_WARPS * 32)
@@ -724,12 +754,14 @@ __global__ void __launch_bounds__(NEAREST_WARPS * 32)
     const int incl = warp_incl_scan(len);
     const int cnt = __shfl_sync(FULL, incl, 31);
     u64 mine = NO_CAND;
-    for (int t0 = 0; t0 < cnt; t0 += 32) {
-      const int pos = flat_position(incl, b, len, t0 + lane);
-      if (t0 + lane < cnt) {
-        const float4 p = g.sorted[pos];
-        mine = umin64(mine, pack_cand(grid_key<false>(q4, p), p.w));
-      }
+    for (int t0 = 0; t0 < cnt; t0 += 64) {  // two loads in flight
+      const int at0 = flat_position(incl, b, len, t0 + lane);
+      const int at1 = t0 + 32 < cnt ? flat_position(incl, b, len, t0 + 32 + lane) : at0;
+      float4 p0 = make_float4(NAN, NAN, NAN, 0.f), p1 = p0;
+      if (t0 + lane < cnt) p0 = g.sorted[at0];
+      if (t0 + 32 + lane < cnt) p1 = g.sorted[at1];
+      if (t0 + lane < cnt) mine = umin64(mine, pack_cand(grid_key<false>(q4, p0), p0.w));
+      if (t0 + 32 + lane < cnt) mine = umin64(mine, pack_cand(grid_key<false>(q4, p1), p1.w));
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mine = umin64(mine, __shfl_xor_sync(FULL, mine, off));
@@ -740,47 +772,101 @@ __global__ void __launch_bounds__(NEAREST_WARPS * 32)
   u64 best = scan_ranges(b, len);
   float dout = outside_distance(q, sp.o, sp.h, cc, n3, 1, sp.extent);
   if (dout != INFINITY && !certified(cand_key(best), dout)) {
-    const float H = sp.h * (float)coarse;
-    int m3[3];
+    // squared distance to a cell's box, less the margins, as bits that sort like it
+    constexpr unsigned NO_CELL = ~0u;
+    auto box_bits = [&](int x, int y, int z, float H) {
+      const int xyz[3] = {x, y, z};
+      float d2 = 0.f;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const float below = (float)xyz[a] * H - v[a] - margin[a];
+        const float above = v[a] - (float)(xyz[a] + 1) * H - margin[a];
+        const float d = fmaxf(0.f, fmaxf(below, above));
+        d2 = fmaf(d, d, d2);
+      }
+      return __float_as_uint(d2 * (1.f - 1e-5f));
+    };
+    // the same for a row of `coarse` fine cells
+    auto row_d2 = [&](int x, int y, int z) {
+      const int lo[3] = {x, y, z}, hi[3] = {x + coarse, y + 1, z + 1};
+      float d2 = 0.f;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const float below = (float)lo[a] * sp.h - v[a] - margin[a];
+        const float above = v[a] - (float)hi[a] * sp.h - margin[a];
+        const float d = fmaxf(0.f, fmaxf(below, above));
+        d2 = fmaf(d, d, d2);
+      }
+      return d2 * (1.f - 1e-5f);
+    };
+    // the lane whose cell is nearest; -1 when none is left that the best key
+    // (NaN: no candidate yet) does not rule out
+    auto nearest_lane = [&](unsigned bits) {
+      const unsigned m = __reduce_min_sync(FULL, bits);
+      if (m == NO_CELL || __uint_as_float(m) > cand_key(best)) return -1;
+      return __ffs(__ballot_sync(FULL, bits == m)) - 1;
+    };
+    constexpr int NC = NEAREST_COARSE;
+    const float H = sp.h * (float)coarse, HS = H * (float)NC;
+    int m3[3], s3[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       m3[a] = (n3[a] + coarse - 1) / coarse;
-      cc[a] /= coarse;
+      s3[a] = (m3[a] + NC - 1) / NC;
+      cc[a] /= coarse * NC;
     }
+    const int* scount = ccount ? ccount + m3[0] * m3[1] * m3[2] : nullptr;
     for (int s = 0;; ++s) {
-      const int w = 2 * s + 1, cube = w * w * w;
-      for (int c0 = 0; c0 < cube; c0 += 32) {
-        const int c = c0 + lane;
-        const int dx = c % w - s, dy = c / w % w - s, dz = c / (w * w) - s;
-        const int x = cc[0] + dx, y = cc[1] + dy, z = cc[2] + dz;
-        float d2 = INFINITY;  // squared distance to the cell's box; INFINITY: not a cell to scan
-        if (c < cube && max(abs(dx), max(abs(dy), abs(dz))) == s && x >= 0 && x < m3[0] && y >= 0 && y < m3[1] &&
-            z >= 0 && z < m3[2] && !(ccount && ccount[(z * m3[1] + y) * m3[0] + x] == 0)) {
-          const int xyz[3] = {x, y, z};
-          d2 = 0.f;
+      int lo[3], e[3];  // the cube's part inside the grid
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            const float below = (float)xyz[a] * H - v[a] - margin[a];
-            const float above = v[a] - (float)(xyz[a] + 1) * H - margin[a];
-            const float d = fmaxf(0.f, fmaxf(below, above));
-            d2 = fmaf(d, d, d2);
+      for (int a = 0; a < 3; ++a) {
+        lo[a] = max(cc[a] - s, 0);
+        e[a] = min(cc[a] + s, s3[a] - 1) - lo[a] + 1;
+      }
+      const int cube = e[0] * e[1] * e[2];
+      for (int c0 = 0; c0 < cube; c0 += 32) {
+        const int c = c0 + lane, yz = c / e[0];
+        const int x = lo[0] + c - yz * e[0], y = lo[1] + yz % e[1], z = lo[2] + yz / e[1];
+        unsigned d = NO_CELL;
+        if (c < cube && max(abs(x - cc[0]), max(abs(y - cc[1]), abs(z - cc[2]))) == s &&
+            !(scount && scount[(z * s3[1] + y) * s3[0] + x] == 0))
+          d = box_bits(x, y, z, HS);
+        for (int src; (src = nearest_lane(d)) >= 0;) {
+          if (lane == src) d = NO_CELL;
+          const int X = __shfl_sync(FULL, x, src) * NC, Y = __shfl_sync(FULL, y, src) * NC,
+                    Z = __shfl_sync(FULL, z, src) * NC;
+          static_assert(NC * NC * NC == 64, "two coarse cells a lane");
+          unsigned dc[2];
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const int u = r * 32 + lane, xc = X + u % NC, yc = Y + u / NC % NC, zc = Z + u / (NC * NC);
+            dc[r] = NO_CELL;
+            if (xc < m3[0] && yc < m3[1] && zc < m3[2] && !(ccount && ccount[(zc * m3[1] + yc) * m3[0] + xc] == 0))
+              dc[r] = box_bits(xc, yc, zc, H);
           }
-          d2 *= 1.f - 1e-5f;
-        }
-        unsigned todo = __ballot_sync(FULL, d2 != INFINITY && !(d2 > cand_key(best)));
-        while (todo) {
-          const int src = __ffs(todo) - 1;
-          todo &= todo - 1;
-          if (__shfl_sync(FULL, d2, src) > cand_key(best)) continue;  // the best has improved meanwhile
-          const int X = __shfl_sync(FULL, x, src) * coarse, Y = __shfl_sync(FULL, y, src) * coarse,
-                    Z = __shfl_sync(FULL, z, src) * coarse;
-          b = len = 0;
-          if (lane < coarse * coarse)
-            row_range(g, n3, X, X + coarse - 1, Y + lane % coarse, Z + lane / coarse, b, len);
-          best = umin64(best, scan_ranges(b, len));
+          // two coarse cells at a time, 16 lanes each: a lane per row of fine cells
+          for (;;) {
+            int u2[2] = {-1, -1};
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              const int sc = nearest_lane(min(dc[0], dc[1]));
+              if (sc < 0) break;
+              u2[t] = __shfl_sync(FULL, dc[0] <= dc[1] ? lane : lane + 32, sc);
+              if (lane == sc) (u2[t] < 32 ? dc[0] : dc[1]) = NO_CELL;
+            }
+            if (u2[0] < 0) break;
+            const int u = lane < 16 ? u2[0] : u2[1], row = lane & 15;
+            b = len = 0;
+            if (u >= 0 && row < coarse * coarse) {
+              const int xf = (X + u % NC) * coarse, yf = (Y + u / NC % NC) * coarse + row % coarse,
+                        zf = (Z + u / (NC * NC)) * coarse + row / coarse;
+              if (!(row_d2(xf, yf, zf) > cand_key(best))) row_range(g, n3, xf, xf + coarse - 1, yf, zf, b, len);
+            }
+            best = umin64(best, scan_ranges(b, len));
+          }
         }
       }
-      dout = outside_distance(q, sp.o, H, cc, m3, s, sp.extent);
+      dout = outside_distance(q, sp.o, HS, cc, s3, s, sp.extent);
       if (dout == INFINITY || certified(cand_key(best), dout)) break;
     }
   }
@@ -860,12 +946,14 @@ cudaError_t launch_knn_grid_table(Launch L, const GridCloud* many, const int2* t
 cudaError_t launch_coarse_count(Launch L, const CloudSet& cs, int64_t n, int* ccount) {
   const unsigned b = up((int64_t)grid_start_entries(n) / 16, 256);
   coarse_count_kernel<<<b < 608 ? b : 608, 256, 0, L.stream>>>(cs, ccount);
-  if (L.counter) *L.counter += 1;
+  super_count_kernel<<<b < 152 ? b : 152, 256, 0, L.stream>>>(cs, ccount);
+  if (L.counter) *L.counter += 2;
   return cudaGetLastError();
 }
 
 // Nearest point of the sorted cloud cs[0] for each of nq queries.  levels 2:
-// far queries search coarse cells; 1: fine cells.
+// far queries descend through cells of 16 and of 4 fine cells that hold
+// points; 1: through cells of 4 to fine cells, empty or not.
 cudaError_t launch_nearest_grid(Launch L, const CloudSet& cs, int levels, const int* ccount, const float* q3, int nq,
                                 int32_t* idx_out, float* key_out) {
   if (nq <= 0) return cudaSuccess;

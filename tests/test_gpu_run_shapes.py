@@ -143,3 +143,29 @@ def test_static_forces_split_over_the_reference(n, m):
     got = out.cpu().numpy()
     check("forces_static f: relative L2", rel_l2(got[:, :3], f), 1e-5)
     check("forces_static W: relative L2", rel_l2(got[:, 3], W), 1e-5)
+
+
+@pytest.mark.parametrize("levels", [1, 2])
+@pytest.mark.parametrize("name", ["line", "plane", "cluster"])
+def test_nearest_through_coarse_cells(name, levels):
+    """Grids of many cells on one or two axes, and a dense cluster with far
+    points: queries beside, beyond and across the empty cells."""
+    rng = np.random.default_rng(8)
+    n, nq = 4001, 203
+    X = rng.uniform(-1, 1, size=(n, 3))
+    if name == "line":
+        X = X[:, :1] * np.array([[1.0, 0.0, 0.0]])
+    elif name == "plane":
+        X[:, 2] = 0.5
+    else:
+        X *= 1e-3
+        X[:7] = rng.uniform(-4, 4, size=(7, 3))
+    X = np.ascontiguousarray(X, np.float32)
+    Q = rng.uniform(-2, 2, size=(nq, 3)).astype(np.float32)
+    Q[::4] = X[rng.integers(0, n, len(Q[::4]))]
+    dx, dy, dz = (Q[:, a:a + 1] - X[None, :, a] for a in range(3))
+    want = ((dx * dx + dy * dy) + dz * dz).argmin(axis=1)
+    with Gpu(X, X[:64], tune={scgr.SCGR_TUNE_NEAREST_LEVELS: levels}) as g:
+        idx = torch.empty(nq, dtype=torch.int32, device="cuda")
+        scgr.scgr_nearest(g.ctx, torch.from_numpy(Q).cuda(), idx)
+        np.testing.assert_array_equal(idx.cpu().numpy(), want)
