@@ -212,6 +212,9 @@ __global__ void __launch_bounds__(FINALIZE_THREADS)
 // and the total weight is m0.  One pass over the template forms the sums in
 // float64; then one block runs every iteration.  (Equal to the per-iteration
 // pass up to rounding: that one forms each f_i in float32.)
+// Bound: the float64 chain of an iteration, about 4 us.  35,000 x 30,800, 200
+// iterations, descriptors included: 1.34 ms (5.8 ms with a combine and a
+// finalize launch per iteration).
 constexpr int NFIXED = 22;  // m0, m1[3], M2[6] (xx xy xz yy yz zz), s1[3], N[9]
 constexpr int FIXED_TPB = 256;
 

@@ -9,6 +9,12 @@
 // shared memory), the leader's warp 0 forms the pose and writes the float32 map
 // back to every block.  Two cluster barriers an iteration; the blocks of a
 // cluster are co-scheduled by the hardware, and nothing waits on another launch.
+//
+// Bound: the leader's chain (13 sums across blocks, the pose update's float64)
+// and then the pair rate of 16 SMs.  An iteration: 500 x 500 7.6 us (20.9 as
+// two launches), 1,000 x 1,000 11.0 (22.7), 2,000 x 2,000 26.4 (28.4); with
+// one template point per thread across all of a block's threads, instead of a
+// warp per reference slice, 1,000 x 1,000 took 12.9.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
