@@ -461,7 +461,14 @@ __device__ __forceinline__ u64 warp_merge(u64 v) {  // v bitonic
 // Bound: issue slots and the look-ups' latency.  1M + 1M points, k = 16: 2.5 ms
 // for both clouds (12.2 ms with a sorted list of 16 per query that every
 // candidate was inserted into); 5,003 + 4,801 points: 43 us (brute force: 350).
-constexpr int QUERY_WARPS = 8;
+//
+// Two warps a block: queries differ in length and a block keeps its warps'
+// places until the last is done (8 warps: 32 of 64 warps active on average).
+// 1M + 1M points, the whole descriptor pass: 8 warps and 5 blocks an SM 3406
+// us, 4 and 10 3223, 2 and 20 3225, 2 and 24 (40 registers) 3121.  A batch's
+// table entries are chunks of queries that 8 warps share.
+constexpr int QUERY_WARPS = 2, QUERY_BLOCKS = 24;
+constexpr int QUERY_TABLE_WARPS = 8, QUERY_TABLE_BLOCKS = 5;
 constexpr int QUERY_CAP = 256;  // candidates a warp keeps
 constexpr int QUERY_PER = QUERY_CAP / 32;
 
@@ -646,21 +653,21 @@ __device__ __forceinline__ void knn_query(const GridCloud& g, int t, int k, u64*
 
 // Cloud blockIdx.y, one query per warp; or (a batch, whose clouds differ in
 // size) the KNN_TABLE_CHUNK queries from table[b].y of cloud table[b].x.
-template <bool FUSED>
-__global__ void __launch_bounds__(QUERY_WARPS * 32, 5)
+template <bool FUSED, int WARPS, int BLOCKS>
+__global__ void __launch_bounds__(WARPS * 32, BLOCKS)
     knn_query_kernel(const CloudSet cs, const int2* __restrict__ table, int k) {
-  __shared__ __align__(16) u64 bufs[QUERY_WARPS][QUERY_CAP];
+  __shared__ __align__(16) u64 bufs[WARPS][QUERY_CAP];
   const int warp = threadIdx.x >> 5;
   if (!table) {
     const GridCloud& g = cs[blockIdx.y];
-    const int t = blockIdx.x * QUERY_WARPS + warp;
+    const int t = blockIdx.x * WARPS + warp;
     if (t < g.n) knn_query<FUSED>(g, t, k, bufs[warp]);
     return;
   }
   const int2 e = table[blockIdx.x];
   const GridCloud& g = cs[e.x];
   const int end = min(g.n, e.y + KNN_TABLE_CHUNK);
-  for (int t = e.y + warp; t < end; t += QUERY_WARPS) {
+  for (int t = e.y + warp; t < end; t += WARPS) {
     knn_query<FUSED>(g, t, k, bufs[warp]);
     __syncwarp();
   }
@@ -728,9 +735,11 @@ __global__ void __launch_bounds__(256) super_count_kernel(const CloudSet cs, int
 // interiors enumerated, 300,000 reference points, 250,007 queries: 823 us;
 // now 566 us: 154 for the 231,563 queries within a cell edge of the surface, the rest for 18,444
 // farther ones, 20 to 200 us of chain each.)
-constexpr int NEAREST_WARPS = 4;
+// Two warps a block (4: 584 us a change mask, 8: 597, 2: 552); more blocks an SM
+// by fewer registers cost more than they hide (2 and 20 blocks: 594).
+constexpr int NEAREST_WARPS = 2;
 
-__global__ void __launch_bounds__(NEAREST_WARPS * 32)
+__global__ void __launch_bounds__(NEAREST_WARPS * 32, 16)
     nearest_query_kernel(const CloudSet cs, int coarse, const int* __restrict__ ccount, const float* __restrict__ q3,
                          int nq, int32_t* __restrict__ idx_out, float* __restrict__ key_out) {
   const GridCloud& g = cs[0];
@@ -926,8 +935,8 @@ cudaError_t launch_grid_sort(Launch L, const CloudSet& cs, int nclouds, int most
 // form of clouds below the brute-force limit (grid_key).
 cudaError_t launch_knn_grid(Launch L, const CloudSet& cs, int nclouds, int most, int k, bool fused) {
   const dim3 grid(up(most, QUERY_WARPS), nclouds);
-  if (fused) knn_query_kernel<true><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, nullptr, k);
-  else knn_query_kernel<false><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, nullptr, k);
+  if (fused) knn_query_kernel<true, QUERY_WARPS, QUERY_BLOCKS><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, nullptr, k);
+  else knn_query_kernel<false, QUERY_WARPS, QUERY_BLOCKS><<<grid, QUERY_WARPS * 32, 0, L.stream>>>(cs, nullptr, k);
   if (L.counter) *L.counter += 1;
   return cudaGetLastError();
 }
@@ -938,7 +947,8 @@ cudaError_t launch_knn_grid_table(Launch L, const GridCloud* many, const int2* t
   if (nblocks <= 0) return cudaSuccess;
   CloudSet cs{};
   cs.many = many;
-  knn_query_kernel<true><<<nblocks, QUERY_WARPS * 32, 0, L.stream>>>(cs, table, k);
+  knn_query_kernel<true, QUERY_TABLE_WARPS, QUERY_TABLE_BLOCKS>
+      <<<nblocks, QUERY_TABLE_WARPS * 32, 0, L.stream>>>(cs, table, k);
   if (L.counter) *L.counter += 1;
   return cudaGetLastError();
 }
