@@ -458,7 +458,7 @@ __device__ __forceinline__ u64 warp_merge(u64 v) {  // v bitonic
 // in one or two steps) and each candidate's rank is the number of smaller
 // ones.  If fewer than k remain the cube grows.  A cube with more candidates
 // than the buffer holds goes to knn_stream.
-// Bound: issue slots and the look-ups' latency.  1M + 1M points, k = 16: 2.5 ms
+// Bound: issue slots and the look-ups' latency.  1M + 1M points, k = 16: 2.2 ms
 // for both clouds (12.2 ms with a sorted list of 16 per query that every
 // candidate was inserted into); 5,003 + 4,801 points: 43 us (brute force: 350).
 //
@@ -733,8 +733,8 @@ __global__ void __launch_bounds__(256) super_count_kernel(const CloudSet cs, int
 // Bound: issue slots and the latency of the range look-ups; a query on the
 // surface costs about two hundred warp instructions.  (Shells of coarse cells,
 // interiors enumerated, 300,000 reference points, 250,007 queries: 823 us;
-// now 566 us: 154 for the 231,563 queries within a cell edge of the surface, the rest for 18,444
-// farther ones, 20 to 200 us of chain each.)
+// now 566 us: 154 for the 231,563 queries within a cell edge of the surface, the
+// rest for 18,444 farther ones, 20 to 200 us of chain each.)
 // Two warps a block (4: 584 us a change mask, 8: 597, 2: 552); more blocks an SM
 // by fewer registers cost more than they hide (2 and 20 blocks: 594).
 constexpr int NEAREST_WARPS = 2;
