@@ -169,3 +169,30 @@ def test_nearest_through_coarse_cells(name, levels):
         idx = torch.empty(nq, dtype=torch.int32, device="cuda")
         scgr.scgr_nearest(g.ctx, torch.from_numpy(Q).cuda(), idx)
         np.testing.assert_array_equal(idx.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("want_pose,want_points", [(True, True), (True, False), (False, True)])
+def test_potential_autograd_equals_the_entry_point(want_pose, want_points):
+    """The gradients that forward forms beside U are the entry point's own bits,
+    for each set of inputs that want one, twice over a kept graph; a pose
+    changed between forward and backward is still refused."""
+    X, Y0 = clouds(700, 650)
+    with Gpu(X, Y0, p=2.0) as g:
+        pose = torch.tensor([0.3, -0.2, 0.5, 0.1, 0.2, -0.3, 1.2], dtype=torch.float64, requires_grad=want_pose)
+        Y = g.Y0.clone().requires_grad_(want_points)
+        gx = torch.empty((650, 3), dtype=torch.float32, device="cuda")
+        U, g7 = scgr.scgr_potential(g.ctx, pose.detach().numpy(), grad_xyz_out=gx)
+        u = scgr.potential(pose, Y, g.ctx)
+        assert u.item() == U
+        inputs = [t for t, w in ((pose, want_pose), (Y, want_points)) if w]
+        want = [t for t, w in ((torch.from_numpy(g7), want_pose), (gx, want_points)) if w]
+        for _ in range(2):
+            for got, ref in zip(torch.autograd.grad(2.0 * u, inputs, retain_graph=True), want):
+                assert torch.equal(got, ref * 2.0)
+        if want_pose:
+            with torch.no_grad():
+                pose += 1.0
+            with pytest.raises(RuntimeError):
+                torch.autograd.grad(u, inputs)
+        with torch.no_grad():
+            assert not scgr.potential(pose.detach(), Y, g.ctx).requires_grad
