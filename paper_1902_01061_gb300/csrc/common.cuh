@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 
+#include "grid_spec.cuh"
+
 namespace scgr {
 
 constexpr int ERR_NONFINITE = 1;
@@ -262,15 +264,6 @@ struct BatchPair {
                      // (512-point blocks, running sums in shared memory), 0 for 2 points x 128 threads
 };
 
-// Uniform grid of the exact grid searches (on the device): origin, cell edge,
-// cells per axis and in all, the cloud's largest extent.
-struct GridSpec {
-  float o[3];
-  float h, inv_h, extent;
-  int g[3];
-  int ncell;
-};
-constexpr int GRID_CELLS_PER_POINT = 4;  // at most this many cells per point
 constexpr int SCAN_B = 4096;             // cells per block of the count scan
 constexpr int CLOUD_PARTS = 256;         // blocks of a cloud's reductions, at most
 // scratch of launch_clouds for two clouds: 6 doubles, then 6 floats a part
@@ -318,7 +311,6 @@ cudaError_t launch_records_multi(Launch L, const float4* X4, const double* aX64,
                                  const DevStats* stats, float4* Xr, float2* XA, float4* Y0r);
 cudaError_t launch_sigma_multi(Launch L, const double* aX64, const BatchPair* pairs, int npairs, double sigma_user,
                                DevStats* out);
-size_t grid_start_entries(int64_t n);
 size_t grid_tot_entries(int64_t n);
 cudaError_t launch_clouds(Launch L, const CloudSet& cs, int nclouds, int most, bool scatter, bool sorted, double* part,
                           float* bpart);

@@ -90,42 +90,6 @@ __global__ void __launch_bounds__(RED_THREADS) cloud_sums_kernel(const CloudSet 
   }
 }
 
-// Grid of a cloud from its box: cell edge h = sqrt(8 A / n), A the box's
-// surface area (about 8 points per occupied cell on a surface sample), at most
-// GRID_CELLS_PER_POINT n cells and 2^16 per axis.
-__device__ void make_grid_spec(const float* lo, const float* hi, int n, GridSpec* out) {
-  float e[3], emax = 0.f;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    e[a] = hi[a] - lo[a];
-    emax = fmaxf(emax, e[a]);
-  }
-  // in units of the largest extent, so that no product overflows
-  const float ie = emax > 0.f ? 1.f / emax : 0.f;
-  const float x = e[0] * ie, y = e[1] * ie, z = e[2] * ie;
-  const float A = 2.f * (x * y + y * z + z * x);
-  float h = fmaxf(sqrtf(8.f * A / (float)n), fmaxf(8.f / (float)n, 1.f / 65536.f));
-  const float most = (float)GRID_CELLS_PER_POINT * (float)n;
-  int g[3];
-  for (int it = 0; it < 96; ++it) {
-    g[0] = max(1, (int)ceilf(x / h + 1e-4f));
-    g[1] = max(1, (int)ceilf(y / h + 1e-4f));
-    g[2] = max(1, (int)ceilf(z / h + 1e-4f));
-    if ((float)g[0] * (float)g[1] * (float)g[2] <= most) break;
-    h *= 1.25f;
-  }
-  h = emax > 0.f ? h * emax : 1.f;
-  out->h = h;
-  out->inv_h = 1.f / h;
-  out->extent = emax;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    out->o[a] = lo[a];
-    out->g[a] = g[a];
-  }
-  out->ncell = g[0] * g[1] * g[2];
-}
-
 // One block per cloud: its mean, box and grid.
 __global__ void __launch_bounds__(RED_THREADS) cloud_mean_kernel(const CloudSet cs, const double* __restrict__ part,
                                                                  const float* __restrict__ bpart) {
@@ -889,7 +853,6 @@ __global__ void __launch_bounds__(NEAREST_WARPS * 32, 16)
 
 static inline unsigned up(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
-size_t grid_start_entries(int64_t n) { return (size_t)GRID_CELLS_PER_POINT * n + 64 + 1; }
 size_t grid_tot_entries(int64_t n) { return grid_start_entries(n) / SCAN_B + 2; }
 
 // Means, boxes and grids of the clouds; scatter matrices and largest
