@@ -349,18 +349,45 @@ __device__ __forceinline__ bool certified(float key, float dout) {
   return dout > 0.f && key < dout * dout * (1.f - 1e-5f);  // false for a NaN key (no candidate)
 }
 
-// Sorted positions [b, b + len) of cells x0..x1 (clamped) of row (y, z); len
-// 0 where the row is outside the grid.
-__device__ __forceinline__ void row_range(const GridCloud& g, const int (&n)[3], int x0, int x1, int y, int z, int& b,
+// Sorted positions [b, b + len) of cells x0..x1 (clamped) of the grid's row (y, z).
+__device__ __forceinline__ void row_cells(const GridCloud& g, const int (&n)[3], int x0, int x1, int y, int z, int& b,
                                           int& len) {
   b = len = 0;
   x0 = max(x0, 0);
   x1 = min(x1, n[0] - 1);
-  if (y < 0 || y >= n[1] || z < 0 || z >= n[2] || x0 > x1) return;
+  if (x0 > x1) return;
   const int c = (z * n[1] + y) * n[0];
   b = cell_start(g, c + x0);
   len = cell_start(g, c + x1 + 1) - b;
 }
+// The same for any row; len 0 where it is outside the grid.
+__device__ __forceinline__ void row_range(const GridCloud& g, const int (&n)[3], int x0, int x1, int y, int z, int& b,
+                                          int& len) {
+  b = len = 0;
+  if (y >= 0 && y < n[1] && z >= 0 && z < n[2]) row_cells(g, n, x0, x1, y, z, b, len);
+}
+
+// The rows of cells inside the grid of the cube within s of cell cc.
+struct CubeRows {
+  int y0, z0, ey, count;
+  __device__ __forceinline__ CubeRows(const int (&cc)[3], const int (&n)[3], int s) {
+    y0 = max(cc[1] - s, 0);
+    z0 = max(cc[2] - s, 0);
+    ey = min(cc[1] + s, n[1] - 1) - y0 + 1;
+    count = ey * (min(cc[2] + s, n[2] - 1) - z0 + 1);
+  }
+  __device__ __forceinline__ void row(int r, int& y, int& z) const {
+    z = r / ey;
+    y = y0 + r - z * ey;
+    z += z0;
+  }
+  // r < 2^16: a float quotient, at least 1 / (2 ey) from a whole number
+  __device__ __forceinline__ void row_of_few(int r, int& y, int& z) const {
+    z = (int)__fdividef((float)r + 0.5f, (float)ey);
+    y = y0 + r - z * ey;
+    z += z0;
+  }
+};
 
 __device__ __forceinline__ int warp_incl_scan(int v) {
   const int lane = threadIdx.x & 31;
@@ -438,7 +465,7 @@ constexpr int QUERY_PER = QUERY_CAP / 32;
 
 // The search without a limit on the candidates: those below the k-th key so
 // far wait in the buffer, 32 of them are sorted across the lanes and merged
-// into the warp's sorted list of the best 32.  The cube grows by shells.
+// into the warp's sorted list of the best 32.
 template <bool FUSED>
 __device__ __noinline__ void knn_stream(const GridCloud& g, float4 q, const float (&q3)[3], const int (&cc)[3],
                                         const int (&n3)[3], int k, u64* buf) {
@@ -456,24 +483,25 @@ __device__ __noinline__ void knn_stream(const GridCloud& g, float4 q, const floa
     buf[lane] = rest;
     cnt = cnt > 32 ? cnt - 32 : 0;
   };
-  // s = 1 scans the whole cube (3 x 3 rows of 3 cells), larger s the shell:
-  // whole rows on its faces, else the two end cells of a row
-  for (int s = 1;; ++s) {
-    const int w = 2 * s + 1;
-    const int nr = s == 1 ? 9 : 2 * w * w;
-    for (int r0 = 0; r0 < nr; r0 += 32) {
-      const int r = r0 + lane;
+  // The cube's rows: two entries a row, its parts on either side of the cube
+  // scanned so far (the whole row in the first where that cube does not reach
+  // it).  Only rows inside the grid are listed, so a grid a few cells thick
+  // costs a few entries however far the cube goes, and the cube grows by a
+  // quarter, so a query across a gap of s cells takes some log s steps.
+  for (int s = 1, done = -1;; done = s, s += 1 + s / 4) {
+    const CubeRows rows(cc, n3, s);
+    const unsigned nr = 2u * (unsigned)rows.count;
+    for (unsigned r0 = 0; r0 < nr; r0 += 32) {
+      const unsigned r = r0 + lane;
       int b = 0, len = 0;
       if (r < nr) {
-        const int row = s == 1 ? r : r >> 1, end = s == 1 ? 0 : r & 1;
-        const int dz = row / w - s, dy = row % w - s;
-        const bool whole = s == 1 || dz == -s || dz == s || dy == -s || dy == s;
-        if (whole) {
-          if (!end) row_range(g, n3, cc[0] - s, cc[0] + s, cc[1] + dy, cc[2] + dz, b, len);
-        } else {
-          const int x = end ? cc[0] + s : cc[0] - s;
-          row_range(g, n3, x, x, cc[1] + dy, cc[2] + dz, b, len);
-        }
+        const bool second = r & 1;
+        int y, z;
+        rows.row((int)(r >> 1), y, z);
+        if (abs(y - cc[1]) <= done && abs(z - cc[2]) <= done)
+          row_cells(g, n3, second ? cc[0] + done + 1 : cc[0] - s, second ? cc[0] + s : cc[0] - done - 1, y, z, b, len);
+        else if (!second)
+          row_cells(g, n3, cc[0] - s, cc[0] + s, y, z, b, len);
       }
       const int incl = warp_incl_scan(len);
       const int total = __shfl_sync(FULL, incl, 31);
@@ -512,13 +540,17 @@ __device__ __forceinline__ void knn_query(const GridCloud& g, int t, int k, u64*
   for (int s = 1; s <= 32; s += s < 4 ? 1 : s >> 1) {
     const float dout = outside_distance(q3, sp.o, sp.h, cc, n3, s, sp.extent);
     float lim = dout > 0.f ? dout * dout * (1.f - 1e-5f) : 0.f;  // INFINITY where the cube covers the grid
-    const int w = 2 * s + 1, rows = w * w;
+    const CubeRows rows(cc, n3, s);
     int cnt = 0;
     __syncwarp();
-    for (int r0 = 0; r0 < rows && cnt <= QUERY_CAP; r0 += 32) {
+    for (int r0 = 0; r0 < rows.count && cnt <= QUERY_CAP; r0 += 32) {
       const int r = r0 + lane;
       int b = 0, len = 0;
-      if (r < rows) row_range(g, n3, cc[0] - s, cc[0] + s, cc[1] + r % w - s, cc[2] + r / w - s, b, len);
+      if (r < rows.count) {
+        int y, z;
+        rows.row_of_few(r, y, z);  // at most 57 x 57
+        row_cells(g, n3, cc[0] - s, cc[0] + s, y, z, b, len);
+      }
       const int incl = warp_incl_scan(len);
       const int total = __shfl_sync(FULL, incl, 31);
       for (int t0 = 0; t0 < total && cnt <= QUERY_CAP; t0 += 32) {

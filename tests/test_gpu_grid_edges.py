@@ -1,6 +1,7 @@
 """Grid searches at the edges of their geometry, against the oracle's brute
 force (indices and keys equal): boxes of subnormal and of very small extent,
-whose reciprocals would overflow."""
+whose reciprocals would overflow; thin grids with fewer than k points beyond a
+gap of up to tens of thousands of cells."""
 import numpy as np
 import pytest
 import torch
@@ -43,3 +44,44 @@ def test_boxes_of_tiny_extent(extent):
         want_idx, want_key = brute_nearest(P, q)
         np.testing.assert_array_equal(idx, want_idx)
         np.testing.assert_array_equal(key, want_key)
+
+
+def gapped(name, n):
+    """n points of which 5 lie beyond a gap that is most of the cloud's length."""
+    rng = np.random.default_rng(n)
+    P = rng.uniform(0.0, 0.1, size=(n, 3))
+    P[-5:] = [[1.0, 0, 0], [0.99, 0, 0], [1.0, 0.1, 0.1], [0.985, 0.05, 0.1], [1.0, 0.1, 0]]
+    if name == "line":
+        P[:, 1:] = 0.25
+    elif name == "pole":
+        P[:, 1:] *= 0.01
+    elif name == "plane":
+        P[:, 2] = -1.5
+    return np.ascontiguousarray(P, np.float32)
+
+
+@pytest.mark.parametrize("grid_min", [None, 0])
+@pytest.mark.parametrize("name,n,k", [("line", 4000, 16), ("line", 150000, 16), ("pole", 5000, 8), ("pole", 30000, 32),
+                                      ("plane", 60000, 16), ("box", 40000, 6)])
+def test_few_points_beyond_a_gap(name, n, k, grid_min):
+    """All points where the grid's key is asked for and the oracle is quick, else the isolated ones and a sample."""
+    P = gapped(name, n)
+    rows = np.arange(n) if n <= 5000 else np.concatenate([np.arange(n - 5, n), np.arange(0, n - 5, n // 300)])
+    with Gpu(P, P[: max(k, 64)], k=k, tune={} if grid_min is None else {scgr.SCGR_TUNE_KNN_GRID_MIN: grid_min}) as g:
+        got = g.knn(0)[rows]
+    want = np.concatenate([first_k(P, P[r], k) for r in np.array_split(rows, 1 + len(rows) * n // 20_000_000)])
+    if grid_min == 0 or n >= 20000:
+        np.testing.assert_array_equal(got, want)
+    else:  # near ties may fall either way with the smaller clouds' key (one rounding less)
+        np.testing.assert_allclose(dist64(P, rows, got), dist64(P, rows, want), rtol=1e-6)
+
+
+def first_k(P, q, k):
+    d = q[:, None, :] - P[None, :, :]
+    key = (d[..., 0] * d[..., 0] + d[..., 1] * d[..., 1]) + d[..., 2] * d[..., 2]
+    return np.argsort(key, axis=1, kind="stable")[:, :k]
+
+
+def dist64(P, rows, idx):
+    P = P.astype(np.float64)
+    return np.linalg.norm(P[idx] - P[rows][:, None, :], axis=2)
