@@ -875,9 +875,12 @@ __global__ void __launch_bounds__(NEAREST_WARPS * 32, 16)
       if (dout == INFINITY || certified(cand_key(best), dout)) break;
     }
   }
+  // an infinite or NaN key (a query whose squared distances leave float32's
+  // range) is no candidate, as in the brute-force search
   if (lane == 0) {
-    if (idx_out) idx_out[t] = (int32_t)(unsigned)best;
-    if (key_out) key_out[t] = cand_key(best);
+    const bool found = cand_key(best) < INFINITY;
+    if (idx_out) idx_out[t] = found ? (int32_t)(unsigned)best : INT_MAX;
+    if (key_out) key_out[t] = found ? cand_key(best) : INFINITY;
   }
 }
 

@@ -1,7 +1,7 @@
 """Grid searches at the edges of their geometry, against the oracle's brute
 force (indices and keys equal): boxes of subnormal and of very small extent,
 whose reciprocals would overflow; thin grids with fewer than k points beyond a
-gap of up to tens of thousands of cells."""
+gap of up to tens of thousands of cells; and queries beyond float32's range."""
 import numpy as np
 import pytest
 import torch
@@ -85,3 +85,20 @@ def first_k(P, q, k):
 def dist64(P, rows, idx):
     P = P.astype(np.float64)
     return np.linalg.norm(P[idx] - P[rows][:, None, :], axis=2)
+
+
+@pytest.mark.parametrize("n", [600, 1500, 70000])
+def test_queries_beyond_float32_range(n):
+    """Where no key is finite the brute-force search (600 points) finds no
+    point: index 2^31 - 1, key infinity.  The grid answers the same, whatever
+    the finite queries beside them."""
+    P = np.ascontiguousarray(synth.mild(n=n).X, np.float32)
+    bad = np.float32([[1e30, 0, 0], [0, -3e38, 0], [np.inf, 0, 0], [0, 0, -np.inf], [np.nan, 0, 0], [np.nan] * 3])
+    q = np.concatenate([bad, P[:40] + np.float32(0.01), P[:3] * np.float32(1e15), bad])
+    with Gpu(P, P[:100], k=8) as g:
+        idx, key = nearest(g, q)
+    want_idx, want_key = brute_nearest(P, q[6:-6])
+    np.testing.assert_array_equal(idx[6:-6], want_idx)
+    np.testing.assert_array_equal(key[6:-6], want_key)
+    for part in (slice(0, 6), slice(len(q) - 6, len(q))):
+        assert np.all(idx[part] == 2**31 - 1) and np.all(np.isposinf(key[part]))
