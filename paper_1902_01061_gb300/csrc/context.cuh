@@ -92,6 +92,7 @@ struct scgr_ctx {
   DevBuf gspec, gcell[2], gstart[2], gtot[2], gsorted[2], gccount;
   bool grid_ok[2] = {false, false};  // sorted into grid cells
   bool coarse_ok = false;            // the reference's coarse cell counts (gccount)
+  bool replayed_X = false;           // the reference or its grid has been set inside a caller's capture
   int nearest_levels = 2;       // 2: two-level nearest search (default), 1: fine shells only (tunable)
   bool small_ok = false;        // the device runs small_run's cluster
   int fused_tail = 1;           // 1: one combine-finalize launch for small templates (tunable)

@@ -92,6 +92,14 @@ scgr_status read_error_word(scgr_ctx* c) {
   return fail(c, SCGR_ERR_NUMERIC, "the iteration step became non-finite (zero or non-finite total weight)");
 }
 
+// Whether a caller is capturing the stream (a stream that cannot be asked is not being captured).
+static bool stream_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
+}
+
 scgr_status set_cloud(scgr_ctx* c, const float* xyz, int64_t n, bool host, bool ref) {
   if (!c) return SCGR_ERR_INVALID_ARG;
   c->err.clear();
@@ -108,7 +116,13 @@ scgr_status set_cloud(scgr_ctx* c, const float* xyz, int64_t n, bool host, bool 
     src = (const float*)c->stage.p;
   }
   SCGR_CK(c, launch_pack(c->L(), src, n, (float4*)dst.p, c->errword));
-  if (ref) { c->n = n; c->have_X = true; c->grid_ok[0] = c->coarse_ok = false; }
+  if (ref) {
+    c->n = n;
+    c->have_X = true;
+    c->grid_ok[0] = c->coarse_ok = false;
+    // a replay of the capture will change the reference without a call
+    if (stream_capturing(c->stream)) c->replayed_X = true;
+  }
   else { c->m = n; c->have_Y = true; c->grid_ok[1] = false; }
   c->have_desc = false;
   return SCGR_OK;
@@ -195,6 +209,7 @@ static bool grid_knn(const scgr_ctx* c, int which) {
 // launch; nothing waits for the host.
 scgr_status prepare_clouds(scgr_ctx* c) {
   c->grid_ok[0] = c->grid_ok[1] = false;
+  if (stream_capturing(c->stream)) c->replayed_X = true;  // the grid is there once it is replayed
   SCGR_CK(c, ensure(c->gspec, 2 * sizeof(GridSpec)));
   CloudSet cs{};
   for (int w = 0; w < 2; ++w) {
@@ -252,17 +267,24 @@ static scgr_status knn_clouds(scgr_ctx* c) {
 // two-level grid search over the reference (the same result): fine cells
 // around the query, then coarse cells that skip empty space.  The reference's
 // grid is the descriptor pass's, or built here on the first query, and kept
-// until the reference changes.  While the stream is being captured a grid
-// that is not there yet is not built (no allocation): brute force.
+// until the reference changes.
+//
+// A search that a caller captures may be replayed after the reference has
+// changed, and brute force reads the points as they then are; from
+// CAPTURED_GRID_MIN points on a captured search keeps the grid it finds
+// (without one it is brute force: nothing can be allocated).  Where the
+// reference itself was set inside a capture, a replay changes it without a
+// call, and where the descriptor pass was captured its grid is there only after
+// a replay: from then on the grid is built again for every search.
+constexpr int64_t CAPTURED_GRID_MIN = 65536;
 scgr_status nearest_reference(scgr_ctx* c, const float* q3, int nq, int32_t* idx_out, float* key_out) {
   const float4* X4 = (const float4*)c->X4.p;
   const int n = (int)c->n;
   bool grid = (int64_t)n >= c->nearest_grid_min;
-  if (grid && !(c->grid_ok[0] && c->coarse_ok)) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    SCGR_CK(c, cudaStreamIsCapturing(c->stream, &cap));
-    grid = cap == cudaStreamCaptureStatusNone;
-  }
+  if (grid && stream_capturing(c->stream))
+    grid = (int64_t)n >= CAPTURED_GRID_MIN && c->grid_ok[0] && c->coarse_ok && !c->replayed_X;
+  else if (c->replayed_X)
+    c->grid_ok[0] = c->coarse_ok = false;
   if (!grid) {
     SCGR_CK(c, launch_nearest(c->L(), X4, n, q3, nq, idx_out, key_out));
     return SCGR_OK;
