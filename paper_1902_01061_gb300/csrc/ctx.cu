@@ -203,6 +203,20 @@ static bool grid_knn(const scgr_ctx* c, int which) {
   return c->prm.neigh_mode == 0 && (which == 0 ? c->n : c->m) >= (c->knn_grid_min < 0 ? 0 : c->knn_grid_min);
 }
 
+// One cloud's grid alone, without statistics.
+static scgr_status build_grid(scgr_ctx* c, int which) {
+  SCGR_CK(c, ensure(c->gspec, 2 * sizeof(GridSpec)));
+  const scgr_status st = grid_buffers(c, which);
+  if (st != SCGR_OK) return st;
+  CloudSet cs{};
+  cs.one[0] = grid_cloud(c, which, true, false);
+  SCGR_CK(c, launch_clouds(c->L(), cs, 1, cs.one[0].n, false, false, c->red, (float*)(c->red + 2 * CLOUD_PARTS * 6)));
+  SCGR_CK(c, launch_grid_sort(c->L(), cs, 1, cs.one[0].n, c->red));
+  c->grid_ok[which] = true;
+  if (which == 0) c->coarse_ok = false;
+  return SCGR_OK;
+}
+
 // The descriptor pass's first part: means, scatter matrices and largest
 // eigenvalues of both clouds, their boxes, and the points sorted into grid
 // cells where the neighbour search wants that.  Both clouds share each
@@ -236,24 +250,31 @@ scgr_status prepare_clouds(scgr_ctx* c) {
   return SCGR_OK;
 }
 
-// k nearest neighbours of both clouds (after prepare_clouds): the grid search
-// where the cloud was sorted, else brute force.  Clouds of fewer than
-// KNN_FUSED_KEY points keep the key rounding of the brute-force search, which
-// served them before (grid_key).
+// k nearest neighbours of both clouds: the grid search or brute force by the
+// size and the knob alone, whatever grids earlier calls have left.  Clouds of
+// fewer than KNN_FUSED_KEY points keep the key rounding of the brute-force
+// search, which served them before (grid_key).
 static scgr_status knn_clouds(scgr_ctx* c) {
   const int k = c->prm.k;
-  bool fused[2];
-  for (int w = 0; w < 2; ++w) fused[w] = c->knn_grid_min < 0 && (w == 0 ? c->n : c->m) < KNN_FUSED_KEY;
+  bool grid[2], fused[2];
   CloudSet cs{};
-  for (int w = 0; w < 2; ++w) cs.one[w] = grid_cloud(c, w, c->grid_ok[w], false);
-  if (c->grid_ok[0] && c->grid_ok[1] && fused[0] == fused[1]) {
+  for (int w = 0; w < 2; ++w) {
+    grid[w] = grid_knn(c, w);
+    fused[w] = c->knn_grid_min < 0 && (w == 0 ? c->n : c->m) < KNN_FUSED_KEY;
+    if (grid[w] && !c->grid_ok[w]) {  // the knob has changed since the descriptor pass
+      const scgr_status st = build_grid(c, w);
+      if (st != SCGR_OK) return st;
+    }
+    cs.one[w] = grid_cloud(c, w, grid[w], false);
+  }
+  if (grid[0] && grid[1] && fused[0] == fused[1]) {
     SCGR_CK(c, launch_knn_grid(c->L(), cs, 2, (int)(c->n > c->m ? c->n : c->m), k, fused[0]));
     return SCGR_OK;
   }
   for (int w = 0; w < 2; ++w) {
     CloudSet one{};
     one.one[0] = cs.one[w];
-    if (c->grid_ok[w]) {
+    if (grid[w]) {
       SCGR_CK(c, launch_knn_grid(c->L(), one, 1, one.one[0].n, k, fused[w]));
     } else {
       SCGR_CK(c, launch_knn(c->L(), one.one[0].P, one.one[0].n, k, one.one[0].knn));
@@ -289,17 +310,11 @@ scgr_status nearest_reference(scgr_ctx* c, const float* q3, int nq, int32_t* idx
     SCGR_CK(c, launch_nearest(c->L(), X4, n, q3, nq, idx_out, key_out));
     return SCGR_OK;
   }
-  CloudSet cs{};
   if (!c->grid_ok[0]) {
-    SCGR_CK(c, ensure(c->gspec, 2 * sizeof(GridSpec)));
-    const scgr_status st = grid_buffers(c, 0);
+    const scgr_status st = build_grid(c, 0);
     if (st != SCGR_OK) return st;
-    cs.one[0] = grid_cloud(c, 0, true, false);
-    SCGR_CK(c, launch_clouds(c->L(), cs, 1, n, false, false, c->red, (float*)(c->red + 2 * CLOUD_PARTS * 6)));
-    SCGR_CK(c, launch_grid_sort(c->L(), cs, 1, n, c->red));
-    c->grid_ok[0] = true;
-    c->coarse_ok = false;
   }
+  CloudSet cs{};
   cs.one[0] = grid_cloud(c, 0, true, false);
   if (!c->coarse_ok) {
     SCGR_CK(c, ensure(c->gccount, grid_start_entries(n) * sizeof(int)));

@@ -102,3 +102,27 @@ def test_queries_beyond_float32_range(n):
     np.testing.assert_array_equal(key[6:-6], want_key)
     for part in (slice(0, 6), slice(len(q) - 6, len(q))):
         assert np.all(idx[part] == 2**31 - 1) and np.all(np.isposinf(key[part]))
+
+
+def lattice(n):
+    """Points whose neighbour keys tie or nearly tie."""
+    g = np.stack(np.meshgrid(*[np.arange(n) * np.float32(0.1)] * 3, indexing="ij"), -1)
+    return np.ascontiguousarray(g.reshape(-1, 3), np.float32)
+
+
+@pytest.mark.parametrize("first,then", [(10**9, 10**9), (10**9, 0), (0, 10**9)])
+def test_neighbours_do_not_depend_on_earlier_calls(first, then):
+    """After a nearest-point search has built the reference's grid, or with the
+    knob changed since the descriptors, the neighbours are those of a context
+    that had the knob from the start (the two searches round the key differently)."""
+    P = lattice(12)
+    with Gpu(P, P, k=16, tune={scgr.SCGR_TUNE_KNN_GRID_MIN: then}) as g:
+        want = [g.knn(0), g.knn(1)]
+    if then == 0:
+        np.testing.assert_array_equal(want[0], O.knn(P, 16))
+    with Gpu(P, P, k=16, tune={scgr.SCGR_TUNE_KNN_GRID_MIN: first}) as g:
+        nearest(g, P[:64])
+        scgr.scgr_set_tuning(g.ctx, scgr.SCGR_TUNE_KNN_GRID_MIN, then)
+        scgr.scgr_set_neighbourhood(g.ctx, k=16)
+        np.testing.assert_array_equal(g.knn(0), want[0])
+        np.testing.assert_array_equal(g.knn(1), want[1])
