@@ -5,6 +5,7 @@
 #include <climits>
 
 #include "common.cuh"
+#include "pointsum.cuh"
 
 namespace scgr {
 
@@ -466,23 +467,36 @@ cudaError_t launch_curvature2(Launch L, const float4* X, const int32_t* nx, int 
 // covariance (radius sqrt(e), Sec. IV).  Its 1/|N| covariance gives
 // a = lambda_min / trace.
 //
-// One pass over the cloud sums the count, the offsets d = q - p and their
-// products, so accurately that the covariance S2/k - m m^T keeps a small
-// eigenvalue: a sum is a pair (acc, lo).  acc starts at c = 1.5 * 2^k, 2^k
+// One pass over the cloud sums the count, the members' offsets and the products
+// of the offsets, so accurately that the covariance S2/k - m m^T keeps a small
+// eigenvalue.  A float32 difference of two coordinates may round, so each
+// coordinate is split exactly, x = xh + xl with xh a multiple of u = 2^-21 r (r
+// up to a power of two, the bound on |d|): differences h of the xh are exact, and the
+// covariance of the offsets h + xl is that of the points (they differ from q - p by
+// the constant xl of p).  A sum is a pair (acc, lo): acc starts at c = 1.5 * 2^k, 2^k
 // above twice what a run of 32 points can add, so t = fma(x, y, acc) stays in
-// acc's binade, z = t - acc is exact, and so is acc's sum of the z; lo
-// collects fma(x, y, -z), the exact rest rounded once.  That is 4 float32
-// operations per sum and pair, with an error of 2^-42 of the bound on |d|^2
-// per pair; a float pair (two-sum) carries the totals from run to run.
+// acc's binade, acc - t is exact, and so is acc's sum of such steps; lo collects
+// fma(x, y, acc - t), the exact rest rounded once, and the products with xl.  lo is a
+// plain float32 sum over a tile's lane (128 points): its rounding is the error, some
+// 2^-42 of the bound B on |d|^2 per point; a float pair (two-sum) carries the totals.
+//
+// That error is relative to B, not to the neighbourhood, so where the smallest
+// eigenvalue is below 2^-17 B (few, tight or very flat neighbours) the point's
+// covariance is summed again in float64 by its warp (none of 20,011 sampled
+// surface points at scale 1, at most 1 in 500 at scale 0.5 and 500 points; an
+// exact plane: all).  Above it the relative error of the eigenvalue is at most about 2^-25
+// (emulated: 20 to 1,500 members, 3e-8 at 2^-17 B, 5e-10 at 1e-3 B; with offsets rounded to
+// float32 4e-6 and 7e-7).
 //
 // Bound: the FP32 pipe.  A pair costs 8 lane operations for the key, 4 for
-// the scaled offsets and the count and 36 for the nine sums: 2.6 pairs per
-// clock per SM, 8.3e11 pairs/s; a group of four points that no query of the
+// the offsets and the count, 36 for the nine sums and 15 for the xl terms:
+// 2.0 pairs per clock per SM; a group of four points that no query of the
 // warp reaches costs only the keys.  Large clouds come in Morton order
 // (order.cu): a warp's queries and a run of 32 points are then compact, and a
 // run whose box lies beyond the radius of the warp's box costs nothing.
 // (20,011 + 17,611 points, scale 1, the whole descriptor pass: 30.2 ms with
-// two passes of 12 float64 operations per member; 1.49 ms unordered; 0.62 ms.)
+// two passes of 12 float64 operations per member; 1.49 ms unordered; 0.62 ms
+// with offsets rounded to float32.)
 //
 // Members' offsets are scaled by a power of two that brings the bound on
 // |d|^2 (the smaller of the squared radius and three squared box extents)
@@ -491,11 +505,14 @@ constexpr int RAD_TPB = 128;
 constexpr int RAD_TILE = 256;
 constexpr int RAD_RUN = 32;
 constexpr int RAD_NS = 10;  // count, d (3), d d^T (6: xx xy xz yy yz zz)
+constexpr float RAD_FLAT = 0x1p-17f;  // smallest eigenvalue / B below which the sums are repeated in float64
 
 struct RadiusScale {
   float s;         // power of two applied to the offsets
   float r2;        // squared radius (not scaled)
+  float B;         // bound on |d|^2, scaled
   float c1, c2;    // acc's starting value for the offsets and for their products
+  float cu, small; // 1.5 * 2^23 u; coordinates below `small` are split, larger ones are multiples of u / 2
 };
 __device__ __forceinline__ RadiusScale radius_scale_of(const double* e_dev, double scale2, const GridSpec* spec) {
   const float r2 = (float)(scale2 * e_dev[0]);
@@ -506,6 +523,10 @@ __device__ __forceinline__ RadiusScale radius_scale_of(const double* e_dev, doub
   o.s = ldexpf(1.f, h);
   o.r2 = r2;
   const float Bs = (B * o.s) * o.s;
+  o.B = Bs;
+  const int e = (ilogbf(B) >> 1) + 1;  // r < 2^e
+  o.cu = ldexpf(1.5f, e + 2);
+  o.small = ldexpf(1.f, e + 1);
   // Bs < 2^(ilogb + 1), sqrt(Bs) < 2^((ilogb >> 1) + 1): 2^(k - 1) >= the
   // RAD_RUN / 2 = 16 terms of a lane
   o.c2 = 1.5f * ldexpf(1.f, ilogbf(Bs) + 6);
@@ -513,11 +534,16 @@ __device__ __forceinline__ RadiusScale radius_scale_of(const double* e_dev, doub
   return o;
 }
 
+// The multiple of u next to x (x itself where it is a multiple of u / 2): x - high is
+// exact, and the difference of two within r of each other fits 23 bits.
+__device__ __forceinline__ float radius_high(float x, const RadiusScale& sc) {
+  return fabsf(x) < sc.small ? __fsub_rn(__fadd_rn(x, sc.cu), sc.cu) : x;
+}
+
 // (acc, lo) += x y in both lanes
 __device__ __forceinline__ void split_fma2(u64& acc, u64& lo, u64 x, u64 y) {
   const u64 t = fma2(x, y, acc);
-  const u64 z = sub2(t, acc);
-  lo = add2(lo, fma2(x, y, sub2(0ull, z)));
+  lo = add2(lo, fma2(x, y, sub2(acc, t)));
   acc = t;
 }
 __device__ __forceinline__ void split_add2(u64& acc, u64& lo, u64 x) {
@@ -531,17 +557,28 @@ __device__ __forceinline__ float member_mask(float key, float r2) {
   return m;
 }
 
+// Covariance of points from their count, sum and sum of products.
+__device__ __forceinline__ void covariance_of_sums(const double (&v)[RAD_NS], double* C) {
+  const double ik = 1.0 / v[0];
+  const double mx = v[1] * ik, my = v[2] * ik, mz = v[3] * ik;
+  C[0] = fma(v[4], ik, -mx * mx); C[1] = fma(v[5], ik, -mx * my); C[2] = fma(v[6], ik, -mx * mz);
+  C[4] = fma(v[7], ik, -my * my); C[5] = fma(v[8], ik, -my * mz); C[8] = fma(v[9], ik, -mz * mz);
+  C[3] = C[1]; C[6] = C[2]; C[7] = C[5];
+}
+
 // Query i's sums over the points of tiles [t0, t1) of split blockIdx.y, written
 // as doubles to part[split][sum][n] (in scaled coordinates).
-__global__ void __launch_bounds__(RAD_TPB)
+__global__ void __launch_bounds__(RAD_TPB, 5)
     radius_sums_kernel(const float4* __restrict__ P, int n, const float* __restrict__ box,
                        const double* __restrict__ e_dev, double scale2, const GridSpec* __restrict__ spec,
                        int tiles_per_split, double* __restrict__ part) {
-  __shared__ __align__(16) float tile[3][RAD_TILE];
+  __shared__ __align__(16) float tile[9][RAD_TILE];  // x, y, z; their high parts, scaled; their low parts, scaled
   const int i = blockIdx.x * RAD_TPB + threadIdx.x;
   const RadiusScale sc = radius_scale_of(e_dev, scale2, spec);
   const float4 q4 = P[i < n ? i : n - 1];
-  const u64 q2x = pk2(q4.x, q4.x), q2y = pk2(q4.y, q4.y), q2z = pk2(q4.z, q4.z), s2 = pk2(sc.s, sc.s);
+  const u64 q2x = pk2(q4.x, q4.x), q2y = pk2(q4.y, q4.y), q2z = pk2(q4.z, q4.z);
+  const float hx = radius_high(q4.x, sc) * sc.s, hy = radius_high(q4.y, sc) * sc.s, hz = radius_high(q4.z, sc) * sc.s;
+  const u64 h2x = pk2(hx, hx), h2y = pk2(hy, hy), h2z = pk2(hz, hz);
   float H[RAD_NS], Lo[RAD_NS];
 #pragma unroll
   for (int f = 0; f < RAD_NS; ++f) H[f] = Lo[f] = 0.f;
@@ -577,9 +614,14 @@ __global__ void __launch_bounds__(RAD_TPB)
     for (int t = threadIdx.x; t < RAD_TILE; t += RAD_TPB) {
       // past the end: a point at NaN, whose key is never <= r2
       const float4 c = base + t < t1 ? P[base + t] : make_float4(NAN, NAN, NAN, 0.f);
-      tile[0][t] = c.x;
-      tile[1][t] = c.y;
-      tile[2][t] = c.z;
+      const float cv[3] = {c.x, c.y, c.z};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const float high = base + t < t1 ? radius_high(cv[a], sc) : 0.f;
+        tile[a][t] = cv[a];
+        tile[3 + a][t] = high * sc.s;
+        tile[6 + a][t] = base + t < t1 ? __fsub_rn(cv[a], high) * sc.s : 0.f;
+      }
     }
     __syncthreads();
     u64 acc[RAD_NS], lo[RAD_NS];
@@ -615,25 +657,36 @@ __global__ void __launch_bounds__(RAD_TPB)
         if (!__any_sync(0xffffffffu, any)) continue;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          float m0, m1, x0, x1, y0, y1, z0, z1;
-          upk2(m[h], m0, m1);
-          upk2(d[h][0], x0, x1);
-          upk2(d[h][1], y0, y1);
-          upk2(d[h][2], z0, z1);
-          // a select before the product: a point past the end has NaN offsets
-          const u64 x = mul2(pk2(m0 != 0.f ? x0 : 0.f, m1 != 0.f ? x1 : 0.f), s2);
-          const u64 y = mul2(pk2(m0 != 0.f ? y0 : 0.f, m1 != 0.f ? y1 : 0.f), s2);
-          const u64 z = mul2(pk2(m0 != 0.f ? z0 : 0.f, m1 != 0.f ? z1 : 0.f), s2);
+          // of others than members the high parts' offsets are 0 and the low parts count 0 times
+          auto offset = [&](int a, u64 q2) {
+            float m0, m1, v0, v1;
+            upk2(m[h], m0, m1);
+            upk2(sub2(*reinterpret_cast<const u64*>(&tile[3 + a][j + 2 * h]), q2), v0, v1);
+            return pk2(m0 != 0.f ? v0 : 0.f, m1 != 0.f ? v1 : 0.f);
+          };
+          const u64 x = offset(0, h2x), y = offset(1, h2y), z = offset(2, h2z);
+          const u64 xl = *reinterpret_cast<const u64*>(&tile[6][j + 2 * h]);
+          const u64 yl = *reinterpret_cast<const u64*>(&tile[7][j + 2 * h]);
+          const u64 zl = *reinterpret_cast<const u64*>(&tile[8][j + 2 * h]);
           acc[0] = add2(acc[0], m[h]);
           split_add2(acc[1], lo[1], x);
           split_add2(acc[2], lo[2], y);
           split_add2(acc[3], lo[3], z);
+          lo[1] = fma2(m[h], xl, lo[1]);
+          lo[2] = fma2(m[h], yl, lo[2]);
+          lo[3] = fma2(m[h], zl, lo[3]);
           split_fma2(acc[4], lo[4], x, x);
           split_fma2(acc[5], lo[5], x, y);
           split_fma2(acc[6], lo[6], x, z);
           split_fma2(acc[7], lo[7], y, y);
           split_fma2(acc[8], lo[8], y, z);
           split_fma2(acc[9], lo[9], z, z);
+          lo[4] = fma2(x, add2(xl, xl), lo[4]);
+          lo[5] = fma2(x, yl, fma2(y, xl, lo[5]));
+          lo[6] = fma2(x, zl, fma2(z, xl, lo[6]));
+          lo[7] = fma2(y, add2(yl, yl), lo[7]);
+          lo[8] = fma2(y, zl, fma2(z, yl, lo[8]));
+          lo[9] = fma2(z, add2(zl, zl), lo[9]);
         }
       }
 #pragma unroll
@@ -658,13 +711,62 @@ __global__ void __launch_bounds__(RAD_TPB)
   for (int f = 0; f < RAD_NS; ++f) part[((size_t)blockIdx.y * RAD_NS + f) * n + i] = (double)H[f] + (double)Lo[f];
 }
 
+// Point i's count, sums of offsets and of their products in float64, by one warp
+// (all lanes call it; lane 2 f gets sum f).
+__device__ __noinline__ double radius_sums_float64(const float4* __restrict__ P, int n, const float* __restrict__ box,
+                                                   float r2, int i) {
+  const int lane = threadIdx.x & 31;
+  const float4 q = P[i];
+  double v[16];
+#pragma unroll
+  for (int f = 0; f < 16; ++f) v[f] = 0.0;
+  auto add = [&](const float4 c) {
+    if (!(knn_key(c, q) <= r2)) return;
+    const double x = (double)c.x - q.x, y = (double)c.y - q.y, z = (double)c.z - q.z;
+    v[0] += 1.0; v[1] += x; v[2] += y; v[3] += z;
+    v[4] = fma(x, x, v[4]); v[5] = fma(x, y, v[5]); v[6] = fma(x, z, v[6]);
+    v[7] = fma(y, y, v[7]); v[8] = fma(y, z, v[8]); v[9] = fma(z, z, v[9]);
+  };
+  if (!box) {
+    for (int j0 = lane; j0 < n; j0 += 32 * 8) {  // eight loads in flight
+      float4 c[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) c[u] = j0 + 32 * u < n ? P[j0 + 32 * u] : make_float4(NAN, NAN, NAN, 0.f);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) add(c[u]);
+    }
+  }
+  const int runs = box ? (n + RAD_RUN - 1) / RAD_RUN : 0;
+  for (int b0 = 0; b0 < runs; b0 += 32) {
+    // the runs of 32 points that the point may reach, a lane each
+    bool reach = b0 + lane < runs;
+    if (reach) {
+      const float* b = box + 6 * (size_t)(b0 + lane);
+      const float gx = fmaxf(0.f, fmaxf(b[0] - q.x, q.x + b[3])), gy = fmaxf(0.f, fmaxf(b[1] - q.y, q.y + b[4])),
+                  gz = fmaxf(0.f, fmaxf(b[2] - q.z, q.z + b[5]));
+      reach = !(fmaf(gz, gz, fmaf(gy, gy, gx * gx)) * (1.f - 1e-5f) > r2);
+    }
+    for (unsigned todo = __ballot_sync(0xffffffffu, reach); todo; todo &= todo - 1) {
+      const int j = (b0 + __ffs(todo) - 1) * RAD_RUN + lane;
+      if (j < n) add(P[j]);
+    }
+  }
+  __syncwarp();
+  warp_reduce16(v);
+  return v[0];
+}
+
 // The splits' sums of a point added in order, its covariance (a power-of-two
-// scaling leaves a = lambda_min / trace unchanged) and its curvature.
+// scaling leaves a = lambda_min / trace unchanged) and its curvature; in
+// float64 from the points where the sums do not resolve it (RAD_FLAT).
 __global__ void __launch_bounds__(CURV_TPB)
-    radius_curvature_kernel(const double* __restrict__ part, int S, int n, const float4* __restrict__ sorted,
-                            double* __restrict__ a64, float* __restrict__ a32, double* __restrict__ sigma_out) {
+    radius_curvature_kernel(const double* __restrict__ part, int S, int n, const float4* __restrict__ P,
+                            const float* __restrict__ box, const double* __restrict__ e_dev, double scale2,
+                            const GridSpec* __restrict__ spec, double* __restrict__ a64, float* __restrict__ a32,
+                            double* __restrict__ sigma_out) {
   const int i0 = blockIdx.x * CURV_TPB + threadIdx.x;
   const int i = min(i0, n - 1);
+  const RadiusScale sc = radius_scale_of(e_dev, scale2, spec);
   double v[RAD_NS];
 #pragma unroll
   for (int f = 0; f < RAD_NS; ++f) v[f] = part[(size_t)f * n + i];
@@ -672,15 +774,28 @@ __global__ void __launch_bounds__(CURV_TPB)
 #pragma unroll
     for (int f = 0; f < RAD_NS; ++f) v[f] += part[((size_t)s * RAD_NS + f) * n + i];
   }
-  const double ik = 1.0 / v[0];
-  const double mx = v[1] * ik, my = v[2] * ik, mz = v[3] * ik;
   double C[9];
-  C[0] = fma(v[4], ik, -mx * mx); C[1] = fma(v[5], ik, -mx * my); C[2] = fma(v[6], ik, -mx * mz);
-  C[4] = fma(v[7], ik, -my * my); C[5] = fma(v[8], ik, -my * mz); C[8] = fma(v[9], ik, -mz * mz);
-  C[3] = C[1]; C[6] = C[2]; C[7] = C[5];
-  const double a = surface_variation(C);
+  covariance_of_sums(v, C);
+  double a = v[0] > 3.0 ? surface_variation(C) : 0.0;  // three points or fewer lie in a plane
+  const bool again = i0 < n && v[0] > 3.0 && !(a * (C[0] + C[4] + C[8]) >= (double)(RAD_FLAT * sc.B));
+  unsigned todo = __ballot_sync(0xffffffffu, again);
+  if (todo) {
+    for (; todo; todo &= todo - 1) {
+      const int src = __ffs(todo) - 1;
+      const double w = radius_sums_float64(P, n, box, sc.r2, __shfl_sync(0xffffffffu, i, src));
+#pragma unroll
+      for (int f = 0; f < RAD_NS; ++f) {
+        const double t = __shfl_sync(0xffffffffu, w, 2 * f);
+        if ((threadIdx.x & 31) == src) v[f] = t;
+      }
+    }
+    if (again) {
+      covariance_of_sums(v, C);
+      a = surface_variation(C);
+    }
+  }
   if (i0 < n) {
-    const int o = sorted ? __float_as_int(sorted[i].w) : i;
+    const int o = box ? __float_as_int(P[i].w) : i;
     a64[o] = a;
     a32[o] = (float)a;
   }
@@ -712,8 +827,8 @@ cudaError_t launch_radius_curvature(Launch L, const float4* P, int n, const floa
   const int S = radius_splits(n, num_sms, box != nullptr);
   radius_sums_kernel<<<dim3(blocks, S), RAD_TPB, 0, L.stream>>>(P, n, box, e_dev, scale2, spec, (ntiles + S - 1) / S,
                                                                 part);
-  radius_curvature_kernel<<<(n + CURV_TPB - 1) / CURV_TPB, CURV_TPB, 0, L.stream>>>(part, S, n, box ? P : nullptr, a64,
-                                                                                   a32, sigma_out);
+  radius_curvature_kernel<<<(n + CURV_TPB - 1) / CURV_TPB, CURV_TPB, 0, L.stream>>>(part, S, n, P, box, e_dev, scale2,
+                                                                                   spec, a64, a32, sigma_out);
   if (L.counter) *L.counter += 2;
   return cudaGetLastError();
 }
