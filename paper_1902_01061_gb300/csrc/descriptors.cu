@@ -347,12 +347,18 @@ __device__ __forceinline__ void two_sum_add(float& h, float& l, float x) {
 // the k neighbours; lambda_min clamped at 0; 0 for a zero trace.
 //
 // The offsets from the point itself are exact float pairs (two-difference),
-// their sums and products float pairs too (two-sum, fma remainder), good to
-// about 2^-46; only the covariance, its polynomial and the last Newton steps
-// are float64.  Where the offsets' squares leave float32's comfortable range,
-// all of it is float64.
+// their sums and products float pairs too (two-sum, fma remainder); only the
+// covariance, its polynomial and the last Newton steps are float64.  The pairs
+// leave an error in a of 2^-50 to 2^-48 rms (k = 8 to 32; emulated on patches
+// of random orientation), so a point flatter than CURV_FLAT, where that would
+// show in a float32 result, has its covariance formed again in float64 about
+// the neighbours' mean, and so has one whose offsets' squares leave float32's
+// comfortable range.  (A smooth surface of 1M points, k = 16, has a about 3e-7;
+// none of its points is that flat.)
 // Bound: float64 issue (about 80 such instructions a point, each 64 cycles of
 // a warp scheduler on GB300) and the gather of the neighbours.
+constexpr double CURV_FLAT = 0x1p-26;
+
 __device__ __noinline__ void covariance_float64(const float4* __restrict__ P, const int32_t* __restrict__ nb, int k,
                                                 double* C) {
   double mx = 0, my = 0, mz = 0;
@@ -410,22 +416,27 @@ __device__ __forceinline__ double point_curvature(const float4* __restrict__ P, 
         pl[f] = __fadd_rn(pl[f], r);
       }
   }
-  double C[9];
+  double C[9], a = 0.0;
   const float tr = ph[0] + ph[3] + ph[5];
-  if (!(tr > 1e-18f && tr < 1e30f)) {
-    covariance_float64(P, nb, k, C);
-    return surface_variation(C);
+  bool again = !(tr > 1e-18f && tr < 1e30f);
+  if (!again) {
+    const double ik = 1.0 / (double)k;
+    double mu[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) mu[d] = ((double)sh[d] + (double)sl[d]) * ik;
+#pragma unroll
+    for (int d = 0, f = 0; d < 3; ++d)
+#pragma unroll
+      for (int b = d; b < 3; ++b, ++f)
+        C[d * 3 + b] = C[b * 3 + d] = fma((double)ph[f] + (double)pl[f], ik, -mu[d] * mu[b]);
+    a = surface_variation(C);
+    again = a < CURV_FLAT;
   }
-  const double ik = 1.0 / (double)k;
-  double mu[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) mu[a] = ((double)sh[a] + (double)sl[a]) * ik;
-#pragma unroll
-  for (int a = 0, f = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = a; b < 3; ++b, ++f)
-      C[a * 3 + b] = C[b * 3 + a] = fma((double)ph[f] + (double)pl[f], ik, -mu[a] * mu[b]);
-  return surface_variation(C);
+  if (again) {
+    covariance_float64(P, nb, k, C);
+    a = surface_variation(C);
+  }
+  return a;
 }
 
 struct CurvatureIn {
