@@ -161,11 +161,10 @@ scgr_status scgr_force_vjp(scgr_ctx* c, const float* v_dev, float* grad_dev) {
   c->err.clear();
   if (!c->have_desc) return fail(c, SCGR_ERR_STATE, "compute descriptors first");
   if (c->rows >= 0) return fail(c, SCGR_ERR_STATE, "the VJP needs the whole template (a row range is set)");
-  // the force pass's split partials are the scratch of this pass's splits (nothing reads them between calls)
-  SCGR_CK(c, launch_force_vjp(c->L(), (const float4*)c->Xr.p, (const float2*)c->XA.p, (int)(c->npad / FORCE_TJ),
-                              (const float4*)c->Y0r.p, (int)c->mpad, (const double*)c->aY64.p, c->prm.g_mode,
-                              (int)c->m, c->pose, c->prm.p, v_dev, grad_dev, (float*)c->partial.p, c->partial.cap,
-                              c->num_sms));
+  SCGR_CK(c, launch_force_vjp(c->L(), c->vjp, (const float4*)c->Xr.p, (const float2*)c->XA.p,
+                              (int)(c->npad / FORCE_TJ), (const float4*)c->Y0r.p, (int)c->mpad,
+                              (const double*)c->aY64.p, c->prm.g_mode, (int)c->m, c->pose, c->prm.p, v_dev, grad_dev,
+                              (float*)(vjp_part_bytes(c->vjp, c->mpad) > c->partial.cap ? c->vjppart.p : c->partial.p)));
   return SCGR_OK;
 }
 

@@ -438,9 +438,16 @@ cudaError_t launch_combine_batch(Launch L, int nblocks, const int* cpair, const 
 cudaError_t launch_finalize_multi(Launch L, const double* blockpart, const BatchPair* pairs, int npairs,
                                   DevPose* poses, const DevStats* stats, StepParams sp, int* err);
 cudaError_t launch_pose_init_multi(Launch L, DevPose* poses, const DevStats* stats, int npairs, int E);
-cudaError_t launch_force_vjp(Launch L, const float4* Xr, const float2* XA, int ntiles, const float4* Y0r, int mpad,
-                             const double* aY64, int g_mode, int m, const DevPose* ps, double p, const float* v,
-                             float* grad, float* part, size_t part_bytes, int num_sms);
+// Grid of the force VJP: P template points per thread, `blocks` of them, `splits`
+// of the reference, nc sums a point.
+struct VjpPlan {
+  int P, blocks, tiles_per_split, splits, nc;
+};
+VjpPlan plan_vjp(int64_t m, int64_t npad, double p, int num_sms, int force_splits);
+size_t vjp_part_bytes(const VjpPlan& v, int64_t mpad);
+cudaError_t launch_force_vjp(Launch L, const VjpPlan& vp, const float4* Xr, const float2* XA, int ntiles,
+                             const float4* Y0r, int mpad, const double* aY64, int g_mode, int m, const DevPose* ps,
+                             double p, const float* v, float* grad, float* part);
 // Stored pair terms: W is M rows of npad floats (npad = the padded reference
 // length of the records, a multiple of 256).
 cudaError_t launch_store_pairs(Launch L, const float2* XA, const float4* Xr, int npad, const float4* Y0r,

@@ -58,6 +58,7 @@ struct scgr_ctx {
   int64_t launches = 0;
   ForcePlan fp{};
   ForcePlan fpot{};        // the potential's pair pass
+  scgr::VjpPlan vjp{};     // the force VJP's
   float qexp = 0.f;        // (p - 1) / 2, exponent of d^2 in the weight
 
   DevBuf X4, Y4, stage, knnX, knnY, aX64, aY64, aX32, aY32, Xr, XA, Y0r, partial, blockpart,
@@ -87,7 +88,7 @@ struct scgr_ctx {
   int64_t nearest_grid_min = 1024; // references with at least this many points: grid nearest search (tunable)
   ForceTuning ftune;            // force-plan overrides (tunable)
   int reuse_pose_free = 1;      // p = 1: one force pass per scgr_run (tunable)
-  DevBuf cd_key, cd_moved, wstore, wupart, wpartial, mpart, mom, radpart, sigpart, fixpart, upart, ord[2];
+  DevBuf cd_key, cd_moved, wstore, wupart, wpartial, mpart, mom, radpart, sigpart, fixpart, upart, vjppart, ord[2];
   // grids of the reference [0] and the template [1], kept until the cloud changes
   DevBuf gspec, gcell[2], gstart[2], gtot[2], gsorted[2], gccount;
   bool grid_ok[2] = {false, false};  // sorted into grid cells

@@ -397,6 +397,7 @@ scgr_status plan_buffers(scgr_ctx* c) {
   t.occ = 0;
   ForcePlan& fu = c->fpot;
   fu = plan_force(mloc, c->npad, c->prm.p, c->num_sms, t);
+  const int force_splits = fu.splits;
   const int64_t ntiles = c->npad / FORCE_TJ, cap = (int64_t)c->fp.splits;
   if (fu.half || fu.splits > cap) {
     const int64_t S = fu.half ? (cap < ntiles ? cap : ntiles) : cap;
@@ -409,6 +410,11 @@ scgr_status plan_buffers(scgr_ctx* c) {
   SCGR_CK(c, ensure(c->blockpart, (size_t)combine_blocks(c->mpad) * 13 * sizeof(double)));
   SCGR_CK(c, ensure(c->fixpart, fixed_part_bytes(c->num_sms)));
   SCGR_CK(c, ensure(c->upart, (size_t)fu.splits * fu.iblocks * sizeof(double)));
+  c->vjp = plan_vjp(mloc, c->npad, c->prm.p, c->num_sms, force_splits);
+  // its scratch is the force pass's partials (nothing reads them between calls) where they suffice, as they do
+  // unless a knob has made them small
+  const size_t vjp_bytes = vjp_part_bytes(c->vjp, c->mpad);
+  if (vjp_bytes > c->partial.cap) SCGR_CK(c, ensure(c->vjppart, vjp_bytes));
   return SCGR_OK;
 }
 

@@ -522,40 +522,52 @@ __global__ void __launch_bounds__(VJP_TPB)
 }
 
 // Splits of the reference range: enough blocks for about eight per SM (two
-// waves of the four to five that are resident), at least one tile each, and
-// at most what the scratch of `part_bytes` bytes holds (one split needs
-// none).  With few blocks even so, one template point per thread instead of
-// two.
-template <int PM>
-static void launch_vjp_pm(Launch L, const float* Xr, const float* XA, int ntiles, const float4* Y0r, int mpad,
-                          const double* aY64, int g_mode, int m, const DevPose* ps, double pm1, const float* v,
-                          float* grad, float* part, size_t part_bytes, int num_sms) {
-  constexpr int nc = PM == 1 ? 1 : VJP_NC;
-  const int64_t want = 8 * (int64_t)num_sms;
-  const int64_t cap = (int64_t)(part_bytes / ((size_t)nc * mpad * sizeof(float)));
-  const int64_t most = cap < ntiles ? (cap < 1 ? 1 : cap) : ntiles;
-  const int b2 = (m + 2 * VJP_TPB - 1) / (2 * VJP_TPB), b1 = (m + VJP_TPB - 1) / VJP_TPB;
-  const bool two = (int64_t)b2 * most >= want;
-  const int blocks = two ? b2 : b1;
-  int64_t S = (want + blocks - 1) / blocks;
+// waves of the four to five that are resident), at least one tile each, and at
+// most 4 / nc times the force pass's splits by its own rule (force_splits), which
+// keeps a block's run of tiles long enough to pay for its start (10,007 x 9,001,
+// p = 2: 10 splits of 4 tiles 88 us, 20 splits of 2 tiles 107 us).  With few
+// blocks even so, one template point per thread instead of two.  From the sizes
+// alone, so that the same call gives the same bits whatever the context has held
+// before and whatever knobs shape the force pass.
+VjpPlan plan_vjp(int64_t m, int64_t npad, double p, int num_sms, int force_splits) {
+  const int64_t want = 8 * (int64_t)num_sms, ntiles = npad / FORCE_TJ;
+  VjpPlan v;
+  v.nc = p == 1.0 ? 1 : VJP_NC;
+  int64_t most = 4 * (int64_t)force_splits / v.nc;
+  most = most < 1 ? 1 : most < ntiles ? most : ntiles;
+  const int64_t b2 = (m + 2 * VJP_TPB - 1) / (2 * VJP_TPB), b1 = (m + VJP_TPB - 1) / VJP_TPB;
+  v.P = b2 * most >= want ? 2 : 1;
+  v.blocks = (int)(v.P == 2 ? b2 : b1);
+  int64_t S = (want + v.blocks - 1) / v.blocks;
   if (S > most) S = most;
-  const int tps = (int)((ntiles + S - 1) / S);
-  const int splits = (ntiles + tps - 1) / tps;
-  const dim3 grid(blocks, splits);
-  if (two)
-    force_vjp_kernel<2, PM><<<grid, VJP_TPB, 0, L.stream>>>(Xr, XA, ntiles, tps, Y0r, mpad, aY64, g_mode, m, ps, pm1, v, grad, part);
-  else
-    force_vjp_kernel<1, PM><<<grid, VJP_TPB, 0, L.stream>>>(Xr, XA, ntiles, tps, Y0r, mpad, aY64, g_mode, m, ps, pm1, v, grad, part);
+  v.tiles_per_split = (int)((ntiles + S - 1) / S);
+  v.splits = (int)((ntiles + v.tiles_per_split - 1) / v.tiles_per_split);
+  return v;
+}
+// Scratch of the splits' sums (one split needs none).
+size_t vjp_part_bytes(const VjpPlan& v, int64_t mpad) {
+  return v.splits > 1 ? (size_t)v.splits * v.nc * mpad * sizeof(float) : 0;
+}
+
+template <int PM>
+static void launch_vjp_pm(Launch L, const VjpPlan& vp, const float* Xr, const float* XA, int ntiles, const float4* Y0r,
+                          int mpad, const double* aY64, int g_mode, int m, const DevPose* ps, double pm1,
+                          const float* v, float* grad, float* part) {
+  const dim3 grid(vp.blocks, vp.splits);
+  const auto k = vp.P == 2 ? force_vjp_kernel<2, PM> : force_vjp_kernel<1, PM>;
+  k<<<grid, VJP_TPB, 0, L.stream>>>(Xr, XA, ntiles, vp.tiles_per_split, Y0r, mpad, aY64, g_mode, m, ps, pm1, v, grad,
+                                    part);
   if (L.counter) ++*L.counter;
-  if (splits > 1) {
-    vjp_combine_kernel<<<b1, VJP_TPB, 0, L.stream>>>(part, splits, nc, mpad, aY64, g_mode, m, pm1, v, grad);
+  if (vp.splits > 1) {
+    vjp_combine_kernel<<<(m + VJP_TPB - 1) / VJP_TPB, VJP_TPB, 0, L.stream>>>(part, vp.splits, vp.nc, mpad, aY64,
+                                                                              g_mode, m, pm1, v, grad);
     if (L.counter) ++*L.counter;
   }
 }
 
-cudaError_t launch_force_vjp(Launch L, const float4* Xr, const float2* XA, int ntiles, const float4* Y0r, int mpad,
-                             const double* aY64, int g_mode, int m, const DevPose* ps, double p, const float* v,
-                             float* grad, float* part, size_t part_bytes, int num_sms) {
+cudaError_t launch_force_vjp(Launch L, const VjpPlan& vp, const float4* Xr, const float2* XA, int ntiles,
+                             const float4* Y0r, int mpad, const double* aY64, int g_mode, int m, const DevPose* ps,
+                             double p, const float* v, float* grad, float* part) {
   if (m <= 0) return cudaSuccess;
   const float* xr = reinterpret_cast<const float*>(Xr);
   const float* xa = reinterpret_cast<const float*>(XA);
@@ -563,7 +575,7 @@ cudaError_t launch_force_vjp(Launch L, const float4* Xr, const float2* XA, int n
                       : p == 2.0 ? launch_vjp_pm<2>
                       : p == 3.0 ? launch_vjp_pm<3>
                                  : launch_vjp_pm<0>;
-  launch(L, xr, xa, ntiles, Y0r, mpad, aY64, g_mode, m, ps, p - 1.0, v, grad, part, part_bytes, num_sms);
+  launch(L, vp, xr, xa, ntiles, Y0r, mpad, aY64, g_mode, m, ps, p - 1.0, v, grad, part);
   return cudaGetLastError();
 }
 
