@@ -465,7 +465,7 @@ def _potential_function():
     class Potential(torch.autograd.Function):
         """U(pose7, Y0) on a context whose template is Y0 (descriptors fixed).
 
-        forward: the potential, and where an input wants a gradient the
+        forward: the potential, and where a gradient is recorded (want) the
         hand-written adjoint with it (scgr_potential with gradients), since
         one pair pass gives both; backward: the scaling by the incoming
         gradient.  No N x M pair terms are stored.  (50,000 x 50,000: forward
@@ -473,8 +473,7 @@ def _potential_function():
         gradient is never taken 1.20 ms, without gradients 0.93 ms.)"""
 
         @staticmethod
-        def forward(fctx, pose7, Y0, handle):
-            want = any(fctx.needs_input_grad[:2])
+        def forward(fctx, pose7, Y0, handle, want):
             gx = torch.empty((Y0.shape[0], 3), dtype=torch.float32, device=Y0.device) if want else None
             U, fctx.g7 = scgr_potential(handle, pose7.detach().double().cpu().numpy(), want_grad=want, grad_xyz_out=gx)
             fctx.save_for_backward(pose7, gx)
@@ -485,7 +484,7 @@ def _potential_function():
             pose7, gx = fctx.saved_tensors
             g = float(gU)
             gp = torch.from_numpy(fctx.g7).to(pose7.dtype) * g
-            return gp.to(pose7.device), gx * g, None
+            return gp.to(pose7.device), gx * g, None, None
 
     return Potential
 
@@ -499,7 +498,11 @@ def potential(pose7, Y0, handle):
     global _POTENTIAL
     if _POTENTIAL is None:
         _POTENTIAL = _potential_function()
-    return _POTENTIAL.apply(pose7, Y0, handle)
+    import torch
+    # read here: inside forward the grad mode is off, and needs_input_grad is
+    # set under no_grad too
+    want = torch.is_grad_enabled() and (pose7.requires_grad or Y0.requires_grad)
+    return _POTENTIAL.apply(pose7, Y0, handle, want)
 
 
 # ---- convenience wrapper ----------------------------------------------------
