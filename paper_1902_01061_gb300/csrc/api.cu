@@ -97,7 +97,7 @@ void scgr_destroy(scgr_ctx* c) {
                     &c->bgclouds, &c->bgspec, &c->bgcell, &c->bgsorted, &c->bgstart, &c->bgtot, &c->bgpart,
                     &c->gspec, &c->gcell[0], &c->gcell[1], &c->gstart[0], &c->gstart[1], &c->gtot[0], &c->gtot[1],
                     &c->gsorted[0], &c->gsorted[1], &c->gccount,
-                    &c->cd_key, &c->cd_moved, &c->wstore, &c->wupart, &c->wpartial, &c->mpart, &c->mom, &c->radpart, &c->sigpart, &c->fixpart, &c->upart, &c->vjppart, &c->ord[0], &c->ord[1]};
+                    &c->cd_key, &c->cd_moved, &c->wstore, &c->wupart, &c->wpartial, &c->mpart, &c->mom, &c->radpart, &c->sigpart, &c->fixpart, &c->upart, &c->ppart, &c->vjppart, &c->ord[0], &c->ord[1]};
   for (DevBuf* b : bufs) release(*b);
   if (c->pose) cudaFree(c->pose);
   if (c->pose_eval) cudaFree(c->pose_eval);

@@ -114,12 +114,15 @@ scgr_status scgr_potential(scgr_ctx* c, const double pose7[7], double* U_out, do
   const bool grad = grad_pose7 || grad_xyz_dev;
   SCGR_CK(c, launch_pose_from_host(L, hp, c->pose_eval, c->stats));
   const ForcePlan& fu = c->fpot;
+  // the split partials: the force pass's (nothing reads them between calls) where they suffice
+  const size_t need = (size_t)fu.splits * c->mpad * sizeof(float4);
+  if (grad && need > c->partial.cap) SCGR_CK(c, ensure(c->ppart, need));
+  float4* const part = (float4*)(need > c->partial.cap ? c->ppart.p : c->partial.p);
   SCGR_CK(c, launch_potential(L, fu, grad, (const float4*)c->Xr.p, (const float2*)c->XA.p,
                               (int)(c->npad / c->fp.tile_j), (const float4*)c->Y0r.p, (int)c->mpad, (int)c->m,
-                              (const float*)c->aY32.p, c->prm.g_mode, c->pose_eval, c->qexp, (float4*)c->partial.p,
-                              (double*)c->upart.p));
+                              (const float*)c->aY32.p, c->prm.g_mode, c->pose_eval, c->qexp, part, (double*)c->upart.p));
   if (grad)
-    SCGR_CK(c, launch_adjoint_combine(L, (const float4*)c->partial.p, fu.splits, (int)c->mpad, (int)c->m,
+    SCGR_CK(c, launch_adjoint_combine(L, part, fu.splits, (int)c->mpad, (int)c->m,
                                       (const float4*)c->Y0r.p, (const double*)c->aY64.p, c->prm.g_mode,
                                       c->pose_eval, grad_xyz_dev, (double*)c->blockpart.p));
   return finish_potential(c, (const double*)c->upart.p, (int64_t)fu.splits * fu.iblocks, grad, pose7, hp, U_out,

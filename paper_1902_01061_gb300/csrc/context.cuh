@@ -88,7 +88,7 @@ struct scgr_ctx {
   int64_t nearest_grid_min = 1024; // references with at least this many points: grid nearest search (tunable)
   ForceTuning ftune;            // force-plan overrides (tunable)
   int reuse_pose_free = 1;      // p = 1: one force pass per scgr_run (tunable)
-  DevBuf cd_key, cd_moved, wstore, wupart, wpartial, mpart, mom, radpart, sigpart, fixpart, upart, vjppart, ord[2];
+  DevBuf cd_key, cd_moved, wstore, wupart, wpartial, mpart, mom, radpart, sigpart, fixpart, upart, ppart, vjppart, ord[2];
   // grids of the reference [0] and the template [1], kept until the cloud changes
   DevBuf gspec, gcell[2], gstart[2], gtot[2], gsorted[2], gccount;
   bool grid_ok[2] = {false, false};  // sorted into grid cells

@@ -383,10 +383,10 @@ scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_sca
   return SCGR_OK;
 }
 
-// The force plan of the context's template rows, the potential's plan beside
-// it, and the buffers whose size they set.  The potential runs 1 or 2 points x
-// 128 threads (the shapes its kernel has) in splits that fit the force pass's
-// partials.
+// The force plan of the context's template rows, the plans of the potential
+// and the force VJP beside it, and the buffers whose size they set.  The
+// potential runs 1 or 2 points x 128 threads (the shapes its kernel has) in
+// whole tiles; the force kernel's knobs do not shape it.
 scgr_status plan_buffers(scgr_ctx* c) {
   const int64_t mloc = c->rows >= 0 ? c->rows : c->m;
   c->fp = plan_force(mloc, c->npad, c->prm.p, c->num_sms, c->ftune);
@@ -398,12 +398,9 @@ scgr_status plan_buffers(scgr_ctx* c) {
   ForcePlan& fu = c->fpot;
   fu = plan_force(mloc, c->npad, c->prm.p, c->num_sms, t);
   const int force_splits = fu.splits;
-  const int64_t ntiles = c->npad / FORCE_TJ, cap = (int64_t)c->fp.splits;
-  if (fu.half || fu.splits > cap) {
-    const int64_t S = fu.half ? (cap < ntiles ? cap : ntiles) : cap;
+  if (fu.half) {
     fu.half = 0;
-    fu.tiles_per_split = (int)((ntiles + S - 1) / S);
-    fu.splits = (int)((ntiles + fu.tiles_per_split - 1) / fu.tiles_per_split);
+    fu.splits = (int)(c->npad / FORCE_TJ);  // of one tile
   }
   SCGR_CK(c, ensure(c->Y0r, (size_t)c->mpad * sizeof(float4)));
   SCGR_CK(c, ensure(c->partial, (size_t)c->fp.splits * c->mpad * sizeof(float4)));

@@ -49,3 +49,20 @@ def test_vjp_bits_do_not_depend_on_history_or_knobs(n, m, p):
     assert np.isfinite(got[0]).all() and np.abs(got[0]).max() > 0
     for other in got[1:]:
         np.testing.assert_array_equal(other, got[0])
+
+
+@pytest.mark.parametrize("n,m,p", [(900, 700, 2.0), (5003, 4801, 1.0), (5003, 4801, 1.5), (3000, 9000, 2.0), (257, 70, 3.0)])
+def test_potential_bits_do_not_depend_on_the_force_knobs(n, m, p):
+    X, Y = clouds(n, m)
+    pose = np.array([0.2, -0.1, 0.3, 0.05, 0.0, -0.1, 1.05])
+    got = []
+    for tune in KNOBS:
+        with Gpu(X, Y, p=p, tune=tune) as g:
+            gx = torch.empty((m, 3), dtype=torch.float32, device="cuda")
+            U0, _ = scgr.scgr_potential(g.ctx, pose, want_grad=False)
+            U, g7 = scgr.scgr_potential(g.ctx, pose, grad_xyz_out=gx)
+            got.append((U0, U, g7, gx.cpu().numpy()))
+    assert np.isfinite(got[0][3]).all() and got[0][1] > 0
+    for other in got[1:]:
+        for a, b in zip(other, got[0]):
+            np.testing.assert_array_equal(a, b)
