@@ -387,7 +387,7 @@ scgr_status curvatures(scgr_ctx* c, int k, double radius_scale, double sigma_sca
 // and the force VJP beside it, and the buffers whose size they set.  The
 // potential runs 1 or 2 points x 128 threads (the shapes its kernel has) in
 // whole tiles; the force kernel's knobs do not shape it.
-scgr_status plan_buffers(scgr_ctx* c) {
+static scgr_status plan_and_size(scgr_ctx* c) {
   const int64_t mloc = c->rows >= 0 ? c->rows : c->m;
   c->fp = plan_force(mloc, c->npad, c->prm.p, c->num_sms, c->ftune);
   c->mpad = force_mpad(mloc, c->fp);
@@ -413,6 +413,14 @@ scgr_status plan_buffers(scgr_ctx* c) {
   const size_t vjp_bytes = vjp_part_bytes(c->vjp, c->mpad);
   if (vjp_bytes > c->partial.cap) SCGR_CK(c, ensure(c->vjppart, vjp_bytes));
   return SCGR_OK;
+}
+
+// A failed allocation leaves the plans without their buffers: no pass may run
+// on them, so the descriptors are wanted again.
+scgr_status plan_buffers(scgr_ctx* c) {
+  const scgr_status st = plan_and_size(c);
+  if (st != SCGR_OK) c->have_desc = false;
+  return st;
 }
 
 // Recompute the force plan (after a tuning change) and the buffers and
