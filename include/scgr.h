@@ -127,13 +127,21 @@ SCGR_EXPORT scgr_status scgr_set_template(scgr_ctx* ctx, const float* xyz_dev, i
 SCGR_EXPORT scgr_status scgr_set_template_host(scgr_ctx* ctx, const float* xyz_host, int64_t m);
 
 /* One-time descriptor pass (Sec. III-A, Sec. IV): k-nearest neighbours of
- * every point of X and of Y0 (exact float32 key (dx*dx+dy*dy)+dz*dz, no fused
- * multiply-add, self included, ties to the lower index; an exact
- * uniform-grid search), the curvature
- * a = lambda_min / (lambda_1+lambda_2+lambda_3) of each neighbourhood's
- * covariance (float64), sigma, and the cloud statistics used by the scale
- * model (means, covariances, largest eigenvalues).  Resets the pose to
- * identity and the iteration counter to 0.  STATE if a cloud is missing. */
+ * every point of X and of Y0 (the first k by a float32 squared-distance key,
+ * self included, ties to the lower index; an exact uniform-grid search), the
+ * curvature a = lambda_min / (lambda_1+lambda_2+lambda_3) of each
+ * neighbourhood's covariance (its sums in float32 pairs that leave about 2^-48
+ * in a, in float64 for points flatter than that resolves), sigma, and the cloud
+ * statistics used by the scale model (means, covariances, largest eigenvalues).
+ * Resets the pose to identity and the iteration counter to 0.  STATE if a cloud
+ * is missing.
+ * The key of clouds of 20000 points and more is (dx*dx + dy*dy) + dz*dz with
+ * every operation rounded on its own.  Smaller clouds, and all clouds of
+ * scgr_batch_run, take fma(dz, dz, fma(dx, dx, dy*dy)), one rounding less a sum,
+ * as the packed brute-force search forms it (but for a cloud's last n % 4
+ * points).  The two differ at near ties: in about 1e-5 of the rows of random
+ * samples, in a quarter of the rows of a cubic lattice.
+ * SCGR_TUNE_KNN_GRID_MIN = 0 gives the first key at every size. */
 SCGR_EXPORT scgr_status scgr_compute_descriptors(scgr_ctx* ctx);
 
 /* Enqueue `iterations` iterations (Eq. 5 - Eq. 12) on the context stream.
@@ -184,11 +192,15 @@ SCGR_EXPORT scgr_status scgr_set_curvature(scgr_ctx* ctx, int which, const doubl
 SCGR_EXPORT scgr_status scgr_set_neighbourhood(scgr_ctx* ctx, int k, double radius_scale, double sigma_scale);
 
 /* Nearest reference point of q_dev [nq][3] (float32): index int32 [nq] and
- * float32 key (squared distance, the kNN key of R1) [nq]; either output may
- * be NULL.  Ties go to the lower index.  References of at least
+ * float32 key (squared distance, every operation rounded on its own) [nq];
+ * either output may be NULL.  Ties go to the lower index.  References of at least
  * SCGR_TUNE_NEAREST_GRID_MIN points are searched through an exact uniform grid
  * (same result as brute force; queries may lie outside the reference's box),
- * smaller ones by brute force.  Enqueued.  STATE without a reference. */
+ * smaller ones by brute force.  A query without a finite key (infinite, NaN or
+ * beyond about 1e19) gets index 2^31 - 1 and an infinite key.  Inside a caller's
+ * stream capture references below 65536 points are searched by brute force, so
+ * that a replay answers for the reference of that moment; larger ones keep the
+ * grid of the capture if one is there.  Enqueued.  STATE without a reference. */
 SCGR_EXPORT scgr_status scgr_nearest(scgr_ctx* ctx, const float* q_dev, int64_t nq, int32_t* idx_dev,
                                      float* key_dev);
 
@@ -342,8 +354,9 @@ SCGR_EXPORT scgr_status scgr_step_apply_dev(scgr_ctx* ctx, const double* parts_d
                                          [1, 4096]; until set, by the batch's size (2 or 4) */
 #define SCGR_TUNE_KNN_GRID_MIN 2      /* clouds of at least this many points use the exact grid kNN in
                                          scgr_compute_descriptors, smaller ones brute force (0: always the
-                                         grid).  Until set, the grid serves every cloud; below 20000 points
-                                         it then keys candidates with the brute-force search's rounding */
+                                         grid), the grid with the key that rounds every operation.  Until
+                                         set, the grid serves every cloud, below 20000 points with the
+                                         fused key (scgr_compute_descriptors) */
 #define SCGR_TUNE_NEAREST_GRID_MIN 14 /* references of at least this many points answer scgr_nearest and
                                          scgr_change_mask through the exact grid search (default 1024;
                                          0: always); the result is identical */

@@ -132,8 +132,9 @@ scgr_status read_error_word(scgr_ctx* c);
 scgr_status set_cloud(scgr_ctx* c, const float* xyz, int64_t n, bool host, bool ref);
 scgr_status force_launch(scgr_ctx* c);
 scgr_status collect_timing(scgr_ctx* c);
-// Clouds below this many points were searched by brute force, whose packed
-// key rounds once less; the grid search keeps their neighbours the same.
+// Clouds below this many points were searched by brute force, whose packed key
+// rounds each sum once less (but for the last n % 4 points); the grid search forms
+// that key for them, so that they keep their neighbours (grid_key).
 constexpr int64_t KNN_FUSED_KEY = 20000;
 scgr_status prepare_clouds(scgr_ctx* c);
 scgr_status nearest_reference(scgr_ctx* c, const float* q3, int nq, int32_t* idx_out, float* key_out);

@@ -313,9 +313,11 @@ __global__ void __launch_bounds__(256) cell_scatter_kernel(const CloudSet cs) {
 // ---- queries ---------------------------------------------------------------------
 
 // Squared distance of the (key, index) order.  FUSED = false: (dx*dx + dy*dy)
-// + dz*dz, each operation rounded on its own.  FUSED = true: the rounding of
-// the packed brute-force search, whose sums the assembler fuses with the
-// products they add; its callers keep the neighbours they had.
+// + dz*dz, each operation rounded on its own.  FUSED = true: the sums fused with
+// the products they add, as the assembler does in the packed brute-force search
+// that served clouds below KNN_FUSED_KEY points and batches before; near ties
+// fall as they fell there (its last n % 4 candidates apart, which it keyed one by
+// one without fusing).
 template <bool FUSED>
 __device__ __forceinline__ float grid_key(float4 q, float4 c) {
   const float dx = __fsub_rn(q.x, c.x), dy = __fsub_rn(q.y, c.y), dz = __fsub_rn(q.z, c.z);
