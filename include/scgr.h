@@ -396,9 +396,9 @@ SCGR_EXPORT scgr_status scgr_step_apply_dev(scgr_ctx* ctx, const double* parts_d
                                          special-function unit.  Results agree with 0 to rounding */
 #define SCGR_TUNE_NEAREST_LEVELS 12  /* nearest-point search over a gridded reference (scgr_nearest,
                                          scgr_change_mask): 2 (default) fine cells around the query, then
-                                         cells of 16 and of 4 fine cells a side that skip empty ones and
-                                         ones beyond the best distance so far; 1 cells of 4 and of 1, with
-                                         no counts of the empty ones.  The result is the same */
+                                         cells of 16 and of 4 fine cells a side; 1 cells of 4 and fine
+                                         cells.  Both skip empty cells and ones beyond the best distance
+                                         so far; the result is the same */
 #define SCGR_TUNE_FUSED_TAIL 13      /* 1 (default): for templates of at most 2,048 padded slots one launch
                                          per iteration combines the split partials and updates the pose
                                          (one block), and where the clouds are small enough for one

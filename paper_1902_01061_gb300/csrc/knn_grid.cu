@@ -812,7 +812,9 @@ __global__ void __launch_bounds__(NEAREST_WARPS * 32, 16)
       s3[a] = (m3[a] + NC - 1) / NC;
       cc[a] /= coarse * NC;
     }
-    const int* scount = ccount ? ccount + m3[0] * m3[1] * m3[2] : nullptr;
+    // counts of the large cells, and (levels 2) of the coarse ones; levels 1 asks the fine cells themselves
+    const bool fine = coarse == 1;
+    const int* scount = fine ? ccount : ccount + m3[0] * m3[1] * m3[2];
     for (int s = 0;; ++s) {
       int lo[3], e[3];  // the cube's part inside the grid
 #pragma unroll
@@ -826,7 +828,7 @@ __global__ void __launch_bounds__(NEAREST_WARPS * 32, 16)
         const int x = lo[0] + c - yz * e[0], y = lo[1] + yz % e[1], z = lo[2] + yz / e[1];
         unsigned d = NO_CELL;
         if (c < cube && max(abs(x - cc[0]), max(abs(y - cc[1]), abs(z - cc[2]))) == s &&
-            !(scount && scount[(z * s3[1] + y) * s3[0] + x] == 0))
+            scount[(z * s3[1] + y) * s3[0] + x] != 0)
           d = box_bits(x, y, z, HS);
         for (int src; (src = nearest_lane(d)) >= 0;) {
           if (lane == src) d = NO_CELL;
@@ -838,8 +840,10 @@ __global__ void __launch_bounds__(NEAREST_WARPS * 32, 16)
           for (int r = 0; r < 2; ++r) {
             const int u = r * 32 + lane, xc = X + u % NC, yc = Y + u / NC % NC, zc = Z + u / (NC * NC);
             dc[r] = NO_CELL;
-            if (xc < m3[0] && yc < m3[1] && zc < m3[2] && !(ccount && ccount[(zc * m3[1] + yc) * m3[0] + xc] == 0))
-              dc[r] = box_bits(xc, yc, zc, H);
+            if (xc < m3[0] && yc < m3[1] && zc < m3[2]) {
+              const int c1 = (zc * m3[1] + yc) * m3[0] + xc;
+              if (fine ? cell_start(g, c1 + 1) > cell_start(g, c1) : ccount[c1] != 0) dc[r] = box_bits(xc, yc, zc, H);
+            }
           }
           // two coarse cells at a time, 16 lanes each: a lane per row of fine cells
           for (;;) {
@@ -953,12 +957,12 @@ cudaError_t launch_coarse_count(Launch L, const CloudSet& cs, int64_t n, int* cc
 
 // Nearest point of the sorted cloud cs[0] for each of nq queries.  levels 2:
 // far queries descend through cells of 16 and of 4 fine cells that hold
-// points; 1: through cells of 4 to fine cells, empty or not.
+// points; 1: through cells of 4 and fine cells that do.
 cudaError_t launch_nearest_grid(Launch L, const CloudSet& cs, int levels, const int* ccount, const float* q3, int nq,
                                 int32_t* idx_out, float* key_out) {
   if (nq <= 0) return cudaSuccess;
   nearest_query_kernel<<<up(nq, NEAREST_WARPS), NEAREST_WARPS * 32, 0, L.stream>>>(
-      cs, levels == 1 ? 1 : NEAREST_COARSE, levels == 1 ? nullptr : ccount, q3, nq, idx_out, key_out);
+      cs, levels == 1 ? 1 : NEAREST_COARSE, ccount, q3, nq, idx_out, key_out);
   if (L.counter) *L.counter += 1;
   return cudaGetLastError();
 }
