@@ -327,10 +327,10 @@ scgr_status nearest_reference(scgr_ctx* c, const float* q3, int nq, int32_t* idx
 
 // Radius neighbourhoods in Morton order from this size of the larger cloud on:
 // the order costs seven launches and saves the pairs beyond the radius (scale 1
-// and 0.5, the descriptor pass of n + 0.9 n points, in index order 4,000: 178 and
-// 188 us, 8,000: 346 and 342, 40,000: 5704 and 5606; in Morton order 200 and
-// 200, 275 and 242, 1532 and 824).
-constexpr int RADIUS_ORDER_MIN = 6144;
+// and 0.5, the descriptor pass of n + 0.9 n points, in index order 4,000: 190 and
+// 209 us, 6,000: 276 and 274, 8,000: 404 and 399, 40,000: 7222 and 7089; in Morton
+// order 209 and 197, 247 and 214, 284 and 242, 1860 and 984).
+constexpr int RADIUS_ORDER_MIN = 5120;
 
 // Curvature of both clouds for the current neighbourhood mode (k nearest or
 // radius), then sigma (scaled by sigma_scale).

@@ -506,8 +506,8 @@ cudaError_t launch_curvature2(Launch L, const float4* X, const int32_t* nx, int 
 // (order.cu): a warp's queries and a run of 32 points are then compact, and a
 // run whose box lies beyond the radius of the warp's box costs nothing.
 // (20,011 + 17,611 points, scale 1, the whole descriptor pass: 30.2 ms with
-// two passes of 12 float64 operations per member; 1.49 ms unordered; 0.62 ms
-// with offsets rounded to float32.)
+// two passes of 12 float64 operations per member; 1.87 ms in index order, 0.66 ms
+// in Morton order; 0.58 ms with offsets rounded to float32.)
 //
 // Members' offsets are scaled by a power of two that brings the bound on
 // |d|^2 (the smaller of the squared radius and three squared box extents)
@@ -815,8 +815,8 @@ __global__ void __launch_bounds__(CURV_TPB)
 
 // Splits of the cloud, so that a small one still gives every SM about eight
 // blocks (at least one tile each); in order, where a block's work is the tiles
-// near its queries, 32 (20,011 + 18,009 points, scale 1: 733 us with 8, 621
-// with 16, 615 with 32; 40,000: 2172, 1772, 1532).
+// near its queries, 32 (20,011 + 18,009 points, scale 1: 895 us with 8, 727
+// with 16, 711 with 32; 40,000: 2731, 2180, 1860).
 int radius_splits(int n, int num_sms, bool ordered) {
   const int blocks = (n + RAD_TPB - 1) / RAD_TPB, ntiles = (n + RAD_TILE - 1) / RAD_TILE;
   int S = ((ordered ? 32 : 8) * num_sms + blocks - 1) / blocks;
