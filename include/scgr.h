@@ -225,8 +225,9 @@ SCGR_EXPORT scgr_status scgr_forces(scgr_ctx* ctx, float* f4_dev);
  * pose7 = (omega[3], t[3], s): Y = s * Y0 @ R + t with R = exp([omega]_x)^T
  * (axis-angle, row-vector convention).  Optional outputs: grad_pose7 (host,
  * 7 doubles: dU/domega, dU/dt, dU/ds) and grad_xyz_dev (device float32
- * [m][3]: dU/dY0).  The gradient pass recomputes the pair tiles of the force
- * kernel (no N x M storage); sums are float64 in a fixed order.  The
+ * [m][3]: dU/dY0).  One pass over the pair tiles gives U and the points'
+ * gradient sums (no N x M storage).  A point's sums are float32 with Kahan
+ * compensation, the sums over points float64, all in a fixed order.  The
  * registration pose is not touched.  Synchronises.  STATE before
  * descriptors; INVALID_ARG for a non-finite pose or s <= 0. */
 SCGR_EXPORT scgr_status scgr_potential(scgr_ctx* ctx, const double pose7[7], double* U_out,
@@ -360,6 +361,8 @@ SCGR_EXPORT scgr_status scgr_step_apply_dev(scgr_ctx* ctx, const double* parts_d
 #define SCGR_TUNE_NEAREST_GRID_MIN 14 /* references of at least this many points answer scgr_nearest and
                                          scgr_change_mask through the exact grid search (default 1024;
                                          0: always); the result is identical */
+/* The SCGR_TUNE_FORCE_* knobs shape the force pass of scgr_forces, scgr_run and the
+ * stepwise calls; the potential and the force VJP have grids of their own. */
 #define SCGR_TUNE_FORCE_P 3           /* force kernel template points per thread: 0 auto, 1, 2, 4 */
 #define SCGR_TUNE_FORCE_TPB 4         /* force kernel threads per block: 0 auto, 128, 256 */
 #define SCGR_TUNE_FORCE_SPLITS 5      /* force kernel reference splits: 0 auto (wave-filling), >= 1 */

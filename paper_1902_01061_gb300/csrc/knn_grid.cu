@@ -446,7 +446,8 @@ __device__ __forceinline__ u64 warp_merge(u64 v) {  // v bitonic
 // Two warps a block: queries differ in length and a block keeps its warps'
 // places until the last is done (8 warps: 32 of 64 warps active on average).
 // 1M + 1M points, the whole descriptor pass: 8 warps and 5 blocks an SM 3406
-// us, 4 and 10 3223, 2 and 20 3225, 2 and 24 (40 registers) 3121.  A batch's
+// us, 4 and 10 3223, 2 and 20 3225, 2 and 24 (40 registers) 3121; with rows
+// inside the grid only 3067.  A batch's
 // table entries are chunks of queries that 8 warps share.
 constexpr int QUERY_WARPS = 2, QUERY_BLOCKS = 24;
 constexpr int QUERY_TABLE_WARPS = 8, QUERY_TABLE_BLOCKS = 5;

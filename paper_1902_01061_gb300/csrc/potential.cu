@@ -95,8 +95,9 @@ __device__ __forceinline__ void potential_pair2(u64 xv, u64 yv, u64 zv, u64 nv, 
 // Bound and layout are the force kernel's: ex2 and sqrt on the special-function
 // unit (10.6 pairs per clock per SM), 12 FP32 lane operations a pair with
 // gradients, 8 without; packed pairs, broadcast tiles, Kahan sums across tiles.
-// Forward and adjoint at 50,000 x 50,000: 3.6 ms as two general-p passes and a
-// float64 combine, 2.3 ms as this one pass.
+// Value and gradients at 50,000 x 50,000, p = 2: this pass 1.1 ms, the whole call
+// through autograd 1.38 ms (3.6 ms as two general-p passes and a float64 combine;
+// 2.3 ms with this pass run twice, in forward and again in backward).
 constexpr int POT_TPB = 128;
 
 template <int P, int PM, bool GRAD>
@@ -351,7 +352,7 @@ __global__ void __launch_bounds__(RED_THREADS) column_sum13_kernel(const double*
 // independent chains hide the special-function latency), the reference range
 // split over grid.y so that a small template still fills the GPU, and the
 // tile sums added across tiles with Kahan compensation.  Measured on GB300 at
-// 10,007 x 9,001, p = 2: 91 us a call (5.2 ms with one scalar thread per
+// 10,007 x 9,001, p = 2: 88 us a call (5.2 ms with one scalar thread per
 // template point, no split, and exp2f, log2f and a division per pair); the
 // error against float64 went from 2.5e-7 to 1.4e-7.
 constexpr int VJP_TPB = 128;
@@ -525,8 +526,8 @@ __global__ void __launch_bounds__(VJP_TPB)
 // waves of the four to five that are resident), at least one tile each, and at
 // most 4 / nc times the force pass's splits by its own rule (force_splits), which
 // keeps a block's run of tiles long enough to pay for its start (10,007 x 9,001,
-// p = 2: 10 splits of 4 tiles 88 us, 20 splits of 2 tiles 107 us).  With few
-// blocks even so, one template point per thread instead of two.  From the sizes
+// p = 2: 8 splits of 5 tiles, 1 point a thread 88 us; 20 of 2 tiles, 2 points 107
+// us).  With few blocks even so, one template point per thread instead of two.  From the sizes
 // alone, so that the same call gives the same bits whatever the context has held
 // before and whatever knobs shape the force pass.
 VjpPlan plan_vjp(int64_t m, int64_t npad, double p, int num_sms, int force_splits) {
